@@ -96,3 +96,23 @@ def test_training_lowers_the_loss():
         mlp_adam(W32, W, gW, Mw, Vw, B, gb, Mb, Vb, t, 3e-3)
     last = float(mlp_loss_grad(X, YP, YL, W, B)[0])
     assert last < 0.35 * first, (first, last)
+
+
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 1217, 4863, 4864, 4897, 32768, 32769])
+def test_tiles_of_rows_match_oracle(rows):
+    """Partly filled tiles, one tile and several tiles per block, both tile heights, and both ways
+    the labels are counted.  Every sum has at most 64 FP32 terms per layer and `rows` terms in
+    random order per weight: 64 * 4 * 2^-24 plus sqrt(rows) 2^-24 stays below 1e-4 of the norm."""
+    from paper_1201_5430_gb300.api import mlp_forward, mlp_loss_grad
+    w, b = _params(8)
+    x, yp, yl = _batch(rows, rows)
+    W, B = _dev(w, b)
+    cuda = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    z = mlp_forward(cuda(x), W, B).cpu().numpy()
+    want = mlp.forward(x, w, b)
+    assert np.abs(z - want).max() <= 1e-5 * (np.abs(want).max() + 1.0)
+    loss, gW, gb = mlp_loss_grad(cuda(x), cuda(yp), cuda(yl), W, B)
+    l0, gw0, gb0 = mlp.loss_and_grad(x, yp, yl, w, b)
+    assert abs(float(loss) - l0) <= 1e-5 * abs(l0)
+    assert np.linalg.norm(gW.cpu().numpy() - gw0) <= 1e-4 * np.linalg.norm(gw0)
+    assert np.linalg.norm(gb.cpu().numpy() - gb0) <= 1e-4 * np.linalg.norm(gb0)
