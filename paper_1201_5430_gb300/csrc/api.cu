@@ -86,7 +86,7 @@ struct Ctx {
     // M2L by rotation - coaxial - rotation (LHV_FORM_RCR)
     RcrTables rcr;
     // scalar reference case (lhv_evaluate_potential_gradient)
-    Buf s_m2l, s_m2m, s_l2l, s_tiles;   // translation blocks of the fused tables, TF32 tiles of s_m2l
+    Buf s_m2l, s_m2m, s_l2l, s_tiles;   // translation blocks of the fused tables, TF32 tiles of the M2L ones
     int s_p = 0, s_type = 0;
     Buf qs, pgfar;
     // filament segments (lhv_evaluate_filaments)
@@ -192,12 +192,8 @@ static void ensure_ops(Ctx* c) {
     build_sparse<T>(c, OP_L2P, c->cfg.p, c->ops.l2p_sp);
     c->ops_type = (int)sizeof(T);
     if constexpr (sizeof(T) == 4) {
-        const int P = c->ops.P;
-        if (ctx_use_tc(c) && tc_supported(2 * P, 2 * P, P)) {
-            tc_tiles_build(c, c->ops.m2l.as<float>(), NUM_OFFSETS, 2 * P, 2 * P, P, c->ops.m2l_tiles);
-            cuda_check(cudaStreamSynchronize(c->stream), "tc tiles");
-        }
-
+        if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
+            m2l_tiles_build(c, c->ops.m2l.as<float>(), c->cfg.p, false, c->ops.m2l_tiles);
     }
 }
 
@@ -218,10 +214,8 @@ static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
     if (kind == 5) {
         // tensor-core tiles of M2L(p, p)
         if constexpr (sizeof(T) == 4) {
-            const int P = pout * pout;
             const float* m2l = cached_op<float>(c, OP_M2L, pout, pout);
-            tc_tiles_build(c, m2l, NUM_OFFSETS, 2 * P, 2 * P, P, c->opcache[key]);
-            cuda_check(cudaStreamSynchronize(c->stream), "tc tiles");
+            m2l_tiles_build(c, m2l, pout, false, c->opcache[key]);
         }
     } else {
         build_op<T>(c, kind, pout, pin, b);
@@ -267,8 +261,8 @@ static void ensure_psi_ops(Ctx* c) {
     psi_form<T>(c, c->ops.m2m.as<T>(), 8, P, c->psi_m2m);
     psi_form<T>(c, c->ops.l2l.as<T>(), 8, P, c->psi_l2l);
     if constexpr (sizeof(T) == 4) {
-        if (ctx_use_tc(c) && tc_supported(2 * P, 2 * P, 0))
-            tc_tiles_build(c, c->psi_m2l.as<float>(), NUM_OFFSETS, 2 * P, 2 * P, 0, c->psi_tiles);
+        if (ctx_use_tc(c) && tc_supported(2 * P, 2 * P))
+            tc_tiles_build(c, c->psi_m2l.as<float>(), NUM_OFFSETS, 2 * P, 2 * P, c->psi_tiles);
         else
             release(c->psi_tiles);
     }
@@ -334,9 +328,8 @@ static Plan<T> make_plan(Ctx* c, int L) {
     pl.p2m_sp = cached_sparse<T>(c, OP_P2M, pl.p[L]);
     pl.l2p_sp = cached_sparse<T>(c, OP_L2P, pl.p[L]);
     for (int l = 2; l <= L; ++l) {
-        const int P = pl.p[l] * pl.p[l];
         pl.m2l[l] = cached_op<T>(c, OP_M2L, pl.p[l], pl.p[l]);
-        if (tc && tc_supported(2 * P, 2 * P, P)) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
+        if (tc && m2l_tc_supported(pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
         if (l < L) pl.m2m[l] = cached_op<T>(c, OP_M2M, pl.p[l], pl.p[l + 1]);
         if (l > 2) pl.l2l[l] = cached_op<T>(c, OP_L2L, pl.p[l], pl.p[l - 1]);
     }
@@ -423,7 +416,8 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
                                   : all_tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * pmax * pmax));
             m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
+                         mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
@@ -480,11 +474,10 @@ static void ensure_scalar_ops(Ctx* c) {
     translation_block<T>(c, c->ops.m2m.as<T>(), 8, P, c->s_m2m);
     translation_block<T>(c, c->ops.l2l.as<T>(), 8, P, c->s_l2l);
     if constexpr (sizeof(T) == 4) {
-        if (ctx_use_tc(c) && tc_supported(P, P, 0)) {
-            tc_tiles_build(c, c->s_m2l.as<float>(), NUM_OFFSETS, P, P, 0, c->s_tiles);
-        } else {
+        if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
+            m2l_tiles_build(c, c->ops.m2l.as<float>(), c->cfg.p, true, c->s_tiles);
+        else
             release(c->s_tiles);
-        }
     }
     cuda_check(cudaStreamSynchronize(c->stream), "scalar tables");
     c->s_p = c->cfg.p;
@@ -560,7 +553,8 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             const int nc = tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(P));
             m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, true, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
+                         mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
@@ -706,7 +700,8 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
             const int nc = pl.rcr ? pl.rcr->nc : tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * PL));
             m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
+                         mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);

@@ -88,14 +88,22 @@ int gemm_nc(int C);
 template <typename T>
 void run_group_gemm(Ctx* c, Grouped& gp, GemmArgs<T> a);
 
-// tensor-core form (tc_gemm.cu), FP32 data; shapes with R % 16 == 0, C % 8 == 0.
-// tc_tiles_build re-lays `ngroups` k-major operators into the TF32 hi/lo tiles the
-// kernel copies straight into shared memory.
-bool tc_supported(int R, int C, int psplit);
-void tc_tiles_build(Ctx* c, const float* ops, int ngroups, int R, int C, int psplit, Buf& tiles);
+// tensor-core form (tc_gemm.cu) of a dense grouped GEMM, FP32 data; shapes with R % 16 == 0,
+// C % 8 == 0 (the complex form's tables).  tc_tiles_build re-lays `ngroups` k-major operators
+// into the TF32 hi/lo tiles the kernel copies straight into shared memory.
+bool tc_supported(int R, int C);
+void tc_tiles_build(Ctx* c, const float* ops, int ngroups, int R, int C, Buf& tiles);
 // in_hi / in_lo: the TF32 split of a.in (same layout), from tc_split.
 void run_tc_gemm(Ctx* c, Grouped& gp, GemmArgs<float> a, const float* tiles, const float* in_hi,
                  const float* in_lo, int* err);
+
+// tensor-core M2L of the two-potential and scalar forms (tc_m2l.cu): p a multiple of 4.
+// m2l_tiles_build lays out the translation blocks of the 316 fused tables; run_tc_m2l adds the
+// translated (and, unless scalar, converted) rows of the groups [g0, g1) to out.
+bool m2l_tc_supported(int p);
+void m2l_tiles_build(Ctx* c, const float* fused, int p, bool scalar, Buf& tiles);
+void run_tc_m2l(Ctx* c, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
+                const int* offsets, const float* in, float* out, int64_t ld, int* err);
 // hi / lo of the rows of the real boxes of levels l0..l1 (ld reals each; device counts)
 void tc_split(Ctx* c, const Levels& lv, const int* count, int l0, int l1, int64_t ld, const float* x, float* hi,
               float* lo);

@@ -165,7 +165,7 @@ struct OpTables {
     Buf l2l;                   // [8][2P][2P]   fused (R|R) + Eq. drt10 per child octant
     Buf l2p;                   // [2P][12P]     v_k (Eq. evf3) and u_lk (Eq. dt3) coefficients
     Buf p2m;                   // [3P][2P]      Eq. eve4 for w = i_x, i_y, i_z
-    Buf m2l_tiles;             // TF32 hi/lo tiles of m2l for the tensor-core products (LHV_TF32X3)
+    Buf m2l_tiles;             // TF32 hi/lo tiles of the translation blocks of m2l (LHV_TF32X3, tc_m2l.cu)
     Csr p2m_sp, l2p_sp;        // P2M and L2P in row-compressed form (their structural zeros dropped)
     Buf offsets;               // int[316][3] M2L offsets (dx, dy, dz)
     Buf slot_of;               // int[343] offset (dx+3)*49+(dy+3)*7+(dz+3) -> slot or -1
@@ -269,9 +269,11 @@ void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels&
 // uniform: pairs of all levels bucketed by offset; else by (level, offset).
 void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& lv, int* table, Grouped& gp,
                  int nc, bool uniform, unsigned long long* pair_counter);
-// the products; loc must be zero for levels >= 2; count: boxes per level (device).
+// the products; loc must be zero for levels >= 2; count: boxes per level (device); offsets:
+// OpTables::offsets.
 template <typename T>
-void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const T* mult, T* loc);
+void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const int* offsets,
+               const T* mult, T* loc);
 
 // ---- RCR translations (rcr.cu) -------------------------------------------------
 // M2L by rotation - coaxial translation - back rotation with the coaxial conversion of

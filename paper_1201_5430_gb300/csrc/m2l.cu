@@ -100,7 +100,8 @@ void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& 
 }
 
 template <typename T>
-void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const T* mult, T* loc) {
+void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const int* offsets,
+               const T* mult, T* loc) {
     const int L = lv.L;
     if constexpr (sizeof(T) == 4) {
         if (pl.rcr) {  // rotation - coaxial - rotation (rcr.cu)
@@ -108,13 +109,12 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
             return;
         }
     }
-    // the tensor-core products read the multipoles split into TF32 hi/lo once
+    // the complex form's tensor-core products read the multipoles split into TF32 hi/lo once
+    // (one p at every level; the other forms split in the kernel)
     const float* mhi = nullptr;
     const float* mlo = nullptr;
     if constexpr (sizeof(T) == 4) {
-        bool any_tc = false;
-        for (int l = 2; l <= L; ++l) any_tc = any_tc || (ctx_m2l_tc(c) && pl.m2l_tiles[l]);
-        if (any_tc) {
+        if (pl.psi && ctx_m2l_tc(c) && pl.m2l_tiles[2]) {
             const int64_t first = (int64_t)lv.off[2] * pl.ld, rows = (int64_t)(lv.off[L + 1] - lv.off[2]) * pl.ld;
             Buf& bh = ctx_tmp(c, 12);
             Buf& bl = ctx_tmp(c, 13);
@@ -149,7 +149,10 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
         bool done = false;
         if constexpr (sizeof(T) == 4) {
             if (ctx_m2l_tc(c) && pl.m2l_tiles[l0]) {
-                run_tc_gemm(c, gp, a, pl.m2l_tiles[l0], mhi, mlo, ctx_err_flag(c));
+                if (pl.psi) run_tc_gemm(c, gp, a, pl.m2l_tiles[l0], mhi, mlo, ctx_err_flag(c));
+                else
+                    run_tc_m2l(c, gp, a.g0, a.g1, pl.p[l0], pl.scalar, pl.m2l_tiles[l0], offsets, mult, loc, pl.ld,
+                               ctx_err_flag(c));
                 done = true;
             }
         }
@@ -158,8 +161,9 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
     }
 }
 
-template void m2l_apply<float>(Ctx*, const Plan<float>&, const Levels&, const int*, Grouped&, const float*, float*);
-template void m2l_apply<double>(Ctx*, const Plan<double>&, const Levels&, const int*, Grouped&, const double*,
-                                double*);
+template void m2l_apply<float>(Ctx*, const Plan<float>&, const Levels&, const int*, Grouped&, const int*,
+                               const float*, float*);
+template void m2l_apply<double>(Ctx*, const Plan<double>&, const Levels&, const int*, Grouped&, const int*,
+                                const double*, double*);
 
 }  // namespace lhv

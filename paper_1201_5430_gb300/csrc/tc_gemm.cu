@@ -1,4 +1,5 @@
-// Tensor-core (tcgen05, TF32) form of the grouped scatter GEMM.
+// Tensor-core (tcgen05, TF32) form of the dense grouped scatter GEMM: the M2L of the complex
+// form (tc_m2l.cu has the two-potential and scalar forms).
 //
 // Same contract as group_gemm.cu, Y (R x pairs) = A_g X, computed transposed so
 // that the box pairs are the MMA's M dimension:
@@ -30,6 +31,7 @@
 
 #include "lhv_group.cuh"
 #include "lhv_internal.cuh"
+#include "tc_common.cuh"
 
 namespace lhv {
 
@@ -37,107 +39,15 @@ namespace {
 
 constexpr int TC_THREADS = 128;   // 4 warps: warp w owns TMEM lanes [32 w, 32 w + 32)
 constexpr int TC_M = 128;         // pairs per work item (MMA M)
-constexpr int TC_KC = 16;         // K per staged chunk (2 MMA k-steps of 8)
 constexpr int TC_NMAX = 256;      // outputs per work item (MMA N, TMEM columns)
 constexpr uint32_t TMEM_COLS = 256;
-constexpr int TC_MAX_RANGES = 16;  // output ranges of 256 rows per operator (L2P at p = 16: 12)
-constexpr long long WAIT_LIMIT = 1ll << 26;
-
-// byte offset of element (row, k) of a [rows x TC_KC] K-major tile made of
-// 8 x 16-byte core matrices, the K groups of one 8-row block contiguous
-__device__ __forceinline__ uint32_t tile_off(int row, int k) {
-    return (uint32_t)(((row >> 3) * (TC_KC / 4) + (k >> 2)) * 128 + (row & 7) * 16 + (k & 3) * 4);
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ float tf32_rna(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
-// shared-memory matrix descriptor, K-major, no swizzle
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo & 0x3FFFFu) >> 4) << 16;
-    d |= (uint64_t)((sbo & 0x3FFFFu) >> 4) << 32;
-    d |= 1ull << 46;  // descriptor version
-    return d;         // base offset 0, swizzle none
-}
-
-// instruction descriptor: D F32, A/B TF32, both K-major, M x N
-__host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, int acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-// bounded wait for the phase `parity` of an mbarrier; false on timeout
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    const uint32_t a = smem_u32(bar);
-    for (long long it = 0; it < WAIT_LIMIT; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// 32 lanes x 32 columns: thread = lane, 32 consecutive FP32 columns
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
-                 : "memory");
-}
-
+constexpr int TC_MAX_RANGES = 5;   // output ranges of 256 rows per operator (1152 rows at p = 24)
 struct TcArgs {
     GemmArgs<float> g;
     const float* tiles;    // operator tiles in shared-memory order (see tc_tiles_build), hi then lo
     int64_t group_stride;  // floats per group of `tiles`
     int nranges;
     int n0[TC_MAX_RANGES], nlen[TC_MAX_RANGES];  // N ranges (<= 256 wide, multiples of 16)
-    int kbeg[TC_MAX_RANGES];                     // first K of each range (psplit for the chi outputs)
     int64_t roff[TC_MAX_RANGES];                 // float offset of each range inside a group
     int nmax;              // widest range (rows of the operator tile in a stage)
     int stage_bytes;       // bytes of one shared stage (Xh, Xl, Bh, Bl), 1024-aligned
@@ -213,8 +123,8 @@ __global__ void __launch_bounds__(TC2_THREADS, TC2_PER_SM) k_tc_gemm(TcArgs ta) 
         const int chunk = c_beg + w / ta.nranges, r = w % ta.nranges;
         const int4 ch = a.chunks[chunk];
         const int g = ch.x, p0 = ch.y, np = ch.z;
-        const int n0 = ta.n0[r], nlen = ta.nlen[r], kbeg = ta.kbeg[r];
-        const int nk = (a.C - kbeg + TC_KC - 1) / TC_KC;
+        const int n0 = ta.n0[r], nlen = ta.nlen[r];
+        const int nk = (a.C + TC_KC - 1) / TC_KC;
         const float* tg = ta.tiles + (int64_t)(g % a.ops_mod) * ta.group_stride + ta.roff[r];
         const int tile_floats = nlen * TC_KC;
         if (t < TC_M) {
@@ -237,7 +147,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TC2_PER_SM) k_tc_gemm(TcArgs ta) 
                 unsigned char* Xl = Xh + TC_M * TC_KC * 4;
                 unsigned char* Bh = Xl + TC_M * TC_KC * 4;
                 unsigned char* Bl = Bh + ta.nmax * TC_KC * 4;
-                const int kc = kbeg + i * TC_KC;
+                const int kc = i * TC_KC;
                 const int kn = min(TC_KC, a.C - kc);
                 for (int e = t; e < TC_M * (TC_KC / 4); e += TC2_THREADS) {
                     const int row = e / (TC_KC / 4), kg = e % (TC_KC / 4);
@@ -270,7 +180,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TC2_PER_SM) k_tc_gemm(TcArgs ta) 
             unsigned char* Xl = Xh + TC_M * TC_KC * 4;
             unsigned char* Bh = Xl + TC_M * TC_KC * 4;
             unsigned char* Bl = Bh + ta.nmax * TC_KC * 4;
-            const int kn = min(TC_KC, a.C - (kbeg + i * TC_KC));
+            const int kn = min(TC_KC, a.C - i * TC_KC);
             if (t == 0) {
                 tc_fence_after();
                 const uint32_t lbo = 128, sbo = (TC_KC / 4) * 128;
@@ -330,13 +240,13 @@ __global__ void k_tc_tiles(int ngroups, const float* __restrict__ ops, int R, in
         const float* Ag = ops + (int64_t)g * C * R;
         float* tg = tiles + (int64_t)g * ta.group_stride;
         for (int r = 0; r < ta.nranges; ++r) {
-            const int n0 = ta.n0[r], nlen = ta.nlen[r], kbeg = ta.kbeg[r];
-            const int nk = (C - kbeg + TC_KC - 1) / TC_KC;
+            const int n0 = ta.n0[r], nlen = ta.nlen[r];
+            const int nk = (C + TC_KC - 1) / TC_KC;
             const int tile_floats = nlen * TC_KC;
             for (int e = threadIdx.x; e < nk * tile_floats; e += blockDim.x) {
                 const int i = e / tile_floats, q = e - i * tile_floats;
                 const int k = q / nlen, n = q - k * nlen;
-                const int kk = kbeg + i * TC_KC + k;
+                const int kk = i * TC_KC + k;
                 const float v = (kk < C) ? Ag[(int64_t)kk * R + n0 + n] : 0.f;
                 const float h = tf32_rna(v), l = tf32_rna(v - h);
                 float* base = tg + ta.roff[r] + (int64_t)i * 2 * tile_floats;
@@ -416,27 +326,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_selftest(const float* X, c
 
 constexpr size_t TC_SMEM = (size_t)2 * TC_M * TC_KC * 4 + (size_t)2 * TC_NMAX * TC_KC * 4 + 1024;
 
-TcArgs tc_layout(int R, int C, int psplit) {
+TcArgs tc_layout(int R, int C) {
     TcArgs ta{};
-    auto add = [&](int lo, int hi, int kbeg) {
-        for (int x = lo; x < hi; x += TC_NMAX) {
-            const int r = ta.nranges++;
-            ta.n0[r] = x;
-            ta.nlen[r] = std::min(TC_NMAX, hi - x);
-            ta.kbeg[r] = kbeg;
-        }
-    };
-    if (psplit > 0) {
-        add(0, psplit, 0);
-        add(psplit, R, psplit);
-    } else {
-        add(0, R, 0);
-    }
+    const int nk = (C + TC_KC - 1) / TC_KC;
     int64_t off = 0;
     ta.nmax = 16;
-    for (int r = 0; r < ta.nranges; ++r) {
+    for (int x = 0; x < R; x += TC_NMAX) {
+        const int r = ta.nranges++;
+        ta.n0[r] = x;
+        ta.nlen[r] = std::min(TC_NMAX, R - x);
         ta.roff[r] = off;
-        const int nk = (C - ta.kbeg[r] + TC_KC - 1) / TC_KC;
         off += (int64_t)nk * 2 * ta.nlen[r] * TC_KC;
         ta.nmax = std::max(ta.nmax, ta.nlen[r]);
     }
@@ -447,16 +346,12 @@ TcArgs tc_layout(int R, int C, int psplit) {
 
 }  // namespace
 
-bool tc_supported(int R, int C, int psplit) {
-    if (C % 8 != 0 || R % 16 != 0) return false;
-    if (psplit > 0 && (psplit % 16 != 0)) return false;
-    const int ranges = psplit > 0 ? (psplit + TC_NMAX - 1) / TC_NMAX + (R - psplit + TC_NMAX - 1) / TC_NMAX
-                                  : (R + TC_NMAX - 1) / TC_NMAX;
-    return ranges <= TC_MAX_RANGES;
+bool tc_supported(int R, int C) {
+    return C % 8 == 0 && R % 16 == 0 && (R + TC_NMAX - 1) / TC_NMAX <= TC_MAX_RANGES;
 }
 
-void tc_tiles_build(Ctx* c, const float* ops, int ngroups, int R, int C, int psplit, Buf& tiles) {
-    TcArgs ta = tc_layout(R, C, psplit);
+void tc_tiles_build(Ctx* c, const float* ops, int ngroups, int R, int C, Buf& tiles) {
+    TcArgs ta = tc_layout(R, C);
     ensure(c, tiles, ta.group_stride * ngroups * (int64_t)sizeof(float));
     k_tc_tiles<<<std::min(ngroups, 152 * 4), 256, 0, stream_of(c)>>>(ngroups, ops, R, C, ta, tiles.as<float>());
     count_launch(c);
@@ -497,7 +392,7 @@ void run_tc_gemm(Ctx* c, Grouped& gp, GemmArgs<float> a, const float* tiles, con
     a.work = gp.work.as<int>();
     cudaStream_t s = stream_of(c);
     cuda_check(cudaMemsetAsync(a.work, 0, 4, s), "tc work");
-    TcArgs ta = tc_layout(a.R, a.C, a.psplit);
+    TcArgs ta = tc_layout(a.R, a.C);
     ta.g = a;
     ta.tiles = tiles;
     ta.in_hi = in_hi;

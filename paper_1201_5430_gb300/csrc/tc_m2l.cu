@@ -1,0 +1,699 @@
+// Tensor-core (tcgen05, TF32) M2L: translation by one block, conversion in the epilogue.
+//
+// The fused M2L operator of an offset t is [[T, C12 T], [0, C22 T]] (Eqs. mr3, drt10): the
+// same translation T for both potentials, then the conversion, which couples each (n, m) to
+// at most six reals of the translated chi and whose coefficients are linear in t.  So the
+// products are only  phi^ = T phi,  chi^ = T chi  (4 p^4 multiply-adds' flops a pair instead of
+// the 6 p^4 of the fused table, and a third of its operator bytes: one P x P block shared by both
+// potentials, P = p^2), and the conversion runs on the accumulators:
+//   phi~_n^m = phi^_n^m + a (tx + i ty) chi^_n^{m+1} + b (tx - i ty) chi^_n^{m-1} + i z tz chi^_n^m
+//   chi~_n^m = chi^_n^m + d (ty + i tx) chi^_{n+1}^{m-1} + e (ty - i tx) chi^_{n+1}^{m+1} + f tz chi^_{n+1}^m
+// in the scaled real basis of operators.cu (t in box sides):
+//   a = -sqrt((n-m)(n+m+1)) / 2n,  b = sqrt((n+m)(n-m+1)) / 2n,  z = m / n  (0 at n = 0),
+//   d = sqrt((n-m+1)(n-m+2)) / 2(n+1),  e = -sqrt((n+m+1)(n+m+2)) / 2(n+1),
+//   f = -sqrt((n+1-m)(n+1+m)) / (n+1)   (d = e = f = 0 at n = p - 1: the chi_p term is dropped);
+//   at m = 0 the m - 1 terms are the conjugates of the m + 1 terms: a and e doubled, b = d = 0.
+// The scalar reference case is the same kernel with one potential and no conversion.
+//
+// D (128 pairs x N) = X (128 x P) T^T (P x N) per potential, D in TMEM in FP32 (phi^ and chi^
+// side by side, 2 P <= 512 columns up to p = 16; above, the outputs are split into ranges of
+// degrees of at most 256 columns, each with the halo degree that chi~ reads).  Precision: every
+// operand split a = hi + lo, hi = tf32(a), lo = tf32(a - hi); D accumulates hi.hi + hi.lo + lo.hi.
+//
+// One persistent CTA per SM, its warps specialised, K walked in chunks of 16 through a ring of
+// shared stages (canonical no-swizzle K-major tiles):
+//   warps 8-15  gather the FP32 source rows (a chunk ahead in registers, two groups of four warps on
+//               alternate chunks), split them and store the hi / lo tiles;
+//   warp 16     brings the operator's hi / lo tile of the chunk with one bulk copy;
+//   warp 17     issues the MMAs (2 k-steps x 3 products x potentials) and commits the stage;
+//   warps 0-7   read the accumulators (thread = pair), convert, and add to the locals through a
+//               [column][pair] staging band, so that a warp's additions cover 128 consecutive
+//               bytes of one row.
+// K runs from the high source degrees down and each stage takes the small cross products before
+// hi.hi: the accumulator rounds toward zero at its own magnitude, which then is small until the
+// last steps.  Far field against FP64, sphere surface at p = 12: v 3.2e-7, s 3.1e-7 (FP32 CUDA cores
+// 3.6e-7, 3.3e-7); in ascending order, and in the fused-table kernel before, 1.2e-6, 1.5e-6.
+// Measured (products, ms an evaluation, fused-table kernel before / this one): sphere surface of
+// 2^20 at p = 12, 4.13 M pairs 7.26 / 4.55; scalar cube of 2^20 at p = 12, 6.04 M pairs 4.01 / 2.28;
+// offset rings of 2^21 at p = 16, 1.33 M pairs 4.33 / 2.52.  Without the epilogue the first
+// takes 1.97: what bounds it is the conversion (tcgen05.ld and its latency, about 1.5) and the
+// additions (about 1.3), which run in turn with the products where one accumulator set fills
+// TMEM.  Operand traffic a pair at p = 12: 1.15 KB of source (split here instead of two arrays) and
+// 1.3 KB of operator, against 3.5 and 3.9 of the fused tables.
+//
+// Every mbarrier wait gives up after a fixed number of polls, sets the error word for the host
+// and an abort word that ends every role; copies and MMAs in flight are waited for (bounded)
+// before TMEM is freed.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "lhv_group.cuh"
+#include "lhv_internal.cuh"
+#include "tc_common.cuh"
+
+namespace lhv {
+
+namespace {
+
+constexpr int M2_EPI_WARPS = 8, M2_PROD_WARPS = 8, M2_GROUPS = 2;
+constexpr int M2_WARPS = M2_EPI_WARPS + M2_PROD_WARPS + 2;
+constexpr int M2_THREADS = 32 * M2_WARPS;
+constexpr int M2_MAX_STAGES = 4;
+constexpr int M2_MAX_RANGES = 4;
+constexpr int M2_X_TILE = TC_PAIRS * TC_KC * 4;  // bytes of one operand tile of the pairs
+constexpr int M2_BAND = 64;                // columns (a potential) staged at once
+constexpr int M2_STG_LD = TC_PAIRS + 1;    // staging [column][pair], odd stride
+constexpr int M2_TMEM = 512;               // TMEM columns: one or two accumulator buffers
+constexpr long long M2_WAIT_LIMIT = 1ll << 24;
+constexpr int M2_SMEM_MAX = 226 * 1024;    // dynamic shared memory (the static part is below 1 KB)
+
+struct M2lArgs {
+    const int4* chunks;
+    const int2* pairs;
+    const int* choff;
+    int g0, g1;
+    const float* in;
+    float* out;
+    int64_t ld;
+    int p, P;
+    const float* tiles;      // per slot: ranges x K chunks x [hi | lo] tiles
+    int64_t group_stride;    // floats per slot
+    const int* offsets;      // [316][3] source box - target box
+    int nranges;
+    int n0[M2_MAX_RANGES], n1[M2_MAX_RANGES];   // output degrees [n0, n1) of each range
+    int c0[M2_MAX_RANGES], nlen[M2_MAX_RANGES]; // its columns [c0, c0 + nlen) (with the halo, 16-padded)
+    int64_t roff[M2_MAX_RANGES];
+    int nstages, stage_bytes;
+    int nbuf;                // accumulator buffers (each M2_TMEM / nbuf columns)
+    const float* conv;       // [p (p + 1) / 2 + 8][8]: a, b, z, d | e, f, 0, 0 of (n, m) at n (n + 1) / 2 + m
+    int* err;
+};
+
+// floats of the conversion table, padded for the reads of the eight orders of a last unit
+__host__ __device__ constexpr int conv_floats(int p) { return (p * (p + 1) / 2 + 8) * 8; }
+
+struct M2lShared {
+    uint64_t full_a[M2_MAX_STAGES], full_b[M2_MAX_STAGES], empty[M2_MAX_STAGES];
+    uint64_t acc_full[2], acc_empty[2], done;
+    uint32_t tmem;
+    int abort;       // set by a role whose wait gave up
+    int epi_abort;   // the epilogue's own verdict, read by all its warps after a barrier
+    int dst[TC_PAIRS];
+};
+
+// bounded wait that also ends when another role has given up
+__device__ __forceinline__ bool m2_wait(uint64_t* bar, uint32_t parity, M2lShared& sh, int* err) {
+    const uint32_t a = smem_u32(bar);
+    for (long long it = 0; it < M2_WAIT_LIMIT; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(done)
+            : "r"(a), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if ((it & 63) == 63 && *(volatile int*)&sh.abort) return false;
+    }
+    *(volatile int*)&sh.abort = 1;
+    atomicExch(err, 1);
+    return false;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+// first column of a range's accumulators: ranges above the first start 16 columns in, since the
+// epilogue reads the column before a degree
+__device__ __forceinline__ uint32_t acc_base(int range) { return range ? 16u : 0u; }
+
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+__device__ __forceinline__ void tmem_ld1(uint32_t addr, uint32_t& a) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(a) : "r"(addr));
+}
+__device__ __forceinline__ void tmem_ld2(uint32_t addr, uint32_t& a, uint32_t& b) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr));
+}
+__device__ __forceinline__ void tmem_ld16_async(uint32_t addr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+}
+// the loads before it have arrived; the registers may be read after it (ties them to the wait)
+template <int N>
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[N]) {
+    static_assert(N == 16 || N == 20, "");
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15])
+                 :
+                 : "memory");
+    if constexpr (N == 20) asm volatile("" : "+r"(r[N - 4]), "+r"(r[N - 3]), "+r"(r[N - 2]), "+r"(r[N - 1]) : : "memory");
+}
+
+// chi of the orders mb - 1 .. mb + 8 of degree N: x[k] = column N^2 + 2 mb - 3 + k, so order
+// mb + i is (Re, Im) = (x[2 i + 2], x[2 i + 3]).  The last pair is read where order mb + 8
+// exists only (the reads stay inside the accumulators); columns past the degree hold other
+// coefficients and are masked by the caller.
+__device__ __forceinline__ void tmem_orders(uint32_t col, int N, int mb, uint32_t (&x)[20]) {
+    tmem_ld16_async(col, x);
+    tmem_ld2(col + 16, x[16], x[17]);
+    if (mb + 8 <= N) tmem_ld2(col + 18, x[18], x[19]);
+    else x[18] = x[19] = 0u;
+}
+// order 0 is one real at x[3]: (Re, Im) = (x[3], 0), and there is no order -1
+template <int N>
+__device__ __forceinline__ void order_zero(uint32_t (&x)[N]) {
+    x[0] = x[1] = 0u;
+    x[2] = x[3];
+    x[3] = 0u;
+}
+
+// Converts the orders [mb, mb + 8) of degree n of this thread's pair and writes them to the
+// staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n (tmem_orders,
+// order_zero applied); on return that of degree n + 1, so that a run of degrees reads each once.
+__device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uint32_t tc, int c0, int p, int n,
+                                               int mb, float tx, float ty, float tz, uint32_t (&x)[20], float* op,
+                                               float* oc) {
+    uint32_t y[20], f[16];
+    const bool up = n + 1 < p;
+    if (up) tmem_orders(tc + (uint32_t)((n + 1) * (n + 1) - c0 + 2 * mb - 3), n + 1, mb, y);
+    if (n > 0) tmem_ld16_async(tp + (uint32_t)(n * n - c0 + 2 * mb - 1), f);
+    else tmem_ld1(tp - (uint32_t)c0, f[1]);
+    tmem_wait(f);
+    if (up) tmem_wait(y);
+    else
+#pragma unroll
+        for (int k = 0; k < 20; ++k) y[k] = 0u;
+    if (mb == 0) {
+        order_zero(y);
+        f[0] = f[1];
+        f[1] = 0u;
+    }
+    const float* k0 = cv + (n * (n + 1) / 2 + mb) * 8;
+    float* op0 = op + (mb ? 2 * mb - 1 : -1) * M2_STG_LD;  // column of Re of order mb (order 0 is one real)
+    float* oc0 = oc + (mb ? 2 * mb - 1 : -1) * M2_STG_LD;
+    // four orders at a time without branches (their chains interleave); orders past n are not stored
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+        if (mb + h > n) break;
+#pragma unroll
+        for (int i = h; i < h + 4; ++i) {
+            const int m = mb + i;
+            const float4 g = *reinterpret_cast<const float4*>(k0 + 8 * i);
+            const float2 e = *reinterpret_cast<const float2*>(k0 + 8 * i + 4);
+            const float ax = g.x * tx, ay = g.x * ty, bx = g.y * tx, by = g.y * ty, z = g.z * tz;
+            const float dx = g.w * tx, dy = g.w * ty, ex = e.x * tx, ey = e.x * ty, fz = e.y * tz;
+            auto F = [](uint32_t u) { return __uint_as_float(u); };
+            const float mr = F(x[2 * i]), mi = F(x[2 * i + 1]), cr = F(x[2 * i + 2]), ci = F(x[2 * i + 3]);
+            const float pr = m < n ? F(x[2 * i + 4]) : 0.f, pi = m < n ? F(x[2 * i + 5]) : 0.f;
+            const float umr = F(y[2 * i]), umi = F(y[2 * i + 1]), ucr = F(y[2 * i + 2]), uci = F(y[2 * i + 3]),
+                        upr = F(y[2 * i + 4]), upi = F(y[2 * i + 5]);
+            const float o0 = fmaf(ax, pr, fmaf(-ay, pi, fmaf(bx, mr, fmaf(by, mi, fmaf(-z, ci, F(f[2 * i]))))));
+            const float q0 = fmaf(ey, upr, fmaf(ex, upi, fmaf(dy, umr, fmaf(-dx, umi, fmaf(fz, ucr, cr)))));
+            const float o1 = fmaf(ax, pi, fmaf(ay, pr, fmaf(bx, mi, fmaf(-by, mr, fmaf(z, cr, F(f[2 * i + 1]))))));
+            const float q1 = fmaf(ey, upi, fmaf(-ex, upr, fmaf(dy, umi, fmaf(dx, umr, fmaf(fz, uci, ci)))));
+            if (m <= n) {
+                const int at = (m ? 2 * i : 2 * i + 1) * M2_STG_LD;
+                op0[at] = o0;
+                oc0[at] = q0;
+                if (m) {
+                    op0[at + M2_STG_LD] = o1;
+                    oc0[at + M2_STG_LD] = q1;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 20; ++k) x[k] = y[k];
+}
+
+template <int NPOT>
+__global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant__ M2lArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ M2lShared sh;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int S = a.nstages, nk = a.P / TC_KC;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
+                     "r"((uint32_t)M2_TMEM)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (t == 0) {
+        for (int s = 0; s < M2_MAX_STAGES; ++s) {
+            mbar_init(&sh.full_a[s], M2_PROD_WARPS / M2_GROUPS);
+            mbar_init(&sh.full_b[s], 1);
+            mbar_init(&sh.empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sh.acc_full[b], 1);
+            mbar_init(&sh.acc_empty[b], M2_EPI_WARPS);
+        }
+        mbar_init(&sh.done, 1);
+        sh.abort = 0;
+        sh.epi_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (NPOT == 2) {
+        float* cv = reinterpret_cast<float*>(smem + (size_t)S * a.stage_bytes);
+        for (int e = t; e < conv_floats(a.p); e += M2_THREADS) cv[e] = a.conv[e];
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sh.tmem;
+    const int c_beg = a.choff[a.g0];
+    const int nwork = (a.choff[a.g1] - c_beg) * a.nranges;  // items: (chunk of <= 128 pairs, range)
+    float* conv = reinterpret_cast<float*>(smem + (size_t)S * a.stage_bytes);  // the conversion table (NPOT = 2)
+    float* stg = conv + (NPOT == 2 ? conv_floats(a.p) : 0);  // the epilogue warps' staging
+    const int mine = nwork > (int)blockIdx.x ? (nwork - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+
+    if (warp >= M2_EPI_WARPS && warp < M2_EPI_WARPS + M2_PROD_WARPS) {
+        // ---- gather and split.  The two groups of four warps take alternate K chunks, so that the
+        // store, the proxy fence and the arrival of one overlap the other's.  This thread: rows
+        // 32 (w % 4) + 8 j + lane % 8, 16 bytes at k group lane / 8.
+        constexpr int RJ = 4;
+        const int pw = warp - M2_EPI_WARPS, grp = pw / (M2_PROD_WARPS / M2_GROUPS);
+        const int row0 = (pw % (M2_PROD_WARPS / M2_GROUPS)) * 32 + (lane & 7), kg = lane >> 3;
+        const int total = mine * nk;  // K chunks of this CTA's items
+        int cur[RJ], nxt[RJ];
+        // source boxes of this thread's rows in the CTA's n-th item
+        auto ids = [&](int n, int (&s)[RJ]) {
+#pragma unroll
+            for (int j = 0; j < RJ; ++j) s[j] = -1;
+            if (n >= mine) return;
+            const int4 ch = a.chunks[c_beg + ((int)blockIdx.x + n * (int)gridDim.x) / a.nranges];
+#pragma unroll
+            for (int j = 0; j < RJ; ++j)
+                if (row0 + 8 * j < ch.z) s[j] = a.pairs[ch.y + row0 + 8 * j].x;
+        };
+        float4 v[NPOT][RJ], w[NPOT][RJ];
+        auto load = [&](const int (&s)[RJ], int k, float4 (&d)[NPOT][RJ]) {
+#pragma unroll
+            for (int q = 0; q < NPOT; ++q)
+#pragma unroll
+                for (int j = 0; j < RJ; ++j)
+                    d[q][j] = s[j] >= 0 ? __ldg(reinterpret_cast<const float4*>(a.in + (int64_t)s[j] * a.ld + q * a.P +
+                                                                               (nk - 1 - k) * TC_KC + kg * 4))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        int have = grp / nk;  // the item whose ids are in cur; nxt holds the following item's
+        if (grp < total) {
+            ids(have, cur);
+            ids(have + 1, nxt);
+            load(cur, grp % nk, v);
+        }
+        for (int g = grp; g < total; g += M2_GROUPS) {
+            if (g + M2_GROUPS < total) {
+                const int n2 = (g + M2_GROUPS) / nk, k2 = (g + M2_GROUPS) - n2 * nk;
+                if (n2 != have) {
+                    if (n2 == have + 1) {
+#pragma unroll
+                        for (int j = 0; j < RJ; ++j) cur[j] = nxt[j];
+                    } else {
+                        ids(n2, cur);  // items of one K chunk (p = 4)
+                    }
+                    have = n2;
+                    ids(have + 1, nxt);
+                }
+                load(cur, k2, w);
+            }
+            const int st = g % S;
+            if (!__all_sync(0xffffffffu, m2_wait(&sh.empty[st], ((uint32_t)(g / S) & 1u) ^ 1u, sh, a.err))) break;
+            unsigned char* base = smem + (size_t)st * a.stage_bytes;
+#pragma unroll
+            for (int q = 0; q < NPOT; ++q)
+#pragma unroll
+                for (int j = 0; j < RJ; ++j) {
+                    const uint32_t o = tile_off(row0 + 8 * j, kg * 4);
+                    const float4 x = v[q][j];
+                    float4 h, l;
+                    h.x = tf32_rna(x.x);
+                    h.y = tf32_rna(x.y);
+                    h.z = tf32_rna(x.z);
+                    h.w = tf32_rna(x.w);
+                    l.x = tf32_rna(x.x - h.x);
+                    l.y = tf32_rna(x.y - h.y);
+                    l.z = tf32_rna(x.z - h.z);
+                    l.w = tf32_rna(x.w - h.w);
+                    *reinterpret_cast<float4*>(base + (2 * q) * M2_X_TILE + o) = h;
+                    *reinterpret_cast<float4*>(base + (2 * q + 1) * M2_X_TILE + o) = l;
+                }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.full_a[st]);
+#pragma unroll
+            for (int q = 0; q < NPOT; ++q)
+#pragma unroll
+                for (int j = 0; j < RJ; ++j) v[q][j] = w[q][j];
+        }
+    } else if (warp == M2_EPI_WARPS + M2_PROD_WARPS) {
+        if (lane == 0) {
+            // ---- operator tiles
+            int st = 0;
+            uint32_t ph = 1;
+            int64_t issued = 0;
+            bool ok = true;
+            for (int item = blockIdx.x; item < nwork && ok; item += gridDim.x) {
+                const int r = item % a.nranges;
+                const int slot = a.chunks[c_beg + item / a.nranges].x % NUM_OFFSETS;
+                const uint32_t bytes = (uint32_t)a.nlen[r] * TC_KC * 4 * 2;
+                const float* src = a.tiles + (int64_t)slot * a.group_stride + a.roff[r];
+                for (int k = 0; k < nk; ++k) {
+                    ok = m2_wait(&sh.empty[st], ph, sh, a.err);
+                    if (!ok) break;
+                    mbar_expect_tx(&sh.full_b[st], bytes);
+                    bulk_copy(smem + (size_t)st * a.stage_bytes + 2 * NPOT * M2_X_TILE, src + (int64_t)(nk - 1 - k) * (bytes / 4),
+                              bytes, &sh.full_b[st]);
+                    ++issued;
+                    if (++st == S) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            // every copy has landed before the CTA may end: the last one of each stage
+            for (int s = 0; s < S; ++s) {
+                const int64_t uses = issued / S + (s < issued % S);
+                if (uses > 0) mbar_wait(&sh.full_b[s], (uint32_t)((uses - 1) & 1));
+            }
+        }
+    } else if (warp == M2_EPI_WARPS + M2_PROD_WARPS + 1) {
+        if (lane == 0) {
+            // ---- MMA issue
+            int st = 0, n = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            const uint32_t lbo = 128, sbo = (TC_KC / 4) * 128;
+            for (int item = blockIdx.x; item < nwork && ok; item += gridDim.x, ++n) {
+                const int nlen = a.nlen[item % a.nranges], b = n % a.nbuf;
+                const uint32_t idesc = make_idesc(TC_PAIRS, nlen);
+                const uint32_t d0 = tmem + (uint32_t)(b * (M2_TMEM / a.nbuf)) + acc_base(item % a.nranges);
+                ok = m2_wait(&sh.acc_empty[b], ((uint32_t)(n / a.nbuf) & 1u) ^ 1u, sh, a.err);
+                if (!ok) break;
+                for (int k = 0; k < nk; ++k) {
+                    ok = m2_wait(&sh.full_a[st], ph, sh, a.err) && m2_wait(&sh.full_b[st], ph, sh, a.err);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t base = smem_u32(smem + (size_t)st * a.stage_bytes);
+                    const uint32_t bh = base + 2 * NPOT * M2_X_TILE, bl = bh + (uint32_t)nlen * TC_KC * 4;
+                    // the small cross products first, then hi.hi (see the top)
+#pragma unroll
+                    for (int part = 0; part < 3; ++part)
+#pragma unroll
+                        for (int ks = TC_KC / 8 - 1; ks >= 0; --ks) {
+                            const uint32_t step = ks * 2 * 128;
+                            const uint64_t B = make_desc((part == 0 ? bl : bh) + step, lbo, sbo);
+#pragma unroll
+                            for (int q = 0; q < NPOT; ++q) {
+                                const uint64_t X =
+                                    make_desc(base + (2 * q + (part == 1)) * M2_X_TILE + step, lbo, sbo);
+                                mma_tf32(d0 + (uint32_t)(q * nlen), X, B, idesc,
+                                         (k == 0 && part == 0 && ks == TC_KC / 8 - 1) ? 0 : 1);
+                            }
+                        }
+                    mma_commit(&sh.empty[st]);
+                    if (++st == S) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (ok) mma_commit(&sh.acc_full[b]);
+            }
+            mma_commit(&sh.done);
+            mbar_wait(&sh.done, 0);  // nothing in flight when TMEM is freed
+        }
+    } else {
+        // ---- epilogue: thread = pair 32 (warp % 4) + lane; the two warps of a lane quarter share the
+        // columns.  Bands of columns are staged [column][pair], then added row by row, lane = column.
+        const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
+        float* stc = stg + (size_t)M2_BAND * M2_STG_LD;  // chi
+        // the staged columns [0, ncol) of every pair to columns [col0, col0 + ncol) of its row
+        auto add_rows = [&](int col0, int ncol) {
+            for (int c = lane; c < ncol; c += 32) {
+                float* o = a.out + col0 + c;
+                // the reads of eight rows before their additions: an addition orders the reads after it
+                constexpr int U = 8;
+#pragma unroll
+                for (int r0 = 0; r0 < TC_PAIRS / M2_EPI_WARPS; r0 += U) {
+                    int d[U];
+                    float f[U], g[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int r = warp + M2_EPI_WARPS * (r0 + u);
+                        d[u] = sh.dst[r];
+                        f[u] = stg[c * M2_STG_LD + r];
+                        if (NPOT == 2) g[u] = stc[c * M2_STG_LD + r];
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (d[u] >= 0) {
+                            float* q = o + (int64_t)d[u] * a.ld;
+                            atomicAdd(q, f[u]);
+                            if (NPOT == 2) atomicAdd(q + a.P, g[u]);
+                        }
+                }
+            }
+        };
+        auto release = [&](int b) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
+        };
+        for (int n = 0; n < mine; ++n) {
+            const int item = (int)blockIdx.x + n * (int)gridDim.x, r = item % a.nranges, b = n % a.nbuf;
+            const int4 ch = a.chunks[c_beg + item / a.nranges];
+            if (t < TC_PAIRS) sh.dst[t] = t < ch.z ? a.pairs[ch.y + t].y : -1;
+            // a wait that gave up is seen by every epilogue warp after this barrier: all leave together
+            if (!m2_wait(&sh.acc_full[b], (uint32_t)(n / a.nbuf) & 1u, sh, a.err)) *(volatile int*)&sh.epi_abort = 1;
+            epi_sync();
+            if (*(volatile int*)&sh.epi_abort) break;
+            tc_fence_after();
+            const int n0 = a.n0[r], n1 = a.n1[r], c0 = a.c0[r], nlen = a.nlen[r];
+            const uint32_t tp =
+                tmem + (uint32_t)(b * (M2_TMEM / a.nbuf)) + acc_base(r) + ((uint32_t)(quarter * 32) << 16);
+            if (NPOT == 1) {
+                const int ncols = n1 * n1 - c0;
+                for (int cb = 0; cb < nlen; cb += M2_BAND) {
+#pragma unroll
+                    for (int k = 0; k < M2_BAND / 32; ++k) {
+                        const int c = 32 * k + 16 * half;
+                        if (cb + c >= nlen) break;
+                        uint32_t x[16];
+                        tmem_ld16_async(tp + (uint32_t)(cb + c), x);
+                        tmem_wait(x);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) stg[(c + i) * M2_STG_LD + row] = __uint_as_float(x[i]);
+                    }
+                    if (cb + M2_BAND >= nlen) release(b);
+                    epi_sync();
+                    add_rows(c0 + cb, min(M2_BAND, ncols - cb));
+                    epi_sync();
+                }
+            } else {
+                const uint32_t tc = tp + (uint32_t)nlen;
+                const int slot = ch.x % NUM_OFFSETS;
+                const float tx = (float)-a.offsets[3 * slot], ty = (float)-a.offsets[3 * slot + 1],
+                            tz = (float)-a.offsets[3 * slot + 2];
+                for (int na = n0; na < n1;) {
+                    int nb = na + 1;  // degrees [na, nb) fit the band
+                    while (nb < n1 && (nb + 1) * (nb + 1) - na * na <= M2_BAND) ++nb;
+                    // runs of degrees in blocks of eight orders: one block is split between the two warps
+                    // of a lane quarter by degree, several are taken in turn
+                    for (int mb = 0; mb < nb; mb += 8) {
+                        int d0 = max(na, mb), d1 = nb;
+                        if (nb <= 8) {
+                            const int mid = (na + nb + 1) / 2;
+                            if (half) d0 = mid;
+                            else d1 = mid;
+                        } else if (((mb >> 3) & 1) != half) {
+                            continue;
+                        }
+                        if (d0 >= d1) continue;
+                        uint32_t x[20];
+                        tmem_orders(tc + (uint32_t)(d0 * d0 - c0 + 2 * mb - 3), d0, mb, x);
+                        tmem_wait(x);
+                        if (mb == 0) order_zero(x);
+                        for (int dn = d0; dn < d1; ++dn) {
+                            const int at = (dn * dn - na * na) * M2_STG_LD + row;
+                            convert_orders(conv, tp, tc, c0, a.p, dn, mb, tx, ty, tz, x, stg + at, stc + at);
+                        }
+                    }
+                    if (nb == n1) release(b);
+                    epi_sync();
+                    add_rows(na * na, nb * nb - na * na);
+                    epi_sync();
+                    na = nb;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)M2_TMEM) : "memory");
+}
+
+// tiles[slot][range][k chunk][hi | lo][tile_off order] of the translation block T of the fused
+// tables: T[k][c] = ops[slot][k ldo + c], k, c < P
+__global__ void k_m2l_tiles(const float* __restrict__ ops, int64_t op_floats, int ldo, M2lArgs a,
+                            float* __restrict__ tiles) {
+    for (int g = blockIdx.x; g < NUM_OFFSETS; g += gridDim.x) {
+        const float* Ag = ops + (int64_t)g * op_floats;
+        float* tg = tiles + (int64_t)g * a.group_stride;
+        for (int r = 0; r < a.nranges; ++r) {
+            const int nlen = a.nlen[r], tile = nlen * TC_KC;
+            for (int e = threadIdx.x; e < a.P / TC_KC * tile; e += blockDim.x) {
+                const int i = e / tile, q = e - i * tile, k = q / nlen, c = q - k * nlen;
+                const int kk = i * TC_KC + k, cc = a.c0[r] + c;
+                const float v = cc < a.P ? Ag[(int64_t)kk * ldo + cc] : 0.f;
+                const float h = tf32_rna(v);
+                float* base = tg + a.roff[r] + (int64_t)i * 2 * tile;
+                const uint32_t o = tile_off(c, k) / 4;
+                base[o] = h;
+                base[tile + o] = tf32_rna(v - h);
+            }
+        }
+    }
+}
+
+int m2l_fixed_smem(int p, int npot) {
+    return (npot * M2_BAND * M2_STG_LD + (npot == 2 ? conv_floats(p) : 0)) * 4;
+}
+
+// One past the last column that the epilogue reads of chi of the degrees [n0, n1) and their
+// halo (tmem_orders), counted from the first column of the range.
+int chi_read_end(int p, int n0, int n1) {
+    int end = 0;
+    for (int n = n0; n < n1; ++n)
+        for (int mb = 0; mb <= n; mb += 8)
+            for (int N = n; N <= std::min(n + 1, p - 1); ++N)
+                end = std::max(end, N * N - n0 * n0 + 2 * mb - 3 + 18 + (mb + 8 <= N ? 2 : 0));
+    return end;
+}
+
+// Ranges, strides and stages of truncation number p.  One range of output degrees holds all
+// columns up to p = 16 (2 x 256 of the 512); above, each range carries the halo degree that its
+// conversion reads.  The accumulators are double-buffered where two fit (the scalar case, p <= 8).
+// Splitting p = 12 and 16 into ranges of 256 columns so that two fit was slower (sphere
+// surface of 2^20, p = 12: products 3.6 ms against 1.8 without the epilogue, 9.3 against 4.9 with
+// it): the narrow MMAs are bound by their operand reads from shared memory, and the reads of
+// TMEM queue behind them.
+M2lArgs m2l_layout(int p, int npot) {
+    M2lArgs a{};
+    a.p = p;
+    a.P = p * p;
+    a.nbuf = npot == 1 || p <= 8 ? 2 : 1;
+    int64_t off = 0;
+    int nmax = 0;
+    for (int n0 = 0; n0 < p;) {
+        const int r = a.nranges++, c0 = n0 * n0, room = M2_TMEM / a.nbuf - (r ? 16 : 0);
+        if (r >= M2_MAX_RANGES) throw Error{LHV_EUNSUPPORTED, "M2L output ranges"};
+        auto width = [&](int n1) {  // columns of the degrees [n0, n1) with their halo, in 16s
+            const int hi = n1 < p && npot == 2 ? (n1 + 1) * (n1 + 1) : n1 * n1;
+            return (hi - c0 + 15) / 16 * 16;
+        };
+        auto fits = [&](int n1) {
+            const int w = width(n1);
+            return w <= 256 && npot * w <= room && (npot == 1 || w + chi_read_end(p, n0, n1) <= room);
+        };
+        int n1 = n0 + 1;
+        while (n1 < p && fits(n1 + 1)) ++n1;
+        if (!fits(n1)) throw Error{LHV_EUNSUPPORTED, "M2L accumulators"};
+        a.n0[r] = n0;
+        a.n1[r] = n1;
+        a.c0[r] = c0;
+        a.nlen[r] = width(n1);
+        a.roff[r] = off;
+        off += (int64_t)(a.P / TC_KC) * 2 * a.nlen[r] * TC_KC;
+        nmax = std::max(nmax, a.nlen[r]);
+        n0 = n1;
+    }
+    a.group_stride = off;
+    a.stage_bytes = 2 * npot * M2_X_TILE + 2 * nmax * TC_KC * 4;
+    a.nstages = std::min(M2_MAX_STAGES, (M2_SMEM_MAX - m2l_fixed_smem(p, npot)) / a.stage_bytes);
+    return a;
+}
+
+}  // namespace
+
+bool m2l_tc_supported(int p) { return p % 4 == 0 && p >= 4 && p <= 24; }
+
+void m2l_tiles_build(Ctx* c, const float* fused, int p, bool scalar, Buf& tiles) {
+    M2lArgs a = m2l_layout(p, scalar ? 1 : 2);
+    const int64_t nt = a.group_stride * NUM_OFFSETS;
+    std::vector<float> conv((size_t)conv_floats(p), 0.f);
+    for (int n = 0; n < p; ++n)
+        for (int m = 0; m <= n; ++m) {
+            float* v = &conv[(size_t)(n * (n + 1) / 2 + m) * 8];
+            const double two = m ? 1.0 : 2.0;
+            if (n > 0) {
+                v[0] = (float)(-two * std::sqrt((double)(n - m) * (n + m + 1)) / (2.0 * n));
+                v[1] = m ? (float)(std::sqrt((double)(n + m) * (n - m + 1)) / (2.0 * n)) : 0.f;
+                v[2] = (float)((double)m / n);
+            }
+            if (n + 1 < p) {
+                v[3] = m ? (float)(std::sqrt((double)(n - m + 1) * (n - m + 2)) / (2.0 * (n + 1))) : 0.f;
+                v[4] = (float)(-two * std::sqrt((double)(n + m + 1) * (n + m + 2)) / (2.0 * (n + 1)));
+                v[5] = (float)(-std::sqrt((double)(n + 1 - m) * (n + 1 + m)) / (n + 1));
+            }
+        }
+    ensure(c, tiles, (nt + (int64_t)conv.size()) * (int64_t)sizeof(float));
+    k_m2l_tiles<<<NUM_OFFSETS, 256, 0, stream_of(c)>>>(fused, 4 * (int64_t)a.P * a.P, 2 * a.P, a, tiles.as<float>());
+    count_launch(c);
+    check_launch("m2l tiles");
+    cuda_check(cudaMemcpyAsync(tiles.as<float>() + nt, conv.data(), conv.size() * sizeof(float),
+                               cudaMemcpyHostToDevice, stream_of(c)),
+               "m2l conversion");
+    cuda_check(cudaStreamSynchronize(stream_of(c)), "m2l tiles");
+}
+
+void run_tc_m2l(Ctx* c, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
+                const int* offsets, const float* in, float* out, int64_t ld, int* err) {
+    M2lArgs a = m2l_layout(p, scalar ? 1 : 2);
+    a.chunks = gp.chunks.as<int4>();
+    a.pairs = gp.pairs.as<int2>();
+    a.choff = gp.choff.as<int>();
+    a.g0 = g0;
+    a.g1 = g1;
+    a.in = in;
+    a.out = out;
+    a.ld = ld;
+    a.tiles = tiles;
+    a.conv = tiles + a.group_stride * NUM_OFFSETS;
+    a.offsets = offsets;
+    a.err = err;
+    // above half an SM's shared memory: one CTA (and its 512 TMEM columns) per SM
+    const size_t smem =
+        std::max<size_t>((size_t)a.nstages * a.stage_bytes + m2l_fixed_smem(p, scalar ? 1 : 2), 120 * 1024);
+    auto kernel = scalar ? k_tc_m2l<1> : k_tc_m2l<2>;
+    cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "m2l smem");
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    kernel<<<sms, M2_THREADS, smem, stream_of(c)>>>(a);
+    count_launch(c);
+    check_launch("tc m2l");
+}
+
+}  // namespace lhv

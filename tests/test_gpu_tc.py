@@ -55,3 +55,28 @@ def test_tf32x3_parity(case):
     ev, es = rel(host3(v4), ref.v), rel(host3(s4), ref.s)
     print(f"tf32x3 {case} p=12: rel L2 v {ev:.2e} s {es:.2e}")
     assert ev < 1e-6 and es < 1e-6, (ev, es)
+
+
+@pytest.mark.parametrize("p", [4, 8, 12, 16, 20, 24])
+@pytest.mark.parametrize("n,leaf", [(700, 8), (5000, 16)])
+def test_m2l_converts_like_the_fused_table(p, n, leaf):
+    """One translation block with the conversion in the epilogue against the fused tables on the
+    CUDA cores, far field only: v and s, and the scalar case.  Covers one and several column
+    ranges (p = 20, 24), one and two accumulator buffers, full and partly filled chunks.  Both
+    sides round 2 p^2 FP32 terms a coefficient: sqrt(2 24^2) 2^-24 = 2e-6."""
+    import torch
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n, 9)
+    q = torch.from_numpy(workloads.charges(n, 3)).cuda()
+    got = {}
+    for tc in (1, 0):
+        ctx = LHV(p=p, leaf_max=leaf, core_a=0.0, precision="tf32x3", terms="far")
+        ctx.set_launch_shape(m2l_tensor_cores=tc)
+        v4, s4 = ctx.evaluate_velocity_stretching(dev(x, "fp32"), dev(w, "fp32"))
+        pg = ctx.evaluate_potential_gradient(dev(x, "fp32"), q)
+        st = ctx.stats()  # raises if a tensor-core wait timed out
+        assert st["leaf_level"] >= 2 and st["m2l_pairs"] > 0
+        got[tc] = (host3(v4), host3(s4), pg.cpu().numpy())
+        ctx.close()
+    for a, b in zip(got[1], got[0]):
+        assert rel(a, b) < 2e-6, rel(a, b)
