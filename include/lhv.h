@@ -115,14 +115,15 @@ typedef struct {
                                                 last check (-1: none) */
     int     tuned_p2p_targets_per_thread;    /* launch shapes in use (lhv_autotune) */
     int     tuned_p2p_sources_per_stage;
-    int     tuned_m2l_pairs_per_chunk;       /* 0: the default (128 on the tensor cores, else
-                                                the largest CUDA-core chunk that fits) */
+    int     tuned_m2l_pairs_per_chunk;       /* 0: the default (128 on the tensor cores, else RCR
+                                                translations where they apply, else the largest
+                                                CUDA-core chunk that fits) */
     int     tuned_m2l_tensor_cores;          /* 1 when M2L runs on the tensor cores */
     double  tune_ms[12];                     /* stage times of the candidates, in the order
                                                 P2P 1/2/4 targets per thread at 128 sources per
                                                 stage, the same at 256, then M2L: (TF32x3 only:
                                                 tensor cores 128, 64 pairs,) CUDA cores 64, 32,
-                                                16 pairs */
+                                                16 pairs (, FP32 and FP64 only: the default) */
     int64_t graph_captures;                  /* steps captured as a CUDA graph (lhv_set_graph) */
     int64_t graph_replays;                   /* steps run as one replay of the captured graph */
     int64_t graph_fallbacks;                 /* steps whose tree failed the captured layout's guard
@@ -253,7 +254,7 @@ int lhv_direct_sampled_f64(lhv_ctx* ctx, int64_t n, const double* x4, const doub
  * sources staged in shared memory per step) and the
  * fastest M2L grouping (box pairs of one offset per GEMM chunk: 64, 32 or 16 on
  * the CUDA cores; under TF32X3 also the tensor-core kernel with 128 or 64 pairs
- * per chunk), chosen by CUDA-event stage times (best of 3 after a warm-up).  v4
+ * per chunk, else also the default translations), chosen by CUDA-event stage times (best of 3 after a warm-up).  v4
  * and s4 receive the last evaluation.  The batched twin tunes on a batch
  * (offsets as for lhv_evaluate_batched).  Results do not depend on the choice
  * beyond rounding. */
@@ -302,8 +303,13 @@ int lhv_set_level_p(lhv_ctx* ctx, const int* p, int nlevels);
 int lhv_set_graph(lhv_ctx* ctx, int enable);
 
 /* Representation of the far field (Sec. 4.2).  LHV_FORM_PHI_CHI (the default): the two
- * real potentials phi and chi, p^2 reals each, translated by the fused real tables
- * [[T, C12 T], [0, C22 T]] (translation and conversion, zero block skipped).
+ * real potentials phi and chi, p^2 reals each.  M2L by the fused real tables [[T, C12 T],
+ * [0, C22 T]] (translation and conversion) or by an equal route that costs less: on the
+ * tensor cores (LHV_TF32X3, p a multiple of 4) the translation T of both potentials with
+ * the conversion applied to the sums, on the CUDA cores with one 4 <= p <= 20 at every
+ * level (FP64: up to the p whose tables fit an SM's shared memory, 16) the RCR
+ * translations below, unless lhv_set_launch_shape asks for a CUDA-core chunk of the fused
+ * tables.  The routes agree to rounding.  M2M and L2L use the fused tables.
  * LHV_FORM_PSI: one complex harmonic function Psi = phi + i chi (Eq. chf1), stored as
  * 2 p^2 reals (Re / Im of Psi_n^m for m >= 0, then of Psi_n^{-m}; Im Psi_n^0 in place of
  * the m = 0 entry of the second half), translated by one dense real table per offset or

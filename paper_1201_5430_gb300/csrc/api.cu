@@ -39,6 +39,7 @@ struct Ctx {
     int64_t tree_n = 0;
     OpTables ops;
     int ops_type = 0;  // sizeof(T) of the built tables
+    bool have_m2l = false;              // ops.m2l is built
     Buf tmp[14];
     Buf xs, ws, mult, loc, table, vfar, sfar, counters, W;
     Grouped gp_m2m, gp_m2l, gp_l2l;
@@ -85,6 +86,7 @@ struct Ctx {
     int psi_p = 0, psi_type = 0;
     // M2L by rotation - coaxial - rotation (LHV_FORM_RCR)
     RcrTables rcr;
+    bool rcr_failed = false;            // its tables failed their check: the default form keeps the fused ones
     // scalar reference case (lhv_evaluate_potential_gradient)
     Buf s_m2l, s_m2m, s_l2l, s_tiles;   // translation blocks of the fused tables, TF32 tiles of the M2L ones
     int s_p = 0, s_type = 0;
@@ -182,10 +184,23 @@ static void harvest(Ctx* c) {
 }
 
 // ---- the evaluation pipeline ----------------------------------------------
+// The fused M2L tables (316 x (2 p^2)^2 reals), built when a route needs them: the CUDA-core grouped
+// GEMM, the complex and scalar forms, and the tensor-core tiles.
+template <typename T>
+static const T* fused_m2l(Ctx* c) {
+    if (!c->have_m2l) {
+        StageScope sc(c, LHV_STAGE_OPS);
+        build_op<T>(c, OP_M2L, c->cfg.p, c->cfg.p, c->ops.m2l);
+        c->have_m2l = true;
+    }
+    return c->ops.m2l.as<T>();
+}
+
 template <typename T>
 static void ensure_ops(Ctx* c) {
     if (c->ops.p == c->cfg.p && c->ops_type == (int)sizeof(T)) return;
     free_operators(c->ops);
+    c->have_m2l = false;
     StageScope sc(c, LHV_STAGE_OPS);
     build_operators<T>(c, c->cfg.p, c->ops);
     build_sparse<T>(c, OP_P2M, c->cfg.p, c->ops.p2m_sp);
@@ -193,7 +208,7 @@ static void ensure_ops(Ctx* c) {
     c->ops_type = (int)sizeof(T);
     if constexpr (sizeof(T) == 4) {
         if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
-            m2l_tiles_build(c, c->ops.m2l.as<float>(), c->cfg.p, false, c->ops.m2l_tiles);
+            m2l_tiles_build(c, fused_m2l<float>(c), c->cfg.p, false, c->ops.m2l_tiles);
     }
 }
 
@@ -257,7 +272,7 @@ static void ensure_psi_ops(Ctx* c) {
     if (c->psi_p == c->cfg.p && c->psi_type == (int)sizeof(T)) return;
     StageScope sc(c, LHV_STAGE_OPS);
     const int P = c->ops.P;
-    psi_form<T>(c, c->ops.m2l.as<T>(), NUM_OFFSETS, P, c->psi_m2l);
+    psi_form<T>(c, fused_m2l<T>(c), NUM_OFFSETS, P, c->psi_m2l);
     psi_form<T>(c, c->ops.m2m.as<T>(), 8, P, c->psi_m2m);
     psi_form<T>(c, c->ops.l2l.as<T>(), 8, P, c->psi_l2l);
     if constexpr (sizeof(T) == 4) {
@@ -269,6 +284,23 @@ static void ensure_psi_ops(Ctx* c) {
     cuda_check(cudaStreamSynchronize(c->stream), "psi tables");
     c->psi_p = c->cfg.p;
     c->psi_type = (int)sizeof(T);
+}
+
+// Whether the two-potential form with one p takes M2L by rotation - coaxial translation - back
+// rotation, O(p^3) a pair, instead of the fused tables, O(p^4), on the CUDA cores: always where its
+// tables fit, unless a chunk of the fused-table GEMM was asked for (lhv_set_launch_shape) or the
+// tensor cores run the products.  The far field's error against FP64 is that of the fused tables or
+// smaller (sphere surface, p = 12: v 3.1e-7 against 3.6e-7).  Products of a cube of 100,003 elements
+// (640,584 pairs), RCR against the fused tables, ms: FP32 p = 4 0.24 / 0.32, p = 8 0.62 / 1.13, p = 12
+// 1.48 / 5.76, p = 16 2.94 / 20.9, p = 20 6.34 / 62.6; FP64 (32,768 elements, 640,206 pairs) p = 4
+// 1.29 / 3.72, p = 8 6.80 / 14.3, p = 12 21.5 / 92.9, p = 16 44.3 / 216.  Below p = 4 the tables were
+// not compared.
+constexpr int RCR_MIN_P = 4;
+template <typename T>
+static bool default_rcr(Ctx* c) {
+    if (c->form != LHV_FORM_PHI_CHI || c->tune_nc != 0 || c->rcr_failed || c->cfg.p < RCR_MIN_P) return false;
+    if (sizeof(T) == 4 && ctx_m2l_tc(c) && m2l_tc_supported(c->cfg.p)) return false;
+    return rcr_chunk(c->cfg.p, sizeof(T), nullptr) > 0;
 }
 
 // Truncation numbers and tables of an evaluation over levels 0..L.
@@ -287,11 +319,16 @@ static Plan<T> make_plan(Ctx* c, int L) {
     pl.ld = (2 * pmax * pmax + 7) / 8 * 8;  // 32-byte rows for the vector loads of the tensor-core path
     const bool base = pl.uniform && pl.p[L] == c->cfg.p;
     const bool tc = sizeof(T) == 4 && ctx_use_tc(c);
-    if (c->form == LHV_FORM_RCR) {
-        if (!base || sizeof(T) != 4 || c->cfg.p > RCR_PMAX)
-            throw Error{LHV_EUNSUPPORTED, "RCR translations run FP32 with one truncation number p <= 20 at every level"};
-        if (c->rcr.p != c->cfg.p) rcr_build(c, c->cfg.p, c->rcr);
-        pl.rcr = &c->rcr;
+    if (c->form == LHV_FORM_RCR && (!base || sizeof(T) != 4 || c->cfg.p > RCR_PMAX))
+        throw Error{LHV_EUNSUPPORTED, "RCR translations run FP32 with one truncation number p <= 20 at every level"};
+    if (c->form == LHV_FORM_RCR || (base && default_rcr<T>(c))) {
+        try {
+            if (c->rcr.p != c->cfg.p) rcr_build<T>(c, c->cfg.p, c->rcr);
+            pl.rcr = &c->rcr;
+        } catch (const Error& e) {
+            if (c->form == LHV_FORM_RCR || e.status != LHV_EUNSUPPORTED) throw;
+            c->rcr_failed = true;
+        }
     }
     if (c->form == LHV_FORM_PSI) {
         if (!base)
@@ -311,12 +348,14 @@ static Plan<T> make_plan(Ctx* c, int L) {
         return pl;
     }
     if (base) {
+        const bool tiles = tc && ctx_m2l_tc(c) && c->ops.m2l_tiles.ptr;
+        const T* m2l = pl.rcr || tiles ? nullptr : fused_m2l<T>(c);
         pl.p2m = c->ops.p2m.as<T>();
         pl.l2p = c->ops.l2p.as<T>();
         for (int l = 0; l <= L; ++l) {
             pl.m2m[l] = c->ops.m2m.as<T>();
             pl.l2l[l] = c->ops.l2l.as<T>();
-            pl.m2l[l] = c->ops.m2l.as<T>();
+            pl.m2l[l] = m2l;
             pl.m2l_tiles[l] = c->ops.m2l_tiles.ptr ? c->ops.m2l_tiles.as<float>() : nullptr;
         }
         pl.p2m_sp = view<T>(c->ops.p2m_sp);
@@ -470,12 +509,12 @@ static void ensure_scalar_ops(Ctx* c) {
     if (c->s_p == c->cfg.p && c->s_type == (int)sizeof(T)) return;
     StageScope sc(c, LHV_STAGE_OPS);
     const int P = c->ops.P;
-    translation_block<T>(c, c->ops.m2l.as<T>(), NUM_OFFSETS, P, c->s_m2l);
+    translation_block<T>(c, fused_m2l<T>(c), NUM_OFFSETS, P, c->s_m2l);
     translation_block<T>(c, c->ops.m2m.as<T>(), 8, P, c->s_m2m);
     translation_block<T>(c, c->ops.l2l.as<T>(), 8, P, c->s_l2l);
     if constexpr (sizeof(T) == 4) {
         if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
-            m2l_tiles_build(c, c->ops.m2l.as<float>(), c->cfg.p, true, c->s_tiles);
+            m2l_tiles_build(c, fused_m2l<float>(c), c->cfg.p, true, c->s_tiles);
         else
             release(c->s_tiles);
     }
@@ -825,8 +864,8 @@ static int evaluate_selected(Ctx* c, int64_t n, const vec4_t<T>* x4, const vec4_
 // Times the launch-shape candidates on the caller's workload (stage times from CUDA
 // events, best of `reps` evaluations after one warm-up) and keeps the fastest:
 //   P2P: 1, 2 or 4 targets per thread (128, 64 or 32 threads per tile of 128 targets);
-//   M2L: 64, 32 or 16 pairs per CUDA-core GEMM chunk, and under TF32x3 the tensor-core
-//        kernel with 128 or 64 pairs per chunk.
+//   M2L: 64, 32 or 16 pairs per CUDA-core GEMM chunk, under TF32x3 the tensor-core kernel
+//        with 128 or 64 pairs per chunk, else the default translations.
 template <typename T, typename F>
 static void autotune(Ctx* c, F&& eval) {
     const bool timing = c->timing;
@@ -877,6 +916,7 @@ static void autotune(Ctx* c, F&& eval) {
         cands.push_back({1, 64});
     }
     for (int nc : {64, 32, 16}) cands.push_back({0, nc});
+    if (cands.front().tc == 0) cands.push_back({1, 0});  // the default: rotation - coaxial - rotation
     best = 1e30;
     Cand pick = cands.front();
     for (const Cand& cd : cands) {

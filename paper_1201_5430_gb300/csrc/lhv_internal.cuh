@@ -160,7 +160,7 @@ struct OpTables {
     int p = 0;
     int P = 0;                 // p*p
     // every matrix is k-major: element (input j, output i) at j * rows + i
-    Buf m2l;                   // [316][2P][2P] fused (S|R) + Eq. drt10 per offset slot
+    Buf m2l;                   // [316][2P][2P] fused (S|R) + Eq. drt10 per offset slot (built when a route needs it)
     Buf m2m;                   // [8][2P][2P]   fused (S|S) + Eq. drt11 per child octant
     Buf l2l;                   // [8][2P][2P]   fused (R|R) + Eq. drt10 per child octant
     Buf l2p;                   // [2P][12P]     v_k (Eq. evf3) and u_lk (Eq. dt3) coefficients
@@ -171,7 +171,7 @@ struct OpTables {
     Buf slot_of;               // int[343] offset (dx+3)*49+(dy+3)*7+(dz+3) -> slot or -1
 };
 
-// Builds every table in FP64 on the GPU and stores it in T.
+// Builds every table but m2l in FP64 on the GPU and stores it in T.
 template <typename T>
 void build_operators(Ctx* c, int p, OpTables& ops);
 // One operator family in FP64 -> T: M2L (316 x [2Pin][2Pout], pout == pin), M2M (8 x
@@ -219,7 +219,7 @@ struct Plan {
     bool scalar = false;                   // scalar reference case: one potential, P x P translation
                                            // tables (the T block of the fused operators), no conversion
     bool psi = false;                      // complex form Psi = phi + i chi: dense 2P x 2P tables
-    const RcrTables* rcr = nullptr;        // M2L by rotation - coaxial - rotation (rcr.cu), FP32
+    const RcrTables* rcr = nullptr;        // M2L by rotation - coaxial - rotation (rcr.cu)
     // output / input split of a fused translation table (its zero block is skipped);
     // 0 (dense) in the complex form
     int split_out(int P) const { return (scalar || psi) ? 0 : P; }
@@ -277,13 +277,14 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
 
 // ---- RCR translations (rcr.cu) -------------------------------------------------
 // M2L by rotation - coaxial translation - back rotation with the coaxial conversion of
-// Eq. rcr1 (Sec. 4.4), two-potential form, FP32, one truncation number p <= RCR_PMAX.
+// Eq. rcr1 (Sec. 4.4), two-potential form, FP32 or FP64, one truncation number p <= RCR_PMAX.
 constexpr int RCR_PMAX = 20;
 struct RcrTables {
     int p = 0;
+    int type = 0;         // sizeof(T) of the tables
     int nc = 0;           // box pairs per chunk of the grouped pair list
-    int slot_floats = 0;  // floats of one offset slot's rotation tables [Y fwd | Y back | Z fwd | Z back]
-    int coax_floats = 0;  // floats of one distance's coaxial blocks and conversion coefficients
+    int slot_floats = 0;  // reals of one offset slot's rotation tables [Y fwd | Y back | Z fwd | Z back]
+    int coax_floats = 0;  // reals of one distance's coaxial blocks and conversion coefficients
     int smem = 0;         // dynamic shared memory of the products kernel
     int nsm = 0;          // streaming multiprocessors
     int ctas_per_sm = 1;  // resident CTAs of the products kernel per SM (its grid: nsm x this)
@@ -292,12 +293,17 @@ struct RcrTables {
     Buf coax;             // [distinct |t|][coax_floats]
     Buf dist_of;          // int[316]: distance index of each offset slot
 };
-// Builds the tables (FP64 on the GPU, stored FP32); synchronous.  LHV_EUNSUPPORTED above RCR_PMAX.
+// Pairs per chunk of the products kernel for tables of `size`-byte reals (and its CTAs per SM);
+// 0: not available (p above RCR_PMAX, or the tables exceed shared memory).
+int rcr_chunk(int p, int size, int* ctas);
+// Builds the tables (FP64 on the GPU, stored in T); synchronous.  LHV_EUNSUPPORTED where rcr_chunk is 0.
+template <typename T>
 void rcr_build(Ctx* c, int p, RcrTables& rt);
 void rcr_free(RcrTables& rt);
 // loc += the RCR translation of mult for every pair of gp (chunks of rt.nc pairs bucketed by
 // offset slot); rows of ld reals (phi then chi).
-void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const float* mult, float* loc, int64_t ld);
+template <typename T>
+void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const T* mult, T* loc, int64_t ld);
 // Gauss-Legendre nodes and weights on [-1, 1] (nq points).
 void gauss_legendre_nodes(int nq, double* xi, double* w);
 // The 316 M2L offsets (dx, dy, dz of the source box from the target box) in slot order,

@@ -103,11 +103,9 @@ template <typename T>
 void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const int* offsets,
                const T* mult, T* loc) {
     const int L = lv.L;
-    if constexpr (sizeof(T) == 4) {
-        if (pl.rcr) {  // rotation - coaxial - rotation (rcr.cu)
-            rcr_apply(c, *pl.rcr, gp, mult, loc, pl.ld);
-            return;
-        }
+    if (pl.rcr) {  // rotation - coaxial - rotation (rcr.cu)
+        rcr_apply<T>(c, *pl.rcr, gp, mult, loc, pl.ld);
+        return;
     }
     // the complex form's tensor-core products read the multipoles split into TF32 hi/lo once
     // (one p at every level; the other forms split in the kernel)

@@ -600,7 +600,6 @@ void build_operators(Ctx* c, int p, OpTables& ops) {
     cudaStream_t s = stream_of(c);
     ops.p = p;
     ops.P = p * p;
-    build_op<T>(c, OP_M2L, p, p, ops.m2l);
     build_op<T>(c, OP_M2M, p, p, ops.m2m);
     build_op<T>(c, OP_L2L, p, p, ops.l2l);
     build_op<T>(c, OP_L2P, p, p, ops.l2p);

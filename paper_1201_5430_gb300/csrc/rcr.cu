@@ -1,5 +1,5 @@
 // M2L by rotation - coaxial translation - back rotation (RCR, Sec. 4.4, Eq. rcr1) for the
-// two-potential form: FP32 products on the CUDA cores, tables built in FP64.
+// two-potential form: FP32 or FP64 products on the CUDA cores, tables built in FP64.
 //
 // A translation by t = target - source centre runs in the frame whose z axis is t.  With
 // Q a rotation taking i_z to t/|t| (r = Q r'), each potential's coefficients are rotated
@@ -43,6 +43,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <utility>
 #include <vector>
 
 #include "lhv_group.cuh"
@@ -221,41 +223,42 @@ __device__ inline void atomic_max_pos(float* a, float v) {
     atomicMax(reinterpret_cast<int*>(a), __float_as_int(v));  // non-negative floats order as ints
 }
 
-// One CTA per slot: the slot's table [Yf | Yb | Zf | Zb] (floats) from the dense blocks of its
-// four jobs (4 s + 0: Y(theta), S basis; + 1: Y(-theta), R basis; + 2: Z(phi), S basis;
+// One CTA per slot: the slot's table [Yf | Yb | Zf | Zb] (reals) from the dense blocks of its
+// four jobs (job_of[4 s + 0]: Y(theta), S basis; + 1: Y(-theta), R basis; + 2: Z(phi), S basis;
 // + 3: Z(-phi), R basis); *resid = the largest entry outside the structure.
-__global__ void k_rcr_pack(const double* __restrict__ dense, int p, int per_slot, float* __restrict__ out,
-                           float* __restrict__ resid) {
+template <typename T>
+__global__ void k_rcr_pack(const double* __restrict__ dense, const int* __restrict__ job_of, int p, int per_slot,
+                           T* __restrict__ out, float* __restrict__ resid) {
     const int NE = p * (4 * p * p - 1) / 3;
     const int ysz = y_off(p);
-    float* dst = out + (int64_t)blockIdx.x * per_slot;
+    T* dst = out + (int64_t)blockIdx.x * per_slot;
     float worst = 0.f;
     for (int which = 0; which < 2; ++which) {  // Y blocks
-        const double* X = dense + ((int64_t)blockIdx.x * 4 + which) * NE;
-        float* d = dst + which * ysz;
+        const double* X = dense + (int64_t)job_of[blockIdx.x * 4 + which] * NE;
+        T* d = dst + which * ysz;
         for (int n = 0; n < p; ++n) {
             const int w = 2 * n + 1, base = n * (4 * n * n - 1) / 3;
             const double* Xn = X + base;
             const int ne = n + 1, no = n, Pe = pad4(ne), Po = pad4(no);
-            float* de = d + y_off(n);
-            float* dod = de + ne * Pe;
+            T* de = d + y_off(n);
+            T* dod = de + ne * Pe;
             for (int e = threadIdx.x; e < w * w; e += blockDim.x) {
                 const int jp = e / w, j = e - jp * w;
                 if (is_even(jp) != is_even(j)) worst = fmaxf(worst, (float)fabs(Xn[e]));
             }
             for (int e = threadIdx.x; e < ne * Pe; e += blockDim.x) {
                 const int i = e / Pe, o = e - i * Pe;
-                de[e] = o < ne ? (float)Xn[even_member(o) * w + even_member(i)] : 0.f;
+                de[e] = o < ne ? (T)Xn[even_member(o) * w + even_member(i)] : (T)0;
             }
             for (int e = threadIdx.x; e < no * Po; e += blockDim.x) {
                 const int i = e / Po, o = e - i * Po;
-                dod[e] = o < no ? (float)Xn[odd_member(o) * w + odd_member(i)] : 0.f;
+                dod[e] = o < no ? (T)Xn[odd_member(o) * w + odd_member(i)] : (T)0;
             }
         }
     }
     for (int which = 0; which < 2; ++which) {  // Z: [m][4] = (Re<-Re, Re<-Im, Im<-Re, Im<-Im)
-        const double* X = dense + ((int64_t)blockIdx.x * 4 + 2 + which) * NE;
-        float* d = dst + 2 * ysz + which * 4 * p;
+        const double* X = dense + (int64_t)job_of[blockIdx.x * 4 + 2 + which] * NE;
+        T* d = dst + 2 * ysz + which * 4 * p;
         for (int n = 0; n < p; ++n) {
             const int w = 2 * n + 1, base = n * (4 * n * n - 1) / 3;
             const double* Xn = X + base;
@@ -276,11 +279,11 @@ __global__ void k_rcr_pack(const double* __restrict__ dense, int p, int per_slot
         }
         for (int e = threadIdx.x; e < 4 * p; e += blockDim.x) {
             const int m = e / 4, k = e & 3;
-            float v = 0.f;
+            T v = 0;
             if (m > 0) {
                 const int N = p - 1, W = 2 * N + 1, bN = N * (4 * N * N - 1) / 3;
                 const int jp = 2 * m - 1 + (k >> 1), j = 2 * m - 1 + (k & 1);
-                v = (float)X[bN + jp * W + j];
+                v = (T)X[bN + jp * W + j];
             }
             d[e] = v;
         }
@@ -291,13 +294,14 @@ __global__ void k_rcr_pack(const double* __restrict__ dense, int p, int per_slot
 // One CTA per distance: [A blocks | tau, sigma] of the coaxial translation at |t| = dist.
 // A_m: [input n - m][output n' - m padded to 4]; ts[(n' p + m) 2 + {0, 1}] = tau, sigma.
 // *resid = the largest mismatch of the fused table's conversion blocks against them.
+template <typename T>
 __global__ void k_rcr_coax(const double* __restrict__ fused, const double* __restrict__ dist, int p, int per_dist,
-                           float* __restrict__ out, float* __restrict__ resid) {
+                           T* __restrict__ out, float* __restrict__ resid) {
     const int P = p * p, ld = 2 * P;
     const double* F = fused + (int64_t)blockIdx.x * ld * ld;
     const double t = dist[blockIdx.x];
-    float* dst = out + (int64_t)blockIdx.x * per_dist;
-    float* ts = dst + coax_off(p, p);
+    T* dst = out + (int64_t)blockIdx.x * per_dist;
+    T* ts = dst + coax_off(p, p);
     float worst = 0.f;
     auto tau = [&](int n2, int m) { return n2 > 0 ? t * m / n2 : 0.0; };
     auto sigma = [&](int n2, int m) {
@@ -305,14 +309,14 @@ __global__ void k_rcr_coax(const double* __restrict__ fused, const double* __res
     };
     for (int m = 0; m < p; ++m) {
         const int k = p - m, K = pad4(k), mo = m ? 2 * m - 1 : 0;
-        float* blk = dst + coax_off(p, m);
+        T* blk = dst + coax_off(p, m);
         for (int e = threadIdx.x; e < k * K; e += blockDim.x) {
             const int i = e / K, o = e - i * K;
-            float v = 0.f;
+            T v = 0;
             if (o < k) {
                 const int n = m + i, n2 = m + o;
                 const double a = F[(int64_t)(n * n + mo) * ld + n2 * n2 + mo];
-                v = (float)a;
+                v = (T)a;
                 // check: the phi <- Im chi block is -tau A, the chi <- chi block A - sigma A(n2 + 1)
                 const double an = n2 + 1 < p ? F[(int64_t)(n * n + mo) * ld + (n2 + 1) * (n2 + 1) + mo] : 0.0;
                 const double b = m ? F[(int64_t)(P + n * n + 2 * m) * ld + n2 * n2 + mo] : 0.0;
@@ -326,34 +330,46 @@ __global__ void k_rcr_coax(const double* __restrict__ fused, const double* __res
     }
     for (int e = threadIdx.x; e < 2 * P; e += blockDim.x) {
         const int q = e >> 1, n2 = q / p, m = q - n2 * p;
-        ts[e] = m <= n2 ? (float)((e & 1) ? sigma(n2, m) : tau(n2, m)) : 0.f;
+        ts[e] = m <= n2 ? (T)((e & 1) ? sigma(n2, m) : tau(n2, m)) : (T)0;
     }
     if (worst > 0.f) atomic_max_pos(resid, worst);
 }
 
+// four pairs of one row: one 16-byte (FP32) or two (FP64) shared-memory accesses
+template <typename T> struct alignas(16) Quad {
+    T x, y, z, w;
+};
+
+template <typename T>
+__device__ __forceinline__ Quad<T> make_quad(T x, T y, T z, T w) {
+    return Quad<T>{x, y, z, w};
+}
+
+template <typename T>
 struct RcrArgs {
     const int4* chunks;
     const int2* pairs;
     const int* nchunks;  // device: total chunks (choff[ngroups])
-    const float* rot;    // per slot: [Yf | Yb | Zf | Zb]
-    const float* coax;   // per distance: [A blocks | tau, sigma]
+    const T* rot;    // per slot: [Yf | Yb | Zf | Zb]
+    const T* coax;   // per distance: [A blocks | tau, sigma]
     const int* dist_of;
-    const float* in;
-    float* out;
+    const T* in;
+    T* out;
     int64_t ld;
     int p;
     int slot_floats, coax_floats;
     int nrg_y, nrg_cx;   // register-tile row groups of the Y / coaxial stages
 };
 
-__device__ __forceinline__ void fma44(float (&acc)[4][4], float4 x, float4 v) {
-    const float xs[4] = {x.x, x.y, x.z, x.w};
+template <typename T>
+__device__ __forceinline__ void fma44(T (&acc)[4][4], Quad<T> x, Quad<T> v) {
+    const T xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        acc[j][0] = fmaf(xs[j], v.x, acc[j][0]);
-        acc[j][1] = fmaf(xs[j], v.y, acc[j][1]);
-        acc[j][2] = fmaf(xs[j], v.z, acc[j][2]);
-        acc[j][3] = fmaf(xs[j], v.w, acc[j][3]);
+        acc[j][0] = fma(xs[j], v.x, acc[j][0]);
+        acc[j][1] = fma(xs[j], v.y, acc[j][1]);
+        acc[j][2] = fma(xs[j], v.z, acc[j][2]);
+        acc[j][3] = fma(xs[j], v.w, acc[j][3]);
     }
 }
 
@@ -364,9 +380,9 @@ __device__ __forceinline__ int stage_item(int k) {
 }
 
 // S -> D by the Y blocks: rows q P + n^2 + member(i) of each class of each degree.
-template <int NCP, int NCG>
-__device__ __forceinline__ void y_stage(const RcrArgs& a, const int* rg_y, const int* yo, const float* Y,
-                                        const float* S, float* D) {
+template <typename T, int NCP, int NCG>
+__device__ __forceinline__ void y_stage(const RcrArgs<T>& a, const int* rg_y, const int* yo, const T* Y,
+                                        const T* S, T* D) {
     const int P = a.p * a.p, total = a.nrg_y * NCG;
     for (int k = 0; k * RA_THREADS < total; ++k) {
         const int it = stage_item(k);
@@ -374,36 +390,36 @@ __device__ __forceinline__ void y_stage(const RcrArgs& a, const int* rg_y, const
         const int rg = it / NCG, cg = it - rg * NCG;
         const int code = rg_y[rg], q = code & 1, odd = (code >> 1) & 1, n = (code >> 2) & 31, og = code >> 7;
         const int sz = odd ? n : n + 1, W = pad4(sz);
-        const float* x = Y + yo[n] + (odd ? (n + 1) * pad4(n + 1) : 0) + og * 4;
-        const float* s = S + (q * P + n * n) * NCP + cg * 4;
-        float acc[4][4] = {};
+        const T* x = Y + yo[n] + (odd ? (n + 1) * pad4(n + 1) : 0) + og * 4;
+        const T* s = S + (q * P + n * n) * NCP + cg * 4;
+        T acc[4][4] = {};
         if (odd) {
 #pragma unroll 4
             for (int i = 0; i < sz; ++i)
-                fma44(acc, *reinterpret_cast<const float4*>(x + i * W),
-                      *reinterpret_cast<const float4*>(s + odd_member(i) * NCP));
+                fma44(acc, *reinterpret_cast<const Quad<T>*>(x + i * W),
+                      *reinterpret_cast<const Quad<T>*>(s + odd_member(i) * NCP));
         } else {
 #pragma unroll 4
             for (int i = 0; i < sz; ++i)
-                fma44(acc, *reinterpret_cast<const float4*>(x + i * W),
-                      *reinterpret_cast<const float4*>(s + even_member(i) * NCP));
+                fma44(acc, *reinterpret_cast<const Quad<T>*>(x + i * W),
+                      *reinterpret_cast<const Quad<T>*>(s + even_member(i) * NCP));
         }
-        float* d = D + (q * P + n * n) * NCP + cg * 4;
+        T* d = D + (q * P + n * n) * NCP + cg * 4;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int o = og * 4 + j;
             if (o < sz)
-                *reinterpret_cast<float4*>(d + (odd ? odd_member(o) : even_member(o)) * NCP) =
-                    make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+                *reinterpret_cast<Quad<T>*>(d + (odd ? odd_member(o) : even_member(o)) * NCP) =
+                    make_quad<T>(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
         }
     }
 }
 
 // S (rotated S-basis multipoles) -> D (rotated R-basis locals): the coaxial translation A_m
 // of each order, the same for phi and chi, Re and Im.
-template <int NCP, int NCG>
-__device__ __forceinline__ void coax_stage(const RcrArgs& a, const int* rg_cx, const int* co, const float* CX,
-                                           const float* S, float* D) {
+template <typename T, int NCP, int NCG>
+__device__ __forceinline__ void coax_stage(const RcrArgs<T>& a, const int* rg_cx, const int* co, const T* CX,
+                                           const T* S, T* D) {
     const int p = a.p, P = p * p, total = a.nrg_cx * NCG;
     for (int kk = 0; kk * RA_THREADS < total; ++kk) {
         const int it = stage_item(kk);
@@ -411,45 +427,45 @@ __device__ __forceinline__ void coax_stage(const RcrArgs& a, const int* rg_cx, c
         const int rg = it / NCG, cg = it - rg * NCG;
         const int code = rg_cx[rg], q = code & 1, r = (code >> 1) & 1, m = (code >> 2) & 31, og = code >> 7;
         const int k = p - m, K = pad4(k), mo = m ? 2 * m - 1 : 0;
-        const float* blk = CX + co[m] + og * 4;
-        const float* s = S + (q * P + mo + r) * NCP + cg * 4;
-        float acc[4][4] = {};
+        const T* blk = CX + co[m] + og * 4;
+        const T* s = S + (q * P + mo + r) * NCP + cg * 4;
+        T acc[4][4] = {};
 #pragma unroll 4
         for (int i = 0; i < k; ++i) {
             const int n = m + i;
-            fma44(acc, *reinterpret_cast<const float4*>(blk + i * K), *reinterpret_cast<const float4*>(s + n * n * NCP));
+            fma44(acc, *reinterpret_cast<const Quad<T>*>(blk + i * K), *reinterpret_cast<const Quad<T>*>(s + n * n * NCP));
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n2 = m + og * 4 + j;
             if (n2 < p)
-                *reinterpret_cast<float4*>(D + (q * P + n2 * n2 + mo + r) * NCP + cg * 4) =
-                    make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+                *reinterpret_cast<Quad<T>*>(D + (q * P + n2 * n2 + mo + r) * NCP + cg * 4) =
+                    make_quad<T>(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
         }
     }
 }
 
 // S -> D: the phases Z (per order m: the 2 x 2 map of (Re, Im) at z + 4 m) of both
 // potentials, per (potential, n, m) and 4 pairs.
-template <int NCP, int NCG>
-__device__ __forceinline__ void z_stage(int p, const int* units, const float* Zt, const float* S, float* D) {
+template <typename T, int NCP, int NCG>
+__device__ __forceinline__ void z_stage(int p, const int* units, const T* Zt, const T* S, T* D) {
     const int P = p * p, nu = p * (p + 1) / 2;
     for (int e = threadIdx.x; e < 2 * nu * NCG; e += RA_THREADS) {
         const int u = e / NCG, cg = e - u * NCG, q = u >= nu, info = units[u - q * nu];
         const int n = info & 31, m = info >> 5;
         const int re = q * P + n * n + (m ? 2 * m - 1 : 0);
-        const float4 x = *reinterpret_cast<const float4*>(S + re * NCP + cg * 4);
+        const Quad<T> x = *reinterpret_cast<const Quad<T>*>(S + re * NCP + cg * 4);
         if (m == 0) {
-            *reinterpret_cast<float4*>(D + re * NCP + cg * 4) = x;
+            *reinterpret_cast<Quad<T>*>(D + re * NCP + cg * 4) = x;
         } else {
-            const float4 y = *reinterpret_cast<const float4*>(S + (re + 1) * NCP + cg * 4);
-            const float4 z = *reinterpret_cast<const float4*>(Zt + 4 * m);
-            *reinterpret_cast<float4*>(D + re * NCP + cg * 4) =
-                make_float4(fmaf(z.x, x.x, z.y * y.x), fmaf(z.x, x.y, z.y * y.y), fmaf(z.x, x.z, z.y * y.z),
-                            fmaf(z.x, x.w, z.y * y.w));
-            *reinterpret_cast<float4*>(D + (re + 1) * NCP + cg * 4) =
-                make_float4(fmaf(z.z, x.x, z.w * y.x), fmaf(z.z, x.y, z.w * y.y), fmaf(z.z, x.z, z.w * y.z),
-                            fmaf(z.z, x.w, z.w * y.w));
+            const Quad<T> y = *reinterpret_cast<const Quad<T>*>(S + (re + 1) * NCP + cg * 4);
+            const Quad<T> z = *reinterpret_cast<const Quad<T>*>(Zt + 4 * m);
+            *reinterpret_cast<Quad<T>*>(D + re * NCP + cg * 4) =
+                make_quad<T>(fma(z.x, x.x, z.y * y.x), fma(z.x, x.y, z.y * y.y), fma(z.x, x.z, z.y * y.z),
+                            fma(z.x, x.w, z.y * y.w));
+            *reinterpret_cast<Quad<T>*>(D + (re + 1) * NCP + cg * 4) =
+                make_quad<T>(fma(z.z, x.x, z.w * y.x), fma(z.z, x.y, z.w * y.y), fma(z.z, x.z, z.w * y.z),
+                            fma(z.z, x.w, z.w * y.w));
         }
     }
 }
@@ -467,43 +483,44 @@ __device__ __forceinline__ void block_elem(int e, int& row, int& col) {
 
 // Gathers the source multipoles of a chunk into A (asynchronous 4-byte copies; columns of
 // absent pairs are zero).
-template <int NC, int NCP>
-__device__ __forceinline__ void gather_async(const RcrArgs& a, int p0, int np, float* A) {
+template <typename T, int NC, int NCP>
+__device__ __forceinline__ void gather_async(const RcrArgs<T>& a, int p0, int np, T* A) {
     const int R = 2 * a.p * a.p, R8 = (R + 7) & ~7;
     for (int e = threadIdx.x; e < R8 * NC; e += RA_THREADS) {
         int row, col;
         block_elem<NC>(e, row, col);
         if (row >= R) continue;
-        float* dst = A + row * NCP + col;
+        T* dst = A + row * NCP + col;
         if (col < np) {
             const int src = a.pairs[p0 + col].x;
-            const float* g = a.in + (int64_t)src * a.ld + row;
+            const T* g = a.in + (int64_t)src * a.ld + row;
             const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(g) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(g), "n"((int)sizeof(T)) : "memory");
         } else {
-            *dst = 0.f;
+            *dst = (T)0;
         }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
-template <int NC>
-__global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs a) {
+template <typename T, int NC>
+__global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
     constexpr int NCP = NC + 4;  // row stride of the buffers (16-byte aligned, 4 mod 8)
     constexpr int NCG = NC / 4;
-    extern __shared__ __align__(16) float ra_smem[];
+    extern __shared__ __align__(16) unsigned char ra_raw[];
+    T* ra_smem = reinterpret_cast<T*>(ra_raw);
     const int p = a.p, P = p * p, R = 2 * P;
     const int ysz = y_off(p);
-    float* T = ra_smem;                 // the slot's [Yf | Yb | Zf | Zb]
-    const float* Yf = T;
-    const float* Yb = T + ysz;
-    const float* Zf = T + 2 * ysz;
-    const float* Zb = Zf + 4 * p;
-    float* CX = T + a.slot_floats;      // the distance's [A blocks | tau, sigma]
-    const float* TS = CX + coax_off(p, p);
-    float* A = CX + a.coax_floats;      // gathered multipoles (the next chunk's, while the stages run)
-    float* B = A + R * NCP;
-    float* C = B + R * NCP;
+    T* tab = ra_smem;                 // the slot's [Yf | Yb | Zf | Zb]
+    const T* Yf = tab;
+    const T* Yb = tab + ysz;
+    const T* Zf = tab + 2 * ysz;
+    const T* Zb = Zf + 4 * p;
+    T* CX = tab + a.slot_floats;      // the distance's [A blocks | tau, sigma]
+    const T* TS = CX + coax_off(p, p);
+    T* A = CX + a.coax_floats;      // gathered multipoles (the next chunk's, while the stages run)
+    T* B = A + R * NCP;
+    T* C = B + R * NCP;
     int* rg_y = reinterpret_cast<int*>(C + R * NCP);
     int* rg_cx = rg_y + a.nrg_y;
     int* units = rg_cx + a.nrg_cx;      // [p (p + 1) / 2]: n | m << 5 of every order m <= n
@@ -535,7 +552,7 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs a) {
     const int c0 = (int)((int64_t)blockIdx.x * nch / gridDim.x), c1 = (int)((int64_t)(blockIdx.x + 1) * nch / gridDim.x);
     if (c0 < c1) {
         const int4 ch = a.chunks[c0];
-        gather_async<NC, NCP>(a, ch.y, ch.z, A);
+        gather_async<T, NC, NCP>(a, ch.y, ch.z, A);
     }
     int cur = -1;
     for (int chunk = c0; chunk < c1; ++chunk) {
@@ -543,26 +560,26 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs a) {
         const int slot = ch.x, p0 = ch.y, np = ch.z;
         __syncthreads();  // the previous chunk's epilogue has read B and s_dst
         if (slot != cur) {
-            const float4* sr = reinterpret_cast<const float4*>(a.rot + (int64_t)slot * a.slot_floats);
-            float4* dr = reinterpret_cast<float4*>(T);
-            for (int e = tid; e < a.slot_floats / 4; e += RA_THREADS) dr[e] = __ldg(sr + e);
-            const float4* sc = reinterpret_cast<const float4*>(a.coax + (int64_t)a.dist_of[slot] * a.coax_floats);
-            float4* dc = reinterpret_cast<float4*>(CX);
-            for (int e = tid; e < a.coax_floats / 4; e += RA_THREADS) dc[e] = __ldg(sc + e);
+            const Quad<T>* sr = reinterpret_cast<const Quad<T>*>(a.rot + (int64_t)slot * a.slot_floats);
+            Quad<T>* dr = reinterpret_cast<Quad<T>*>(tab);
+            for (int e = tid; e < a.slot_floats / 4; e += RA_THREADS) dr[e] = sr[e];
+            const Quad<T>* sc = reinterpret_cast<const Quad<T>*>(a.coax + (int64_t)a.dist_of[slot] * a.coax_floats);
+            Quad<T>* dc = reinterpret_cast<Quad<T>*>(CX);
+            for (int e = tid; e < a.coax_floats / 4; e += RA_THREADS) dc[e] = sc[e];
             cur = slot;
         }
         if (tid < NC) s_dst[tid] = tid < np ? a.pairs[p0 + tid].y : -1;
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
-        z_stage<NCP, NCG>(p, units, Zf, A, B);
+        z_stage<T, NCP, NCG>(p, units, Zf, A, B);
         __syncthreads();
         if (chunk + 1 < c1) {  // A is free: the next chunk's multipoles arrive during the stages
             const int4 nx = a.chunks[chunk + 1];
-            gather_async<NC, NCP>(a, nx.y, nx.z, A);
+            gather_async<T, NC, NCP>(a, nx.y, nx.z, A);
         }
-        y_stage<NCP, NCG>(a, rg_y, yo, Yf, B, C);
+        y_stage<T, NCP, NCG>(a, rg_y, yo, Yf, B, C);
         __syncthreads();
-        coax_stage<NCP, NCG>(a, rg_cx, co, CX, C, B);
+        coax_stage<T, NCP, NCG>(a, rg_cx, co, CX, C, B);
         __syncthreads();
         // B -> C: the conversion of Eq. rcr1, per (n, m) and 4 pairs:
         // Re phi~ = Re phi - tau Im chi, Im phi~ = Im phi + tau Re chi, chi~_n = chi_n - sigma chi_{n+1}
@@ -570,49 +587,49 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs a) {
             const int u = e / NCG, cg = e - u * NCG, info = units[u];
             const int n = info & 31, m = info >> 5, parts = m ? 2 : 1;
             const int re = n * n + (m ? 2 * m - 1 : 0);
-            const float tau = TS[(n * p + m) * 2], sigma = TS[(n * p + m) * 2 + 1];
-            float4 ph[2], ch[2];
+            const T tau = TS[(n * p + m) * 2], sigma = TS[(n * p + m) * 2 + 1];
+            Quad<T> ph[2], ch[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (k < parts) {
-                    ph[k] = *reinterpret_cast<const float4*>(B + (re + k) * NCP + cg * 4);
-                    ch[k] = *reinterpret_cast<const float4*>(B + (P + re + k) * NCP + cg * 4);
+                    ph[k] = *reinterpret_cast<const Quad<T>*>(B + (re + k) * NCP + cg * 4);
+                    ch[k] = *reinterpret_cast<const Quad<T>*>(B + (P + re + k) * NCP + cg * 4);
                 }
             }
             if (m > 0) {
-                float4 o0 = ph[0], o1 = ph[1];
-                o0.x = fmaf(-tau, ch[1].x, o0.x);
-                o0.y = fmaf(-tau, ch[1].y, o0.y);
-                o0.z = fmaf(-tau, ch[1].z, o0.z);
-                o0.w = fmaf(-tau, ch[1].w, o0.w);
-                o1.x = fmaf(tau, ch[0].x, o1.x);
-                o1.y = fmaf(tau, ch[0].y, o1.y);
-                o1.z = fmaf(tau, ch[0].z, o1.z);
-                o1.w = fmaf(tau, ch[0].w, o1.w);
-                *reinterpret_cast<float4*>(C + re * NCP + cg * 4) = o0;
-                *reinterpret_cast<float4*>(C + (re + 1) * NCP + cg * 4) = o1;
+                Quad<T> o0 = ph[0], o1 = ph[1];
+                o0.x = fma(-tau, ch[1].x, o0.x);
+                o0.y = fma(-tau, ch[1].y, o0.y);
+                o0.z = fma(-tau, ch[1].z, o0.z);
+                o0.w = fma(-tau, ch[1].w, o0.w);
+                o1.x = fma(tau, ch[0].x, o1.x);
+                o1.y = fma(tau, ch[0].y, o1.y);
+                o1.z = fma(tau, ch[0].z, o1.z);
+                o1.w = fma(tau, ch[0].w, o1.w);
+                *reinterpret_cast<Quad<T>*>(C + re * NCP + cg * 4) = o0;
+                *reinterpret_cast<Quad<T>*>(C + (re + 1) * NCP + cg * 4) = o1;
             } else {
-                *reinterpret_cast<float4*>(C + re * NCP + cg * 4) = ph[0];
+                *reinterpret_cast<Quad<T>*>(C + re * NCP + cg * 4) = ph[0];
             }
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (k < parts) {
-                    float4 c = ch[k];
+                    Quad<T> c = ch[k];
                     if (n + 1 < p) {  // chi_{n+1}^m: row + 2n + 1
-                        const float4 nx = *reinterpret_cast<const float4*>(B + (P + re + k + 2 * n + 1) * NCP + cg * 4);
-                        c.x = fmaf(-sigma, nx.x, c.x);
-                        c.y = fmaf(-sigma, nx.y, c.y);
-                        c.z = fmaf(-sigma, nx.z, c.z);
-                        c.w = fmaf(-sigma, nx.w, c.w);
+                        const Quad<T> nx = *reinterpret_cast<const Quad<T>*>(B + (P + re + k + 2 * n + 1) * NCP + cg * 4);
+                        c.x = fma(-sigma, nx.x, c.x);
+                        c.y = fma(-sigma, nx.y, c.y);
+                        c.z = fma(-sigma, nx.z, c.z);
+                        c.w = fma(-sigma, nx.w, c.w);
                     }
-                    *reinterpret_cast<float4*>(C + (P + re + k) * NCP + cg * 4) = c;
+                    *reinterpret_cast<Quad<T>*>(C + (P + re + k) * NCP + cg * 4) = c;
                 }
             }
         }
         __syncthreads();
-        y_stage<NCP, NCG>(a, rg_y, yo, Yb, C, B);
+        y_stage<T, NCP, NCG>(a, rg_y, yo, Yb, C, B);
         __syncthreads();
-        z_stage<NCP, NCG>(p, units, Zb, B, C);
+        z_stage<T, NCP, NCG>(p, units, Zb, B, C);
         __syncthreads();
         const int R8 = (R + 7) & ~7;
         for (int e = tid; e < R8 * NC; e += RA_THREADS) {
@@ -639,24 +656,19 @@ int rg_cx_count(int p) {
     return 2 * g;
 }
 
-int apply_smem(int p, int nc) {
+int apply_smem(int p, int nc, int size) {
     const int P = p * p;
     const int floats = slot_floats(p) + coax_floats(p) + 3 * (2 * P) * (nc + 4);
     const int ints = rg_y_count(p) + rg_cx_count(p) + RCR_PMAX * (RCR_PMAX + 1) / 2 + 2 * (RCR_PMAX + 1) + nc;
-    return floats * 4 + ints * 4;
+    return floats * size + ints * 4;
 }
 
-template <int NC>
-void launch_apply(Ctx* c, const RcrTables& rt, const RcrArgs& a) {
-    static int configured = 0;
-    if (configured < rt.smem) {
-        cuda_check(cudaFuncSetAttribute(k_rcr_m2l<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, rt.smem),
-                   "rcr smem");
-        cuda_check(cudaFuncSetAttribute(k_rcr_m2l<NC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100),
-                   "rcr carveout");
-        configured = rt.smem;
-    }
-    k_rcr_m2l<NC><<<rt.nsm * rt.ctas_per_sm, RA_THREADS, rt.smem, stream_of(c)>>>(a);
+template <typename T, int NC>
+void launch_apply(Ctx* c, const RcrTables& rt, const RcrArgs<T>& a) {
+    cuda_check(cudaFuncSetAttribute(k_rcr_m2l<T, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, rt.smem), "rcr smem");
+    cuda_check(cudaFuncSetAttribute(k_rcr_m2l<T, NC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100),
+               "rcr carveout");
+    k_rcr_m2l<T, NC><<<rt.nsm * rt.ctas_per_sm, RA_THREADS, rt.smem, stream_of(c)>>>(a);
 }
 
 void rot_matrix(double theta, double phi, bool inverse, bool y_part, double* q) {
@@ -706,6 +718,26 @@ void gauss_legendre_nodes(int nq, double* xi, double* w) {
     }
 }
 
+// NC a multiple of 8 keeps the row stride NC + 4 at 4 mod 8 (conflict-free columns in FP32); the
+// most resident CTAs per SM up to two (the stages are latency-bound; measured on GB300: p = 12
+// 24 pairs x 2 CTAs 121 ms against 8 x 3 129 ms; p = 16 8 x 2 249 ms against 24 x 1 317 ms),
+// then the largest chunk.  0: the tables do not fit.
+int rcr_chunk(int p, int size, int* ctas) {
+    int best = 0, pick = 0;
+    if (p < 1 || p > RCR_PMAX) return 0;
+    for (int nc : {32, 24, 16, 8}) {
+        const int sm = apply_smem(p, nc, size);
+        if (sm > SMEM_MAX) continue;
+        const int k = std::min(2, SMEM_PER_SM / (sm + 1024));
+        if (k * 64 + nc > best) {
+            best = k * 64 + nc;
+            pick = nc;
+            if (ctas) *ctas = k;
+        }
+    }
+    return pick;
+}
+
 void rcr_free(RcrTables& rt) {
     for (Buf* b : {&rt.rot, &rt.coax, &rt.dist_of}) {
         if (b->ptr) cudaFree(b->ptr);
@@ -715,6 +747,7 @@ void rcr_free(RcrTables& rt) {
     rt.p = 0;
 }
 
+template <typename T>
 void rcr_build(Ctx* c, int p, RcrTables& rt) {
     if (p < 1 || p > RCR_PMAX) throw Error{LHV_EUNSUPPORTED, "RCR translations run p <= 20"};
     cudaStream_t s = stream_of(c);
@@ -722,20 +755,27 @@ void rcr_build(Ctx* c, int p, RcrTables& rt) {
     std::vector<int> offs, slot_of;
     m2l_offsets(offs, slot_of);
     // per slot: t = target - source = -(source offset) = |t| (sin th cos ph, sin th sin ph, cos th)
-    std::vector<RotJob> jobs(NUM_OFFSETS * 4);
+    // the blocks depend on theta or phi alone, which many offsets share: one job per distinct angle
+    std::vector<RotJob> jobs;
+    std::vector<int> job_of;
+    std::map<std::pair<int, long long>, int> known;  // (which of the four, angle in units of 1e-12) -> job
     for (int k = 0; k < NUM_OFFSETS; ++k) {
         const double tx = -offs[3 * k], ty = -offs[3 * k + 1], tz = -offs[3 * k + 2];
         const double tl = std::sqrt(tx * tx + ty * ty + tz * tz);
         const double th = std::acos(std::max(-1.0, std::min(1.0, tz / tl)));
         const double ph = std::atan2(ty, tx);
-        rot_matrix(th, ph, false, true, jobs[4 * k + 0].q);   // Y(theta), S basis
-        jobs[4 * k + 0].r_basis = 0;
-        rot_matrix(th, ph, true, true, jobs[4 * k + 1].q);    // Y(-theta), R basis
-        jobs[4 * k + 1].r_basis = 1;
-        rot_matrix(th, ph, false, false, jobs[4 * k + 2].q);  // Z(phi), S basis
-        jobs[4 * k + 2].r_basis = 0;
-        rot_matrix(th, ph, true, false, jobs[4 * k + 3].q);   // Z(-phi), R basis
-        jobs[4 * k + 3].r_basis = 1;
+        // Y(theta), S basis; Y(-theta), R basis; Z(phi), S basis; Z(-phi), R basis
+        for (int which = 0; which < 4; ++which) {
+            const bool y = which < 2, inverse = (which & 1) != 0;
+            const auto at = known.emplace(std::make_pair(which, std::llround((y ? th : ph) * 1e12)), (int)jobs.size());
+            if (at.second) {
+                jobs.emplace_back();
+                rot_matrix(th, ph, inverse, y, jobs.back().q);
+                jobs.back().r_basis = inverse ? 1 : 0;
+                jobs.back().pad = 0;
+            }
+            job_of.push_back(at.first->second);
+        }
     }
     std::vector<double> xq(p), wq(p);
     gauss_legendre_nodes(p, xq.data(), wq.data());
@@ -760,13 +800,16 @@ void rcr_build(Ctx* c, int p, RcrTables& rt) {
     }
     const int P = p * p, NE = p * (4 * p * p - 1) / 3;
     const int sf = slot_floats(p), cf = coax_floats(p);
-    Buf djobs, dq, dense, fused, ddist, dres;
+    Buf djobs, djob_of, dq, dense, fused, ddist, dres;
     float resid = 0.f;
     auto cleanup = [&] {
-        for (Buf* b : {&djobs, &dq, &dense, &fused, &ddist, &dres}) cudaFree(b->ptr);
+        for (Buf* b : {&djobs, &djob_of, &dq, &dense, &fused, &ddist, &dres}) cudaFree(b->ptr);
     };
     try {
         ensure(c, djobs, (int64_t)jobs.size() * sizeof(RotJob));
+        ensure(c, djob_of, (int64_t)job_of.size() * 4);
+        cuda_check(cudaMemcpyAsync(djob_of.ptr, job_of.data(), job_of.size() * 4, cudaMemcpyHostToDevice, s),
+                   "rcr job index");
         ensure(c, dq, 2 * p * 8);
         ensure(c, dense, (int64_t)jobs.size() * NE * 8);
         ensure(c, dres, 16);
@@ -782,15 +825,15 @@ void rcr_build(Ctx* c, int p, RcrTables& rt) {
                                                                     dq.as<double>() + p, dense.as<double>());
         count_launch(c);
         check_launch("rcr rotations");
-        ensure(c, rt.rot, (int64_t)NUM_OFFSETS * sf * 4);
-        k_rcr_pack<<<NUM_OFFSETS, 256, 0, s>>>(dense.as<double>(), p, sf, rt.rot.as<float>(), dres.as<float>());
+        ensure(c, rt.rot, (int64_t)NUM_OFFSETS * sf * (int64_t)sizeof(T));
+        k_rcr_pack<T><<<NUM_OFFSETS, 256, 0, s>>>(dense.as<double>(), djob_of.as<int>(), p, sf, rt.rot.as<T>(), dres.as<float>());
         count_launch(c);
         check_launch("rcr pack");
         build_m2l_at(c, p, t3, fused);
         ensure(c, ddist, (int64_t)dist.size() * 8);
         cuda_check(cudaMemcpyAsync(ddist.ptr, dist.data(), dist.size() * 8, cudaMemcpyHostToDevice, s), "rcr dist");
-        ensure(c, rt.coax, (int64_t)d2s.size() * cf * 4);
-        k_rcr_coax<<<(int)d2s.size(), 256, 0, s>>>(fused.as<double>(), ddist.as<double>(), p, cf, rt.coax.as<float>(),
+        ensure(c, rt.coax, (int64_t)d2s.size() * cf * (int64_t)sizeof(T));
+        k_rcr_coax<T><<<(int)d2s.size(), 256, 0, s>>>(fused.as<double>(), ddist.as<double>(), p, cf, rt.coax.as<T>(),
                                                    dres.as<float>() + 1);
         count_launch(c);
         check_launch("rcr coaxial");
@@ -813,41 +856,27 @@ void rcr_build(Ctx* c, int p, RcrTables& rt) {
         throw Error{LHV_EUNSUPPORTED, "RCR tables failed their structural check"};
     }
     rt.p = p;
+    rt.type = (int)sizeof(T);
     rt.slot_floats = sf;
     rt.coax_floats = cf;
     rt.resid = resid;
-    // NC a multiple of 8 keeps the row stride NC + 4 at 4 mod 8 (conflict-free columns); the
-    // most resident CTAs per SM up to two (the stages are latency-bound; measured on GB300: p = 12
-    // 24 pairs x 2 CTAs 121 ms against 8 x 3 129 ms; p = 16 8 x 2 249 ms against 24 x 1 317 ms),
-    // then the largest chunk
-    rt.nc = 0;
-    rt.ctas_per_sm = 1;
-    int best = 0;
-    for (int nc : {32, 24, 16, 8}) {
-        const int sm = apply_smem(p, nc);
-        if (sm > SMEM_MAX) continue;
-        const int k = std::min(2, SMEM_PER_SM / (sm + 1024));
-        if (k * 64 + nc > best) {
-            best = k * 64 + nc;
-            rt.nc = nc;
-            rt.ctas_per_sm = k;
-        }
-    }
+    rt.nc = rcr_chunk(p, sizeof(T), &rt.ctas_per_sm);
     if (rt.nc == 0) throw Error{LHV_EUNSUPPORTED, "RCR tables exceed shared memory"};
-    rt.smem = apply_smem(p, rt.nc);
+    rt.smem = apply_smem(p, rt.nc, sizeof(T));
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     rt.nsm = sms > 0 ? sms : 152;
 }
 
-void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const float* mult, float* loc, int64_t ld) {
-    RcrArgs a{};
+template <typename T>
+void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const T* mult, T* loc, int64_t ld) {
+    RcrArgs<T> a{};
     a.chunks = gp.chunks.as<int4>();
     a.pairs = gp.pairs.as<int2>();
     a.nchunks = gp.choff.as<int>() + gp.ngroups;
-    a.rot = rt.rot.as<float>();
-    a.coax = rt.coax.as<float>();
+    a.rot = rt.rot.as<T>();
+    a.coax = rt.coax.as<T>();
     a.dist_of = rt.dist_of.as<int>();
     a.in = mult;
     a.out = loc;
@@ -858,13 +887,18 @@ void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const float* mult, floa
     a.nrg_y = rg_y_count(rt.p);
     a.nrg_cx = rg_cx_count(rt.p);
     switch (rt.nc) {
-        case 32: launch_apply<32>(c, rt, a); break;
-        case 24: launch_apply<24>(c, rt, a); break;
-        case 16: launch_apply<16>(c, rt, a); break;
-        default: launch_apply<8>(c, rt, a); break;
+        case 32: launch_apply<T, 32>(c, rt, a); break;
+        case 24: launch_apply<T, 24>(c, rt, a); break;
+        case 16: launch_apply<T, 16>(c, rt, a); break;
+        default: launch_apply<T, 8>(c, rt, a); break;
     }
     count_launch(c);
     check_launch("rcr m2l");
 }
+
+template void rcr_build<float>(Ctx*, int, RcrTables&);
+template void rcr_build<double>(Ctx*, int, RcrTables&);
+template void rcr_apply<float>(Ctx*, const RcrTables&, Grouped&, const float*, float*, int64_t);
+template void rcr_apply<double>(Ctx*, const RcrTables&, Grouped&, const double*, double*, int64_t);
 
 }  // namespace lhv

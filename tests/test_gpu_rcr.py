@@ -89,3 +89,53 @@ def test_unsupported():
         with pytest.raises(LHVError) as e:
             c.evaluate_velocity_stretching(dev(x, kw["prec"]), dev(w, kw["prec"]))
         assert e.value.status == -6
+
+
+def _default_and_fused(run, **kw):
+    """run(context) with the default M2L of the two-potential form and with the fused tables
+    (chosen by a CUDA-core chunk)."""
+    from paper_1201_5430_gb300 import LHV
+    out = []
+    for nc in (0, 64):
+        c = LHV(**kw)
+        c.set_launch_shape(m2l_pairs_per_chunk=nc)
+        out.append(run(c))
+        assert c.stats()["m2l_pairs"] > 0
+        c.close()
+    return out
+
+
+@pytest.mark.parametrize("prec,p", [("fp32", p) for p in (3, 4, 5, 7, 8, 10, 13, 17, 20, 21)]
+                         + [("fp64", p) for p in (4, 7, 12, 16, 17)] + [("tf32x3", 10)])
+@pytest.mark.parametrize("n,leaf", [(700, 8), (6000, 16)])
+def test_default_translations_equal_the_fused_tables(prec, p, n, leaf):
+    """The default M2L of the two-potential form (RCR where its tables fit) against the fused
+    tables, far field only, few and many pairs a chunk, p outside RCR's range included.  Both
+    sides round about 2 p^2 terms: sqrt(2 21^2) 2^-24 = 2e-6 in FP32; in FP64 the quadrature of the
+    rotation blocks adds 2 p^2 terms of its own, 1e-12."""
+    x, w = workloads.cube(n, 11)
+    e = "fp64" if prec == "fp64" else "fp32"
+
+    def run(c):
+        v4, s4 = c.evaluate_velocity_stretching(dev(x, e), dev(w, e))
+        return host3(v4), host3(s4)
+
+    a, b = _default_and_fused(run, p=p, leaf_max=leaf, core_a=0.0, precision=prec, terms="far")
+    tol = 1e-12 if prec == "fp64" else 2e-6
+    assert rel(a[0], b[0]) < tol and rel(a[1], b[1]) < tol, (rel(a[0], b[0]), rel(a[1], b[1]))
+
+
+def test_default_translations_of_filaments_and_batches():
+    import torch
+    th = 2 * np.pi * np.arange(3000) / 3000
+    x = np.stack([np.cos(th), np.sin(th), np.zeros(3000)], axis=1).astype(np.float32)
+    g = torch.ones(3000, device="cuda")
+    a, b = _default_and_fused(lambda c: host3(c.evaluate_filaments([0, 3000], [True], dev(x, "fp32"), g)),
+                              p=12, leaf_max=16, core_a=0.0, precision="fp32", terms="far")
+    assert rel(a, b) < 2e-6, rel(a, b)
+    systems = workloads.blob_systems(nsys=3, seed=9, n_lo=1e3, n_hi=4e3)
+    xs, ws = (np.concatenate([q[k] for q in systems]) for k in (0, 1))
+    off = np.cumsum([0] + [q[0].shape[0] for q in systems]).tolist()
+    a, b = _default_and_fused(lambda c: host3(c.evaluate_batched(off, dev(xs, "fp32"), dev(ws, "fp32"))[0]),
+                              p=8, leaf_max=16, core_a=0.0, precision="fp32", terms="far")
+    assert rel(a, b) < 2e-6, rel(a, b)

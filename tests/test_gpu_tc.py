@@ -71,7 +71,7 @@ def test_m2l_converts_like_the_fused_table(p, n, leaf):
     got = {}
     for tc in (1, 0):
         ctx = LHV(p=p, leaf_max=leaf, core_a=0.0, precision="tf32x3", terms="far")
-        ctx.set_launch_shape(m2l_tensor_cores=tc)
+        ctx.set_launch_shape(m2l_pairs_per_chunk=64, m2l_tensor_cores=tc)
         v4, s4 = ctx.evaluate_velocity_stretching(dev(x, "fp32"), dev(w, "fp32"))
         pg = ctx.evaluate_potential_gradient(dev(x, "fp32"), q)
         st = ctx.stats()  # raises if a tensor-core wait timed out
