@@ -1,74 +1,32 @@
 // Generated by gen_core_fit.py -- do not edit.
-// Gaussian core of Eq. vem1, x = r/a, u = x^2 (the FP32 near-field kernel).
-// x < 1.5: K/x^3 = sqrt(2/pi) sum_k kSerF[k] s^k, d/du = sqrt(2/pi) sum_k kSerFp[k] s^k,
-//   s = (2u - 2.25)/2.25; max rel. errors 3.4e-08, 5.7e-08 (coefficients in FP32).
-// 1.5 <= x < 6.5: 1 - K = exp(-u/2) (sum_k kCoreFit[k] t^k + sqrt(2/pi) x), y = 1/x,
-//   t = (2y - 0.82051282051282048)/0.51282051282051277; max rel. error 8.2e-07 of the sum.
-//   Packed kernel: 1 - K = exp(-u/2) x G(y), G = y E + sqrt(2/pi) = -sum_k kCoreFitG2[k] t^k;
-//   max rel. error 5.7e-08 of G.
+// Gaussian core of Eq. vem1, x = r/a, u = x^2 (the packed FP32 near-field kernel; host arrays,
+// the kernel gets them with their powers of a).
+// x < 1.5: d(K/x^3)/du = sqrt(2/pi) sum_k kSerFp[k] s^k, s = (2u - 2.25)/2.25; max rel.
+//   error 5.7e-08 (coefficients in FP32); K/x^3 = (sqrt(2/pi) exp(-u/2) - 2u d(K/x^3)/du) / 3.
+// 1.5 <= x < 6.5: 1 - K = exp(-u/2) x G(y), G = sum_k kCoreFitG[k] t^k, y = 1/x,
+//   t = (2y - 0.82051282051282048)/0.51282051282051277; evaluated in FP32 the error of G
+//   makes at most 8.9e-08 (rms 1.4e-08) of K/r^3 and 2.3e-07 (2.6e-08) of its derivative term.
 #pragma once
 #define LHV_CORE_SER_DEG 7
-#define LHV_CORE_FIT_DEG 7
+#define LHV_CORE_G_DEG 5
 #define LHV_CORE_U_SER 2.25f
 #define LHV_CORE_Y_SCALE 3.900000000e+00f
 #define LHV_CORE_Y_SHIFT -1.600000000e+00f
-static __device__ __constant__ const float kSerF[8] = {
-    2.404837310e-01f,
-    -7.583419234e-02f,
-    1.466703136e-02f,
-    -2.087964211e-03f,
-    2.362600353e-04f,
-    -2.221878458e-05f,
-    1.804490580e-06f,
-    -1.267918179e-07f,
+static const double kSerFp[8] = {
+    -6.74081702080310124e-02,
+    2.60747194054093585e-02,
+    -5.56790498970447228e-03,
+    8.40070911140781257e-04,
+    -9.87481726321254294e-05,
+    9.53937180547165568e-06,
+    -7.90512838604255385e-07,
+    5.63989132908741876e-08,
 };
-static __device__ __constant__ const float kSerFp[8] = {
-    -6.740816683e-02f,
-    2.607471868e-02f,
-    -5.567905027e-03f,
-    8.400708903e-04f,
-    -9.874817624e-05f,
-    9.539371604e-06f,
-    -7.905128427e-07f,
-    5.639891398e-08f,
-};
-static __device__ __constant__ const float kCoreFit[8] = {
-    2.884729803e-01f,
-    1.443179101e-01f,
-    -2.340069599e-02f,
-    1.839783392e-03f,
-    6.155305309e-04f,
-    -3.799752740e-04f,
-    1.085868716e-04f,
-    -1.276623516e-05f,
-};
-static __device__ __constant__ const float2 kSerF2[8] = {
-    {2.404837310e-01f, 2.404837310e-01f},
-    {-7.583419234e-02f, -7.583419234e-02f},
-    {1.466703136e-02f, 1.466703136e-02f},
-    {-2.087964211e-03f, -2.087964211e-03f},
-    {2.362600353e-04f, 2.362600353e-04f},
-    {-2.221878458e-05f, -2.221878458e-05f},
-    {1.804490580e-06f, 1.804490580e-06f},
-    {-1.267918179e-07f, -1.267918179e-07f},
-};
-static __device__ __constant__ const float2 kSerFp2[8] = {
-    {-6.740816683e-02f, -6.740816683e-02f},
-    {2.607471868e-02f, 2.607471868e-02f},
-    {-5.567905027e-03f, -5.567905027e-03f},
-    {8.400708903e-04f, 8.400708903e-04f},
-    {-9.874817624e-05f, -9.874817624e-05f},
-    {9.539371604e-06f, 9.539371604e-06f},
-    {-7.905128427e-07f, -7.905128427e-07f},
-    {5.639891398e-08f, 5.639891398e-08f},
-};
-static __device__ __constant__ const float2 kCoreFitG2[8] = {
-    {-9.162324667e-01f, -9.162324667e-01f},
-    {-1.331747770e-01f, -1.331747770e-01f},
-    {-2.740348876e-02f, -2.740348876e-02f},
-    {5.245395470e-03f, 5.245395470e-03f},
-    {-7.283564191e-04f, -7.283564191e-04f},
-    {-1.941047685e-06f, -1.941047685e-06f},
-    {5.942788630e-05f, 5.942788630e-05f},
-    {-2.260535803e-05f, -2.260535803e-05f},
+static const double kCoreFitG[6] = {
+    9.16232455621992070e-01,
+    1.33175404977378425e-01,
+    2.74009021387655836e-02,
+    -5.24410439707704169e-03,
+    7.46741134718980314e-04,
+    -5.25932156033631076e-05,
 };

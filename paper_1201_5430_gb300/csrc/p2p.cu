@@ -8,15 +8,13 @@
 //   s_i = (sum_j f w_j) x w_i + sum_j g (w_i . d) (w_j x d),   g = f'/r.
 // K evaluation, x = r/a:
 //   x >= x_cut  : K = 1 to the working precision (f = 1/r^3, g = -3/r^5);
-//   x <  x_ser  : K/x^3 as a function of x^2 (dK/dx = sqrt(2/pi) x^2 e^{-x^2/2}
-//                 integrates term by term into a series without the cancellation
-//                 of the closed form at small x): in FP32 a degree-7 Chebyshev
-//                 interpolant of it and of its derivative on x^2 < 2.25, in FP64
-//                 the series itself below x = 1;
-//   otherwise   : K = 1 - exp(-x^2/2) R(x), R(x) = exp(x^2/2) erfc(x/sqrt 2) +
-//                 sqrt(2/pi) x with its first term a degree-7 Chebyshev
-//                 interpolant in 1/x (FP32; the packed kernel interpolates
-//                 G = R / x instead, so that K / r^3 = 1/r^3 - exp(-x^2/2) G / (a r^2)),
+//   x <  x_ser  : in FP32 the derivative of K/x^3 by x^2 as a degree-7 Chebyshev interpolant on
+//                 x^2 < 2.25, and K/x^3 from it (dK/dx = sqrt(2/pi) x^2 e^{-x^2/2}, so
+//                 K/x^3 = (sqrt(2/pi) e^{-x^2/2} - 2 x^2 (K/x^3)') / 3, a sum of positive terms
+//                 without the cancellation of the closed form at small x); in FP64 the
+//                 series of both below x = 1;
+//   otherwise   : K = 1 - exp(-x^2/2) x G(1/x), G(1/x) = exp(x^2/2) erfc(x/sqrt 2) / x + sqrt(2/pi) a
+//                 degree-5 polynomial in 1/x (FP32: K / r^3 = 1/r^3 - exp(-x^2/2) G / (a r^2)),
 //                 or Eq. vem1 with erf (FP64).
 // The self pair j = i is excluded only in the source chunk that can hold it.
 // The far-field result (L2P) of the same element is added and the sum is
@@ -36,14 +34,14 @@ namespace lhv {
 namespace {
 
 template <typename T> struct CoreConsts {
-    T a, inv_a, inv_a2, c3, c5;  // a, 1/a, 1/a^2, sqrt(2/pi)/a^3, sqrt(2/pi)/a^5
-    T x2_cut;                 // (r/a)^2 beyond which K = 1 in this precision
-    T u_series;               // (r/a)^2 below which the Taylor series is used
-    // packed FP32x2 kernel: r^2 cut, a LHV_CORE_Y_SCALE, -sqrt(2/pi)/(3 a^3), -(2/3) sqrt(2/pi)/a^5
-    T r2_cut, t_scale, c3_3n, c5_g;
-    // packed kernel, fit region: log2(exp(-u/2) / a) = ue_scale r^2 + ue_shift; -sqrt(2/pi)/(3 a^2);
-    // (r/a)^2 of the series region as r^2
-    T ue_scale, ue_shift, c3_3a, r2_series;
+    // FP64 kernel: 1/a, 1/a^2, sqrt(2/pi)/a^3, sqrt(2/pi)/a^5, (r/a)^2 beyond which K = 1 and
+    // (r/a)^2 below which the series is used
+    T inv_a, inv_a2, c3, c5, x2_cut, u_series;
+    // packed FP32x2 kernel: r^2 cut, a LHV_CORE_Y_SCALE; exp(-u/2) = 2^(e_scale r^2); c33 =
+    // sqrt(2/pi)/(3 a^3); bound of the series region as r^2, its s = ser_scale r^2 - 1
+    T r2_cut, t_scale, e_scale, c33, r2_series, ser_scale;
+    float2 gfit[LHV_CORE_G_DEG + 1];    // -G / a in powers of t (both lanes alike)
+    float2 sfit[LHV_CORE_SER_DEG + 1];  // -(2/3) sqrt(2/pi) / a^5 F' in powers of s
     int smooth;
 };
 
@@ -79,44 +77,8 @@ __device__ __forceinline__ float ex2_ftz(float x) {
     return y;
 }
 
-// f = K/r^3 and g = f'/r for one pair.  The singular part 1/r^3 is shared; the
-// core correction (divergent, only for r < x_cut a) replaces it.
-template <bool SMOOTH>
-__device__ __forceinline__ void kernel_fg(float r2, const CoreConsts<float>& cc, float& f, float& g) {
-    const float ri = rsqrt_ftz(r2);
-    const float ri2 = ri * ri;
-    f = ri * ri2;
-    if (SMOOTH) {
-        const float u = r2 * cc.inv_a2;
-        if (u < cc.x2_cut) {
-            if (u < cc.u_series) {
-                const float s = fmaf(u, 2.0f / LHV_CORE_U_SER, -1.0f);
-                float F = kSerF[LHV_CORE_SER_DEG], Fp = kSerFp[LHV_CORE_SER_DEG];
-#pragma unroll
-                for (int k = LHV_CORE_SER_DEG - 1; k >= 0; --k) {
-                    F = fmaf(F, s, kSerF[k]);
-                    Fp = fmaf(Fp, s, kSerFp[k]);
-                }
-                f = cc.c3 * F;
-                g = 2.0f * cc.c5 * Fp;
-                return;
-            }
-            const float t = fmaf(cc.a * ri, LHV_CORE_Y_SCALE, LHV_CORE_Y_SHIFT);  // y = 1/x = a/r
-            float E = kCoreFit[LHV_CORE_FIT_DEG];
-#pragma unroll
-            for (int k = LHV_CORE_FIT_DEG - 1; k >= 0; --k) E = fmaf(E, t, kCoreFit[k]);
-            const float x = r2 * ri * cc.inv_a;
-            const float R = fmaf(0.79788456080286535588f, x, E);
-            const float e = ex2_ftz(u * -0.72134752044448170368f);  // exp(-u/2)
-            const float K = fmaf(-e, R, 1.0f);
-            f *= K;
-            g = (cc.c3 * e - 3.0f * f) * ri2;
-            return;
-        }
-    }
-    g = -3.0f * f * ri2;
-}
-
+// f = K/r^3 and g = f'/r for one pair (FP64).  The singular part 1/r^3 is shared; the core
+// correction (divergent, only for r < x_cut a) replaces it.
 template <bool SMOOTH>
 __device__ __forceinline__ void kernel_fg(double r2, const CoreConsts<double>& cc, double& f, double& g) {
     if (SMOOTH) {
@@ -331,66 +293,68 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-// kernel_fg for two pairs at once, returning f and gm = -g/3 (the factor -3
-// is applied to the finished sums).  fg2_singular gives the packed singular
-// part; fg2_core then replaces it where either lane lies inside x_cut a: the
-// interpolant of each region that a lane needs is evaluated for both lanes and
-// taken by the lanes in that region.  Inside the fit region f = f_s (1 - e R)
-// with f_s = 1/r^3 and e = exp(-u/2), and gm = (f - sqrt(2/pi) e / (3 a^3)) / r^2.
-__device__ __forceinline__ void fg2_singular(float2 r2, float2& ri, float2& ri2, float2& f, float2& gm) {
+// f and gm = -g/3 of two pairs at once (the factor -3 is applied to the finished sums).
+// fg2_singular gives ri = 1/r, ri2 = 1/r^2 and f = f_s = 1/r^3; fg2_core then gives gm = f / r^2,
+// or where any lane of the warp lies inside x_cut a the core's f and gm: inside the fit region
+// f = f_s - e (G / a) / r^2 with e = exp(-u/2), and gm = (f - sqrt(2/pi) e / (3 a^3)) / r^2.
+__device__ __forceinline__ void fg2_singular(float2 r2, float2& ri, float2& ri2, float2& f) {
     ri.x = rsqrt_ftz(r2.x);
     ri.y = rsqrt_ftz(r2.y);
     ri2 = mul2(ri, ri);
     f = mul2(ri, ri2);
-    gm = mul2(f, ri2);
 }
 
 // Core correction for SU source pairs at once (their chains interleave).  The
 // branches are warp-uniform votes: every lane of the warp runs the pair loop.
 // The fit-region form is exact to FP32 rounding for every x >= 1.5 (beyond
-// x_cut, e R and e/(3 a^3) r^3 are below the unit roundoff, so f and gm come out
+// x_cut, e G / (a r^2) and e/(3 a^3) are below the unit roundoff of f, so f and gm come out
 // unchanged), so it is applied to every lane without a per-lane choice; the
 // series then overrides the lanes with x < 1.5.
+// Bound by the FMA pipe like the pair loop.  Packed operations a source pair: fit 10 (t, degree-5
+// Horner, exponent, three products and two sums, less the singular gm), series 10 more.  With a degree-7 G, an
+// interpolant each for the series' f and g and the singular gm formed before the vote (13 and 18), and
+// log2(a) in the exponent, a launch took 137.4 ms on the leapfrog pair of 2^22 and 1.33 ms on the ring
+// of 2^18, against 134.4 and 1.26 ms; near field against FP64 on that ring: v 5.9e-8 both, s 7.9e-7 and
+// 7.8e-7.
 template <int SU>
 __device__ __forceinline__ void fg2_core(const float2 (&r2)[SU], const float2 (&ri)[SU], const float2 (&ri2)[SU],
                                          const CoreConsts<float>& cc, float2 (&f)[SU], float2 (&gm)[SU]) {
     float rmin = fminf(r2[0].x, r2[0].y);
 #pragma unroll
     for (int v = 1; v < SU; ++v) rmin = fminf(rmin, fminf(r2[v].x, r2[v].y));
-    if (!__any_sync(0xffffffffu, rmin < cc.r2_cut)) return;
-    // 1 - K = exp(-u/2) x G(y), so f K = f - (exp(-u/2) / a) G / r^2 (f r^3 = 1, x = r/a):
-    // e = exp(-u/2) / a in one fma and one ex2, the fit -G in y = a/r
+    if (!__any_sync(0xffffffffu, rmin < cc.r2_cut)) {
+#pragma unroll
+        for (int v = 0; v < SU; ++v) gm[v] = mul2(f[v], ri2[v]);
+        return;
+    }
+    // 1 - K = exp(-u/2) x G(y), so f K = f - exp(-u/2) (G / a) / r^2 (f r^3 = 1, x = r/a).  The power
+    // of a stays out of the exponent, where log2(a) would cost e a few units of its last place.
+    float2 e[SU];
 #pragma unroll
     for (int v = 0; v < SU; ++v) {
         const float2 t = fma2(ri[v], dup2(cc.t_scale), dup2(LHV_CORE_Y_SHIFT));  // from y = 1/x = a/r
-        float2 nG = kCoreFitG2[LHV_CORE_FIT_DEG];
+        float2 nG = cc.gfit[LHV_CORE_G_DEG];
 #pragma unroll
-        for (int k = LHV_CORE_FIT_DEG - 1; k >= 0; --k) nG = fma2(nG, t, kCoreFitG2[k]);  // -G(y)
-        const float2 ue = fma2(r2[v], dup2(cc.ue_scale), dup2(cc.ue_shift));
-        float2 e;
-        e.x = ex2_ftz(ue.x);
-        e.y = ex2_ftz(ue.y);
-        f[v] = fma2(mul2(ri2[v], e), nG, f[v]);
-        gm[v] = mul2(fma2(e, dup2(cc.c3_3a), f[v]), ri2[v]);
+        for (int k = LHV_CORE_G_DEG - 1; k >= 0; --k) nG = fma2(nG, t, cc.gfit[k]);  // -G(y) / a
+        const float2 ue = mul2(r2[v], dup2(cc.e_scale));
+        e[v].x = ex2_ftz(ue.x);
+        e[v].y = ex2_ftz(ue.y);
+        f[v] = fma2(mul2(ri2[v], e[v]), nG, f[v]);
+        gm[v] = mul2(fma2(e[v], dup2(-cc.c33), f[v]), ri2[v]);
     }
     if (!__any_sync(0xffffffffu, rmin < cc.r2_series)) return;
 #pragma unroll
     for (int v = 0; v < SU; ++v) {
-        const float2 u = mul2(r2[v], dup2(cc.inv_a2));
-        const float2 s = fma2(u, dup2(2.0f / LHV_CORE_U_SER), dup2(-1.0f));
-        float2 F = kSerF2[LHV_CORE_SER_DEG], Fp = kSerFp2[LHV_CORE_SER_DEG];
+        const float2 s = fma2(r2[v], dup2(cc.ser_scale), dup2(-1.0f));
+        float2 gs = cc.sfit[LHV_CORE_SER_DEG];
 #pragma unroll
-        for (int k = LHV_CORE_SER_DEG - 1; k >= 0; --k) {
-            F = fma2(F, s, kSerF2[k]);
-            Fp = fma2(Fp, s, kSerFp2[k]);
-        }
-        const float2 fs = mul2(dup2(cc.c3), F);
-        const float2 gs = mul2(dup2(cc.c5_g), Fp);
-        if (u.x < cc.u_series) {
+        for (int k = LHV_CORE_SER_DEG - 1; k >= 0; --k) gs = fma2(gs, s, cc.sfit[k]);
+        const float2 fs = fma2(r2[v], gs, mul2(e[v], dup2(cc.c33)));
+        if (r2[v].x < cc.r2_series) {
             f[v].x = fs.x;
             gm[v].x = gs.x;
         }
-        if (u.y < cc.u_series) {
+        if (r2[v].y < cc.r2_series) {
             f[v].y = fs.y;
             gm[v].y = gs.y;
         }
@@ -561,9 +525,14 @@ __global__ void __launch_bounds__(32 * P2P_WARPS) k_p2p_x2(const int* __restrict
                             dy[u] = add2(XI[q][1], nyj[u]);
                             dz[u] = add2(XI[q][2], nzj[u]);
                             r2[u] = fma2(dz[u], dz[u], fma2(dy[u], dy[u], mul2(dx[u], dx[u])));
-                            fg2_singular(r2[u], ri[u], ri2[u], f[u], gm[u]);
+                            fg2_singular(r2[u], ri[u], ri2[u], f[u]);
                         }
-                        if (SMOOTH) fg2_core<SU>(r2, ri, ri2, cc, f, gm);
+                        if constexpr (SMOOTH) {
+                            fg2_core<SU>(r2, ri, ri2, cc, f, gm);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < SU; ++u) gm[u] = mul2(f[u], ri2[u]);
+                        }
 #pragma unroll
                         for (int u = 0; u < SU; ++u) {
                             if (decltype(check)::value) {
@@ -1069,7 +1038,6 @@ void run_p2p(Ctx* c, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs, 
     cc.smooth = a > 0.0;
     if (cc.smooth) {
         const double s2pi = 0.79788456080286535588;
-        cc.a = (T)a;
         cc.inv_a = (T)(1.0 / a);
         cc.inv_a2 = (T)(1.0 / (a * a));
         cc.c3 = (T)(s2pi / (a * a * a));
@@ -1077,19 +1045,25 @@ void run_p2p(Ctx* c, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs, 
         // beyond x_cut, 1 - K and the K' term are below the unit roundoff
         const double xc = sizeof(T) == 4 ? 6.5 : 9.0;
         cc.x2_cut = (T)(xc * xc);
-        cc.u_series = (T)(sizeof(T) == 4 ? LHV_CORE_U_SER : 1.0);
+        cc.u_series = (T)1.0;
         // the packed FP32 kernel's warp vote: the core fit runs for a step only if a pair lies
         // inside r_K (1 - K < eps/10 beyond it, the criterion of the tree's core rule and of the
         // far field, which takes K = 1 for every pair it handles), capped at x_cut a
         const double rv = ctx_rK(c) > 0.0 ? std::min(xc * a, ctx_rK(c)) : xc * a;
         cc.r2_cut = (T)(rv * rv);
         cc.t_scale = (T)(a * (double)LHV_CORE_Y_SCALE);
-        cc.c3_3n = (T)(-s2pi / (3.0 * a * a * a));
-        cc.c5_g = (T)(-2.0 / 3.0 * s2pi / (a * a * a * a * a));
-        cc.ue_scale = (T)(-0.5 / (a * a * 0.69314718055994530942));  // -u/2 in base 2
-        cc.ue_shift = (T)(-std::log2(a));
-        cc.c3_3a = (T)(-s2pi / (3.0 * a * a));
-        cc.r2_series = (T)((sizeof(T) == 4 ? LHV_CORE_U_SER : 1.0) * a * a);
+        cc.e_scale = (T)(-0.5 / (a * a * 0.69314718055994530942));  // -u/2 in base 2
+        cc.c33 = (T)(s2pi / (3.0 * a * a * a));
+        cc.r2_series = (T)(LHV_CORE_U_SER * a * a);
+        cc.ser_scale = (T)(2.0 / (LHV_CORE_U_SER * a * a));
+        for (int k = 0; k <= LHV_CORE_G_DEG; ++k) {
+            const float g = (float)(-kCoreFitG[k] / a);
+            cc.gfit[k] = make_float2(g, g);
+        }
+        for (int k = 0; k <= LHV_CORE_SER_DEG; ++k) {
+            const float g = (float)(-2.0 / 3.0 * s2pi / (a * a * a * a * a) * kSerFp[k]);
+            cc.sfit[k] = make_float2(g, g);
+        }
     }
     int* work = reinterpret_cast<int*>(ctx_tmp(c, 6).ptr);
     ensure(c, ctx_tmp(c, 6), 64);
