@@ -281,6 +281,154 @@ __global__ void __launch_bounds__(P2P_TILE / TPT) k_p2p(const int* __restrict__ 
     if (threadIdx.x == 0 && my_pairs) atomicAdd(pairs, my_pairs);
 }
 
+// The same sums with S source strands (FP64): a block of P2P_TILE threads takes P2P_TILE / S targets
+// of a tile, thread t target t % (P2P_TILE / S) over the sources of strand t / (P2P_TILE / S) of every
+// stage; the strands' totals are added at the end.  A leaf of ten elements fills 8 % of k_p2p's
+// block and 62 % of this one's at S = 8; past P2P_TILE / 2 elements a leaf S = 1 (k_p2p) wastes less than
+// half.  FP64 ring of 32768 elements (10 a leaf): 12.4 ms a launch with k_p2p, 4.4 ms with
+// S = 8.
+template <typename T, bool SMOOTH, int S, int CH>
+__global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict__ ntiles_dev,
+                                                         const int2* __restrict__ tiles, int* __restrict__ work,
+                                                         const int* __restrict__ bbeg, const int* __restrict__ bend,
+                                                         const int* __restrict__ bcol,
+                                                         const vec4_t<T>* __restrict__ xs,
+                                                         const vec4_t<T>* __restrict__ ws,
+                                                         const int* __restrict__ perm,
+                                                         const vec4_t<T>* __restrict__ vfar,
+                                                         const vec4_t<T>* __restrict__ sfar,
+                                                         vec4_t<T>* __restrict__ vout, vec4_t<T>* __restrict__ sout,
+                                                         CoreConsts<T> cc, int near,
+                                                         unsigned long long* __restrict__ pairs) {
+    constexpr int TW = P2P_TILE / S;     // targets per work item
+    constexpr int NA = 9;
+    __shared__ vec4_t<T> sx[CH];
+    __shared__ vec4_t<T> sw[CH];
+    __shared__ int sid[CH];
+    __shared__ T part[NA][P2P_TILE];
+    __shared__ int cbeg[27], cpre[28];
+    __shared__ int cur;
+    const int nitems = *ntiles_dev * S;
+    const int strand = threadIdx.x / TW, tg = threadIdx.x % TW;
+    unsigned long long my_pairs = 0;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) cur = atomicAdd(work, 1);
+        __syncthreads();
+        const int item = cur;
+        if (item >= nitems) break;
+        const int2 tw = tiles[item / S];
+        const int leaf = tw.x, t0 = tw.y + (item % S) * TW;
+        const int tend = min(bend[leaf], tw.y + P2P_TILE);
+        if (t0 >= tend) continue;  // block-uniform
+        if (threadIdx.x < 32) {  // lane q < 27 reads colleague q; a warp scan gives the prefix counts
+            int cnt = 0, beg = 0;
+            if (threadIdx.x < 27) {
+                const int cb = bcol[(int64_t)leaf * 27 + threadIdx.x];
+                if (cb >= 0) {
+                    beg = bbeg[cb];
+                    cnt = bend[cb] - beg;
+                }
+            }
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (threadIdx.x >= o) incl += v;
+            }
+            if (threadIdx.x < 27) {
+                cbeg[threadIdx.x] = beg;
+                cpre[threadIdx.x] = incl - cnt;
+            }
+            if (threadIdx.x == 26) cpre[27] = incl;
+        }
+        const int ti = t0 + tg;
+        const bool act = ti < tend;
+        const vec4_t<T> xi = act ? xs[ti] : vec4_t<T>{};
+        const vec4_t<T> wi = act ? ws[ti] : vec4_t<T>{};
+        T hi[NA], lo[NA];
+#pragma unroll
+        for (int a = 0; a < NA; ++a) hi[a] = lo[a] = 0;
+        __syncthreads();
+        const int nsrc = near ? cpre[27] : 0;
+        if (threadIdx.x == 0 && near)
+            my_pairs += (unsigned long long)min(TW, tend - t0) * (unsigned long long)(nsrc - 1);
+        int qrun = 0;  // colleague of this thread's last staged source (its sources only move forward)
+        for (int s0 = 0; s0 < nsrc; s0 += CH) {
+            for (int v = s0 + threadIdx.x; v < min(nsrc, s0 + CH); v += P2P_TILE) {
+                while (cpre[qrun + 1] <= v) ++qrun;
+                const int j = cbeg[qrun] + (v - cpre[qrun]);
+                sx[v - s0] = xs[j];
+                sw[v - s0] = ws[j];
+                sid[v - s0] = j;
+            }
+            __syncthreads();
+            const int ns = min(CH, nsrc - s0);
+            T acc[NA];
+#pragma unroll
+            for (int a = 0; a < NA; ++a) acc[a] = 0;
+            if (act)
+                for (int k = strand; k < ns; k += S) {
+                    const vec4_t<T> xj = sx[k];
+                    const vec4_t<T> wj = sw[k];
+                    const T dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
+                    T f, g;
+                    kernel_fg<SMOOTH>(dx * dx + dy * dy + dz * dz, cc, f, g);
+                    if (sid[k] == ti) {
+                        f = 0;
+                        g = 0;
+                    }
+                    const T cx = wj.y * dz - wj.z * dy;
+                    const T cy = wj.z * dx - wj.x * dz;
+                    const T cz = wj.x * dy - wj.y * dx;
+                    acc[0] += f * cx;
+                    acc[1] += f * cy;
+                    acc[2] += f * cz;
+                    acc[3] += f * wj.x;
+                    acc[4] += f * wj.y;
+                    acc[5] += f * wj.z;
+                    const T h = g * (wi.x * dx + wi.y * dy + wi.z * dz);
+                    acc[6] += h * cx;
+                    acc[7] += h * cy;
+                    acc[8] += h * cz;
+                }
+#pragma unroll
+            for (int a = 0; a < NA; ++a) two_sum_acc(hi[a], lo[a], acc[a]);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) part[a][threadIdx.x] = hi[a] + lo[a];
+        __syncthreads();
+        if (strand == 0 && act) {
+            T r[NA];
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                r[a] = part[a][tg];
+                for (int q = 1; q < S; ++q) r[a] += part[a][q * TW + tg];
+            }
+            vec4_t<T> vf{}, sf{};
+            if (vfar) {
+                vf = vfar[ti];
+                sf = sfar[ti];
+            }
+            vec4_t<T> vo, so;
+            vo.x = vf.x + r[0];
+            vo.y = vf.y + r[1];
+            vo.z = vf.z + r[2];
+            vo.w = 0;
+            // (sum_j f w_j) x w_i + sum_j g (w_i . d)(w_j x d)
+            so.x = sf.x + (r[4] * wi.z - r[5] * wi.y) + r[6];
+            so.y = sf.y + (r[5] * wi.x - r[3] * wi.z) + r[7];
+            so.z = sf.z + (r[3] * wi.y - r[4] * wi.x) + r[8];
+            so.w = 0;
+            const int o = perm[ti];
+            vout[o] = vo;
+            sout[o] = so;
+        }
+    }
+    if (threadIdx.x == 0 && my_pairs) atomicAdd(pairs, my_pairs);
+}
+
 // ---- packed FP32x2 form of the same pair loop (float only) ----
 // Each add/mul/fma of the pair loop works on a float2 holding two sources of
 // the stage (2m, 2m+1); the target's values are duplicated into both lanes.
@@ -1107,7 +1255,29 @@ void run_p2p(Ctx* c, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs, 
     using C128 = std::integral_constant<int, 128>;
     using C256 = std::integral_constant<int, 256>;
     const bool wide = ctx_p2p_sources(c) == 256;
-    switch (ctx_p2p_tpt(c)) {
+    // FP64 at one target per thread (the default): source strands where the mean leaf fills less
+    // than half of a tile
+    int strands = 1;
+    if constexpr (!std::is_same<T, float>::value) {
+        if (ctx_p2p_tpt(c) == 1)
+            while (strands < 8 && n * strands < (int64_t)lv.nbox[L] * (P2P_TILE / 2)) strands *= 2;
+        auto launch_strands = [&](auto st) {
+            constexpr int S = decltype(st)::value;
+            int per_sm = 1, sms = 152, dev = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            auto kern = cc.smooth ? k_p2p_strands<T, true, S, 128> : k_p2p_strands<T, false, S, 128>;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P2P_TILE, 0);
+            const int grid = (int)std::min<int64_t>(max_tiles * S, (int64_t)sms * std::max(per_sm, 1));
+            kern<<<grid, P2P_TILE, 0, s>>>(tb.tile_count.as<int>(), tb.tiles.as<int2>(), work, tb.bbeg.as<int>() + o,
+                                           tb.bend.as<int>() + o, tb.bcol.as<int>() + (int64_t)o * 27, xs, ws, perm,
+                                           vfar, sfar, v_out, s_out, cc, near ? 1 : 0, pair_counter);
+        };
+        if (strands == 2) launch_strands(I2{});
+        else if (strands == 4) launch_strands(I4{});
+        else if (strands == 8) launch_strands(std::integral_constant<int, 8>{});
+    }
+    if (strands == 1) switch (ctx_p2p_tpt(c)) {
         case 2: wide ? launch(I2{}, C256{}) : launch(I2{}, C128{}); break;
         case 4: wide ? launch(I4{}, C256{}) : launch(I4{}, C128{}); break;
         default: wide ? launch(I1{}, C256{}) : launch(I1{}, C128{}); break;

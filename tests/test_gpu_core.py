@@ -44,3 +44,24 @@ def test_pairs_across_the_core(a, tpt):
         sv, ss = f * nj * r, (f + np.abs(g) * r * r) * nj * ni
         assert np.max(np.linalg.norm(v[i::2] - ve, axis=1) / sv) < 1.5e-6
         assert np.max(np.linalg.norm(s[i::2] - se, axis=1) / ss) < 1.5e-6
+
+
+@pytest.mark.parametrize("n,leaf", [(300, 4), (2000, 12), (4000, 24), (4000, 48), (3001, 150)])
+@pytest.mark.parametrize("a", [0.0, 0.03])
+def test_fp64_source_strands_equal_one_strand(n, leaf, a):
+    """FP64 near field with 1 to 8 source strands (mean leaves from a few elements to more than a
+    tile) against the unsplit kernel (two targets per thread): the same terms in another order,
+    n 2^-53 of the sum of their sizes at most; s cancels to about 1e-3 of it."""
+    import workloads
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n, 3)
+    got = []
+    for tpt in (1, 2):
+        c = LHV(p=4, leaf_max=leaf, core_a=a, precision="fp64", terms="near")
+        c.set_launch_shape(p2p_targets_per_thread=tpt)
+        v4, s4 = c.evaluate_velocity_stretching(dev(x, "fp64"), dev(w, "fp64"))
+        got.append((host3(v4), host3(s4), c.stats()["p2p_pairs"]))
+        c.close()
+    assert got[0][2] == got[1][2]
+    for p, q in zip(got[0][:2], got[1][:2]):
+        assert np.linalg.norm(p - q) < n * 2.0 ** -53 * 1e3 * np.linalg.norm(q)
