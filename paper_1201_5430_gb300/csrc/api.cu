@@ -425,7 +425,6 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
         const int64_t nleaf = lv.nbox[L];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
         ensure(c, c->loc, nbt * pl.ld * (int64_t)sizeof(T));
-        ensure(c, c->table, (nbt - lv.off[2]) * (int64_t)NUM_OFFSETS * 4);
         ensure(c, c->W, nleaf * 3 * PL * (int64_t)sizeof(T));
         ensure(c, c->vfar, n * (int64_t)sizeof(vec4_t<T>));
         ensure(c, c->sfar, n * (int64_t)sizeof(vec4_t<T>));
@@ -453,7 +452,7 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
             // the tensor-core kernel takes 128 pairs per MMA; the CUDA-core kernel at most 64
             const int nc = pl.rcr ? pl.rcr->nc
                                   : all_tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * pmax * pmax));
-            m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, pl.uniform, cnt + 1);
+            m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
             m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
                          mult, loc);
@@ -573,7 +572,6 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
         const int64_t nbt = lv.off[L + 1];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
         ensure(c, c->loc, nbt * pl.ld * (int64_t)sizeof(T));
-        ensure(c, c->table, (nbt - lv.off[2]) * (int64_t)NUM_OFFSETS * 4);
         ensure(c, c->pgfar, n * (int64_t)sizeof(vec4_t<T>));
         T* mult = c->mult.as<T>();
         T* loc = c->loc.as<T>();
@@ -590,7 +588,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             fill_level_rows<T>(c, lv, c->tb.counts.as<int>(), 2, L, pl.ld, 0, loc, (T)0);  // zero locals
             const bool tc = sizeof(T) == 4 && ctx_m2l_tc(c) && pl.m2l_tiles[2];
             const int nc = tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(P));
-            m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, true, cnt + 1);
+            m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, true, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
             m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
                          mult, loc);
@@ -718,7 +716,6 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
         const int64_t nbt = lv.off[L + 1];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
         ensure(c, c->loc, nbt * pl.ld * (int64_t)sizeof(T));
-        ensure(c, c->table, (nbt - lv.off[2]) * (int64_t)NUM_OFFSETS * 4);
         ensure(c, c->W, (int64_t)lv.nbox[L] * 3 * PL * (int64_t)sizeof(T));
         ensure(c, c->vfar, n * (int64_t)sizeof(vec4_t<T>));
         ensure(c, c->sfar, n * (int64_t)sizeof(vec4_t<T>));
@@ -737,7 +734,7 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
             fill_level_rows<T>(c, lv, c->tb.counts.as<int>(), 2, L, pl.ld, 0, loc, (T)0);
             const bool tc = sizeof(T) == 4 && ctx_m2l_tc(c) && pl.m2l_tiles[2];
             const int nc = pl.rcr ? pl.rcr->nc : tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * PL));
-            m2l_prepare(c, c->ops, c->tb, lv, c->table.as<int>(), c->gp_m2l, nc, pl.uniform, cnt + 1);
+            m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
             m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
                          mult, loc);

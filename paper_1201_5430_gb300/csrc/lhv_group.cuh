@@ -141,14 +141,12 @@ struct OctItems {
     }
 };
 
-// M2L: rows of the interaction table (global target box, 316 slots -> global source box or -1).
-// by_level = false: group = offset slot (pairs of all levels share the operator);
-// by_level = true : group = (level - 2) * 316 + slot (each level has its own p).
+// M2L with a truncation number per level: rows of the interaction table (global target box, 316
+// slots -> global source box or -1); group = (level - 2) * 316 + slot.
 struct M2LItems {
     const int* table;  // rows for the target slots [t0, ...)
     const int* loff;   // real boxes before each level (device)
     int t0;
-    bool by_level;
     int L;
     int off[MAX_LEVELS + 2];  // global box offsets of the levels
     __device__ int64_t limit() const { return (int64_t)(loff[L + 1] - loff[2]) * NUM_OFFSETS; }
@@ -159,9 +157,8 @@ struct M2LItems {
         d = off[l] + (rb - loff[l]);
         const int src = table[(int64_t)(d - t0) * NUM_OFFSETS + slot];
         if (src < 0) return false;
-        g = slot;
+        g = (l - 2) * NUM_OFFSETS + slot;
         s = src;
-        if (by_level) g += (l - 2) * NUM_OFFSETS;
         return true;
     }
 };

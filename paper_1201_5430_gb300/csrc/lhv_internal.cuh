@@ -265,9 +265,9 @@ void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels&
                     const T* loc, vec4_t<T>* pgfar);
 
 // ---- M2L (m2l.cu) ------------------------------------------------------------
-// table: (off[L+1] - off[2]) * 316 ints; nc: pairs per GEMM chunk (gemm_nc).
-// uniform: pairs of all levels bucketed by offset; else by (level, offset).
-void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& lv, int* table, Grouped& gp,
+// The pair list gp: nc pairs per GEMM chunk (gemm_nc).  uniform: pairs of all levels bucketed by
+// offset; else by (level, offset), through the interaction table in `table_buf`.
+void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& lv, Buf& table_buf, Grouped& gp,
                  int nc, bool uniform, unsigned long long* pair_counter);
 // the products; loc must be zero for levels >= 2; count: boxes per level (device); offsets:
 // OpTables::offsets.

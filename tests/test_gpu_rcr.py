@@ -139,3 +139,43 @@ def test_default_translations_of_filaments_and_batches():
     a, b = _default_and_fused(lambda c: host3(c.evaluate_batched(off, dev(xs, "fp32"), dev(ws, "fp32"))[0]),
                               p=8, leaf_max=16, core_a=0.0, precision="fp32", terms="far")
     assert rel(a, b) < 2e-6, rel(a, b)
+
+
+@pytest.mark.parametrize("n,leaf,nsys", [(65, 1, 1), (700, 1, 1), (3000, 8, 1), (20000, 4, 1), (900, 4, 7)])
+def test_pair_list_against_the_definition(n, leaf, nsys):
+    """The M2L pair list (blocks of target boxes, pairs ranked per offset slot): as many pairs as the
+    interaction lists of the exported boxes hold, and as the list of the route with a truncation number
+    per level (the interaction table); few and many boxes a block, several systems.  What the pairs
+    carry is compared with the oracle elsewhere."""
+    from paper_1201_5430_gb300 import LHV
+    rng = np.random.default_rng(n)
+    x = rng.random((n * nsys, 3)).astype(np.float32)
+    w = rng.standard_normal((n * nsys, 3)).astype(np.float32)
+    off = [n * k for k in range(nsys + 1)]
+    got = []
+    for mixed in (False, True):
+        c = LHV(p=6, leaf_max=leaf, core_a=0.0, precision="fp32", terms="far")
+        c.set_launch_shape(m2l_pairs_per_chunk=64)
+        if mixed:
+            c.set_level_p([0, 0, 5])
+        c.evaluate_batched(off, dev(x, "fp32"), dev(w, "fp32"))
+        st = c.stats()
+        if not mixed:
+            L = st["leaf_level"]
+            want = 0
+            for l in range(2, L + 1):
+                keys = c.export("box_keys", l).cpu().numpy().astype(np.uint64)
+                sysid = keys >> np.uint64(3 * l)
+                q = np.zeros((keys.size, 3), dtype=np.int64)
+                for b in range(l):
+                    for d in range(3):
+                        q[:, d] |= ((keys >> np.uint64(3 * b + d)) & np.uint64(1)).astype(np.int64) << b
+                for i in range(keys.size):
+                    same = sysid == sysid[i]
+                    far = np.abs(q - q[i]).max(axis=1) > 1
+                    near_parent = np.abs((q >> 1) - (q[i] >> 1)).max(axis=1) <= 1
+                    want += int(np.sum(same & far & near_parent))
+            assert st["m2l_pairs"] == want
+        got.append(st["m2l_pairs"])
+        c.close()
+    assert got[0] == got[1]
