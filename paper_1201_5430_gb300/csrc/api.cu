@@ -49,7 +49,8 @@ struct Ctx {
     int level_p[MAX_LEVELS + 1] = {};   // lhv_set_level_p (0: cfg.p)
     std::map<int, Buf> opcache;         // tables of other (kind, p_out, p_in) than ops, type opcache_type
     int opcache_type = 0;
-    std::map<int, Csr> spcache;         // sparse P2M / L2P of other p than ops, type spcache_type
+    std::map<int, Sell> spcache;        // sparse P2M / L2P of other p than ops, type spcache_type
+    std::map<int, Buf> qtabs;           // harmonics' recurrence tables of other p, type spcache_type
     int spcache_type = 0;
     int eval_p[MAX_LEVELS + 1] = {};    // truncation numbers of the last evaluation's expansions
     int eval_ld = 0;                    // their stride (reals per box)
@@ -203,8 +204,9 @@ static void ensure_ops(Ctx* c) {
     c->have_m2l = false;
     StageScope sc(c, LHV_STAGE_OPS);
     build_operators<T>(c, c->cfg.p, c->ops);
-    build_sparse<T>(c, OP_P2M, c->cfg.p, c->ops.p2m_sp);
-    build_sparse<T>(c, OP_L2P, c->cfg.p, c->ops.l2p_sp);
+    build_sparse<T>(c, OP_P2M, c->cfg.p, 0, c->ops.p2m_sp);
+    build_sparse<T>(c, OP_L2P, c->cfg.p, 0, c->ops.l2p_sp);
+    build_qtab<T>(c, c->cfg.p, c->ops.qtab);
     c->ops_type = (int)sizeof(T);
     if constexpr (sizeof(T) == 4) {
         if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
@@ -239,31 +241,44 @@ static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
 }
 
 template <typename T>
-static CsrView<T> view(const Csr& m) {
-    CsrView<T> v;
-    v.rowptr = m.rowptr.as<int>();
+static SellView<T> view(const Sell& m) {
+    SellView<T> v;
+    v.sptr = m.sptr.as<int>();
     v.col = m.col.as<int>();
     v.val = m.val.as<T>();
     v.rows = m.rows;
     return v;
 }
 
-// P2M / L2P of truncation number p in row-compressed form, from the cache.
+// P2M / L2P of truncation number p as a sparse map from the cache; v_only: the v_k rows of L2P.
 template <typename T>
-static CsrView<T> cached_sparse(Ctx* c, int kind, int p) {
+static SellView<T> cached_sparse(Ctx* c, int kind, int p, bool v_only = false) {
     if (c->spcache_type != (int)sizeof(T)) {
-        for (auto& kv : c->spcache) free_csr(kv.second);
+        for (auto& kv : c->spcache) free_sparse(kv.second);
         c->spcache.clear();
+        for (auto& kv : c->qtabs) release(kv.second);
+        c->qtabs.clear();
         c->spcache_type = (int)sizeof(T);
     }
-    const int key = kind | (p << 8);
+    const int key = kind | (p << 8) | (v_only ? 1 << 16 : 0);
     auto it = c->spcache.find(key);
     if (it == c->spcache.end()) {
         StageScope sc(c, LHV_STAGE_OPS);
-        build_sparse<T>(c, kind, p, c->spcache[key]);
+        build_sparse<T>(c, kind, p, v_only ? 3 * p * p : 0, c->spcache[key]);
         it = c->spcache.find(key);
     }
     return view<T>(it->second);
+}
+
+// The v_k rows of L2P(p): filaments and the scalar case need no gradient.
+template <typename T>
+static SellView<T> velocity_rows(Ctx* c, int p) {
+    if (p != c->cfg.p) return cached_sparse<T>(c, OP_L2P, p, true);
+    if (c->ops.l2pv_sp.rows == 0) {
+        StageScope sc(c, LHV_STAGE_OPS);
+        build_sparse<T>(c, OP_L2P, p, 3 * p * p, c->ops.l2pv_sp);
+    }
+    return view<T>(c->ops.l2pv_sp);
 }
 
 // Tables of the complex form Psi = phi + i chi (Sec. 4.2): M F M^-1 of the fused tables.
@@ -335,14 +350,13 @@ static Plan<T> make_plan(Ctx* c, int L) {
             throw Error{LHV_EUNSUPPORTED, "the complex form runs one truncation number at every level"};
         ensure_psi_ops<T>(c);
         pl.psi = true;
-        pl.p2m = c->ops.p2m.as<T>();
-        pl.l2p = c->ops.l2p.as<T>();
         for (int l = 0; l <= L; ++l) {
             pl.m2m[l] = c->psi_m2m.as<T>();
             pl.l2l[l] = c->psi_l2l.as<T>();
             pl.m2l[l] = c->psi_m2l.as<T>();
             pl.m2l_tiles[l] = c->psi_tiles.ptr ? c->psi_tiles.as<float>() : nullptr;
         }
+        pl.qtab = c->ops.qtab.as<T>();
         pl.p2m_sp = view<T>(c->ops.p2m_sp);
         pl.l2p_sp = view<T>(c->ops.l2p_sp);
         return pl;
@@ -350,21 +364,21 @@ static Plan<T> make_plan(Ctx* c, int L) {
     if (base) {
         const bool tiles = tc && ctx_m2l_tc(c) && c->ops.m2l_tiles.ptr;
         const T* m2l = pl.rcr || tiles ? nullptr : fused_m2l<T>(c);
-        pl.p2m = c->ops.p2m.as<T>();
-        pl.l2p = c->ops.l2p.as<T>();
         for (int l = 0; l <= L; ++l) {
             pl.m2m[l] = c->ops.m2m.as<T>();
             pl.l2l[l] = c->ops.l2l.as<T>();
             pl.m2l[l] = m2l;
             pl.m2l_tiles[l] = c->ops.m2l_tiles.ptr ? c->ops.m2l_tiles.as<float>() : nullptr;
         }
+        pl.qtab = c->ops.qtab.as<T>();
         pl.p2m_sp = view<T>(c->ops.p2m_sp);
         pl.l2p_sp = view<T>(c->ops.l2p_sp);
         return pl;
     }
-    pl.p2m = cached_op<T>(c, OP_P2M, pl.p[L], pl.p[L]);
-    pl.l2p = cached_op<T>(c, OP_L2P, pl.p[L], pl.p[L]);
     pl.p2m_sp = cached_sparse<T>(c, OP_P2M, pl.p[L]);
+    Buf& qt = c->qtabs[pl.p[L]];  // emptied with the sparse maps when the type changes
+    if (!qt.ptr) build_qtab<T>(c, pl.p[L], qt);
+    pl.qtab = qt.as<T>();
     pl.l2p_sp = cached_sparse<T>(c, OP_L2P, pl.p[L]);
     for (int l = 2; l <= L; ++l) {
         pl.m2l[l] = cached_op<T>(c, OP_M2L, pl.p[l], pl.p[l]);
@@ -568,7 +582,8 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             pl.m2l[l] = c->s_m2l.as<T>();
             pl.m2l_tiles[l] = c->s_tiles.ptr ? c->s_tiles.as<float>() : nullptr;
         }
-        pl.l2p_sp = view<T>(c->ops.l2p_sp);
+        pl.qtab = c->ops.qtab.as<T>();
+        pl.l2p_sp = velocity_rows<T>(c, p);
         const int64_t nbt = lv.off[L + 1];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
         ensure(c, c->loc, nbt * pl.ld * (int64_t)sizeof(T));
@@ -709,7 +724,8 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
     vec4_t<T>* vfar = nullptr;
     c->have_far = far;
     if (far) {
-        const Plan<T> pl = make_plan<T>(c, L);
+        Plan<T> pl = make_plan<T>(c, L);
+        pl.l2p_sp = velocity_rows<T>(c, pl.p[L]);  // v at the nodes alone
         for (int l = 0; l <= MAX_LEVELS; ++l) c->eval_p[l] = l <= L ? pl.p[l] : 0;
         c->eval_ld = pl.ld;
         const int PL = pl.p[L] * pl.p[L];
@@ -718,7 +734,6 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
         ensure(c, c->loc, nbt * pl.ld * (int64_t)sizeof(T));
         ensure(c, c->W, (int64_t)lv.nbox[L] * 3 * PL * (int64_t)sizeof(T));
         ensure(c, c->vfar, n * (int64_t)sizeof(vec4_t<T>));
-        ensure(c, c->sfar, n * (int64_t)sizeof(vec4_t<T>));
         T* mult = c->mult.as<T>();
         T* loc = c->loc.as<T>();
         {
@@ -745,8 +760,8 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
         }
         vfar = c->vfar.as<vec4_t<T>>();
         {
-            StageScope sc(c, LHV_STAGE_L2P);  // v at the nodes (the s lanes are not used)
-            run_l2p<T>(c, pl, c->tb, lv, xs, segs, loc, vfar, c->sfar.as<vec4_t<T>>());
+            StageScope sc(c, LHV_STAGE_L2P);
+            run_l2p<T>(c, pl, c->tb, lv, xs, segs, loc, vfar, nullptr);
         }
     }
     {
@@ -1246,7 +1261,9 @@ void lhv_destroy(lhv_ctx* ctx) {
     lhv::rcr_free(c.rcr);
     for (auto& kv : c.opcache) lhv::release(kv.second);
     c.opcache.clear();
-    for (auto& kv : c.spcache) lhv::free_csr(kv.second);
+    for (auto& kv : c.spcache) lhv::free_sparse(kv.second);
+    for (auto& kv : c.qtabs) lhv::release(kv.second);
+    c.qtabs.clear();
     c.spcache.clear();
     for (auto* b : {&c.sel_W, &c.sel_b, &c.sel_X, &c.sel_Z, &c.sel_choice, &c.sel_idx, &c.sel_dv, &c.sel_ds, &c.sel_err,
                     &c.s_m2l, &c.s_m2m, &c.s_l2l, &c.s_tiles, &c.qs, &c.pgfar, &c.psi_m2l, &c.psi_m2m,
@@ -1255,7 +1272,7 @@ void lhv_destroy(lhv_ctx* ctx) {
     lhv::TreeBufs& t = c.tb;
     lhv::Buf* tree[] = {&t.keys_a, &t.keys_b, &t.idx_a, &t.idx_b, &t.hist, &t.boxof_a, &t.boxof_b, &t.flags,
                         &t.scan_tmp, &t.perm, &t.params, &t.counts, &t.bkey, &t.bbeg, &t.bend, &t.bparent,
-                        &t.bcbeg, &t.bcend, &t.bcol, &t.tiles, &t.tile_count, &t.cubes, &t.sysoff};
+                        &t.bcbeg, &t.bcend, &t.bcol, &t.tiles, &t.tile_count, &t.geom, &t.cubes, &t.sysoff};
     for (auto* b : tree) lhv::release(*b);
     for (auto& b : c.tmp) lhv::release(b);
     lhv::Buf* rest[] = {&c.xs, &c.ws, &c.mult, &c.loc, &c.table, &c.vfar, &c.sfar, &c.counters, &c.hx, &c.hw,

@@ -9,6 +9,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
+#include <type_traits>
+#include <vector>
 
 #include "lhv_group.cuh"
 #include "lhv_internal.cuh"
@@ -17,22 +20,9 @@ namespace lhv {
 
 namespace {
 
-// Centre and side of a box from its key prefix at `level` (Morton bits interleaved
-// x, y, z from bit 0; the system id above bit 3*level selects the cube).
-__device__ inline void box_geom(const SysCube* __restrict__ cubes, uint64_t key, int level, double& cx, double& cy,
-                                double& cz, double& h) {
-    const SysCube cb = cubes[level > 0 ? (key >> (3 * level)) : key];
-    h = ldexp(cb.side, -level);
-    uint64_t c[3] = {0, 0, 0};
-    for (int b = 0; b < level; ++b)
-        for (int ax = 0; ax < 3; ++ax) c[ax] |= ((key >> (3 * b + ax)) & 1ull) << b;
-    cx = cb.x0[0] + ((double)c[0] + 0.5) * h;
-    cy = cb.x0[1] + ((double)c[1] + 0.5) * h;
-    cz = cb.x0[2] + ((double)c[2] + 0.5) * h;
-}
-
 // Coefficients of the recurrences of Q_n^m for n, m < p (they depend on (n, m)
-// only), built once per block in shared memory from double-precision values:
+// only), formed once per context in double precision (lhv::build_qtab) and copied to shared memory by
+// each block (p = 12: 312 reals; formed by every block they took it 7,000 cycles of the FP64 pipe):
 //   Q_m^m     = cm[m] (x + i y) Q_{m-1}^{m-1},        cm[m] = -sqrt((2m - 1) / (2m)),
 //   Q_{m+1}^m = c1[m] z Q_m^m,                        c1[m] = sqrt(2m + 1),
 //   Q_n^m     = A[m][n] z Q_{n-1}^m - B[m][n] r^2 Q_{n-2}^m,
@@ -47,24 +37,9 @@ struct QTab {
 __host__ __device__ inline int qtab_reals(int p) { return 2 * p * p + 2 * p; }
 
 template <typename T>
-__device__ inline QTab<T> build_qtab(T* base, int p) {
-    QTab<T> q{base, base + p * p, base + 2 * p * p, base + 2 * p * p + p, p};
-    for (int i = threadIdx.x; i < p * p; i += blockDim.x) {
-        const int m = i / p, n = i - m * p;
-        double a = 0.0, b = 0.0;
-        if (n >= m + 2) {
-            const double d = (double)((n + m) * (n - m));
-            a = (double)(2 * n - 1) / sqrt(d);
-            b = sqrt((double)((n + m - 1) * (n - m - 1)) / d);
-        }
-        q.A[i] = (T)a;
-        q.B[i] = (T)b;
-    }
-    for (int m = threadIdx.x; m < p; m += blockDim.x) {
-        q.cm[m] = m > 0 ? (T)(-sqrt((double)(2 * m - 1) / (double)(2 * m))) : (T)0;
-        q.c1[m] = (T)sqrt((double)(2 * m + 1));
-    }
-    return q;
+__device__ inline QTab<T> load_qtab(T* base, const T* __restrict__ src, int p) {
+    for (int i = threadIdx.x; i < qtab_reals(p); i += blockDim.x) base[i] = src[i];
+    return QTab<T>{base, base + p * p, base + 2 * p * p, base + 2 * p * p + p, p};
 }
 
 // Walks every (n, m), 0 <= m <= n < p, of the recurrence of Q_n^m at (x, y, z)
@@ -103,26 +78,50 @@ __device__ inline void for_each_Q(int p, T x, T y, T z, const QTab<T>& q, F&& f,
     }
 }
 
+// out[r] = sum of the sparse map's row r over `in` (shared memory), f(r, sum): the warps of a block
+// take the slices in turn.
+template <typename T, typename F>
+__device__ inline void sparse_rows(const SellView<T>& m, const T* in, int warp, int nwarps, F&& f) {
+    const int lane = threadIdx.x & 31;
+    for (int q = warp; 32 * q < m.rows; q += nwarps) {
+        const int b = m.sptr[q], e = m.sptr[q + 1];
+        T acc = 0;
+#pragma unroll 3
+        for (int i = b + lane; i < e; i += 32) {
+            const T v = m.val[i], x = in[m.col[i]];
+            if (v != (T)0) acc += v * x;  // a padding entry adds nothing, whatever its input holds
+        }
+        const int r = 32 * q + lane;
+        if (r < m.rows) f(r, acc);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // P2M, part 1 (per leaf): W_k = sum_e w_{e,k} g_hat(rho_e), where
 // g_hat_n^m = nu_n^m R_n^{-m}(-rho) = i^m conj(Q_n^m(rho)), rho = (x - c)/h.
 // Part 2 is the grouped GEMM  M_hat = (1/h) [G_x G_y G_z] [W_x; W_y; W_z]
 // with G_k the scaled real form of Eq. eve4 for w = i_k.
 // ---------------------------------------------------------------------------
-constexpr int P2M_THREADS = 128;
-constexpr int P2M_MAX_OUT = (3 * 24 * 24 + P2M_THREADS - 1) / P2M_THREADS;  // W entries per thread, p <= 24
+// Blocks of 128 threads over chunks of up to 128 elements, or of 64 threads over 32 where the mean leaf
+// is small: a block's shared memory then holds the rows of 32 elements, and an SM 11 blocks instead
+// of two (p = 12).  P2M of the sphere surface of 2^20 (15 elements a leaf) 1.86 -> 0.48 ms, of the ring
+// of 32,768 (10) 0.140 -> 0.060; of the leapfrog pair (440), where an entry of the harmonics is
+// now read once for its three strengths, 2.12 -> 1.45 ms at p = 16.
+constexpr int P2M_THREADS = 128, P2M_SMALL = 64;
+constexpr int P2M_SMALL_LEAF = 48;  // mean elements per leaf up to which the small blocks are taken
+constexpr int p2m_max_out(int threads) { return (24 * 24 + threads - 1) / threads; }  // (n, m) entries per thread, p <= 24
 
 // Row stride of the staged harmonics: odd, so that the lanes of a warp, each writing entry k of
 // its own element's row, fall in 32 different shared-memory banks (a stride of p^2 = 256 put all
 // 32 in one bank).
 __host__ __device__ inline int p2m_row_stride(int P) { return P | 1; }
 
-// Shared memory of k_p2m_w and the elements per chunk: the largest chunk (128, 64 or 32
-// elements) whose rows, strengths and recurrence table fit in 80 KB (two blocks per SM).
+// Shared memory of k_p2m_w and the elements per chunk: the largest chunk (`most`, at least 32,
+// halved) whose rows, strengths and recurrence table fit in 80 KB (two blocks per SM).
 template <typename T>
-size_t p2m_smem(int p, int& chunk) {
-    const size_t row = (size_t)p2m_row_stride(p * p) + 3;
-    chunk = 128;
+size_t p2m_smem(int p, int most, int& chunk) {
+    const size_t row = (size_t)p2m_row_stride(p * p) + 4;
+    chunk = most;
     while (chunk > 32 && sizeof(T) * (chunk * row + qtab_reals(p)) > 80 * 1024) chunk /= 2;
     return sizeof(T) * (chunk * row + qtab_reals(p));
 }
@@ -136,37 +135,43 @@ size_t p2m_smem(int p, int& chunk) {
 // SEG (NC = 3): the element is a filament node owning the segment x -> x + l with
 // circulation Gamma, ws = (l, Gamma): W gets (Gamma l / (8 pi h)) sum_j w_j g_hat(rho_j) at
 // the Gauss-Legendre points x + l (1 + xi_j) / 2 (Eqs. vf5, vf6).
-template <typename T, int NC, bool SEG = false>
-__global__ void __launch_bounds__(P2M_THREADS) k_p2m_w(const int* __restrict__ ntiles_dev,
-                                                     const int2* __restrict__ tiles, int level,
-                                                     const uint64_t* __restrict__ bkey, const int* __restrict__ bend,
-                                                     const SysCube* __restrict__ cubes,
+template <typename T, int NC, bool SEG, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_p2m_w(const int* __restrict__ ntiles_dev,
+                                                     const int2* __restrict__ tiles, const dbl4* __restrict__ geom,
+                                                     const T* __restrict__ qtab, const int* __restrict__ bend,
                                                      const vec4_t<T>* __restrict__ xs,
                                                      const vec4_t<T>* __restrict__ ws, const T* __restrict__ qs,
                                                      T* __restrict__ Wout, int64_t ldw, int p, int chunk,
                                                      GaussRule rule = GaussRule{}) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    static_assert(P2M_THREADS % 64 == 0, "warps pair up by the parity of m");
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    static_assert(THREADS % 64 == 0, "warps pair up by the parity of m");
+    constexpr int MAX_OUT = p2m_max_out(THREADS);
     const int P = p * p, gs = p2m_row_stride(P);
     const int par = (threadIdx.x >> 5) & 1;  // parity of the orders m this warp's harmonics take
-    T* gh = reinterpret_cast<T*>(smem_raw);  // [chunk][gs]: the harmonics of an element in a row
-    T* wk = gh + (size_t)chunk * gs;         // [chunk][NC]: strength / h
+    constexpr int WS = NC == 3 ? 4 : 1;      // reals per strength: one vector read
+    T* wk = reinterpret_cast<T*>(smem_raw);  // [chunk][WS]: strength / h
+    T* gh = wk + (size_t)chunk * WS;         // [chunk][gs]: the harmonics of an element in a row
     const int ntiles = *ntiles_dev;
-    const QTab<T> qt = build_qtab(wk + (size_t)chunk * 3, p);  // visible after the tile loop's first barrier
+    const QTab<T> qt = load_qtab(gh + (size_t)chunk * gs, qtab, p);  // visible after the tile loop's first barrier
     // a block takes a contiguous range of tiles; the tiles of a leaf are consecutive, so the
     // partial W of a leaf is summed over its tiles in registers and added once per leaf
     const int t_lo = (int)((int64_t)ntiles * blockIdx.x / gridDim.x);
     const int t_hi = (int)((int64_t)ntiles * (blockIdx.x + 1) / gridDim.x);
-    T acc[P2M_MAX_OUT];  // outputs i = threadIdx.x + q blockDim.x of the current leaf
+    T acc[MAX_OUT][NC];  // entries j = threadIdx.x + q THREADS of the current leaf's NC rows of W
 #pragma unroll
-    for (int q = 0; q < P2M_MAX_OUT; ++q) acc[q] = 0;
+    for (int q = 0; q < MAX_OUT; ++q)
+#pragma unroll
+        for (int k = 0; k < NC; ++k) acc[q][k] = 0;
     auto flush = [&](int leaf) {
         T* Wb = Wout + (int64_t)leaf * ldw;
 #pragma unroll
-        for (int q = 0; q < P2M_MAX_OUT; ++q) {
-            const int i = threadIdx.x + q * blockDim.x;
-            if (i < NC * P) atomicAdd(Wb + i, acc[q]);
-            acc[q] = 0;
+        for (int q = 0; q < MAX_OUT; ++q) {
+            const int j = threadIdx.x + q * THREADS;
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                if (j < P) atomicAdd(Wb + k * P + j, acc[q][k]);
+                acc[q][k] = 0;
+            }
         }
     };
     int cur = -1;
@@ -177,9 +182,8 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_w(const int* __restrict__ n
             if (cur >= 0) flush(cur);
             cur = b;
         }
-        double cx, cy, cz, h;
-        box_geom(cubes, bkey[b], level, cx, cy, cz, h);
-        const T invh = (T)(1.0 / h);
+        const dbl4 bg = geom[b];
+        const T invh = (T)bg.w;
         const int e0 = tw.y, e1 = min(bend[b], tw.y + P2P_TILE);
         for (int c0 = e0; c0 < e1; c0 += chunk) {
             const int ne = min(chunk, e1 - c0);
@@ -194,9 +198,9 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_w(const int* __restrict__ n
                         const vec4_t<T> wv = ws[c0 + e];
                         // M_hat carries 1/h (P2M scaling); a segment's strength is Gamma l / (8 pi)
                         const T sc = SEG ? wv.w * (T)(0.039788735772973833942) * invh : invh;  // 1/(8 pi)
-                        wk[e * 3 + 0] = wv.x * sc;
-                        wk[e * 3 + 1] = wv.y * sc;
-                        wk[e * 3 + 2] = wv.z * sc;
+                        wk[e * 4 + 0] = wv.x * sc;
+                        wk[e * 4 + 1] = wv.y * sc;
+                        wk[e * 4 + 2] = wv.z * sc;
                     } else {
                         wk[e] = qs[c0 + e] * invh;
                     }
@@ -214,7 +218,7 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_w(const int* __restrict__ n
                         pz += t * (double)wv.z;
                         wq = (T)rule.w[j];
                     }
-                    const T rx = (T)((px - cx) / h), ry = (T)((py - cy) / h), rz = (T)((pz - cz) / h);
+                    const T rx = (T)((px - bg.x) * bg.w), ry = (T)((py - bg.y) * bg.w), rz = (T)((pz - bg.z) * bg.w);
                     for_each_Q<T>(p, rx, ry, rz, qt, [&](int n, int m, T qr, T qi) {
                         T re, im;  // i^m conj(Q)
                         switch (m & 3) {
@@ -235,26 +239,42 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_w(const int* __restrict__ n
                 }
             }
             __syncthreads();
+            // an entry of the harmonics serves the NC strengths of its element
 #pragma unroll
-            for (int q = 0; q < P2M_MAX_OUT; ++q) {
-                const int i = threadIdx.x + q * blockDim.x;
-                if (i >= NC * P) break;
-                const int k = i / P, j = i - k * P;
-                T s = 0;
-                for (int e = 0; e < ne; ++e) s += wk[e * NC + k] * gh[(size_t)e * gs + j];
-                acc[q] += s;
+            for (int q = 0; q < MAX_OUT; ++q) {
+                const int j = threadIdx.x + q * THREADS;
+                if (j >= P) break;
+                T s[NC];
+#pragma unroll
+                for (int k = 0; k < NC; ++k) s[k] = 0;
+#pragma unroll 4
+                for (int e = 0; e < ne; ++e) {
+                    const T g = gh[(size_t)e * gs + j];
+                    if constexpr (NC == 3) {
+                        const vec4_t<T> w = *reinterpret_cast<const vec4_t<T>*>(wk + e * 4);
+                        s[0] += w.x * g;
+                        s[1] += w.y * g;
+                        s[2] += w.z * g;
+                    } else {
+                        s[0] += wk[e] * g;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < NC; ++k) acc[q][k] += s[k];
             }
         }
     }
     if (cur >= 0) flush(cur);
 }
 
-// P2M, part 2 (per leaf): M_hat = G W with G the P2M map of Eq. eve4 in row-compressed form
-// (its structural zeros dropped); one block per leaf, W staged in shared memory.
+// P2M, part 2 (per leaf): M_hat = G W with G the sparse P2M map of Eq. eve4; one block per leaf, W
+// staged in shared memory.
+constexpr int P2M_APPLY_THREADS = 96;
 template <typename T>
-__global__ void __launch_bounds__(P2M_THREADS) k_p2m_apply(const int* __restrict__ nleaf_dev, const T* __restrict__ W,
-                                                          int P, CsrView<T> g, T* __restrict__ mult, int64_t ld) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+__global__ void __launch_bounds__(P2M_APPLY_THREADS) k_p2m_apply(const int* __restrict__ nleaf_dev,
+                                                                const T* __restrict__ W, int P, SellView<T> g,
+                                                                T* __restrict__ mult, int64_t ld) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     T* w = reinterpret_cast<T*>(smem_raw);  // [3P]
     const int nleaf = *nleaf_dev;
     for (int b = blockIdx.x; b < nleaf; b += gridDim.x) {
@@ -262,18 +282,14 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_apply(const int* __restrict
         for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) w[i] = W[(int64_t)b * 3 * P + i];
         __syncthreads();
         T* out = mult + (int64_t)b * ld;
-        for (int r = threadIdx.x; r < g.rows; r += blockDim.x) {
-            T acc = 0;
-            for (int k = g.rowptr[r]; k < g.rowptr[r + 1]; ++k) acc += g.val[k] * w[g.col[k]];
-            out[r] = acc;
-        }
+        sparse_rows(g, w, threadIdx.x >> 5, P2M_APPLY_THREADS / 32, [&](int r, T v) { out[r] = v; });
     }
 }
 
 // ---------------------------------------------------------------------------
 // L2P (per tile of a leaf; the 12 coefficient vectors cf = E L_hat of v_k (Eq. evf3)
 // and u_lk = D_{i_l} v_k (Eq. dt3) come from the leaf's local expansion through the
-// row-compressed map E, in shared memory):
+// sparse map E, in shared memory):
 //   v_k = (1/h) c_k . b(rho),   u_lk = (1/h^2) c_{3+3l+k} . b(rho),
 //   s_k = sum_l w_l u_lk (Eq. evf6),
 // b = real form of R_hat = nu R:  b[n^2] = R_hat_n^0,  2 Re R_hat_n^m,  -2 Im R_hat_n^m,
@@ -281,22 +297,22 @@ __global__ void __launch_bounds__(P2M_THREADS) k_p2m_apply(const int* __restrict
 // ---------------------------------------------------------------------------
 constexpr int L2P_THREADS = 128;
 
-template <typename T>
-__global__ void __launch_bounds__(L2P_THREADS) k_l2p_eval(const int* __restrict__ ntiles_dev,
-                                                        const int2* __restrict__ tiles, int level,
-                                                        const uint64_t* __restrict__ bkey,
-                                                        const int* __restrict__ bend,
-                                                        const SysCube* __restrict__ cubes,
+// GRAD: the 12 vectors of v and grad v, else the 3 of v (sfar unused)
+template <typename T, int THREADS, bool GRAD>
+__global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ ntiles_dev,
+                                                        const int2* __restrict__ tiles, const dbl4* __restrict__ geom,
+                                                        const T* __restrict__ qtab, const int* __restrict__ bend,
                                                         const vec4_t<T>* __restrict__ xs,
                                                         const vec4_t<T>* __restrict__ ws, const T* __restrict__ loc,
-                                                        int64_t ld, CsrView<T> e, vec4_t<T>* __restrict__ vfar,
+                                                        int64_t ld, SellView<T> e, vec4_t<T>* __restrict__ vfar,
                                                         vec4_t<T>* __restrict__ sfar, int p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int NV = GRAD ? 12 : 3, CS = GRAD ? 12 : 4;  // vectors, and their stride in shared memory
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     const int P = p * p;
-    T* cf = reinterpret_cast<T*>(smem_raw);  // [P][12]
-    T* lh = cf + 12 * P;                     // [2P] the leaf's local expansion
+    T* cf = reinterpret_cast<T*>(smem_raw);  // [P][CS]
+    T* lh = cf + CS * P;                     // [2P] the leaf's local expansion
     const int ntiles = *ntiles_dev;
-    const QTab<T> qt = build_qtab(lh + 2 * P, p);  // visible after the tile loop's first barrier
+    const QTab<T> qt = load_qtab(lh + 2 * P, qtab, p);  // visible after the tile loop's first barrier
     // a block takes a contiguous range of tiles; the tiles of a leaf are consecutive, so the
     // leaf's coefficient vectors are staged once per leaf, not once per tile
     const int t_lo = (int)((int64_t)ntiles * blockIdx.x / gridDim.x);
@@ -305,30 +321,27 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p_eval(const int* __restrict_
     for (int t = t_lo; t < t_hi; ++t) {
         const int2 tw = tiles[t];
         const int b = tw.x;
-        double cx, cy, cz, h;
-        box_geom(cubes, bkey[b], level, cx, cy, cz, h);
+        const dbl4 bg = geom[b];
         if (b != staged) {
             __syncthreads();
             for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) lh[i] = loc[(int64_t)b * ld + i];
             __syncthreads();
-            for (int r = threadIdx.x; r < 12 * P; r += blockDim.x) {  // output r = j P + i: vector j, entry i
-                T acc = 0;
-                for (int k = e.rowptr[r]; k < e.rowptr[r + 1]; ++k) acc += e.val[k] * lh[e.col[k]];
+            sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {  // r = j P + i: vector j, entry i
                 const int j = r / P, i = r - j * P;
-                cf[i * 12 + j] = acc;
-            }
+                cf[i * CS + j] = v;
+            });
             __syncthreads();
             staged = b;
         }
-        const T invh = (T)(1.0 / h);
+        const T invh = (T)bg.w;
         const int e1 = min(bend[b], tw.y + P2P_TILE);
         for (int e = tw.y + threadIdx.x; e < e1; e += blockDim.x) {
-            vec4_t<T> xv = xs[e], wv = ws[e];
-            const T rx = (T)(((double)xv.x - cx) / h), ry = (T)(((double)xv.y - cy) / h),
-                    rz = (T)(((double)xv.z - cz) / h);
-            T acc[12];
+            const vec4_t<T> xv = xs[e];
+            const T rx = (T)(((double)xv.x - bg.x) * bg.w), ry = (T)(((double)xv.y - bg.y) * bg.w),
+                    rz = (T)(((double)xv.z - bg.z) * bg.w);
+            T acc[NV];
 #pragma unroll
-            for (int j = 0; j < 12; ++j) acc[j] = 0;
+            for (int j = 0; j < NV; ++j) acc[j] = 0;
             for_each_Q<T>(p, rx, ry, rz, qt, [&](int n, int m, T qr, T qi) {
                 T re, im;  // (-1)^n i^m Q
                 switch (m & 3) {
@@ -342,29 +355,33 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p_eval(const int* __restrict_
                     im = -im;
                 }
                 if (m == 0) {
-                    const T* c = cf + (n * n) * 12;
+                    const T* c = cf + (n * n) * CS;
 #pragma unroll
-                    for (int j = 0; j < 12; ++j) acc[j] += c[j] * re;
+                    for (int j = 0; j < NV; ++j) acc[j] += c[j] * re;
                 } else {
-                    const T* c1 = cf + (n * n + 2 * m - 1) * 12;
-                    const T* c2 = c1 + 12;
+                    const T* c1 = cf + (n * n + 2 * m - 1) * CS;
+                    const T* c2 = c1 + CS;
                     const T b1 = 2 * re, b2 = -2 * im;
 #pragma unroll
-                    for (int j = 0; j < 12; ++j) acc[j] += c1[j] * b1 + c2[j] * b2;
+                    for (int j = 0; j < NV; ++j) acc[j] += c1[j] * b1 + c2[j] * b2;
                 }
             });
-            vec4_t<T> v, s;
+            vec4_t<T> v;
             v.x = acc[0] * invh;
             v.y = acc[1] * invh;
             v.z = acc[2] * invh;
             v.w = 0;
-            const T invh2 = invh * invh;
-            s.x = (wv.x * acc[3] + wv.y * acc[6] + wv.z * acc[9]) * invh2;
-            s.y = (wv.x * acc[4] + wv.y * acc[7] + wv.z * acc[10]) * invh2;
-            s.z = (wv.x * acc[5] + wv.y * acc[8] + wv.z * acc[11]) * invh2;
-            s.w = 0;
             vfar[e] = v;
-            sfar[e] = s;
+            if constexpr (GRAD) {
+                const vec4_t<T> wv = ws[e];
+                const T invh2 = invh * invh;
+                vec4_t<T> s;
+                s.x = (wv.x * acc[3] + wv.y * acc[6] + wv.z * acc[9]) * invh2;
+                s.y = (wv.x * acc[4] + wv.y * acc[7] + wv.z * acc[10]) * invh2;
+                s.z = (wv.x * acc[5] + wv.y * acc[8] + wv.z * acc[11]) * invh2;
+                s.w = 0;
+                sfar[e] = s;
+            }
         }
     }
 }
@@ -374,47 +391,39 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p_eval(const int* __restrict_
 // and grad phi_k = (1/h) c_k . b(rho), with c_k the velocity rows of the L2P map (Eq. evf3)
 // applied to (L_hat, 0): with chi = 0, v = grad phi (Eq. 4).  Lanes of the output: grad phi
 // in x, y, z, phi in w.
-template <typename T>
-__global__ void __launch_bounds__(L2P_THREADS) k_l2p_scalar(const int* __restrict__ ntiles_dev,
-                                                          const int2* __restrict__ tiles, int level,
-                                                          const uint64_t* __restrict__ bkey,
-                                                          const int* __restrict__ bend,
-                                                          const SysCube* __restrict__ cubes,
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_l2p_scalar(const int* __restrict__ ntiles_dev,
+                                                          const int2* __restrict__ tiles, const dbl4* __restrict__ geom,
+                                                        const T* __restrict__ qtab, const int* __restrict__ bend,
                                                           const vec4_t<T>* __restrict__ xs, const T* __restrict__ loc,
-                                                          int64_t ld, CsrView<T> e, vec4_t<T>* __restrict__ pgfar,
+                                                          int64_t ld, SellView<T> e, vec4_t<T>* __restrict__ pgfar,
                                                           int p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     const int P = p * p;
     T* cf = reinterpret_cast<T*>(smem_raw);  // [P][4]
     T* lh = cf + 4 * P;                      // [2P] (L_hat, 0)
     const int ntiles = *ntiles_dev;
-    const QTab<T> qt = build_qtab(lh + 2 * P, p);
+    const QTab<T> qt = load_qtab(lh + 2 * P, qtab, p);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int2 tw = tiles[t];
         const int b = tw.x;
-        double cx, cy, cz, h;
-        box_geom(cubes, bkey[b], level, cx, cy, cz, h);
+        const dbl4 bg = geom[b];
         __syncthreads();
         for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) lh[i] = i < P ? loc[(int64_t)b * ld + i] : (T)0;
         __syncthreads();
-        for (int r = threadIdx.x; r < 4 * P; r += blockDim.x) {  // vector j = 0: phi itself, 1..3: rows of v_x, v_y, v_z
+        // vector j = 0: phi itself, 1..3: rows of v_x, v_y, v_z
+        for (int i = threadIdx.x; i < P; i += blockDim.x) cf[i * 4] = lh[i];
+        sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {
             const int j = r / P, i = r - j * P;
-            T acc = 0;
-            if (j == 0) {
-                acc = lh[i];
-            } else {
-                const int row = r - P;
-                for (int k = e.rowptr[row]; k < e.rowptr[row + 1]; ++k) acc += e.val[k] * lh[e.col[k]];
-            }
-            cf[i * 4 + j] = acc;
-        }
+            cf[i * 4 + 1 + j] = v;
+        });
         __syncthreads();
-        const T invh = (T)(1.0 / h);
+        const T invh = (T)bg.w;
         const int e1 = min(bend[b], tw.y + P2P_TILE);
         for (int el = tw.y + threadIdx.x; el < e1; el += blockDim.x) {
             const vec4_t<T> xv = xs[el];
-            const T rx = (T)(((double)xv.x - cx) / h), ry = (T)(((double)xv.y - cy) / h),
-                    rz = (T)(((double)xv.z - cz) / h);
+            const T rx = (T)(((double)xv.x - bg.x) * bg.w), ry = (T)(((double)xv.y - bg.y) * bg.w),
+                    rz = (T)(((double)xv.z - bg.z) * bg.w);
             T acc[4] = {0, 0, 0, 0};
             for_each_Q<T>(p, rx, ry, rz, qt, [&](int n, int m, T qr, T qi) {
                 T re, im;  // (-1)^n i^m Q
@@ -453,28 +462,97 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p_scalar(const int* __restric
 }  // namespace
 
 template <typename T>
-void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
-             const vec4_t<T>* ws, T* W, T* mult) {
-    const int L = lv.L, nl = lv.nbox[L], o = lv.off[L], p = pl.p[L], P = p * p;
-    int chunk;
-    const size_t smem = p2m_smem<T>(p, chunk);
-    cuda_check(cudaFuncSetAttribute(k_p2m_w<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-               "p2m attr");
-    const int* count = tb.counts.as<int>();
-    fill_level_rows<T>(c, lv, count, L, L, 3 * P, o, W, (T)0);  // W of the real leaves
-    const int64_t max_tiles = nl + lv.n / P2P_TILE + 1;
-    k_p2m_w<T, 3><<<grid_for(max_tiles, 1, 152 * 16), P2M_THREADS, smem, stream_of(c)>>>(
-        tb.tile_count.as<int>(), tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o, tb.bend.as<int>() + o,
-        tb.cubes.as<SysCube>(), xs, ws, nullptr, W, (int64_t)3 * P, p, chunk);
-    count_launch(c);
-    check_launch("p2m w");
-    const size_t smem2 = sizeof(T) * 3 * P;
-    cuda_check(cudaFuncSetAttribute(k_p2m_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2),
-               "p2m apply attr");
-    k_p2m_apply<T><<<grid_for(nl, 1, 152 * 16), P2M_THREADS, smem2, stream_of(c)>>>(count + L, W, P, pl.p2m_sp,
-                                                                                   mult + (int64_t)o * pl.ld, pl.ld);
+void build_qtab(Ctx* c, int p, Buf& dst) {
+    std::vector<T> h((size_t)qtab_reals(p), (T)0);
+    T *A = h.data(), *B = A + p * p, *cm = B + p * p, *c1 = cm + p;
+    for (int m = 0; m < p; ++m) {
+        for (int n = m + 2; n < p; ++n) {
+            const double d = (double)((n + m) * (n - m));
+            A[m * p + n] = (T)((2 * n - 1) / std::sqrt(d));
+            B[m * p + n] = (T)std::sqrt((double)((n + m - 1) * (n - m - 1)) / d);
+        }
+        cm[m] = m > 0 ? (T)-std::sqrt((2.0 * m - 1.0) / (2.0 * m)) : (T)0;
+        c1[m] = (T)std::sqrt(2.0 * m + 1.0);
+    }
+    ensure(c, dst, (int64_t)(h.size() * sizeof(T)));
+    cuda_check(cudaMemcpy(dst.ptr, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice), "recurrence table");
+}
+
+// Blocks of a persistent kernel: as many as are resident at once, at most `items`.
+template <typename K>
+static int resident_grid(K kernel, int threads, size_t smem, int64_t items) {
+    int per_sm = 1, sms = 152, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)sms * std::max(per_sm, 1)));
+}
+
+// W of the leaves (rows of ldw reals, zeroed) by blocks that suit their mean size.
+template <typename T, int NC, bool SEG>
+static void launch_p2m_w(Ctx* c, const TreeBufs& tb, const Levels& lv, int p, const T* qtab, const vec4_t<T>* xs, const vec4_t<T>* ws,
+                         const T* qs, T* W, int64_t ldw, const GaussRule& rule) {
+    const int L = lv.L, o = lv.off[L];
+    auto launch = [&](auto threads, int most) {
+        constexpr int TH = decltype(threads)::value;
+        int chunk;
+        const size_t smem = p2m_smem<T>(p, most, chunk);
+        auto kernel = k_p2m_w<T, NC, SEG, TH>;
+        cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "p2m attr");
+        kernel<<<tile_grid(kernel, TH, smem, lv), TH, smem, stream_of(c)>>>(
+            tb.tile_count.as<int>(), tb.tiles.as<int2>(), tb.geom.as<dbl4>(), qtab, tb.bend.as<int>() + o, xs, ws, qs, W, ldw, p, chunk, rule);
+        count_launch(c);
+        check_launch("p2m w");
+    };
+    if (lv.n <= (int64_t)lv.leaves * P2M_SMALL_LEAF) launch(std::integral_constant<int, P2M_SMALL>{}, 32);
+    else launch(std::integral_constant<int, P2M_THREADS>{}, 128);
+}
+
+template <typename T>
+static void launch_p2m_apply(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const T* W, T* mult) {
+    const int L = lv.L, P = pl.p[L] * pl.p[L];
+    const size_t smem = sizeof(T) * 3 * P;
+    k_p2m_apply<T><<<resident_grid(k_p2m_apply<T>, P2M_APPLY_THREADS, smem, lv.nbox[L]), P2M_APPLY_THREADS, smem,
+                     stream_of(c)>>>(tb.counts.as<int>() + L, W, P, pl.p2m_sp, mult + (int64_t)lv.off[L] * pl.ld, pl.ld);
     count_launch(c);
     check_launch("p2m apply");
+}
+
+// Blocks of a kernel whose blocks take contiguous ranges of the near-field tiles: one tile a block
+// where that is less than eight a resident block (their unevenness would set the time: L2P of
+// the FP64 ring of 32,768, 1.8 tiles a resident block, 1.10 ms against 0.92), 16 blocks an SM where a
+// leaf holds several tiles (P2M, L2P of the leapfrog pair, 440 elements a leaf: 1.8, 1.86 ms with the
+// resident blocks, 1.45, 1.74 with 16), else those resident at once (sphere surface, 15 a leaf:
+// 0.48, 1.32 ms against 0.54, 1.59 with 16).
+constexpr int BIG_LEAF = 64;
+template <typename K>
+static int tile_grid(K kernel, int threads, size_t smem, const Levels& lv) {
+    const int64_t tiles = lv.nbox[lv.L] + lv.n / P2P_TILE + 1;
+    const int resident = resident_grid(kernel, threads, smem, tiles);
+    if (lv.leaves + lv.n / P2P_TILE < 8 * (int64_t)resident) return grid_for(tiles, 1, 8 * resident);
+    if (lv.n > (int64_t)lv.leaves * BIG_LEAF) return grid_for(tiles, 1, 152 * 16);
+    return resident;
+}
+
+// Threads of an L2P block of three or four vectors for the mean leaf: f(integral_constant).  Narrow
+// blocks put more leaves on an SM (scalar cube, 32 a leaf: 0.29 ms against 0.35 with 128 threads); with
+// twelve vectors the sparse map takes half of the work and wants the wide block (sphere
+// surface 1.52 against 1.32).
+template <typename F>
+static void l2p_threads(const Levels& lv, F&& f) {
+    const int64_t nl = lv.leaves;
+    if (lv.n <= nl * 32) f(std::integral_constant<int, 32>{});
+    else if (lv.n <= nl * 64) f(std::integral_constant<int, 64>{});
+    else f(std::integral_constant<int, L2P_THREADS>{});
+}
+
+template <typename T>
+void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
+             const vec4_t<T>* ws, T* W, T* mult) {
+    const int L = lv.L, P = pl.p[L] * pl.p[L];
+    fill_level_rows<T>(c, lv, tb.counts.as<int>(), L, L, 3 * P, lv.off[L], W, (T)0);  // W of the real leaves
+    launch_p2m_w<T, 3, false>(c, tb, lv, pl.p[L], pl.qtab, xs, ws, nullptr, W, 3 * P, GaussRule{});
+    launch_p2m_apply<T>(c, pl, tb, lv, W, mult);
 }
 
 template <typename T>
@@ -561,15 +639,20 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
 template <typename T>
 void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
              const vec4_t<T>* ws, const T* loc, vec4_t<T>* vfar, vec4_t<T>* sfar) {
-    const int L = lv.L, nl = lv.nbox[L], o = lv.off[L], p = pl.p[L], P = p * p;
-    const size_t smem = sizeof(T) * (14 * P + qtab_reals(p));
-    cuda_check(cudaFuncSetAttribute(k_l2p_eval<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "l2p attr");
-    const int64_t max_tiles = nl + lv.n / P2P_TILE + 1;
-    k_l2p_eval<T><<<grid_for(max_tiles, 1, 152 * 16), L2P_THREADS, smem, stream_of(c)>>>(
-        tb.tile_count.as<int>(), tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o, tb.bend.as<int>() + o,
-        tb.cubes.as<SysCube>(), xs, ws, loc + (int64_t)o * pl.ld, pl.ld, pl.l2p_sp, vfar, sfar, p);
-    count_launch(c);
-    check_launch("l2p");
+    const int L = lv.L, o = lv.off[L], p = pl.p[L], P = p * p;
+    auto launch = [&](auto threads, auto grad) {
+        constexpr int TH = decltype(threads)::value;
+        constexpr bool GRAD = decltype(grad)::value;
+        const size_t smem = sizeof(T) * ((GRAD ? 14 : 6) * P + qtab_reals(p));
+        auto kernel = k_l2p_eval<T, TH, GRAD>;
+        cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "l2p attr");
+        kernel<<<tile_grid(kernel, TH, smem, lv), TH, smem, stream_of(c)>>>(
+            tb.tile_count.as<int>(), tb.tiles.as<int2>(), tb.geom.as<dbl4>(), pl.qtab, tb.bend.as<int>() + o, xs, ws, loc + (int64_t)o * pl.ld, pl.ld, pl.l2p_sp, vfar, sfar, p);
+        count_launch(c);
+        check_launch("l2p");
+    };
+    if (sfar) launch(std::integral_constant<int, L2P_THREADS>{}, std::true_type{});
+    else l2p_threads(lv, [&](auto th) { launch(th, std::false_type{}); });
 }
 
 
@@ -578,63 +661,40 @@ void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
 template <typename T>
 void run_p2m_segments(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
                       const vec4_t<T>* seg, const GaussRule& rule, T* W, T* mult) {
-    const int L = lv.L, nl = lv.nbox[L], o = lv.off[L], p = pl.p[L], P = p * p;
-    int chunk;
-    const size_t smem = p2m_smem<T>(p, chunk);
-    cuda_check(cudaFuncSetAttribute(k_p2m_w<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-               "p2m attr");
-    const int* count = tb.counts.as<int>();
-    fill_level_rows<T>(c, lv, count, L, L, 3 * P, o, W, (T)0);
-    const int64_t max_tiles = nl + lv.n / P2P_TILE + 1;
-    k_p2m_w<T, 3, true><<<grid_for(max_tiles, 1, 152 * 16), P2M_THREADS, smem, stream_of(c)>>>(
-        tb.tile_count.as<int>(), tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o, tb.bend.as<int>() + o,
-        tb.cubes.as<SysCube>(), xs, seg, nullptr, W, (int64_t)3 * P, p, chunk, rule);
-    count_launch(c);
-    check_launch("p2m segments");
-    const size_t smem2 = sizeof(T) * 3 * P;
-    cuda_check(cudaFuncSetAttribute(k_p2m_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2),
-               "p2m apply attr");
-    k_p2m_apply<T><<<grid_for(nl, 1, 152 * 16), P2M_THREADS, smem2, stream_of(c)>>>(count + L, W, P, pl.p2m_sp,
-                                                                                   mult + (int64_t)o * pl.ld, pl.ld);
-    count_launch(c);
-    check_launch("p2m apply");
+    const int L = lv.L, P = pl.p[L] * pl.p[L];
+    fill_level_rows<T>(c, lv, tb.counts.as<int>(), L, L, 3 * P, lv.off[L], W, (T)0);
+    launch_p2m_w<T, 3, true>(c, tb, lv, pl.p[L], pl.qtab, xs, seg, nullptr, W, 3 * P, rule);
+    launch_p2m_apply<T>(c, pl, tb, lv, W, mult);
 }
 
 // Scalar reference case: P2M of the monopoles straight into the leaf multipoles.
 template <typename T>
 void run_p2m_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
                     const T* qs, T* mult) {
-    const int L = lv.L, nl = lv.nbox[L], o = lv.off[L], p = pl.p[L];
-    int chunk;
-    const size_t smem = p2m_smem<T>(p, chunk);
-    cuda_check(cudaFuncSetAttribute(k_p2m_w<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-               "p2m attr");
-    T* leaf_rows = mult + (int64_t)o * pl.ld;
+    const int L = lv.L;
     fill_level_rows<T>(c, lv, tb.counts.as<int>(), L, L, pl.ld, 0, mult, (T)0);
-    const int64_t max_tiles = nl + lv.n / P2P_TILE + 1;
-    k_p2m_w<T, 1><<<grid_for(max_tiles, 1, 152 * 16), P2M_THREADS, smem, stream_of(c)>>>(
-        tb.tile_count.as<int>(), tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o, tb.bend.as<int>() + o,
-        tb.cubes.as<SysCube>(), xs, nullptr, qs, leaf_rows, pl.ld, p, chunk);
-    count_launch(c);
-    check_launch("p2m scalar");
+    launch_p2m_w<T, 1, false>(c, tb, lv, pl.p[L], pl.qtab, xs, nullptr, qs, mult + (int64_t)lv.off[L] * pl.ld, pl.ld,
+                              GaussRule{});
 }
 
 template <typename T>
 void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
                     const T* loc, vec4_t<T>* pgfar) {
-    const int L = lv.L, nl = lv.nbox[L], o = lv.off[L], p = pl.p[L], P = p * p;
+    const int L = lv.L, o = lv.off[L], p = pl.p[L], P = p * p;
     const size_t smem = sizeof(T) * (6 * P + qtab_reals(p));
-    cuda_check(cudaFuncSetAttribute(k_l2p_scalar<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-               "l2p attr");
-    const int64_t max_tiles = nl + lv.n / P2P_TILE + 1;
-    k_l2p_scalar<T><<<grid_for(max_tiles, 1, 152 * 16), L2P_THREADS, smem, stream_of(c)>>>(
-        tb.tile_count.as<int>(), tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o, tb.bend.as<int>() + o,
-        tb.cubes.as<SysCube>(), xs, loc + (int64_t)o * pl.ld, pl.ld, pl.l2p_sp, pgfar, p);
-    count_launch(c);
-    check_launch("l2p scalar");
+    l2p_threads(lv, [&](auto threads) {
+        constexpr int TH = decltype(threads)::value;
+        auto kernel = k_l2p_scalar<T, TH>;
+        cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "l2p attr");
+        kernel<<<tile_grid(kernel, TH, smem, lv), TH, smem, stream_of(c)>>>(
+            tb.tile_count.as<int>(), tb.tiles.as<int2>(), tb.geom.as<dbl4>(), pl.qtab, tb.bend.as<int>() + o, xs, loc + (int64_t)o * pl.ld, pl.ld, pl.l2p_sp, pgfar, p);
+        count_launch(c);
+        check_launch("l2p scalar");
+    });
 }
 
 #define LHV_INST(T)                                                                                              \
+    template void build_qtab<T>(Ctx*, int, Buf&);                                                                \
     template void run_p2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,            \
                              const vec4_t<T>*, T*, T*);                                                         \
     template void run_m2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, Grouped&, T*);              \

@@ -66,6 +66,8 @@ struct Levels {
     int off[MAX_LEVELS + 1] = {0};   // global box index of the first box of each level
     int cap_off[MAX_LEVELS + 1] = {0};
     int64_t n = 0;                   // elements of the tree
+    int leaves = 0;                  // leaves of the last tree whose counts the host read (a captured
+                                     // step follows one of the same level): picks block shapes
 };
 
 struct Ctx;
@@ -114,6 +116,7 @@ struct TreeBufs {
     Buf counts;                // int32[64] (device)
     Buf bkey, bbeg, bend, bparent, bcbeg, bcend, bcol;  // per box (global index)
     Buf tiles, tile_count;     // P2P work items: int2 (leaf, first element)
+    Buf geom;                  // dbl4 per leaf: centre, 1 / side
 };
 
 // Builds keys, sort, levels and lists for n positions (device [n][4] of T) of
@@ -141,16 +144,16 @@ void gather_sorted(Ctx* c, int64_t n, const int* perm, const vec4_t<T>* x4, cons
                    vec4_t<T>* xs, vec4_t<T>* ws);
 
 // ---- operators (operators.cu) -----------------------------------------------
-// Row-compressed form of a sparse map (rows = outputs): out[r] = sum val[k] in[col[k]],
-// k in [rowptr[r], rowptr[r+1]).
-struct Csr {
-    Buf rowptr, col, val;
+// Sliced form of a sparse map (rows = outputs): out[row] = sum val in[col].  The rows lie in slices of
+// 32; entry k of a slice's rows is a run of 32 values from sptr[slice] + 32 k (short rows padded
+// with zeros), so a warp reads its slice coalesced, and neighbouring rows read neighbouring inputs.
+struct Sell {
+    Buf sptr, col, val;
     int rows = 0;
-    int64_t nnz = 0;
 };
 template <typename T>
-struct CsrView {
-    const int* rowptr = nullptr;
+struct SellView {
+    const int* sptr = nullptr;
     const int* col = nullptr;
     const T* val = nullptr;
     int rows = 0;
@@ -163,10 +166,11 @@ struct OpTables {
     Buf m2l;                   // [316][2P][2P] fused (S|R) + Eq. drt10 per offset slot (built when a route needs it)
     Buf m2m;                   // [8][2P][2P]   fused (S|S) + Eq. drt11 per child octant
     Buf l2l;                   // [8][2P][2P]   fused (R|R) + Eq. drt10 per child octant
-    Buf l2p;                   // [2P][12P]     v_k (Eq. evf3) and u_lk (Eq. dt3) coefficients
-    Buf p2m;                   // [3P][2P]      Eq. eve4 for w = i_x, i_y, i_z
     Buf m2l_tiles;             // TF32 hi/lo tiles of the translation blocks of m2l (LHV_TF32X3, tc_m2l.cu)
-    Csr p2m_sp, l2p_sp;        // P2M and L2P in row-compressed form (their structural zeros dropped)
+    // sparse maps (structural zeros dropped): P2M 3P -> 2P (Eq. eve4 for w = i_x, i_y, i_z), L2P
+    // 2P -> 12P (v_k of Eq. evf3, u_lk of Eq. dt3), and the 3P rows v_k of it alone (built on first use)
+    Sell p2m_sp, l2p_sp, l2pv_sp;
+    Buf qtab;                  // recurrence coefficients of the harmonics (qtab_reals(p) reals of T)
     Buf offsets;               // int[316][3] M2L offsets (dx, dy, dz)
     Buf slot_of;               // int[343] offset (dx+3)*49+(dy+3)*7+(dz+3) -> slot or -1
 };
@@ -180,10 +184,11 @@ void build_operators(Ctx* c, int p, OpTables& ops);
 enum OpKind : int { OP_M2L = 0, OP_M2M = 1, OP_L2L = 2, OP_L2P = 3, OP_P2M = 4 };
 template <typename T>
 void build_op(Ctx* c, int kind, int pout, int pin, Buf& dst);
-// P2M (2P x 3P) or L2P (12P x 2P) of truncation number p, rows = outputs, in T.
+// P2M (2P x 3P) or L2P (12P x 2P) of truncation number p, rows = outputs, in T; the first `rows`
+// outputs (0: all).
 template <typename T>
-void build_sparse(Ctx* c, int kind, int p, Csr& dst);
-void free_csr(Csr& m);
+void build_sparse(Ctx* c, int kind, int p, int rows, Sell& dst);
+void free_sparse(Sell& m);
 void free_operators(OpTables& ops);
 // dst = the translation block T ([P][P] per group, k-major) of ngroups fused [2P][2P] tables.
 template <typename T>
@@ -208,13 +213,12 @@ struct Plan {
     int L = 0;
     int p[MAX_LEVELS + 1] = {};            // truncation number of the expansions of level l
     int ld = 0;                            // reals per box in mult / loc: 2 max_l p[l]^2 (l = 2..L)
-    const T* p2m = nullptr;                // P2M(p[L])          [3P][2P]
-    const T* l2p = nullptr;                // L2P(p[L])          [2P][12P]
     const T* m2m[MAX_LEVELS + 1] = {};     // [l]: level l+1 -> l, 8 x [2P(l+1)][2P(l)]
     const T* l2l[MAX_LEVELS + 1] = {};     // [l]: level l-1 -> l, 8 x [2P(l-1)][2P(l)]
     const T* m2l[MAX_LEVELS + 1] = {};     // [l]: 316 x [2P(l)][2P(l)]
     const float* m2l_tiles[MAX_LEVELS + 1] = {};  // tensor-core tiles of m2l[l] (LHV_TF32X3), or null
-    CsrView<T> p2m_sp, l2p_sp;             // P2M(p[L]), L2P(p[L]) in row-compressed form
+    const T* qtab = nullptr;               // recurrence coefficients of the harmonics for p[L]
+    SellView<T> p2m_sp, l2p_sp;            // P2M(p[L]), L2P(p[L]) (v_k alone: filaments, scalar case)
     bool uniform = true;                   // p[l] equal over l = 2..L
     bool scalar = false;                   // scalar reference case: one potential, P x P translation
                                            // tables (the T block of the fused operators), no conversion
@@ -227,6 +231,9 @@ struct Plan {
 };
 
 // ---- expansions (expansions.cu) ----------------------------------------------
+// Coefficients of the recurrences of the harmonics for truncation number p, into dst.
+template <typename T>
+void build_qtab(Ctx* c, int p, Buf& dst);
 // P2M into mult (leaf level), work buffer W: nleaf * 3P reals.
 template <typename T>
 void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
@@ -237,7 +244,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
 // L2L for all levels 2 -> 3 .. L-1 -> L (adds into loc).
 template <typename T>
 void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Grouped& gp, T* loc);
-// L2P at the leaves.
+// L2P at the leaves (sfar null: v alone, with the v_k rows of the map in pl.l2p_sp).
 template <typename T>
 void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
              const vec4_t<T>* ws, const T* loc, vec4_t<T>* vfar, vec4_t<T>* sfar);

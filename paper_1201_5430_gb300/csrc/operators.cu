@@ -24,6 +24,7 @@
 // (m >= 0; Eqs. rsbf2 and rsbf4), and the symmetry above for m < 0.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -404,33 +405,32 @@ int m2l_slot_host(int dx, int dy, int dz) {
 }
 
 void free_operators(OpTables& ops) {
-    Buf* all[] = {&ops.m2l, &ops.m2m, &ops.l2l, &ops.l2p, &ops.p2m, &ops.offsets, &ops.slot_of, &ops.m2l_tiles};
+    Buf* all[] = {&ops.m2l, &ops.m2m, &ops.l2l, &ops.qtab, &ops.offsets, &ops.slot_of, &ops.m2l_tiles};
     for (Buf* b : all) {
         if (b->ptr) cudaFree(b->ptr);
         b->ptr = nullptr;
         b->cap = 0;
     }
-    free_csr(ops.p2m_sp);
-    free_csr(ops.l2p_sp);
+    for (Sell* m : {&ops.p2m_sp, &ops.l2p_sp, &ops.l2pv_sp}) free_sparse(*m);
     ops.p = 0;
 }
 
-void free_csr(Csr& m) {
-    for (Buf* b : {&m.rowptr, &m.col, &m.val}) {
+void free_sparse(Sell& m) {
+    for (Buf* b : {&m.sptr, &m.col, &m.val}) {
         if (b->ptr) cudaFree(b->ptr);
         b->ptr = nullptr;
         b->cap = 0;
     }
     m.rows = 0;
-    m.nnz = 0;
 }
 
 template <typename T>
-void build_sparse(Ctx* c, int kind, int p, Csr& dst) {
+void build_sparse(Ctx* c, int kind, int p, int rows, Sell& dst) {
     // the dense FP64 map (k-major [C][R]), read back once and compressed by rows
     const int P = p * p;
     const int R = kind == OP_P2M ? 2 * P : 12 * P;
     const int C = kind == OP_P2M ? 3 * P : 2 * P;
+    const int nr = rows > 0 ? std::min(rows, R) : R;
     Buf dense;
     std::vector<double> h((size_t)R * C);
     try {
@@ -441,29 +441,37 @@ void build_sparse(Ctx* c, int kind, int p, Csr& dst) {
         throw;
     }
     cudaFree(dense.ptr);
-    std::vector<int> rowptr(R + 1, 0), col;
+    std::vector<std::vector<int>> cols(nr);
+    for (int k = 0; k < C; ++k)
+        for (int r = 0; r < nr; ++r)
+            if (h[(size_t)k * R + r] != 0.0) cols[r].push_back(k);
+    const int ns = (nr + 31) / 32;
+    std::vector<int> sptr(ns + 1, 0), col;
     std::vector<T> val;
-    for (int r = 0; r < R; ++r) {
-        for (int k = 0; k < C; ++k) {
-            const double v = h[(size_t)k * R + r];
-            if (v != 0.0) {
-                col.push_back(k);
-                val.push_back((T)v);
+    for (int q = 0; q < ns; ++q) {
+        const int n = std::min(32, nr - 32 * q);
+        size_t width = 0;
+        for (int i = 0; i < n; ++i) width = std::max(width, cols[32 * q + i].size());
+        sptr[q + 1] = sptr[q] + 32 * (int)width;
+        col.resize(sptr[q + 1], 0);
+        val.resize(sptr[q + 1], (T)0);
+        for (int i = 0; i < n; ++i) {
+            const int r = 32 * q + i;
+            for (int k = 0; k < (int)cols[r].size(); ++k) {
+                col[sptr[q] + 32 * k + i] = cols[r][k];
+                val[sptr[q] + 32 * k + i] = (T)h[(size_t)cols[r][k] * R + r];
             }
         }
-        rowptr[r + 1] = (int)col.size();
     }
-    free_csr(dst);
-    ensure(c, dst.rowptr, (int64_t)(R + 1) * 4);
-    ensure(c, dst.col, (int64_t)std::max<size_t>(col.size(), 1) * 4);
-    ensure(c, dst.val, (int64_t)std::max<size_t>(val.size(), 1) * sizeof(T));
-    cuda_check(cudaMemcpy(dst.rowptr.ptr, rowptr.data(), (R + 1) * 4, cudaMemcpyHostToDevice), "sparse rows");
-    if (!col.empty()) {
-        cuda_check(cudaMemcpy(dst.col.ptr, col.data(), col.size() * 4, cudaMemcpyHostToDevice), "sparse cols");
-        cuda_check(cudaMemcpy(dst.val.ptr, val.data(), val.size() * sizeof(T), cudaMemcpyHostToDevice), "sparse vals");
-    }
-    dst.rows = R;
-    dst.nnz = (int64_t)col.size();
+    free_sparse(dst);
+    auto put = [&](Buf& b, const void* src, size_t bytes) {
+        ensure(c, b, (int64_t)bytes);
+        if (bytes) cuda_check(cudaMemcpy(b.ptr, src, bytes, cudaMemcpyHostToDevice), "sparse map");
+    };
+    put(dst.sptr, sptr.data(), sptr.size() * 4);
+    put(dst.col, col.data(), col.size() * 4);
+    put(dst.val, val.data(), val.size() * sizeof(T));
+    dst.rows = nr;
 }
 
 void m2l_offsets(std::vector<int>& offs, std::vector<int>& slot_of) {
@@ -602,8 +610,6 @@ void build_operators(Ctx* c, int p, OpTables& ops) {
     ops.P = p * p;
     build_op<T>(c, OP_M2M, p, p, ops.m2m);
     build_op<T>(c, OP_L2L, p, p, ops.l2l);
-    build_op<T>(c, OP_L2P, p, p, ops.l2p);
-    build_op<T>(c, OP_P2M, p, p, ops.p2m);
     std::vector<int> offs, slot_of;
     m2l_offsets(offs, slot_of);
     ensure(c, ops.offsets, offs.size() * sizeof(int));
@@ -775,8 +781,8 @@ template void psi_form<double>(Ctx*, const double*, int, int, Buf&);
 template void psi_rows<float>(Ctx*, int64_t, int, int64_t, float*, bool);
 template void psi_rows<double>(Ctx*, int64_t, int, int64_t, double*, bool);
 
-template void build_sparse<float>(Ctx*, int, int, Csr&);
-template void build_sparse<double>(Ctx*, int, int, Csr&);
+template void build_sparse<float>(Ctx*, int, int, int, Sell&);
+template void build_sparse<double>(Ctx*, int, int, int, Sell&);
 template void build_op<float>(Ctx*, int, int, int, Buf&);
 template void build_op<double>(Ctx*, int, int, int, Buf&);
 template void build_operators<float>(Ctx*, int, OpTables&);

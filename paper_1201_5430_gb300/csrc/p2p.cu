@@ -1260,7 +1260,7 @@ void run_p2p(Ctx* c, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs, 
     int strands = 1;
     if constexpr (!std::is_same<T, float>::value) {
         if (ctx_p2p_tpt(c) == 1)
-            while (strands < 8 && n * strands < (int64_t)lv.nbox[L] * (P2P_TILE / 2)) strands *= 2;
+            while (strands < 8 && n * strands < (int64_t)lv.leaves * (P2P_TILE / 2)) strands *= 2;
         auto launch_strands = [&](auto st) {
             constexpr int S = decltype(st)::value;
             int per_sm = 1, sms = 152, dev = 0;

@@ -606,10 +606,25 @@ __global__ void k_tile_counts(int nb, const int* __restrict__ nleaf, const int* 
         cnt[b] = b < nl ? (bend[b] - bbeg[b] + P2P_TILE - 1) / P2P_TILE : 0;
 }
 
+// Also the geometry of every leaf, (centre, 1 / side), for P2M and L2P: in FP64 once per leaf (a warp's
+// FP64 instruction takes 16 cycles of the SM), not once per element.
 __global__ void k_tile_fill(int nb, const int* __restrict__ nleaf, const int* __restrict__ bbeg,
-                            const int* __restrict__ bend, const int* __restrict__ first, int2* __restrict__ tiles) {
+                            const int* __restrict__ bend, const int* __restrict__ first, int2* __restrict__ tiles,
+                            int level, const uint64_t* __restrict__ bkey, const SysCube* __restrict__ cubes,
+                            dbl4* __restrict__ geom) {
     const int nl = min(nb, *nleaf);
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nl; b += gridDim.x * blockDim.x) {
+        // key: Morton bits interleaved x, y, z from bit 0; the system id above bit 3 level
+        const uint64_t key = bkey[b];
+        const SysCube cb = cubes[level > 0 ? (key >> (3 * level)) : key];
+        const uint64_t q = level > 0 ? key & ((~0ull) >> (64 - 3 * level)) : 0ull;
+        const double h = ldexp(cb.side, -level);
+        dbl4 g;
+        g.x = cb.x0[0] + ((double)compact3(q) + 0.5) * h;
+        g.y = cb.x0[1] + ((double)compact3(q >> 1) + 0.5) * h;
+        g.z = cb.x0[2] + ((double)compact3(q >> 2) + 0.5) * h;
+        g.w = 1.0 / h;
+        geom[b] = g;
         int nt = (bend[b] - bbeg[b] + P2P_TILE - 1) / P2P_TILE;
         for (int j = 0; j < nt; ++j) tiles[first[b] + j] = make_int2(b, bbeg[b] + j * P2P_TILE);
     }
@@ -825,6 +840,7 @@ int build_tree(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const vec4_t<
             lv.nbox[l] = (l <= L) ? hcounts[l] : 0;
             lv.off[l + 1] = lv.off[l] + lv.nbox[l];
         }
+        lv.leaves = lv.nbox[L];
     }
     LevelTable lt{};
     lt.L = L;
@@ -856,8 +872,10 @@ int build_tree(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const vec4_t<
         exclusive_scan(c, nl, cnt, first, tb.scan_tmp.as<int>(), tb.tile_count.as<int>());
         int64_t max_tiles = nl + nn / P2P_TILE + 1;
         ensure(c, tb.tiles, max_tiles * 8);
+        ensure(c, tb.geom, (int64_t)nl * sizeof(dbl4));
         k_tile_fill<<<grid_for(nl, 256), 256, 0, s>>>(nl, counts + L, tb.bbeg.as<int>() + o, tb.bend.as<int>() + o,
-                                                      first, tb.tiles.as<int2>());
+                                                      first, tb.tiles.as<int2>(), L, tb.bkey.as<uint64_t>() + o,
+                                                      cubes, tb.geom.as<dbl4>());
         count_launch(c);
         check_launch("tiles");
     }
