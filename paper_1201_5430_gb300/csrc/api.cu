@@ -89,7 +89,8 @@ struct Ctx {
     RcrTables rcr;
     bool rcr_failed = false;            // its tables failed their check: the default form keeps the fused ones
     // scalar reference case (lhv_evaluate_potential_gradient)
-    Buf s_m2l, s_m2m, s_l2l, s_tiles;   // translation blocks of the fused tables, TF32 tiles of the M2L ones
+    Buf s_m2l, s_m2m, s_l2l;            // translation blocks of the fused tables
+    Buf s_tiles, s_m2m_tiles, s_l2l_tiles;  // and their TF32 tiles
     int s_p = 0, s_type = 0;
     Buf qs, pgfar;
     // filament segments (lhv_evaluate_filaments)
@@ -209,8 +210,15 @@ static void ensure_ops(Ctx* c) {
     build_qtab<T>(c, c->cfg.p, c->ops.qtab);
     c->ops_type = (int)sizeof(T);
     if constexpr (sizeof(T) == 4) {
-        if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
-            m2l_tiles_build(c, fused_m2l<float>(c), c->cfg.p, false, c->ops.m2l_tiles);
+        if (ctx_use_tc(c)) {
+            const int p = c->cfg.p;
+            if (tc_trans_supported(TRANS_M2L, p))
+                tc_trans_tiles(c, TRANS_M2L, fused_m2l<float>(c), p, false, c->ops.m2l_tiles);
+            if (tc_trans_supported(TRANS_M2M, p))
+                tc_trans_tiles(c, TRANS_M2M, c->ops.m2m.as<float>(), p, false, c->ops.m2m_tiles);
+            if (tc_trans_supported(TRANS_L2L, p))
+                tc_trans_tiles(c, TRANS_L2L, c->ops.l2l.as<float>(), p, false, c->ops.l2l_tiles);
+        }
     }
 }
 
@@ -232,7 +240,7 @@ static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
         // tensor-core tiles of M2L(p, p)
         if constexpr (sizeof(T) == 4) {
             const float* m2l = cached_op<float>(c, OP_M2L, pout, pout);
-            m2l_tiles_build(c, m2l, pout, false, c->opcache[key]);
+            tc_trans_tiles(c, TRANS_M2L, m2l, pout, false, c->opcache[key]);
         }
     } else {
         build_op<T>(c, kind, pout, pin, b);
@@ -314,7 +322,7 @@ constexpr int RCR_MIN_P = 4;
 template <typename T>
 static bool default_rcr(Ctx* c) {
     if (c->form != LHV_FORM_PHI_CHI || c->tune_nc != 0 || c->rcr_failed || c->cfg.p < RCR_MIN_P) return false;
-    if (sizeof(T) == 4 && ctx_m2l_tc(c) && m2l_tc_supported(c->cfg.p)) return false;
+    if (sizeof(T) == 4 && ctx_m2l_tc(c) && tc_trans_supported(TRANS_M2L, c->cfg.p)) return false;
     return rcr_chunk(c->cfg.p, sizeof(T), nullptr) > 0;
 }
 
@@ -373,6 +381,10 @@ static Plan<T> make_plan(Ctx* c, int L) {
         pl.qtab = c->ops.qtab.as<T>();
         pl.p2m_sp = view<T>(c->ops.p2m_sp);
         pl.l2p_sp = view<T>(c->ops.l2p_sp);
+        if (tiles) {
+            pl.m2m_tiles = c->ops.m2m_tiles.as<float>();
+            pl.l2l_tiles = c->ops.l2l_tiles.as<float>();
+        }
         return pl;
     }
     pl.p2m_sp = cached_sparse<T>(c, OP_P2M, pl.p[L]);
@@ -382,7 +394,7 @@ static Plan<T> make_plan(Ctx* c, int L) {
     pl.l2p_sp = cached_sparse<T>(c, OP_L2P, pl.p[L]);
     for (int l = 2; l <= L; ++l) {
         pl.m2l[l] = cached_op<T>(c, OP_M2L, pl.p[l], pl.p[l]);
-        if (tc && m2l_tc_supported(pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
+        if (tc && tc_trans_supported(TRANS_M2L, pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
         if (l < L) pl.m2m[l] = cached_op<T>(c, OP_M2M, pl.p[l], pl.p[l + 1]);
         if (l > 2) pl.l2l[l] = cached_op<T>(c, OP_L2L, pl.p[l], pl.p[l - 1]);
     }
@@ -468,8 +480,7 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
                                   : all_tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * pmax * pmax));
             m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
-                         mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
@@ -526,10 +537,14 @@ static void ensure_scalar_ops(Ctx* c) {
     translation_block<T>(c, c->ops.m2m.as<T>(), 8, P, c->s_m2m);
     translation_block<T>(c, c->ops.l2l.as<T>(), 8, P, c->s_l2l);
     if constexpr (sizeof(T) == 4) {
-        if (ctx_use_tc(c) && m2l_tc_supported(c->cfg.p))
-            m2l_tiles_build(c, fused_m2l<float>(c), c->cfg.p, true, c->s_tiles);
-        else
-            release(c->s_tiles);
+        const int p = c->cfg.p;
+        auto tiles = [&](TransKind kind, const float* fused, Buf& dst) {
+            if (ctx_use_tc(c) && tc_trans_supported(kind, p)) tc_trans_tiles(c, kind, fused, p, true, dst);
+            else release(dst);
+        };
+        tiles(TRANS_M2L, c->ops.m2l.as<float>(), c->s_tiles);
+        tiles(TRANS_M2M, c->ops.m2m.as<float>(), c->s_m2m_tiles);
+        tiles(TRANS_L2L, c->ops.l2l.as<float>(), c->s_l2l_tiles);
     }
     cuda_check(cudaStreamSynchronize(c->stream), "scalar tables");
     c->s_p = c->cfg.p;
@@ -583,6 +598,10 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             pl.m2l_tiles[l] = c->s_tiles.ptr ? c->s_tiles.as<float>() : nullptr;
         }
         pl.qtab = c->ops.qtab.as<T>();
+        if (sizeof(T) == 4 && ctx_m2l_tc(c)) {
+            pl.m2m_tiles = c->s_m2m_tiles.as<float>();
+            pl.l2l_tiles = c->s_l2l_tiles.as<float>();
+        }
         pl.l2p_sp = velocity_rows<T>(c, p);
         const int64_t nbt = lv.off[L + 1];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
@@ -605,8 +624,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             const int nc = tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(P));
             m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, true, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
-                         mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
@@ -751,8 +769,7 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
             const int nc = pl.rcr ? pl.rcr->nc : tc && c->tune_nc == 0 ? TC_PAIRS : ctx_m2l_nc(c, gemm_nc<T>(2 * PL));
             m2l_prepare(c, c->ops, c->tb, lv, c->table, c->gp_m2l, nc, pl.uniform, cnt + 1);
             StageScope sg(c, LHV_STAGE_M2L_PRODUCTS);
-            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, c->ops.offsets.as<int>(),
-                         mult, loc);
+            m2l_apply<T>(c, pl, lv, c->tb.counts.as<int>(), c->gp_m2l, mult, loc);
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
@@ -1266,7 +1283,7 @@ void lhv_destroy(lhv_ctx* ctx) {
     c.qtabs.clear();
     c.spcache.clear();
     for (auto* b : {&c.sel_W, &c.sel_b, &c.sel_X, &c.sel_Z, &c.sel_choice, &c.sel_idx, &c.sel_dv, &c.sel_ds, &c.sel_err,
-                    &c.s_m2l, &c.s_m2m, &c.s_l2l, &c.s_tiles, &c.qs, &c.pgfar, &c.psi_m2l, &c.psi_m2m,
+                    &c.s_m2l, &c.s_m2m, &c.s_l2l, &c.s_tiles, &c.s_m2m_tiles, &c.s_l2l_tiles, &c.qs, &c.pgfar, &c.psi_m2l, &c.psi_m2m,
                     &c.psi_l2l, &c.psi_tiles, &c.f_off, &c.f_closed, &c.f_seg, &c.f_next, &c.f_segs, &c.f_nexts})
         lhv::release(*b);
     lhv::TreeBufs& t = c.tb;

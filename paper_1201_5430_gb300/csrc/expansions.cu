@@ -568,12 +568,29 @@ static OctItems oct_items(const TreeBufs& tb, const Levels& lv, bool up) {
     return it;
 }
 
-// chunk width for the translations between levels: set by the widest input
+// chunk width for the translations between levels: the MMA's on the tensor cores, else set by the
+// widest input
 template <typename T>
-static int oct_nc(const Plan<T>& pl) {
+static int oct_nc(const Plan<T>& pl, const float* tiles) {
+    if (tiles) return TC_PAIRS;
     int pmax = 1;
     for (int l = 2; l <= pl.L; ++l) pmax = std::max(pmax, pl.p[l]);
     return std::min(16, gemm_nc<T>(2 * pmax * pmax));  // levels hold few boxes: many short items
+}
+
+// One level of M2M or L2L on the tensor cores (LHV_TF32X3, one p a multiple of 4), true if it ran
+// there.  The grouped GEMM streams 250 KB of operator for every 16 boxes (p = 12), here one block T for
+// 128; M2M + L2L, ms: sphere surface of 2^20 2.74 -> 0.56, offset rings of 2^21 (p = 16) 1.13 -> 0.43,
+// 16 blob systems 0.61 -> 0.27, a filament's eleven levels of few boxes 1.51 -> 0.94.
+template <typename T>
+static bool oct_tc(Ctx* c, const Plan<T>& pl, TransKind kind, const float* tiles, Grouped& gp, const GemmArgs<T>& a) {
+    if constexpr (sizeof(T) == 4) {
+        if (tiles) {
+            run_tc_trans(c, kind, gp, a.g0, a.g1, pl.p[pl.L], pl.scalar, tiles, a.in, a.out, a.ldin, ctx_err_flag(c));
+            return true;
+        }
+    }
+    return false;
 }
 
 template <typename T>
@@ -583,7 +600,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
     // parents of the levels 2 .. L-1 accumulate atomically
     fill_level_rows<T>(c, lv, tb.counts.as<int>(), 2, L - 1, pl.ld, 0, mult, (T)0);
     const int nitems = lv.off[L + 1] - lv.off[3];
-    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl), oct_items<T>(tb, lv, true));
+    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl, pl.m2m_tiles), oct_items<T>(tb, lv, true));
     for (int l = L - 1; l >= 2; --l) {
         const int Pout = pl.p[l] * pl.p[l], Pin = pl.p[l + 1] * pl.p[l + 1];
         GemmArgs<T> a{};
@@ -603,7 +620,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.scale = (T)1;
         a.pairs_hint = lv.nbox[l + 1];
         a.may_split_k = 1;
-        run_group_gemm<T>(c, gp, a);
+        if (!oct_tc(c, pl, TRANS_M2M, pl.m2m_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }
 
@@ -612,7 +629,7 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
     const int L = lv.L;
     if (L < 3) return;
     const int nitems = lv.off[L + 1] - lv.off[3];
-    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl), oct_items<T>(tb, lv, false));
+    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl, pl.l2l_tiles), oct_items<T>(tb, lv, false));
     for (int l = 2; l < L; ++l) {
         const int Pout = pl.p[l + 1] * pl.p[l + 1], Pin = pl.p[l] * pl.p[l];
         GemmArgs<T> a{};
@@ -632,7 +649,7 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.scale = (T)1;
         a.pairs_hint = lv.nbox[l + 1];
         a.may_split_k = 1;
-        run_group_gemm<T>(c, gp, a);
+        if (!oct_tc(c, pl, TRANS_L2L, pl.l2l_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }
 

@@ -97,13 +97,15 @@ void tc_tiles_build(Ctx* c, const float* ops, int ngroups, int R, int C, Buf& ti
 void run_tc_gemm(Ctx* c, Grouped& gp, GemmArgs<float> a, const float* tiles, const float* in_hi,
                  const float* in_lo, int* err);
 
-// tensor-core M2L of the two-potential and scalar forms (tc_m2l.cu): p a multiple of 4.
-// m2l_tiles_build lays out the translation blocks of the 316 fused tables; run_tc_m2l adds the
-// translated (and, unless scalar, converted) rows of the groups [g0, g1) to out.
-bool m2l_tc_supported(int p);
-void m2l_tiles_build(Ctx* c, const float* fused, int p, bool scalar, Buf& tiles);
-void run_tc_m2l(Ctx* c, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
-                const int* offsets, const float* in, float* out, int64_t ld, int* err);
+// Tensor-core translations of the two-potential and scalar forms (tc_m2l.cu), one p a multiple of
+// 4.  tc_trans_tiles lays out the translation blocks of the fused tables (316 of M2L, 8 of M2M or
+// L2L) and the conversion's tables; run_tc_trans adds the translated (and, unless scalar,
+// converted) rows of the groups [g0, g1) to out.
+enum TransKind : int { TRANS_M2L = 0, TRANS_M2M = 1, TRANS_L2L = 2 };
+bool tc_trans_supported(TransKind kind, int p);
+void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scalar, Buf& tiles);
+void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
+                  const float* in, float* out, int64_t ld, int* err);
 // hi / lo of the rows of the real boxes of levels l0..l1 (ld reals each; device counts)
 void tc_split(Ctx* c, const Levels& lv, const int* count, int l0, int l1, int64_t ld, const float* x, float* hi,
               float* lo);

@@ -166,7 +166,8 @@ struct OpTables {
     Buf m2l;                   // [316][2P][2P] fused (S|R) + Eq. drt10 per offset slot (built when a route needs it)
     Buf m2m;                   // [8][2P][2P]   fused (S|S) + Eq. drt11 per child octant
     Buf l2l;                   // [8][2P][2P]   fused (R|R) + Eq. drt10 per child octant
-    Buf m2l_tiles;             // TF32 hi/lo tiles of the translation blocks of m2l (LHV_TF32X3, tc_m2l.cu)
+    // TF32 hi/lo tiles of the translation blocks of the three tables (LHV_TF32X3, tc_m2l.cu)
+    Buf m2l_tiles, m2m_tiles, l2l_tiles;
     // sparse maps (structural zeros dropped): P2M 3P -> 2P (Eq. eve4 for w = i_x, i_y, i_z), L2P
     // 2P -> 12P (v_k of Eq. evf3, u_lk of Eq. dt3), and the 3P rows v_k of it alone (built on first use)
     Sell p2m_sp, l2p_sp, l2pv_sp;
@@ -217,6 +218,8 @@ struct Plan {
     const T* l2l[MAX_LEVELS + 1] = {};     // [l]: level l-1 -> l, 8 x [2P(l-1)][2P(l)]
     const T* m2l[MAX_LEVELS + 1] = {};     // [l]: 316 x [2P(l)][2P(l)]
     const float* m2l_tiles[MAX_LEVELS + 1] = {};  // tensor-core tiles of m2l[l] (LHV_TF32X3), or null
+    const float* m2m_tiles = nullptr;      // tensor-core tiles of m2m / l2l (LHV_TF32X3, one p), or null
+    const float* l2l_tiles = nullptr;
     const T* qtab = nullptr;               // recurrence coefficients of the harmonics for p[L]
     SellView<T> p2m_sp, l2p_sp;            // P2M(p[L]), L2P(p[L]) (v_k alone: filaments, scalar case)
     bool uniform = true;                   // p[l] equal over l = 2..L
@@ -276,11 +279,9 @@ void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels&
 // offset; else by (level, offset), through the interaction table in `table_buf`.
 void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& lv, Buf& table_buf, Grouped& gp,
                  int nc, bool uniform, unsigned long long* pair_counter);
-// the products; loc must be zero for levels >= 2; count: boxes per level (device); offsets:
-// OpTables::offsets.
+// the products; loc must be zero for levels >= 2; count: boxes per level (device).
 template <typename T>
-void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const int* offsets,
-               const T* mult, T* loc);
+void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const T* mult, T* loc);
 
 // ---- RCR translations (rcr.cu) -------------------------------------------------
 // M2L by rotation - coaxial translation - back rotation with the coaxial conversion of

@@ -224,8 +224,7 @@ void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& 
 }
 
 template <typename T>
-void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const int* offsets,
-               const T* mult, T* loc) {
+void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Grouped& gp, const T* mult, T* loc) {
     const int L = lv.L;
     if (pl.rcr) {  // rotation - coaxial - rotation (rcr.cu)
         rcr_apply<T>(c, *pl.rcr, gp, mult, loc, pl.ld);
@@ -273,8 +272,8 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
             if (ctx_m2l_tc(c) && pl.m2l_tiles[l0]) {
                 if (pl.psi) run_tc_gemm(c, gp, a, pl.m2l_tiles[l0], mhi, mlo, ctx_err_flag(c));
                 else
-                    run_tc_m2l(c, gp, a.g0, a.g1, pl.p[l0], pl.scalar, pl.m2l_tiles[l0], offsets, mult, loc, pl.ld,
-                               ctx_err_flag(c));
+                    run_tc_trans(c, TRANS_M2L, gp, a.g0, a.g1, pl.p[l0], pl.scalar, pl.m2l_tiles[l0], mult, loc, pl.ld,
+                                 ctx_err_flag(c));
                 done = true;
             }
         }
@@ -283,9 +282,8 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
     }
 }
 
-template void m2l_apply<float>(Ctx*, const Plan<float>&, const Levels&, const int*, Grouped&, const int*,
-                               const float*, float*);
-template void m2l_apply<double>(Ctx*, const Plan<double>&, const Levels&, const int*, Grouped&, const int*,
-                                const double*, double*);
+template void m2l_apply<float>(Ctx*, const Plan<float>&, const Levels&, const int*, Grouped&, const float*, float*);
+template void m2l_apply<double>(Ctx*, const Plan<double>&, const Levels&, const int*, Grouped&, const double*,
+                                double*);
 
 }  // namespace lhv

@@ -1,6 +1,6 @@
-// Tensor-core (tcgen05, TF32) M2L: translation by one block, conversion in the epilogue.
+// Tensor-core (tcgen05, TF32) translations: M2L, and M2M and L2L with the same kernel.
 //
-// The fused M2L operator of an offset t is [[T, C12 T], [0, C22 T]] (Eqs. mr3, drt10): the
+// The fused operator of a translation t is [[T, C12 T], [0, C22 T]] (Eqs. mr3, drt10, drt11): the
 // same translation T for both potentials, then the conversion, which couples each (n, m) to
 // at most six reals of the translated chi and whose coefficients are linear in t.  So the
 // products are only  phi^ = T phi,  chi^ = T chi  (4 p^4 multiply-adds' flops a pair instead of
@@ -13,6 +13,12 @@
 //   d = sqrt((n-m+1)(n-m+2)) / 2(n+1),  e = -sqrt((n+m+1)(n+m+2)) / 2(n+1),
 //   f = -sqrt((n+1-m)(n+1+m)) / (n+1)   (d = e = f = 0 at n = p - 1: the chi_p term is dropped);
 //   at m = 0 the m - 1 terms are the conjugates of the m + 1 terms: a and e doubled, b = d = 0.
+// L2L converts in the same (R) basis; its T block carries the change of scale from the parent's
+// box to the child's of phi, and chi takes half of it (one length more, Eq. 4).  M2M converts in
+// the S basis (Eq. drt11), chi~ from the degree below:
+//   a = -sqrt((n-m)(n+m+1)) / 2(n+1),  b = sqrt((n+m)(n-m+1)) / 2(n+1),  z = -m / (n+1),
+//   d = -sqrt((n+m)(n+m-1)) / 2n,  e = sqrt((n-m)(n-m-1)) / 2n,  f = sqrt((n-m)(n+m)) / n  (0 at n = 0),
+// and chi takes twice the T block's scale of phi.
 // The scalar reference case is the same kernel with one potential and no conversion.
 //
 // D (128 pairs x N) = X (128 x P) T^T (P x N) per potential, D in TMEM in FP32 (phi^ and chi^
@@ -81,7 +87,6 @@ struct M2lArgs {
     int p, P;
     const float* tiles;      // per slot: ranges x K chunks x [hi | lo] tiles
     int64_t group_stride;    // floats per slot
-    const int* offsets;      // [316][3] source box - target box
     int nranges;
     int n0[M2_MAX_RANGES], n1[M2_MAX_RANGES];   // output degrees [n0, n1) of each range
     int c0[M2_MAX_RANGES], nlen[M2_MAX_RANGES]; // its columns [c0, c0 + nlen) (with the halo, 16-padded)
@@ -89,6 +94,9 @@ struct M2lArgs {
     int nstages, stage_bytes;
     int nbuf;                // accumulator buffers (each M2_TMEM / nbuf columns)
     const float* conv;       // [p (p + 1) / 2 + 8][8]: a, b, z, d | e, f, 0, 0 of (n, m) at n (n + 1) / 2 + m
+    const float* tvec;       // [ngroups][4]: t of each operator, in box sides of the conversion's basis
+    float chi_scale;         // chi^ = chi_scale T chi (1; L2L 1/2, M2M 2)
+    int ngroups;             // operators (a group's is g % ngroups)
     int* err;
 };
 
@@ -185,15 +193,21 @@ __device__ __forceinline__ void order_zero(uint32_t (&x)[N]) {
     x[3] = 0u;
 }
 
+// What the epilogue does with the translated potentials.
+enum TransMode : int { TM_SCALAR = 0, TM_R = 1, TM_S = 2 };  // one potential; Eq. drt10; Eq. drt11
+
 // Converts the orders [mb, mb + 8) of degree n of this thread's pair and writes them to the
-// staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n (tmem_orders,
-// order_zero applied); on return that of degree n + 1, so that a run of degrees reads each once.
+// staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n (R basis; S basis:
+// n - 1) as read by tmem_orders with order_zero applied; on return that of the next degree, so
+// that a run of degrees reads each once.
+template <int MODE>
 __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uint32_t tc, int c0, int p, int n,
-                                               int mb, float tx, float ty, float tz, uint32_t (&x)[20], float* op,
-                                               float* oc) {
+                                               int mb, float tx, float ty, float tz, float cs, uint32_t (&x)[20],
+                                               float* op, float* oc) {
     uint32_t y[20], f[16];
-    const bool up = n + 1 < p;
-    if (up) tmem_orders(tc + (uint32_t)((n + 1) * (n + 1) - c0 + 2 * mb - 3), n + 1, mb, y);
+    const int nx = MODE == TM_R ? n + 1 : n;  // the degree read here
+    const bool up = nx < p;
+    if (up) tmem_orders(tc + (uint32_t)(nx * nx - c0 + 2 * mb - 3), nx, mb, y);
     if (n > 0) tmem_ld16_async(tp + (uint32_t)(n * n - c0 + 2 * mb - 1), f);
     else tmem_ld1(tp - (uint32_t)c0, f[1]);
     tmem_wait(f);
@@ -221,14 +235,16 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
             const float ax = g.x * tx, ay = g.x * ty, bx = g.y * tx, by = g.y * ty, z = g.z * tz;
             const float dx = g.w * tx, dy = g.w * ty, ex = e.x * tx, ey = e.x * ty, fz = e.y * tz;
             auto F = [](uint32_t u) { return __uint_as_float(u); };
-            const float mr = F(x[2 * i]), mi = F(x[2 * i + 1]), cr = F(x[2 * i + 2]), ci = F(x[2 * i + 3]);
-            const float pr = m < n ? F(x[2 * i + 4]) : 0.f, pi = m < n ? F(x[2 * i + 5]) : 0.f;
-            const float umr = F(y[2 * i]), umi = F(y[2 * i + 1]), ucr = F(y[2 * i + 2]), uci = F(y[2 * i + 3]),
-                        upr = F(y[2 * i + 4]), upi = F(y[2 * i + 5]);
+            const uint32_t* u = MODE == TM_R ? x : y;  // degree n
+            const uint32_t* w = MODE == TM_R ? y : x;  // degree n + 1 (R), n - 1 (S)
+            const float mr = F(u[2 * i]), mi = F(u[2 * i + 1]), cr = F(u[2 * i + 2]), ci = F(u[2 * i + 3]);
+            const float pr = m < n ? F(u[2 * i + 4]) : 0.f, pi = m < n ? F(u[2 * i + 5]) : 0.f;
+            const float umr = F(w[2 * i]), umi = F(w[2 * i + 1]), ucr = F(w[2 * i + 2]), uci = F(w[2 * i + 3]),
+                        upr = F(w[2 * i + 4]), upi = F(w[2 * i + 5]);
             const float o0 = fmaf(ax, pr, fmaf(-ay, pi, fmaf(bx, mr, fmaf(by, mi, fmaf(-z, ci, F(f[2 * i]))))));
-            const float q0 = fmaf(ey, upr, fmaf(ex, upi, fmaf(dy, umr, fmaf(-dx, umi, fmaf(fz, ucr, cr)))));
+            const float q0 = fmaf(ey, upr, fmaf(ex, upi, fmaf(dy, umr, fmaf(-dx, umi, fmaf(fz, ucr, cs * cr)))));
             const float o1 = fmaf(ax, pi, fmaf(ay, pr, fmaf(bx, mi, fmaf(-by, mr, fmaf(z, cr, F(f[2 * i + 1]))))));
-            const float q1 = fmaf(ey, upi, fmaf(-ex, upr, fmaf(dy, umi, fmaf(dx, umr, fmaf(fz, uci, ci)))));
+            const float q1 = fmaf(ey, upi, fmaf(-ex, upr, fmaf(dy, umi, fmaf(dx, umr, fmaf(fz, uci, cs * ci)))));
             if (m <= n) {
                 const int at = (m ? 2 * i : 2 * i + 1) * M2_STG_LD;
                 op0[at] = o0;
@@ -244,8 +260,9 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
     for (int k = 0; k < 20; ++k) x[k] = y[k];
 }
 
-template <int NPOT>
+template <int MODE>
 __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant__ M2lArgs a) {
+    constexpr int NPOT = MODE == TM_SCALAR ? 1 : 2;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ M2lShared sh;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -374,7 +391,7 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
             bool ok = true;
             for (int item = blockIdx.x; item < nwork && ok; item += gridDim.x) {
                 const int r = item % a.nranges;
-                const int slot = a.chunks[c_beg + item / a.nranges].x % NUM_OFFSETS;
+                const int slot = a.chunks[c_beg + item / a.nranges].x % a.ngroups;
                 const uint32_t bytes = (uint32_t)a.nlen[r] * TC_KC * 4 * 2;
                 const float* src = a.tiles + (int64_t)slot * a.group_stride + a.roff[r];
                 for (int k = 0; k < nk; ++k) {
@@ -510,9 +527,7 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                 }
             } else {
                 const uint32_t tc = tp + (uint32_t)nlen;
-                const int slot = ch.x % NUM_OFFSETS;
-                const float tx = (float)-a.offsets[3 * slot], ty = (float)-a.offsets[3 * slot + 1],
-                            tz = (float)-a.offsets[3 * slot + 2];
+                const float4 tv = __ldg(reinterpret_cast<const float4*>(a.tvec) + ch.x % a.ngroups);
                 for (int na = n0; na < n1;) {
                     int nb = na + 1;  // degrees [na, nb) fit the band
                     while (nb < n1 && (nb + 1) * (nb + 1) - na * na <= M2_BAND) ++nb;
@@ -529,12 +544,19 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                         }
                         if (d0 >= d1) continue;
                         uint32_t x[20];
-                        tmem_orders(tc + (uint32_t)(d0 * d0 - c0 + 2 * mb - 3), d0, mb, x);
-                        tmem_wait(x);
-                        if (mb == 0) order_zero(x);
+                        const int dx = MODE == TM_R ? d0 : d0 - 1;
+                        if (dx >= 0) {
+                            tmem_orders(tc + (uint32_t)(dx * dx - c0 + 2 * mb - 3), dx, mb, x);
+                            tmem_wait(x);
+                            if (mb == 0) order_zero(x);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 20; ++k) x[k] = 0u;
+                        }
                         for (int dn = d0; dn < d1; ++dn) {
                             const int at = (dn * dn - na * na) * M2_STG_LD + row;
-                            convert_orders(conv, tp, tc, c0, a.p, dn, mb, tx, ty, tz, x, stg + at, stc + at);
+                            convert_orders<MODE>(conv, tp, tc, c0, a.p, dn, mb, tv.x, tv.y, tv.z, a.chi_scale, x, stg + at,
+                                                 stc + at);
                         }
                     }
                     if (nb == n1) release(b);
@@ -554,11 +576,11 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)M2_TMEM) : "memory");
 }
 
-// tiles[slot][range][k chunk][hi | lo][tile_off order] of the translation block T of the fused
-// tables: T[k][c] = ops[slot][k ldo + c], k, c < P
+// tiles[group][range][k chunk][hi | lo][tile_off order] of the translation block T of the fused
+// tables: T[k][c] = ops[group][k ldo + c], k, c < P
 __global__ void k_m2l_tiles(const float* __restrict__ ops, int64_t op_floats, int ldo, M2lArgs a,
                             float* __restrict__ tiles) {
-    for (int g = blockIdx.x; g < NUM_OFFSETS; g += gridDim.x) {
+    for (int g = blockIdx.x; g < a.ngroups; g += gridDim.x) {
         const float* Ag = ops + (int64_t)g * op_floats;
         float* tg = tiles + (int64_t)g * a.group_stride;
         for (int r = 0; r < a.nranges; ++r) {
@@ -599,10 +621,11 @@ int chi_read_end(int p, int n0, int n1) {
 // surface of 2^20, p = 12: products 3.6 ms against 1.8 without the epilogue, 9.3 against 4.9 with
 // it): the narrow MMAs are bound by their operand reads from shared memory, and the reads of
 // TMEM queue behind them.
-M2lArgs m2l_layout(int p, int npot) {
+M2lArgs m2l_layout(int p, int npot, int ngroups) {
     M2lArgs a{};
     a.p = p;
     a.P = p * p;
+    a.ngroups = ngroups;
     a.nbuf = npot == 1 || p <= 8 ? 2 : 1;
     int64_t off = 0;
     int nmax = 0;
@@ -637,40 +660,62 @@ M2lArgs m2l_layout(int p, int npot) {
 
 }  // namespace
 
-bool m2l_tc_supported(int p) { return p % 4 == 0 && p >= 4 && p <= 24; }
-
-void m2l_tiles_build(Ctx* c, const float* fused, int p, bool scalar, Buf& tiles) {
-    M2lArgs a = m2l_layout(p, scalar ? 1 : 2);
-    const int64_t nt = a.group_stride * NUM_OFFSETS;
-    std::vector<float> conv((size_t)conv_floats(p), 0.f);
-    for (int n = 0; n < p; ++n)
-        for (int m = 0; m <= n; ++m) {
-            float* v = &conv[(size_t)(n * (n + 1) / 2 + m) * 8];
-            const double two = m ? 1.0 : 2.0;
-            if (n > 0) {
-                v[0] = (float)(-two * std::sqrt((double)(n - m) * (n + m + 1)) / (2.0 * n));
-                v[1] = m ? (float)(std::sqrt((double)(n + m) * (n - m + 1)) / (2.0 * n)) : 0.f;
-                v[2] = (float)((double)m / n);
-            }
-            if (n + 1 < p) {
-                v[3] = m ? (float)(std::sqrt((double)(n - m + 1) * (n - m + 2)) / (2.0 * (n + 1))) : 0.f;
-                v[4] = (float)(-two * std::sqrt((double)(n + m + 1) * (n + m + 2)) / (2.0 * (n + 1)));
-                v[5] = (float)(-std::sqrt((double)(n + 1 - m) * (n + 1 + m)) / (n + 1));
-            }
-        }
-    ensure(c, tiles, (nt + (int64_t)conv.size()) * (int64_t)sizeof(float));
-    k_m2l_tiles<<<NUM_OFFSETS, 256, 0, stream_of(c)>>>(fused, 4 * (int64_t)a.P * a.P, 2 * a.P, a, tiles.as<float>());
-    count_launch(c);
-    check_launch("m2l tiles");
-    cuda_check(cudaMemcpyAsync(tiles.as<float>() + nt, conv.data(), conv.size() * sizeof(float),
-                               cudaMemcpyHostToDevice, stream_of(c)),
-               "m2l conversion");
-    cuda_check(cudaStreamSynchronize(stream_of(c)), "m2l tiles");
+bool tc_trans_supported(TransKind kind, int p) {
+    // above p = 16 the accumulators are split into ranges of degrees whose halo is the degree above;
+    // M2M's conversion reads the degree below
+    return p % 4 == 0 && p >= 4 && p <= (kind == TRANS_M2M ? 16 : 24);
 }
 
-void run_tc_m2l(Ctx* c, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
-                const int* offsets, const float* in, float* out, int64_t ld, int* err) {
-    M2lArgs a = m2l_layout(p, scalar ? 1 : 2);
+void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scalar, Buf& tiles) {
+    const int ng = kind == TRANS_M2L ? NUM_OFFSETS : 8;
+    M2lArgs a = m2l_layout(p, scalar ? 1 : 2, ng);
+    const int64_t nt = a.group_stride * ng;
+    // conversion table, then the translation vectors
+    std::vector<float> tab((size_t)conv_floats(p), 0.f);
+    const double in_chi = kind == TRANS_L2L ? 0.5 : 1.0;  // chi^ = in_chi T chi in these coefficients
+    for (int n = 0; n < p; ++n)
+        for (int m = 0; m <= n; ++m) {
+            float* v = &tab[(size_t)(n * (n + 1) / 2 + m) * 8];
+            const double two = m ? 1.0 : 2.0, one = m ? 1.0 : 0.0;
+            const double den = kind == TRANS_M2M ? n + 1.0 : (double)n;
+            if (den > 0.0) {
+                v[0] = (float)(-two * in_chi * std::sqrt((double)(n - m) * (n + m + 1)) / (2.0 * den));
+                v[1] = (float)(one * in_chi * std::sqrt((double)(n + m) * (n - m + 1)) / (2.0 * den));
+                v[2] = (float)((kind == TRANS_M2M ? -1.0 : 1.0) * in_chi * m / den);
+            }
+            if (kind == TRANS_M2M) {
+                if (n > 0) {
+                    v[3] = (float)(-one * std::sqrt((double)(n + m) * (n + m - 1)) / (2.0 * n));
+                    v[4] = (float)(two * std::sqrt((double)(n - m) * std::max(n - m - 1, 0)) / (2.0 * n));
+                    v[5] = (float)(std::sqrt((double)(n - m) * (n + m)) / n);
+                }
+            } else if (n + 1 < p) {
+                v[3] = (float)(one * in_chi * std::sqrt((double)(n - m + 1) * (n - m + 2)) / (2.0 * (n + 1)));
+                v[4] = (float)(-two * in_chi * std::sqrt((double)(n + m + 1) * (n + m + 2)) / (2.0 * (n + 1)));
+                v[5] = (float)(-in_chi * std::sqrt((double)(n + 1 - m) * (n + 1 + m)) / (n + 1));
+            }
+        }
+    std::vector<int> offs, slot_of;
+    m2l_offsets(offs, slot_of);
+    for (int g = 0; g < ng; ++g)
+        for (int k = 0; k < 4; ++k) {
+            // M2L: t = target - source = -offset; child octant o: t = 0.5 - o (M2M), o - 0.5 (L2L), in child sides
+            const float o = (float)((g >> k) & 1);
+            tab.push_back(k == 3 ? 0.f : kind == TRANS_M2L ? (float)-offs[3 * g + k] : kind == TRANS_M2M ? 0.5f - o : o - 0.5f);
+        }
+    ensure(c, tiles, (nt + (int64_t)tab.size()) * (int64_t)sizeof(float));
+    k_m2l_tiles<<<ng, 256, 0, stream_of(c)>>>(fused, 4 * (int64_t)a.P * a.P, 2 * a.P, a, tiles.as<float>());
+    count_launch(c);
+    check_launch("translation tiles");
+    cuda_check(cudaMemcpyAsync(tiles.as<float>() + nt, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice,
+                               stream_of(c)),
+               "translation tables");
+    cuda_check(cudaStreamSynchronize(stream_of(c)), "translation tiles");
+}
+
+void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
+                  const float* in, float* out, int64_t ld, int* err) {
+    M2lArgs a = m2l_layout(p, scalar ? 1 : 2, kind == TRANS_M2L ? NUM_OFFSETS : 8);
     a.chunks = gp.chunks.as<int4>();
     a.pairs = gp.pairs.as<int2>();
     a.choff = gp.choff.as<int>();
@@ -680,20 +725,21 @@ void run_tc_m2l(Ctx* c, const Grouped& gp, int g0, int g1, int p, bool scalar, c
     a.out = out;
     a.ld = ld;
     a.tiles = tiles;
-    a.conv = tiles + a.group_stride * NUM_OFFSETS;
-    a.offsets = offsets;
+    a.conv = tiles + a.group_stride * a.ngroups;
+    a.tvec = a.conv + conv_floats(p);
+    a.chi_scale = kind == TRANS_M2L ? 1.0f : kind == TRANS_L2L ? 0.5f : 2.0f;
     a.err = err;
     // above half an SM's shared memory: one CTA (and its 512 TMEM columns) per SM
     const size_t smem =
         std::max<size_t>((size_t)a.nstages * a.stage_bytes + m2l_fixed_smem(p, scalar ? 1 : 2), 120 * 1024);
-    auto kernel = scalar ? k_tc_m2l<1> : k_tc_m2l<2>;
-    cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "m2l smem");
+    auto kernel = scalar ? k_tc_m2l<TM_SCALAR> : kind == TRANS_M2M ? k_tc_m2l<TM_S> : k_tc_m2l<TM_R>;
+    cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "translation smem");
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     kernel<<<sms, M2_THREADS, smem, stream_of(c)>>>(a);
     count_launch(c);
-    check_launch("tc m2l");
+    check_launch("tc translation");
 }
 
 }  // namespace lhv

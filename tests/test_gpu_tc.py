@@ -80,3 +80,32 @@ def test_m2l_converts_like_the_fused_table(p, n, leaf):
         ctx.close()
     for a, b in zip(got[1], got[0]):
         assert rel(a, b) < 2e-6, rel(a, b)
+
+
+@pytest.mark.parametrize("p", [4, 8, 12, 16, 20])
+@pytest.mark.parametrize("n,leaf,nsys", [(3000, 4, 1), (60, 1, 5)])
+def test_levels_translate_like_the_fused_tables(p, n, leaf, nsys):
+    """M2M and L2L on the tensor cores (several levels, few and many boxes an octant) against the
+    fused tables on the CUDA cores: the exported multipoles of every level, the locals of the leaves
+    and the field.  A coefficient passes up to seven levels of 2 p^2 rounded terms:
+    7 sqrt(2 20^2) 2^-24 = 1.2e-5 at most, 2e-6 a level."""
+    import torch
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n * nsys, 21)
+    off = [n * k for k in range(nsys + 1)]
+    q = torch.from_numpy(workloads.charges(n * nsys, 4)).cuda()
+    got = {}
+    for tc in (1, 0):
+        ctx = LHV(p=p, leaf_max=leaf, core_a=0.0, precision="tf32x3", terms="far")
+        ctx.set_launch_shape(m2l_pairs_per_chunk=64, m2l_tensor_cores=tc)
+        v4, s4 = ctx.evaluate_batched(off, dev(x, "fp32"), dev(w, "fp32"))
+        L = ctx.stats()["leaf_level"]
+        assert L >= 4
+        out = [ctx.export("multipole", l).double().cpu().numpy() for l in range(2, L + 1)]
+        out += [ctx.export("local", l).double().cpu().numpy() for l in range(2, L + 1)]
+        out += [host3(v4), host3(s4)]
+        out.append(ctx.evaluate_potential_gradient(dev(x, "fp32"), q).double().cpu().numpy())
+        got[tc] = out
+        ctx.close()
+    for a, b in zip(got[1], got[0]):
+        assert np.linalg.norm(a - b) < 1.2e-5 * np.linalg.norm(b), np.linalg.norm(a - b) / np.linalg.norm(b)
