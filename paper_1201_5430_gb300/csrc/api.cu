@@ -1287,7 +1287,7 @@ void lhv_destroy(lhv_ctx* ctx) {
                     &c.psi_l2l, &c.psi_tiles, &c.f_off, &c.f_closed, &c.f_seg, &c.f_next, &c.f_segs, &c.f_nexts})
         lhv::release(*b);
     lhv::TreeBufs& t = c.tb;
-    lhv::Buf* tree[] = {&t.keys_a, &t.keys_b, &t.idx_a, &t.idx_b, &t.hist, &t.boxof_a, &t.boxof_b, &t.flags,
+    lhv::Buf* tree[] = {&t.keys_a, &t.keys_b, &t.idx, &t.hist, &t.boxof, &t.flags,
                         &t.scan_tmp, &t.perm, &t.params, &t.counts, &t.bkey, &t.bbeg, &t.bend, &t.bparent,
                         &t.bcbeg, &t.bcend, &t.bcol, &t.tiles, &t.tile_count, &t.geom, &t.cubes, &t.sysoff};
     for (auto* b : tree) lhv::release(*b);

@@ -43,7 +43,8 @@ struct TreeParams {
     int bits;           // Morton bits per axis
     int nsys;
     int L_cap;          // deepest level any tree of these cubes may have: min(L_K, the level cap, bits)
-    int pad[2];
+    int ticket;         // blocks of the running launch that are done
+    int pad;
 };
 
 // Growable device allocation.
@@ -108,9 +109,9 @@ inline int grid_for(int64_t n, int block, int cap = 152 * 32) {
 
 // ---- tree (tree.cu) ---------------------------------------------------------
 struct TreeBufs {
-    Buf keys_a, keys_b, idx_a, idx_b, hist, boxof_a, boxof_b, flags, scan_tmp;
+    Buf keys_a, keys_b, idx, hist, boxof, flags, scan_tmp;
     Buf perm;                  // int32[n]
-    Buf params;                // TreeParams (device)
+    Buf params;                // TreeParams, then a block counter per system (device)
     Buf cubes;                 // SysCube[nsys] (device)
     Buf sysoff;                // int64[nsys + 1] element offsets of the systems (device)
     Buf counts;                // int32[64] (device)
@@ -121,7 +122,7 @@ struct TreeBufs {
 
 // Builds keys, sort, levels and lists for n positions (device [n][4] of T) of
 // nsys systems (host offsets sysoff[0..nsys], sysoff[0] = 0, sysoff[nsys] = n).
-// On return `lv` (host) is filled; two short stream synchronisations happen inside.
+// On return `lv` (host) is filled; one short stream synchronisation happens inside.
 template <typename T>
 int build_tree(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const vec4_t<T>* x4, const vec4_t<T>* w4,
                TreeBufs& tb, Levels& lv, TreeParams& hp, Error& err);

@@ -111,3 +111,33 @@ def test_full_size_ring_keys():
     np.testing.assert_array_equal(ctx.export("keys").cpu().numpy().view(np.uint64), keys[perm])
     np.testing.assert_array_equal(ctx.export("perm").cpu().numpy(), perm)
     assert ctx.stats()["leaf_level"] == T.leaf_level(keys[perm], 64, side, workloads.RING_CORE_A, 1e-6)
+
+
+@pytest.mark.parametrize("n", [1023, 1025, 65536, 65537, 262145, 2097153])
+@pytest.mark.parametrize("kind", ["cloud", "lattice", "thin", "tiny"])
+def test_keys_and_order_at_the_edges_of_the_sort(n, kind):
+    """Sizes around the sort's tile and its changes of tile; positions on cell faces (lattice), far from
+    the origin with an extent near one ulp (thin: many equal keys), and below the float cell's range (tiny)."""
+    from paper_1201_5430_gb300 import LHV
+    if kind != "cloud" and n > 65537:
+        pytest.skip("covered by the smaller sizes")
+    rng = np.random.default_rng(n)
+    x = rng.random((n, 3)).astype(np.float32)
+    if kind == "lattice":
+        x = np.floor(x * np.float32(64.0)) * np.float32(0.75) - np.float32(8.0)
+    elif kind == "thin":
+        x = np.float32(4096.0) + x * np.float32(0.01)
+    elif kind == "tiny":
+        x = x * np.float32(1e-18)
+    ctx = LHV(p=4, leaf_max=64, max_level=4)
+    ctx.build_tree(dev(x, "fp32"))
+    keys, _, _ = T.morton_keys(x)
+    perm = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(ctx.export("keys").cpu().numpy().view(np.uint64), keys[perm])
+    np.testing.assert_array_equal(ctx.export("perm").cpu().numpy(), perm)
+    ctx.close()
+
+
+def test_colleagues_of_many_leaves():
+    """Enough leaves (above 8192) that their colleagues come from the parents'."""
+    _check(workloads.cube(30000, 3)[0], 4)
