@@ -484,7 +484,7 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
         }
         vfar = c->vfar.as<vec4_t<T>>();
         sfar = c->sfar.as<vec4_t<T>>();
@@ -628,7 +628,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
         }
         pgfar = c->pgfar.as<vec4_t<T>>();
         {
@@ -773,7 +773,7 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
         }
         vfar = c->vfar.as<vec4_t<T>>();
         {

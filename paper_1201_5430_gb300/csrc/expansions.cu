@@ -555,19 +555,6 @@ void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
     launch_p2m_apply<T>(c, pl, tb, lv, W, mult);
 }
 
-template <typename T>
-static OctItems oct_items(const TreeBufs& tb, const Levels& lv, bool up) {
-    OctItems it{};
-    it.bkey = tb.bkey.as<uint64_t>();
-    it.bparent = tb.bparent.as<int>();
-    it.loff = tb.counts.as<int>() + 32;  // the level scan's offsets of the real boxes
-    for (int l = 0; l <= MAX_LEVELS; ++l) it.off[l] = lv.off[l];
-    it.lo = 3;
-    it.hi = lv.L;
-    it.up = up;
-    return it;
-}
-
 // chunk width for the translations between levels: the MMA's on the tensor cores, else set by the
 // widest input
 template <typename T>
@@ -581,11 +568,17 @@ static int oct_nc(const Plan<T>& pl, const float* tiles) {
 // One level of M2M or L2L on the tensor cores (LHV_TF32X3, one p a multiple of 4), true if it ran
 // there.  The grouped GEMM streams 250 KB of operator for every 16 boxes (p = 12), here one block T for
 // 128; M2M + L2L, ms: sphere surface of 2^20 2.74 -> 0.56, offset rings of 2^21 (p = 16) 1.13 -> 0.43,
-// 16 blob systems 0.61 -> 0.27, a filament's eleven levels of few boxes 1.51 -> 0.94.
+// 16 blob systems 0.61 -> 0.27.  A level of few boxes (b boxes with b p^4 up to OCT_TC_MIN) stays with the
+// grouped GEMM, which splits its sums over the idle SMs: about 12 us at p = 12, 17 at p = 16, where the
+// MMA's one pass over T and its epilogue take 29 and 36.  M2M + L2L of a filament's eleven levels 0.88 -> 0.71, of the
+// ring of 32,768 elements 0.23 -> 0.20, the others as before (twice the limit: offset rings 0.35 -> 0.37).
+constexpr int64_t OCT_TC_MIN = 16000000;
 template <typename T>
-static bool oct_tc(Ctx* c, const Plan<T>& pl, TransKind kind, const float* tiles, Grouped& gp, const GemmArgs<T>& a) {
+static bool oct_tc(Ctx* c, const Plan<T>& pl, TransKind kind, const float* tiles, const Grouped& gp,
+                   const GemmArgs<T>& a) {
     if constexpr (sizeof(T) == 4) {
-        if (tiles) {
+        const int64_t P = pl.p[pl.L] * pl.p[pl.L];
+        if (tiles && a.pairs_hint * P * P > OCT_TC_MIN) {
             run_tc_trans(c, kind, gp, a.g0, a.g1, pl.p[pl.L], pl.scalar, tiles, a.in, a.out, a.ldin, ctx_err_flag(c));
             return true;
         }
@@ -599,8 +592,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
     if (L < 3) return;
     // parents of the levels 2 .. L-1 accumulate atomically
     fill_level_rows<T>(c, lv, tb.counts.as<int>(), 2, L - 1, pl.ld, 0, mult, (T)0);
-    const int nitems = lv.off[L + 1] - lv.off[3];
-    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl, pl.m2m_tiles), oct_items<T>(tb, lv, true));
+    oct_list(c, tb, lv, gp, oct_nc(pl, pl.m2m_tiles));
     for (int l = L - 1; l >= 2; --l) {
         const int Pout = pl.p[l] * pl.p[l], Pin = pl.p[l + 1] * pl.p[l + 1];
         GemmArgs<T> a{};
@@ -618,18 +610,21 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.ldout = pl.ld;
         a.mode = GEMM_ATOMIC;
         a.scale = (T)1;
-        a.pairs_hint = lv.nbox[l + 1];
+        a.pairs_hint = lv.real[l + 1];
         a.may_split_k = 1;
         if (!oct_tc(c, pl, TRANS_M2M, pl.m2m_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }
 
 template <typename T>
-void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Grouped& gp, T* loc) {
+void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const Grouped& up, Grouped& own, T* loc) {
     const int L = lv.L;
     if (L < 3) return;
-    const int nitems = lv.off[L + 1] - lv.off[3];
-    build_grouped(c, gp, (L - 2) * 8, nitems, nitems, oct_nc(pl, pl.l2l_tiles), oct_items<T>(tb, lv, false));
+    // M2M's list serves with the pairs swapped, unless its chunks have another width (p > 16 on the
+    // tensor cores, which take L2L but not M2M there)
+    const int nc = oct_nc(pl, pl.l2l_tiles);
+    if (up.nc != nc) oct_list(c, tb, lv, own, nc);
+    const Grouped& gp = up.nc != nc ? own : up;
     for (int l = 2; l < L; ++l) {
         const int Pout = pl.p[l + 1] * pl.p[l + 1], Pin = pl.p[l] * pl.p[l];
         GemmArgs<T> a{};
@@ -645,9 +640,10 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.ldin = pl.ld;
         a.out = loc;
         a.ldout = pl.ld;
+        a.swap = 1;
         a.mode = GEMM_ATOMIC;  // one parent per child: the plain sum, issued without waiting for the old value
         a.scale = (T)1;
-        a.pairs_hint = lv.nbox[l + 1];
+        a.pairs_hint = lv.real[l + 1];
         a.may_split_k = 1;
         if (!oct_tc(c, pl, TRANS_L2L, pl.l2l_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
@@ -715,7 +711,7 @@ void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels&
     template void run_p2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,            \
                              const vec4_t<T>*, T*, T*);                                                         \
     template void run_m2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, Grouped&, T*);              \
-    template void run_l2l<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, Grouped&, T*);              \
+    template void run_l2l<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const Grouped&, Grouped&, T*); \
     template void run_l2p<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,            \
                              const vec4_t<T>*, const T*, vec4_t<T>*, vec4_t<T>*);                      \
     template void run_p2m_scalar<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,     \

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lhv_internal.cuh"
 #include "lhv_group.cuh"
@@ -47,6 +48,79 @@ __global__ void k_set_total(int ng, const int* __restrict__ cnt, int* __restrict
     if (threadIdx.x == 0 && blockIdx.x == 0) off[ng] = (ng > 0 ? off[ng - 1] + cnt[ng - 1] : 0);
 }
 
+// The children of the levels 3 .. L by (level, octant).  Block b of nblk takes a contiguous range of the
+// real boxes; FILL = false counts them per group to cnt[group][b], and the last block turns the
+// counts into positions, choff[group] into the group's first chunk (choff[ngroups]: their number)
+// and lists the chunks; FILL = true writes the pairs (child, parent) there.  Two launches where ten (count,
+// scan, totals, cursors, fill, and three for the chunks) took 25 to 60 us, twice an evaluation.
+constexpr int OCT_GROUPS = 8 * MAX_LEVELS;
+struct OctLevels {
+    int L;
+    int off[MAX_LEVELS + 1];
+};
+template <bool FILL>
+__global__ void __launch_bounds__(256) k_oct_list(OctLevels lv, const int* __restrict__ loff,
+                                                  const uint64_t* __restrict__ bkey, const int* __restrict__ bparent,
+                                                  int nblk, int* __restrict__ cnt, int nc, int* __restrict__ choff,
+                                                  int4* __restrict__ chunks, int2* __restrict__ pairs,
+                                                  int* __restrict__ ticket) {
+    __shared__ int at[OCT_GROUPS], first[OCT_GROUPS + 1], chunk0[OCT_GROUPS + 1], lo[MAX_LEVELS + 2];
+    const int ng = (lv.L - 2) * 8, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int l = t; l <= lv.L + 1; l += blockDim.x) lo[l] = loff[l];
+    for (int g = t; g < ng; g += blockDim.x) at[g] = FILL ? cnt[g * nblk + blockIdx.x] : 0;
+    __syncthreads();
+    const int64_t nb = lo[lv.L + 1] - lo[3];
+    const int b0 = lo[3] + (int)(nb * blockIdx.x / nblk), b1 = lo[3] + (int)(nb * (blockIdx.x + 1) / nblk);
+    for (int rb = b0 + t; rb < b1; rb += blockDim.x) {
+        int l = 3;
+        while (l < lv.L && rb >= lo[l + 1]) ++l;
+        const int b = lv.off[l] + (rb - lo[l]);
+        const int pos = atomicAdd(&at[(l - 3) * 8 + (int)(bkey[b] & 7ull)], 1);
+        if (FILL) pairs[pos] = make_int2(b, lv.off[l - 1] + bparent[b]);
+    }
+    if (FILL) return;
+    __syncthreads();
+    for (int g = t; g < ng; g += blockDim.x) __stcg(cnt + g * nblk + blockIdx.x, at[g]);
+    if (!last_block(ticket, nblk)) return;
+    for (int g = warp; g < ng; g += 8) {
+        int carry = 0;
+        for (int i0 = 0; i0 < nblk; i0 += 32) {
+            const int v = i0 + lane < nblk ? __ldcg(cnt + g * nblk + i0 + lane) : 0;
+            int x = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (i0 + lane < nblk) __stcg(cnt + g * nblk + i0 + lane, carry + x - v);
+            carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) at[g] = carry;
+    }
+    __syncthreads();
+    if (t == 0) {
+        int f = 0, c = 0;
+        for (int g = 0; g < ng; ++g) {
+            first[g] = f;
+            chunk0[g] = c;
+            f += at[g];
+            c += (at[g] + nc - 1) / nc;
+        }
+        chunk0[ng] = c;
+    }
+    __syncthreads();
+    for (int i = t; i < ng * nblk; i += blockDim.x) __stcg(cnt + i, __ldcg(cnt + i) + first[i / nblk]);
+    for (int g = t; g <= ng; g += blockDim.x) choff[g] = chunk0[g];
+    for (int c = t; c < chunk0[ng]; c += blockDim.x) {
+        int a = 0, b = ng - 1;  // the last group whose first chunk is <= c
+        while (a < b) {
+            const int mid = (a + b + 1) >> 1;
+            if (chunk0[mid] <= c) a = mid; else b = mid - 1;
+        }
+        const int k = (c - chunk0[a]) * nc;
+        chunks[c] = make_int4(a, first[a] + k, min(nc, at[a] - k), 0);
+    }
+}
+
 constexpr int GG_THREADS = 256;
 constexpr int KC = 16;  // operator rows (input coefficients) staged per step
 constexpr int GG_DEPTH = 4;  // steps of operator rows in flight
@@ -70,28 +144,31 @@ __global__ void __launch_bounds__(GG_THREADS) k_group_gemm(GemmArgs<T> a) {
     // segments' partial products meet in the atomic adds of the epilogue
     const int nks = SPLIT && a.ksplit > 1 ? a.ksplit : 1;
     const int kper = SPLIT ? (a.C + nks * KC - 1) / (nks * KC) * KC : a.C;
-    const int nwork = (c_end - c_beg) * nrt * nks;
+    const int nwork = (c_end - c_beg) * a.sub * nrt * nks;
     int last_key = -1;
-    for (;;) {
+    for (int turn = blockIdx.x;; turn += gridDim.x) {
         __syncthreads();
-        if (t == 0) s_work = atomicAdd(a.work, 1);
-        __syncthreads();
-        const int w = s_work;
+        if (a.work) {
+            if (t == 0) s_work = atomicAdd(a.work, 1);
+            __syncthreads();
+        }
+        const int w = a.work ? s_work : turn;
         if (w >= nwork) break;
         const int ks = SPLIT ? w % nks : 0, wc = SPLIT ? w / nks : w;
-        const int chunk = c_beg + wc / nrt, rt = wc % nrt;
+        const int part = wc / nrt, rt = wc % nrt;  // part: NC pairs of a chunk
         const int kseg0 = ks * kper, kseg1 = SPLIT ? min(a.C, kseg0 + kper) : a.C;
         if (kseg0 >= kseg1) continue;  // block-uniform: an empty last segment
-        const int4 ch = a.chunks[chunk];
-        const int g = ch.x, p0 = ch.y, np = ch.z;
+        const int4 ch = a.chunks[c_beg + part / a.sub];
+        const int g = ch.x, skip = part % a.sub * NC, p0 = ch.y + skip, np = min(NC, ch.z - skip);
+        if (np <= 0) continue;
         const int r0 = rt * RT;
-        const int key = chunk * nks + ks;
+        const int key = part * nks + ks;
         if (key != last_key) {
             if (t < NC) {
                 if (t < np) {
                     const int2 pr = a.pairs[p0 + t];
-                    s_src[t] = pr.x;
-                    s_dst[t] = pr.y;
+                    s_src[t] = a.swap ? pr.y : pr.x;
+                    s_dst[t] = a.swap ? pr.x : pr.y;
                 } else {
                     s_src[t] = -1;
                     s_dst[t] = -1;
@@ -181,7 +258,7 @@ __global__ void __launch_bounds__(GG_THREADS) k_group_gemm(GemmArgs<T> a) {
 }
 
 template <typename T, int NC, int TM, bool SPLIT>
-void launch_gemm(Ctx* c, const GemmArgs<T>& a) {
+void launch_gemm(Ctx* c, GemmArgs<T> a) {
     const size_t smem = sizeof(T) * ((size_t)a.C * (NC + 4) + 2 * (size_t)KC * 16 * TM);
     cuda_check(cudaFuncSetAttribute(k_group_gemm<T, NC, TM, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                "gemm attr");
@@ -191,6 +268,12 @@ void launch_gemm(Ctx* c, const GemmArgs<T>& a) {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // a level whose items all start at once takes them in turn; more, of uneven work (the zero
+    // block), are handed out by a counter, which costs the clearing (FP64 ring of 32,768, M2M 0.90 ms in
+    // turn, 0.75 by the counter)
+    const int64_t items = (a.pairs_hint / NC + (a.g1 - a.g0)) * ((a.R + 16 * TM - 1) / (16 * TM)) * std::max(a.ksplit, 1);
+    if (a.pairs_hint > 0 && items <= (int64_t)sms * per_sm) a.work = nullptr;
+    else cuda_check(cudaMemsetAsync(a.work, 0, 4, stream_of(c)), "gemm work");
     k_group_gemm<T, NC, TM, SPLIT><<<sms * per_sm, GG_THREADS, smem, stream_of(c)>>>(a);
     count_launch(c);
     check_launch("group gemm");
@@ -212,6 +295,30 @@ void grouped_finish(Ctx* c, Grouped& gp, int nc) {
                                                    gp.chunks.as<int4>());
     count_launch(c);
     check_launch("chunks");
+}
+
+void oct_list(Ctx* c, const TreeBufs& tb, const Levels& lv, Grouped& gp, int nc) {
+    const int nb = lv.off[lv.L + 1] - lv.off[3];
+    gp.ngroups = (lv.L - 2) * 8;
+    gp.nc = nc;
+    const int nblk = grid_for(nb, 256, 64);
+    ensure(c, gp.gcount, gp.ngroups * nblk * 4);
+    ensure(c, gp.choff, (gp.ngroups + 1) * 4);
+    ensure(c, gp.pairs, std::max(nb, 1) * (int64_t)8);
+    ensure(c, gp.chunks, (int64_t)(nb / nc + gp.ngroups + 1) * 16);
+    ensure(c, gp.work, 64);
+    OctLevels ol{};
+    ol.L = lv.L;
+    for (int l = 0; l <= MAX_LEVELS; ++l) ol.off[l] = lv.off[l];
+    const auto pass = [&](auto fill) {
+        k_oct_list<decltype(fill)::value><<<nblk, 256, 0, stream_of(c)>>>(
+            ol, tb.counts.as<int>() + 32, tb.bkey.as<uint64_t>(), tb.bparent.as<int>(), nblk, gp.gcount.as<int>(), nc,
+            gp.choff.as<int>(), gp.chunks.as<int4>(), gp.pairs.as<int2>(), &tb.params.as<TreeParams>()->ticket);
+        count_launch(c);
+    };
+    pass(std::false_type{});
+    pass(std::true_type{});
+    check_launch("level pairs");
 }
 
 void grouped_prepare(Ctx* c, Grouped& gp, int ngroups, int64_t max_pairs, int nc) {
@@ -255,13 +362,14 @@ static void launch_tm(Ctx* c, const GemmArgs<T>& a, int tm) {
 }
 
 template <typename T>
-void run_group_gemm(Ctx* c, Grouped& gp, GemmArgs<T> a) {
+void run_group_gemm(Ctx* c, const Grouped& gp, GemmArgs<T> a) {
     a.chunks = gp.chunks.as<int4>();
     a.pairs = gp.pairs.as<int2>();
     a.choff = gp.choff.as<int>();
     a.work = gp.work.as<int>();
-    cuda_check(cudaMemsetAsync(a.work, 0, 4, stream_of(c)), "gemm work");
-    const int nc = gp.nc;
+    // a list of the tensor cores' wide chunks: each as several items of 16 pairs
+    const int nc = gp.nc == TC_PAIRS ? 16 : gp.nc;
+    a.sub = gp.nc / nc;
     // rows per tile 16 TM: the tallest tile that still leaves every SM a few work items
     // (a small level's few chunks would otherwise run as a handful of long serial tiles)
     int tm = 8;
@@ -284,7 +392,7 @@ void run_group_gemm(Ctx* c, Grouped& gp, GemmArgs<T> a) {
 
 template int gemm_nc<float>(int);
 template int gemm_nc<double>(int);
-template void run_group_gemm<float>(Ctx*, Grouped&, GemmArgs<float>);
-template void run_group_gemm<double>(Ctx*, Grouped&, GemmArgs<double>);
+template void run_group_gemm<float>(Ctx*, const Grouped&, GemmArgs<float>);
+template void run_group_gemm<double>(Ctx*, const Grouped&, GemmArgs<double>);
 
 }  // namespace lhv

@@ -23,11 +23,13 @@ struct GemmArgs {
     const int4* chunks;
     const int2* pairs;
     const int* choff;
-    int* work;
+    int* work;            // counter that hands out the items (null: in turn)
     int g0, g1;           // groups [g0, g1) of this launch
     const T* ops;         // operator of group g at ops + (g % ops_mod) * C * R, k-major [C][R]
     int ops_mod;
     int R, C;
+    int sub;              // items of a chunk (set by run_group_gemm where the list's chunks are wider than its kernel)
+    int swap;             // 1: the pairs are (destination, source)
     int psplit;           // > 0: rows >= psplit use inputs >= psplit_c only (zero lower-left block)
     int psplit_c;         // column of that split (0: the same as psplit)
     const T* in;          // source vectors: in + src * ldin, C entries
@@ -82,11 +84,15 @@ void build_grouped(Ctx* c, Grouped& gp, int ngroups, int64_t nitems, int64_t max
     check_launch("grouped pairs");
 }
 
+// The pairs (child, parent) of the levels 3 .. L in groups (level - 3) 8 + octant, and their chunks:
+// M2M's list, and L2L's with the pairs swapped.
+void oct_list(Ctx* c, const TreeBufs& tb, const Levels& lv, Grouped& gp, int nc);
+
 template <typename T>
 int gemm_nc(int C);
 
 template <typename T>
-void run_group_gemm(Ctx* c, Grouped& gp, GemmArgs<T> a);
+void run_group_gemm(Ctx* c, const Grouped& gp, GemmArgs<T> a);
 
 // tensor-core form (tc_gemm.cu) of a dense grouped GEMM, FP32 data; shapes with R % 16 == 0,
 // C % 8 == 0 (the complex form's tables).  tc_tiles_build re-lays `ngroups` k-major operators
@@ -100,7 +106,7 @@ void run_tc_gemm(Ctx* c, Grouped& gp, GemmArgs<float> a, const float* tiles, con
 // Tensor-core translations of the two-potential and scalar forms (tc_m2l.cu), one p a multiple of
 // 4.  tc_trans_tiles lays out the translation blocks of the fused tables (316 of M2L, 8 of M2M or
 // L2L) and the conversion's tables; run_tc_trans adds the translated (and, unless scalar,
-// converted) rows of the groups [g0, g1) to out.
+// converted) rows of the groups [g0, g1) to out (L2L: of the pairs (child, parent) of M2M).
 enum TransKind : int { TRANS_M2L = 0, TRANS_M2M = 1, TRANS_L2L = 2 };
 bool tc_trans_supported(TransKind kind, int p);
 void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scalar, Buf& tiles);
@@ -111,37 +117,6 @@ void tc_split(Ctx* c, const Levels& lv, const int* count, int l0, int l1, int64_
               float* lo);
 
 // Item sources ---------------------------------------------------------------
-
-// Children of the levels [lo, hi] (global box indices off[lo] .. off[hi+1]-1)
-// with their parents; group = (level - lo) * 8 + octant (key & 7).
-// up = true : child -> parent (M2M);  up = false : parent -> child (L2L).
-// Items run over the real boxes, numbered by loff (the device exclusive scan of the counts);
-// a box's slot is off[l] + its index in the level.
-struct OctItems {
-    const uint64_t* bkey;
-    const int* bparent;
-    const int* loff;          // real boxes before each level (device)
-    int off[MAX_LEVELS + 1];
-    int lo, hi;
-    bool up;
-    __device__ int64_t limit() const { return loff[hi + 1] - loff[lo]; }
-    __device__ bool operator()(int64_t i, int& g, int& s, int& d) const {
-        const int rb = loff[lo] + (int)i;
-        int l = lo;
-        while (l < hi && rb >= loff[l + 1]) ++l;
-        const int b = off[l] + (rb - loff[l]);
-        const int par = off[l - 1] + bparent[b];
-        g = (l - lo) * 8 + (int)(bkey[b] & 7ull);
-        if (up) {
-            s = b;
-            d = par;
-        } else {
-            s = par;
-            d = b;
-        }
-        return true;
-    }
-};
 
 // M2L with a truncation number per level: rows of the interaction table (global target box, 316
 // slots -> global source box or -1); group = (level - 2) * 316 + slot.

@@ -67,6 +67,7 @@ struct Levels {
     int off[MAX_LEVELS + 1] = {0};   // global box index of the first box of each level
     int cap_off[MAX_LEVELS + 1] = {0};
     int64_t n = 0;                   // elements of the tree
+    int real[MAX_LEVELS] = {0};      // boxes per level and
     int leaves = 0;                  // leaves of the last tree whose counts the host read (a captured
                                      // step follows one of the same level): picks block shapes
 };
@@ -99,6 +100,21 @@ int ctx_m2l_nc(Ctx* c, int dflt);                    // M2L pairs per SIMT GEMM 
 bool ctx_m2l_tc(Ctx* c);                             // M2L products on the tensor cores (TF32x3, autotuned)
 int ctx_graph_level(Ctx* c);                         // leaf level of a step being captured as a graph (-1: none)
 int* ctx_abort_word(Ctx* c);                         // device word: a captured step must not write its result
+
+// True in the block of a launch that finishes last (all of a group of nblocks blocks that count on
+// `ticket`, which it leaves at zero): it sees what the others wrote before the call.  No block waits.
+__device__ inline bool last_block(int* ticket, int nblocks) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1) == nblocks - 1;
+        if (last) *ticket = 0;
+    }
+    __syncthreads();
+    __threadfence();
+    return last != 0;
+}
 
 inline int grid_for(int64_t n, int block, int cap = 152 * 32) {
     int64_t g = (n + block - 1) / block;
@@ -247,7 +263,7 @@ template <typename T>
 void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Grouped& gp, T* mult);
 // L2L for all levels 2 -> 3 .. L-1 -> L (adds into loc).
 template <typename T>
-void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Grouped& gp, T* loc);
+void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const Grouped& up, Grouped& own, T* loc);
 // L2P at the leaves (sfar null: v alone, with the v_k rows of the map in pl.l2p_sp).
 template <typename T>
 void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,

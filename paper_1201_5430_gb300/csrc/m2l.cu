@@ -90,9 +90,10 @@ __global__ void __launch_bounds__(256) k_m2l_pairs(TableLevels lv, const int* __
     }
 }
 
-// The chunks of at most nc pairs of every slot (one block): first[slot * nblk] is the slot's first
+// The chunks of at most nc pairs of every slot (every block scans the slots, then takes a share of
+// the chunks: 33,000 of the sphere surface took one block 22 us): first[slot * nblk] is the slot's first
 // pair, *npairs the number of pairs; choff[slot] its first chunk, choff[316] their number.
-__global__ void __launch_bounds__(1024) k_m2l_chunks(int nblk, const int* __restrict__ first,
+__global__ void __launch_bounds__(256) k_m2l_chunks(int nblk, const int* __restrict__ first,
                                                      const int* __restrict__ npairs, int nc, int* __restrict__ choff,
                                                      int4* __restrict__ chunks) {
     __shared__ int pair0[NUM_OFFSETS + 1], chunk0[NUM_OFFSETS + 1];
@@ -115,8 +116,9 @@ __global__ void __launch_bounds__(1024) k_m2l_chunks(int nblk, const int* __rest
         if (t == 0) chunk0[NUM_OFFSETS] = carry;
     }
     __syncthreads();
-    for (int g = t; g <= NUM_OFFSETS; g += blockDim.x) choff[g] = chunk0[g];
-    for (int c = t; c < chunk0[NUM_OFFSETS]; c += blockDim.x) {
+    if (blockIdx.x == 0)
+        for (int g = t; g <= NUM_OFFSETS; g += blockDim.x) choff[g] = chunk0[g];
+    for (int c = blockIdx.x * blockDim.x + t; c < chunk0[NUM_OFFSETS]; c += gridDim.x * blockDim.x) {
         int lo = 0, hi = NUM_OFFSETS - 1;  // the last slot whose first chunk is <= c
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -180,8 +182,9 @@ void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& 
     if (uniform) {
         gp.ngroups = NUM_OFFSETS;
         gp.nc = nc;
-        // blocks of at least 64 target boxes; two per SM read and rank the pairs of a large tree
-        const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152, nt / 64));
+        // blocks of at least 16 target boxes, two rounds of the threads (4096 elements, 832 boxes: 20 us a
+        // pass with 64, 10 with 16); two per SM read and rank the pairs of a large tree
+        const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152, nt / 16));
         const int64_t ncnt = (int64_t)NUM_OFFSETS * nblk;
         ensure(c, gp.gcount, (ncnt + 1) * 4);
         ensure(c, gp.choff, (NUM_OFFSETS + 1) * 4);
@@ -199,7 +202,7 @@ void m2l_prepare(Ctx* c, const OpTables& ops, const TreeBufs& tb, const Levels& 
         pass(std::false_type{});
         exclusive_scan(c, ncnt, counts, counts, gp.scan_tmp.as<int>(), counts + ncnt);
         pass(std::true_type{});
-        k_m2l_chunks<<<1, 1024, 0, s>>>(nblk, counts, counts + ncnt, nc, gp.choff.as<int>(), gp.chunks.as<int4>());
+        k_m2l_chunks<<<grid_for(nt * 64 / nc, 256, 152), 256, 0, s>>>(nblk, counts, counts + ncnt, nc, gp.choff.as<int>(), gp.chunks.as<int4>());
         count_launch(c);
         check_launch("m2l pairs");
         return;

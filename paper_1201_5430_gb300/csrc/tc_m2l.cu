@@ -81,6 +81,7 @@ struct M2lArgs {
     const int2* pairs;
     const int* choff;
     int g0, g1;
+    int swap;                // 1: the pairs are (destination, source)
     const float* in;
     float* out;
     int64_t ld;
@@ -320,7 +321,10 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
             const int4 ch = a.chunks[c_beg + ((int)blockIdx.x + n * (int)gridDim.x) / a.nranges];
 #pragma unroll
             for (int j = 0; j < RJ; ++j)
-                if (row0 + 8 * j < ch.z) s[j] = a.pairs[ch.y + row0 + 8 * j].x;
+                if (row0 + 8 * j < ch.z) {
+                    const int2 pr = a.pairs[ch.y + row0 + 8 * j];
+                    s[j] = a.swap ? pr.y : pr.x;
+                }
         };
         float4 v[NPOT][RJ], w[NPOT][RJ];
         auto load = [&](const int (&s)[RJ], int k, float4 (&d)[NPOT][RJ]) {
@@ -498,7 +502,10 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
         for (int n = 0; n < mine; ++n) {
             const int item = (int)blockIdx.x + n * (int)gridDim.x, r = item % a.nranges, b = n % a.nbuf;
             const int4 ch = a.chunks[c_beg + item / a.nranges];
-            if (t < TC_PAIRS) sh.dst[t] = t < ch.z ? a.pairs[ch.y + t].y : -1;
+            if (t < TC_PAIRS) {
+                const int2 pr = t < ch.z ? a.pairs[ch.y + t] : make_int2(-1, -1);
+                sh.dst[t] = a.swap ? pr.x : pr.y;
+            }
             // a wait that gave up is seen by every epilogue warp after this barrier: all leave together
             if (!m2_wait(&sh.acc_full[b], (uint32_t)(n / a.nbuf) & 1u, sh, a.err)) *(volatile int*)&sh.epi_abort = 1;
             epi_sync();
@@ -721,6 +728,7 @@ void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int
     a.choff = gp.choff.as<int>();
     a.g0 = g0;
     a.g1 = g1;
+    a.swap = kind == TRANS_L2L;
     a.in = in;
     a.out = out;
     a.ld = ld;

@@ -68,21 +68,6 @@ __host__ __device__ inline uint64_t morton3(uint64_t qx, uint64_t qy, uint64_t q
 // ---------------------------------------------------------------------------
 // Cube
 // ---------------------------------------------------------------------------
-// True in the block of a launch that finishes last (all of a group of nblocks blocks that count on
-// `ticket`, which it leaves at zero): it sees what the others wrote before the call.  No block waits.
-__device__ inline bool last_block(int* ticket, int nblocks) {
-    __shared__ int last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        last = atomicAdd(ticket, 1) == nblocks - 1;
-        if (last) *ticket = 0;
-    }
-    __syncthreads();
-    __threadfence();
-    return last != 0;
-}
-
 template <typename T>
 __device__ inline T warp_min(T v) {
     for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -1124,6 +1109,7 @@ int build_tree(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const vec4_t<
             lv.nbox[l] = (l <= L) ? hcounts[l] : 0;
             lv.off[l + 1] = lv.off[l] + lv.nbox[l];
         }
+        for (int l = 0; l < MAX_LEVELS; ++l) lv.real[l] = lv.nbox[l];
         lv.leaves = lv.nbox[L];
     }
     LevelTable lt{};

@@ -109,3 +109,10 @@ def test_levels_translate_like_the_fused_tables(p, n, leaf, nsys):
         ctx.close()
     for a, b in zip(got[1], got[0]):
         assert np.linalg.norm(a - b) < 1.2e-5 * np.linalg.norm(b), np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("p,n,leaf", [(4, 100000, 2), (8, 20000, 4)])
+def test_levels_of_many_boxes_take_the_tensor_cores(p, n, leaf):
+    """Low p: a level needs p^4 boxes > 1.6e7 for the tensor cores; the levels above stay with the
+    grouped GEMM, which splits the same list's chunks of 128.  Bound as above."""
+    test_levels_translate_like_the_fused_tables(p, n, leaf, 1)
