@@ -32,20 +32,19 @@
 //               alternate chunks), split them and store the hi / lo tiles;
 //   warp 16     brings the operator's hi / lo tile of the chunk with one bulk copy;
 //   warp 17     issues the MMAs (2 k-steps x 3 products x potentials) and commits the stage;
-//   warps 0-7   read the accumulators (thread = pair), convert, and add to the locals through a
-//               [column][pair] staging band, so that a warp's additions cover 128 consecutive
-//               bytes of one row.
+//   warps 0-7   read the accumulators (thread = pair), convert, and stage bands of columns as
+//               [pair][column]; the copy engine adds a pair's band to its row (bulk reductions).
 // K runs from the high source degrees down and each stage takes the small cross products before
 // hi.hi: the accumulator rounds toward zero at its own magnitude, which then is small until the
 // last steps.  Far field against FP64, sphere surface at p = 12: v 3.2e-7, s 3.1e-7 (FP32 CUDA cores
 // 3.6e-7, 3.3e-7); in ascending order, and in the fused-table kernel before, 1.2e-6, 1.5e-6.
-// Measured (products, ms an evaluation, fused-table kernel before / this one): sphere surface of
-// 2^20 at p = 12, 4.13 M pairs 7.26 / 4.55; scalar cube of 2^20 at p = 12, 6.04 M pairs 4.01 / 2.28;
-// offset rings of 2^21 at p = 16, 1.33 M pairs 4.33 / 2.52.  Without the epilogue the first
-// takes 1.97: what bounds it is the conversion (tcgen05.ld and its latency, about 1.5) and the
-// additions (about 1.3), which run in turn with the products where one accumulator set fills
-// TMEM.  Operand traffic a pair at p = 12: 1.15 KB of source (split here instead of two arrays) and
-// 1.3 KB of operator, against 3.5 and 3.9 of the fused tables.
+// Measured (products, ms an evaluation, fused-table kernel before / this one with the additions by
+// atomicAdd / by bulk reductions): sphere surface of 2^20 at p = 12, 4.13 M pairs 7.26 / 4.56 / 4.24; scalar
+// cube of 2^20 at p = 12, 6.04 M pairs 4.01 / 2.28 / 1.96; offset rings of 2^21 at p = 16, 1.33 M
+// pairs 4.33 / 2.54 / 2.32.  Without the epilogue the first takes 1.97: what bounds it is the
+// conversion (tcgen05.ld and its latency), which runs in turn with the products where one accumulator
+// set fills TMEM.  Operand traffic a pair at p = 12: 1.15 KB of source (split here instead of two
+// arrays) and 1.3 KB of operator, against 3.5 and 3.9 of the fused tables.
 //
 // Every mbarrier wait gives up after a fixed number of polls, sets the error word for the host
 // and an abort word that ends every role; copies and MMAs in flight are waited for (bounded)
@@ -71,7 +70,7 @@ constexpr int M2_MAX_STAGES = 4;
 constexpr int M2_MAX_RANGES = 4;
 constexpr int M2_X_TILE = TC_PAIRS * TC_KC * 4;  // bytes of one operand tile of the pairs
 constexpr int M2_BAND = 64;                // columns (a potential) staged at once
-constexpr int M2_STG_LD = TC_PAIRS + 1;    // staging [column][pair], odd stride
+constexpr int M2_STG_LD = M2_BAND + 4;     // staging [pair][column]: a quad of a pair to a bank group of its own
 constexpr int M2_TMEM = 512;               // TMEM columns: one or two accumulator buffers
 constexpr long long M2_WAIT_LIMIT = 1ll << 24;
 constexpr int M2_SMEM_MAX = 226 * 1024;    // dynamic shared memory (the static part is below 1 KB)
@@ -110,7 +109,6 @@ struct M2lShared {
     uint32_t tmem;
     int abort;       // set by a role whose wait gave up
     int epi_abort;   // the epilogue's own verdict, read by all its warps after a barrier
-    int dst[TC_PAIRS];
 };
 
 // bounded wait that also ends when another role has given up
@@ -149,6 +147,20 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t b
 __device__ __forceinline__ uint32_t acc_base(int range) { return range ? 16u : 0u; }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// the two epilogue warps of a lane quarter
+__device__ __forceinline__ void quarter_sync(int quarter) {
+    asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
+}
+// dst[i] += src[i] in global memory, by the copy engine (16-byte aligned, a multiple of 16 bytes)
+__device__ __forceinline__ void bulk_add(float* dst, const float* src, uint32_t bytes) {
+    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
+                 "r"(smem_u32(src)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// this thread's additions have read their source
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld1(uint32_t addr, uint32_t& a) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(a) : "r"(addr));
@@ -197,6 +209,35 @@ __device__ __forceinline__ void order_zero(uint32_t (&x)[N]) {
 // What the epilogue does with the translated potentials.
 enum TransMode : int { TM_SCALAR = 0, TM_R = 1, TM_S = 2 };  // one potential; Eq. drt10; Eq. drt11
 
+// (Re, Im) of the orders M .. M + 3 (M a multiple of 4) of degree n to d[0 .. 8), d = the column of Re of
+// order M.  Orders past n are not stored, and order 0 is the one real v[1].  An odd degree's
+// orders start on a quad (n^2 - 1 = 0 mod 4), whose first column belongs to the degree below where M = 0;
+// an even one's a column before.
+__device__ __forceinline__ void store_orders(float* d, const float (&v)[8], int M, int n) {
+    if (n & 1) {
+        if (M == 0) {
+            d[1] = v[1];
+            *reinterpret_cast<float2*>(d + 2) = make_float2(v[2], v[3]);
+        } else {
+            *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+        if (M + 2 <= n) *reinterpret_cast<float4*>(d + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
+        if (M > 0) d[0] = v[0];
+        if (M + 2 <= n) {
+            *reinterpret_cast<float4*>(d + 1) = make_float4(v[1], v[2], v[3], v[4]);
+            if (M + 4 <= n) {
+                *reinterpret_cast<float2*>(d + 5) = make_float2(v[5], v[6]);
+                d[7] = v[7];
+            } else {
+                d[5] = v[5];
+            }
+        } else {
+            d[1] = v[1];
+        }
+    }
+}
+
 // Converts the orders [mb, mb + 8) of degree n of this thread's pair and writes them to the
 // staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n (R basis; S basis:
 // n - 1) as read by tmem_orders with order_zero applied; on return that of the next degree, so
@@ -222,12 +263,11 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
         f[1] = 0u;
     }
     const float* k0 = cv + (n * (n + 1) / 2 + mb) * 8;
-    float* op0 = op + (mb ? 2 * mb - 1 : -1) * M2_STG_LD;  // column of Re of order mb (order 0 is one real)
-    float* oc0 = oc + (mb ? 2 * mb - 1 : -1) * M2_STG_LD;
     // four orders at a time without branches (their chains interleave); orders past n are not stored
 #pragma unroll
     for (int h = 0; h < 8; h += 4) {
         if (mb + h > n) break;
+        float vo[8], vq[8];
 #pragma unroll
         for (int i = h; i < h + 4; ++i) {
             const int m = mb + i;
@@ -246,16 +286,14 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
             const float q0 = fmaf(ey, upr, fmaf(ex, upi, fmaf(dy, umr, fmaf(-dx, umi, fmaf(fz, ucr, cs * cr)))));
             const float o1 = fmaf(ax, pi, fmaf(ay, pr, fmaf(bx, mi, fmaf(-by, mr, fmaf(z, cr, F(f[2 * i + 1]))))));
             const float q1 = fmaf(ey, upi, fmaf(-ex, upr, fmaf(dy, umi, fmaf(dx, umr, fmaf(fz, uci, cs * ci)))));
-            if (m <= n) {
-                const int at = (m ? 2 * i : 2 * i + 1) * M2_STG_LD;
-                op0[at] = o0;
-                oc0[at] = q0;
-                if (m) {
-                    op0[at + M2_STG_LD] = o1;
-                    oc0[at + M2_STG_LD] = q1;
-                }
-            }
+            const bool zero = i == 0 && m == 0;
+            vo[2 * (i - h)] = o0;
+            vo[2 * (i - h) + 1] = zero ? o0 : o1;
+            vq[2 * (i - h)] = q0;
+            vq[2 * (i - h) + 1] = zero ? q0 : q1;
         }
+        store_orders(op + (2 * (mb + h) - 1), vo, mb + h, n);
+        store_orders(oc + (2 * (mb + h) - 1), vq, mb + h, n);
     }
 #pragma unroll
     for (int k = 0; k < 20; ++k) x[k] = y[k];
@@ -464,36 +502,11 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
         }
     } else {
         // ---- epilogue: thread = pair 32 (warp % 4) + lane; the two warps of a lane quarter share the
-        // columns.  Bands of columns are staged [column][pair], then added row by row, lane = column.
+        // columns.  Bands of columns are staged [pair][column] and added to the pairs' rows by the copy engine
+        // while the next band is read.
         const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
-        float* stc = stg + (size_t)M2_BAND * M2_STG_LD;  // chi
-        // the staged columns [0, ncol) of every pair to columns [col0, col0 + ncol) of its row
-        auto add_rows = [&](int col0, int ncol) {
-            for (int c = lane; c < ncol; c += 32) {
-                float* o = a.out + col0 + c;
-                // the reads of eight rows before their additions: an addition orders the reads after it
-                constexpr int U = 8;
-#pragma unroll
-                for (int r0 = 0; r0 < TC_PAIRS / M2_EPI_WARPS; r0 += U) {
-                    int d[U];
-                    float f[U], g[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int r = warp + M2_EPI_WARPS * (r0 + u);
-                        d[u] = sh.dst[r];
-                        f[u] = stg[c * M2_STG_LD + r];
-                        if (NPOT == 2) g[u] = stc[c * M2_STG_LD + r];
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (d[u] >= 0) {
-                            float* q = o + (int64_t)d[u] * a.ld;
-                            atomicAdd(q, f[u]);
-                            if (NPOT == 2) atomicAdd(q + a.P, g[u]);
-                        }
-                }
-            }
-        };
+        float* st_p = stg + row * M2_STG_LD;
+        float* st_c = st_p + TC_PAIRS * M2_STG_LD;  // chi
         auto release = [&](int b) {
             tc_fence_before();
             __syncwarp();
@@ -502,10 +515,9 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
         for (int n = 0; n < mine; ++n) {
             const int item = (int)blockIdx.x + n * (int)gridDim.x, r = item % a.nranges, b = n % a.nbuf;
             const int4 ch = a.chunks[c_beg + item / a.nranges];
-            if (t < TC_PAIRS) {
-                const int2 pr = t < ch.z ? a.pairs[ch.y + t] : make_int2(-1, -1);
-                sh.dst[t] = a.swap ? pr.x : pr.y;
-            }
+            const int2 pr = row < ch.z ? a.pairs[ch.y + row] : make_int2(-1, -1);
+            const int dst = a.swap ? pr.x : pr.y;
+            float* out = a.out + (int64_t)dst * a.ld;  // not used where dst < 0
             // a wait that gave up is seen by every epilogue warp after this barrier: all leave together
             if (!m2_wait(&sh.acc_full[b], (uint32_t)(n / a.nbuf) & 1u, sh, a.err)) *(volatile int*)&sh.epi_abort = 1;
             epi_sync();
@@ -515,29 +527,46 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
             const uint32_t tp =
                 tmem + (uint32_t)(b * (M2_TMEM / a.nbuf)) + acc_base(r) + ((uint32_t)(quarter * 32) << 16);
             if (NPOT == 1) {
-                const int ncols = n1 * n1 - c0;
-                for (int cb = 0; cb < nlen; cb += M2_BAND) {
+                const int ncols = n1 * n1 - c0;  // a multiple of 4
+                // each warp stages and adds its own 32 columns of a band
+                for (int cb = 32 * half; cb < nlen; cb += M2_BAND) {
+                    bulk_wait_read();
+                    __syncwarp();
 #pragma unroll
-                    for (int k = 0; k < M2_BAND / 32; ++k) {
-                        const int c = 32 * k + 16 * half;
-                        if (cb + c >= nlen) break;
+                    for (int k = 0; k < 2; ++k) {
+                        if (cb + 16 * k >= nlen) break;
                         uint32_t x[16];
-                        tmem_ld16_async(tp + (uint32_t)(cb + c), x);
+                        tmem_ld16_async(tp + (uint32_t)(cb + 16 * k), x);
                         tmem_wait(x);
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) stg[(c + i) * M2_STG_LD + row] = __uint_as_float(x[i]);
+                        for (int i = 0; i < 16; i += 4)
+                            *reinterpret_cast<uint4*>(st_p + 32 * half + 16 * k + i) =
+                                make_uint4(x[i], x[i + 1], x[i + 2], x[i + 3]);
                     }
-                    if (cb + M2_BAND >= nlen) release(b);
-                    epi_sync();
-                    add_rows(c0 + cb, min(M2_BAND, ncols - cb));
-                    epi_sync();
+                    fence_async_smem();
+                    __syncwarp();
+                    const int nc = min(32, ncols - cb);
+                    if (dst >= 0 && nc > 0) bulk_add(out + c0 + cb, st_p + 32 * half, (uint32_t)nc * 4);
+                    bulk_commit();
                 }
+                release(b);
             } else {
                 const uint32_t tc = tp + (uint32_t)nlen;
                 const float4 tv = __ldg(reinterpret_cast<const float4*>(a.tvec) + ch.x % a.ngroups);
                 for (int na = n0; na < n1;) {
-                    int nb = na + 1;  // degrees [na, nb) fit the band
+                    // degrees [na, nb) fit the band; an even nb where there is one, so that the band
+                    // [s0, s1) of whole quads holds no columns of other degrees (those are zero)
+                    int nb = na + 1;
                     while (nb < n1 && (nb + 1) * (nb + 1) - na * na <= M2_BAND) ++nb;
+                    if ((nb & 1) && nb < n1 && nb > na + 1) --nb;
+                    const int s0 = na * na & ~3, s1 = (nb * nb + 3) & ~3;
+                    bulk_wait_read();
+                    quarter_sync(quarter);
+                    if (half == 0) {
+                        if (na & 1) st_p[0] = st_c[0] = 0.f;
+                        if (nb & 1)
+                            for (int c = nb * nb - s0; c < s1 - s0; ++c) st_p[c] = st_c[c] = 0.f;
+                    }
                     // runs of degrees in blocks of eight orders: one block is split between the two warps
                     // of a lane quarter by degree, several are taken in turn
                     for (int mb = 0; mb < nb; mb += 8) {
@@ -561,19 +590,23 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                             for (int k = 0; k < 20; ++k) x[k] = 0u;
                         }
                         for (int dn = d0; dn < d1; ++dn) {
-                            const int at = (dn * dn - na * na) * M2_STG_LD + row;
-                            convert_orders<MODE>(conv, tp, tc, c0, a.p, dn, mb, tv.x, tv.y, tv.z, a.chi_scale, x, stg + at,
-                                                 stc + at);
+                            const int at = dn * dn - s0;
+                            convert_orders<MODE>(conv, tp, tc, c0, a.p, dn, mb, tv.x, tv.y, tv.z, a.chi_scale, x,
+                                                 st_p + at, st_c + at);
                         }
                     }
                     if (nb == n1) release(b);
-                    epi_sync();
-                    add_rows(na * na, nb * nb - na * na);
-                    epi_sync();
+                    fence_async_smem();
+                    quarter_sync(quarter);
+                    // one warp adds phi, the other chi
+                    if (dst >= 0)
+                        bulk_add(out + half * a.P + s0, half ? st_c : st_p, (uint32_t)(s1 - s0) * 4);
+                    bulk_commit();
                     na = nb;
                 }
             }
         }
+        bulk_wait_all();
     }
     __syncwarp();
     tc_fence_before();
@@ -607,7 +640,7 @@ __global__ void k_m2l_tiles(const float* __restrict__ ops, int64_t op_floats, in
 }
 
 int m2l_fixed_smem(int p, int npot) {
-    return (npot * M2_BAND * M2_STG_LD + (npot == 2 ? conv_floats(p) : 0)) * 4;
+    return (npot * TC_PAIRS * M2_STG_LD + (npot == 2 ? conv_floats(p) : 0)) * 4;
 }
 
 // One past the last column that the epilogue reads of chi of the degrees [n0, n1) and their
@@ -649,7 +682,8 @@ M2lArgs m2l_layout(int p, int npot, int ngroups) {
         };
         int n1 = n0 + 1;
         while (n1 < p && fits(n1 + 1)) ++n1;
-        if (!fits(n1)) throw Error{LHV_EUNSUPPORTED, "M2L accumulators"};
+        if (npot == 1 && n1 < p) n1 &= ~1;  // whole quads of columns
+        if (n1 <= n0 || !fits(n1)) throw Error{LHV_EUNSUPPORTED, "M2L accumulators"};
         a.n0[r] = n0;
         a.n1[r] = n1;
         a.c0[r] = c0;
