@@ -33,12 +33,19 @@
 //   phi~ = phi^ + i tau chi^,  tau = |t| m / n;   chi~_n = chi^_n - sigma chi^_{n+1},
 //   sigma = |t| sqrt((n + 1 - m)(n + 1 + m)) / (n + 1)   (the chi^_p term dropped).
 //
-// Products: one CTA per streaming multiprocessor walks a contiguous range of chunks of the
-// grouped pair list (pairs bucketed by offset slot, m2l_prepare), holds the slot's tables
-// in shared memory, gathers NC source multipoles as columns of A ([row][pair]) and runs
-//   A -Z-> B -Y-> C -coaxial-> B -conversion-> C -Y-> B -Z, atomics-> locals,
-// the Y and coaxial stages as register-tiled products (4 output rows x 4 pairs per thread).
-// The next chunk's gather (asynchronous copies into A) is issued after the first stage.
+// Products: the resident CTAs walk contiguous ranges of chunks of the grouped pair list (pairs
+// bucketed by offset slot, m2l_prepare), hold the slot's tables in shared memory, gather NC source
+// multipoles into A and run
+//   A -transposed-> C -Z-> B -Y-> C -coaxial-> B -conversion-> C -Y-> B -Z-> C -transposed-> B -> locals
+// on [row][pair] buffers, the Y and coaxial stages as register-tiled products (4 output rows x 4 pairs
+// per thread).  The next chunk's gather is issued after the first Z stage.  Where a box's row is a
+// multiple of 16 bytes (FP64; FP32 of even p) the gather copies 16 bytes at a time to [pair][row] and a
+// pair's result leaves as one bulk addition; the index work of 4-byte copies and of one
+// atomicAdd per coefficient was a third of the kernel's instructions.  Products at p = 12, FP32, ms with 4-byte
+// copies and atomicAdd (odd p still) / so: cloud of 100,003, 0.64 M pairs 1.45 / 1.19; ring of 2^18,
+// 0.50 M pairs 1.14 / 0.94; FP64 ring of 2^15 9.15 / 9.11 (FP64 pipe).  What bounds it: issue slots and the
+// shared-memory pipe, each at about 60 % (two 16-byte reads for 16 multiply-adds), and the seven
+// barriers a chunk with 16 warps an SM; 384 and 512 threads a CTA were slower (1.23, 1.47).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -49,6 +56,7 @@
 
 #include "lhv_group.cuh"
 #include "lhv_internal.cuh"
+#include "tc_common.cuh"
 
 namespace lhv {
 
@@ -359,6 +367,7 @@ struct RcrArgs {
     int p;
     int slot_floats, coax_floats;
     int nrg_y, nrg_cx;   // register-tile row groups of the Y / coaxial stages
+    int wide;            // a box's row is a multiple of 16 bytes
 };
 
 template <typename T>
@@ -503,6 +512,48 @@ __device__ __forceinline__ void gather_async(const RcrArgs<T>& a, int p0, int np
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
+// The same where a row is a multiple of 16 bytes: A as [pair][row], in 16-byte pieces, a row one piece
+// longer than R so that one piece of consecutive pairs spreads over the banks.
+template <typename T, int NC>
+__device__ __forceinline__ void gather_wide(const RcrArgs<T>& a, int p0, int np, T* A) {
+    constexpr int VE = 16 / (int)sizeof(T);
+    const int R = 2 * a.p * a.p, pieces = R / VE;
+    for (int e = threadIdx.x; e < pieces * NC; e += RA_THREADS) {
+        const int col = e / pieces, q = e - col * pieces;
+        T* dst = A + col * (R + VE) + q * VE;
+        if (col < np) {
+            const T* g = a.in + (int64_t)a.pairs[p0 + col].x * a.ld + q * VE;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(g) : "memory");
+        } else {
+#pragma unroll
+            for (int k = 0; k < VE; ++k) dst[k] = (T)0;
+        }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+// [pair][row] pieces <-> [row][pair]
+template <typename T, int NC, int NCP, bool IN>
+__device__ __forceinline__ void transpose_block(int R, const T* S, T* D) {
+    constexpr int VE = 16 / (int)sizeof(T);
+    struct alignas(16) Piece {
+        T v[VE];
+    };
+    for (int e = threadIdx.x; e < R / VE * NC; e += RA_THREADS) {
+        const int q = e / NC, col = e - q * NC;
+        if (IN) {
+            const Piece x = *reinterpret_cast<const Piece*>(S + col * (R + VE) + q * VE);
+#pragma unroll
+            for (int k = 0; k < VE; ++k) D[(q * VE + k) * NCP + col] = x.v[k];
+        } else {
+            Piece x;
+#pragma unroll
+            for (int k = 0; k < VE; ++k) x.v[k] = S[(q * VE + k) * NCP + col];
+            *reinterpret_cast<Piece*>(D + col * (R + VE) + q * VE) = x;
+        }
+    }
+}
+
 template <typename T, int NC>
 __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
     constexpr int NCP = NC + 4;  // row stride of the buffers (16-byte aligned, 4 mod 8)
@@ -550,10 +601,11 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
     }
     const int nch = *a.nchunks;
     const int c0 = (int)((int64_t)blockIdx.x * nch / gridDim.x), c1 = (int)((int64_t)(blockIdx.x + 1) * nch / gridDim.x);
-    if (c0 < c1) {
-        const int4 ch = a.chunks[c0];
-        gather_async<T, NC, NCP>(a, ch.y, ch.z, A);
-    }
+    const auto gather = [&](const int4& ch) {
+        if (a.wide) gather_wide<T, NC>(a, ch.y, ch.z, A);
+        else gather_async<T, NC, NCP>(a, ch.y, ch.z, A);
+    };
+    if (c0 < c1) gather(a.chunks[c0]);
     int cur = -1;
     for (int chunk = c0; chunk < c1; ++chunk) {
         const int4 ch = a.chunks[chunk];
@@ -570,12 +622,16 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
         }
         if (tid < NC) s_dst[tid] = tid < np ? a.pairs[p0 + tid].y : -1;
         asm volatile("cp.async.wait_all;\n" ::: "memory");
+        bulk_wait_read();  // the additions of the previous chunk have read B
         __syncthreads();
-        z_stage<T, NCP, NCG>(p, units, Zf, A, B);
+        if (a.wide) {
+            transpose_block<T, NC, NCP, true>(R, A, C);
+            __syncthreads();
+        }
+        z_stage<T, NCP, NCG>(p, units, Zf, a.wide ? C : A, B);
         __syncthreads();
         if (chunk + 1 < c1) {  // A is free: the next chunk's multipoles arrive during the stages
-            const int4 nx = a.chunks[chunk + 1];
-            gather_async<T, NC, NCP>(a, nx.y, nx.z, A);
+            gather(a.chunks[chunk + 1]);
         }
         y_stage<T, NCP, NCG>(a, rg_y, yo, Yf, B, C);
         __syncthreads();
@@ -631,6 +687,15 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
         __syncthreads();
         z_stage<T, NCP, NCG>(p, units, Zb, B, C);
         __syncthreads();
+        if (a.wide) {  // one bulk addition a pair
+            transpose_block<T, NC, NCP, false>(R, C, B);
+            fence_async_smem();
+            __syncthreads();
+            constexpr int VE = 16 / (int)sizeof(T);
+            if (tid < np) bulk_add(a.out + (int64_t)s_dst[tid] * a.ld, B + tid * (R + VE), R * (uint32_t)sizeof(T));
+            bulk_commit();
+            continue;
+        }
         const int R8 = (R + 7) & ~7;
         for (int e = tid; e < R8 * NC; e += RA_THREADS) {
             int row, col;
@@ -639,6 +704,7 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
         }
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
+    bulk_wait_all();
 }
 
 int slot_floats(int p) { return 2 * y_off(p) + 8 * p; }
@@ -886,6 +952,7 @@ void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const T* mult, T* loc, 
     a.coax_floats = rt.coax_floats;
     a.nrg_y = rg_y_count(rt.p);
     a.nrg_cx = rg_cx_count(rt.p);
+    a.wide = 2 * rt.p * rt.p * sizeof(T) % 16 == 0 && ld * sizeof(T) % 16 == 0;
     switch (rt.nc) {
         case 32: launch_apply<T, 32>(c, rt, a); break;
         case 24: launch_apply<T, 24>(c, rt, a); break;

@@ -151,17 +151,6 @@ __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" :::
 __device__ __forceinline__ void quarter_sync(int quarter) {
     asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
 }
-// dst[i] += src[i] in global memory, by the copy engine (16-byte aligned, a multiple of 16 bytes)
-__device__ __forceinline__ void bulk_add(float* dst, const float* src, uint32_t bytes) {
-    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
-                 "r"(smem_u32(src)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// this thread's additions have read their source
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 __device__ __forceinline__ void tmem_ld1(uint32_t addr, uint32_t& a) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(a) : "r"(addr));
 }
