@@ -252,9 +252,9 @@ template <typename T>
 static SellView<T> view(const Sell& m) {
     SellView<T> v;
     v.sptr = m.sptr.as<int>();
-    v.col = m.col.as<int>();
-    v.val = m.val.as<T>();
+    v.ent = m.ent.as<SellEntry<T>>();
     v.rows = m.rows;
+    v.cols = m.cols;
     return v;
 }
 

@@ -78,18 +78,18 @@ __device__ inline void for_each_Q(int p, T x, T y, T z, const QTab<T>& q, F&& f,
     }
 }
 
-// out[r] = sum of the sparse map's row r over `in` (shared memory), f(r, sum): the warps of a block
-// take the slices in turn.
+// out[r] = sum of the sparse map's row r over `in` (shared memory, in[cols] = 0), f(r, sum): the warps of
+// a block take the slices in turn.
 template <typename T, typename F>
 __device__ inline void sparse_rows(const SellView<T>& m, const T* in, int warp, int nwarps, F&& f) {
     const int lane = threadIdx.x & 31;
     for (int q = warp; 32 * q < m.rows; q += nwarps) {
         const int b = m.sptr[q], e = m.sptr[q + 1];
         T acc = 0;
-#pragma unroll 3
+#pragma unroll 4
         for (int i = b + lane; i < e; i += 32) {
-            const T v = m.val[i], x = in[m.col[i]];
-            if (v != (T)0) acc += v * x;  // a padding entry adds nothing, whatever its input holds
+            const SellEntry<T> n = m.ent[i];
+            acc += n.val * in[n.col];
         }
         const int r = 32 * q + lane;
         if (r < m.rows) f(r, acc);
@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(P2M_APPLY_THREADS) k_p2m_apply(const int* __re
                                                                 const T* __restrict__ W, int P, SellView<T> g,
                                                                 T* __restrict__ mult, int64_t ld) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    T* w = reinterpret_cast<T*>(smem_raw);  // [3P]
+    T* w = reinterpret_cast<T*>(smem_raw);  // [3P], then a zero
     const int nleaf = *nleaf_dev;
+    if (threadIdx.x == 0) w[3 * P] = 0;
     for (int b = blockIdx.x; b < nleaf; b += gridDim.x) {
         __syncthreads();
         for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) w[i] = W[(int64_t)b * 3 * P + i];
@@ -310,9 +311,11 @@ __global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ nt
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int P = p * p;
     T* cf = reinterpret_cast<T*>(smem_raw);  // [P][CS]
-    T* lh = cf + CS * P;                     // [2P] the leaf's local expansion
+    T* lh = cf + CS * P;                     // [2P] the leaf's local expansion, then a zero
     const int ntiles = *ntiles_dev;
-    const QTab<T> qt = load_qtab(lh + 2 * P, qtab, p);  // visible after the tile loop's first barrier
+    if (threadIdx.x == 0) lh[2 * P] = 0;
+    const unsigned per = 0xffffffffu / (unsigned)P + 1u;  // r / P = the upper half of r per, r < 12 P
+    const QTab<T> qt = load_qtab(lh + 2 * P + 4, qtab, p);  // visible after the tile loop's first barrier
     // a block takes a contiguous range of tiles; the tiles of a leaf are consecutive, so the
     // leaf's coefficient vectors are staged once per leaf, not once per tile
     const int t_lo = (int)((int64_t)ntiles * blockIdx.x / gridDim.x);
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ nt
             for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) lh[i] = loc[(int64_t)b * ld + i];
             __syncthreads();
             sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {  // r = j P + i: vector j, entry i
-                const int j = r / P, i = r - j * P;
+                const int j = (int)__umulhi((unsigned)r, per), i = r - j * P;
                 cf[i * CS + j] = v;
             });
             __syncthreads();
@@ -401,9 +404,11 @@ __global__ void __launch_bounds__(THREADS) k_l2p_scalar(const int* __restrict__ 
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int P = p * p;
     T* cf = reinterpret_cast<T*>(smem_raw);  // [P][4]
-    T* lh = cf + 4 * P;                      // [2P] (L_hat, 0)
+    T* lh = cf + 4 * P;                      // [2P] (L_hat, 0), then a zero
     const int ntiles = *ntiles_dev;
-    const QTab<T> qt = load_qtab(lh + 2 * P, qtab, p);
+    if (threadIdx.x == 0) lh[2 * P] = 0;
+    const unsigned per = 0xffffffffu / (unsigned)P + 1u;
+    const QTab<T> qt = load_qtab(lh + 2 * P + 4, qtab, p);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int2 tw = tiles[t];
         const int b = tw.x;
@@ -414,7 +419,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_scalar(const int* __restrict__ 
         // vector j = 0: phi itself, 1..3: rows of v_x, v_y, v_z
         for (int i = threadIdx.x; i < P; i += blockDim.x) cf[i * 4] = lh[i];
         sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {
-            const int j = r / P, i = r - j * P;
+            const int j = (int)__umulhi((unsigned)r, per), i = r - j * P;
             cf[i * 4 + 1 + j] = v;
         });
         __syncthreads();
@@ -511,7 +516,7 @@ static void launch_p2m_w(Ctx* c, const TreeBufs& tb, const Levels& lv, int p, co
 template <typename T>
 static void launch_p2m_apply(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const T* W, T* mult) {
     const int L = lv.L, P = pl.p[L] * pl.p[L];
-    const size_t smem = sizeof(T) * 3 * P;
+    const size_t smem = sizeof(T) * (3 * P + 1);
     k_p2m_apply<T><<<resident_grid(k_p2m_apply<T>, P2M_APPLY_THREADS, smem, lv.nbox[L]), P2M_APPLY_THREADS, smem,
                      stream_of(c)>>>(tb.counts.as<int>() + L, W, P, pl.p2m_sp, mult + (int64_t)lv.off[L] * pl.ld, pl.ld);
     count_launch(c);
@@ -523,7 +528,7 @@ static void launch_p2m_apply(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, cons
 // the FP64 ring of 32,768, 1.8 tiles a resident block, 1.10 ms against 0.92), 16 blocks an SM where a
 // leaf holds several tiles (P2M, L2P of the leapfrog pair, 440 elements a leaf: 1.8, 1.86 ms with the
 // resident blocks, 1.45, 1.74 with 16), else those resident at once (sphere surface, 15 a leaf:
-// 0.48, 1.32 ms against 0.54, 1.59 with 16).
+// 0.48, 1.32 ms against 0.54, 1.59 with 16, before the sparse maps were packed).
 constexpr int BIG_LEAF = 64;
 template <typename K>
 static int tile_grid(K kernel, int threads, size_t smem, const Levels& lv) {
@@ -537,7 +542,7 @@ static int tile_grid(K kernel, int threads, size_t smem, const Levels& lv) {
 // Threads of an L2P block of three or four vectors for the mean leaf: f(integral_constant).  Narrow
 // blocks put more leaves on an SM (scalar cube, 32 a leaf: 0.29 ms against 0.35 with 128 threads); with
 // twelve vectors the sparse map takes half of the work and wants the wide block (sphere
-// surface 1.52 against 1.32).
+// surface 1.18 with 64 against 1.06, cloud of 24 a leaf 0.087 against 0.080).
 template <typename F>
 static void l2p_threads(const Levels& lv, F&& f) {
     const int64_t nl = lv.leaves;
@@ -656,7 +661,7 @@ void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
     auto launch = [&](auto threads, auto grad) {
         constexpr int TH = decltype(threads)::value;
         constexpr bool GRAD = decltype(grad)::value;
-        const size_t smem = sizeof(T) * ((GRAD ? 14 : 6) * P + qtab_reals(p));
+        const size_t smem = sizeof(T) * ((GRAD ? 14 : 6) * P + 4 + qtab_reals(p));
         auto kernel = k_l2p_eval<T, TH, GRAD>;
         cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "l2p attr");
         kernel<<<tile_grid(kernel, TH, smem, lv), TH, smem, stream_of(c)>>>(
@@ -694,7 +699,7 @@ template <typename T>
 void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,
                     const T* loc, vec4_t<T>* pgfar) {
     const int L = lv.L, o = lv.off[L], p = pl.p[L], P = p * p;
-    const size_t smem = sizeof(T) * (6 * P + qtab_reals(p));
+    const size_t smem = sizeof(T) * (6 * P + 4 + qtab_reals(p));
     l2p_threads(lv, [&](auto threads) {
         constexpr int TH = decltype(threads)::value;
         auto kernel = k_l2p_scalar<T, TH>;

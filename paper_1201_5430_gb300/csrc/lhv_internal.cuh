@@ -162,18 +162,23 @@ void gather_sorted(Ctx* c, int64_t n, const int* perm, const vec4_t<T>* x4, cons
 
 // ---- operators (operators.cu) -----------------------------------------------
 // Sliced form of a sparse map (rows = outputs): out[row] = sum val in[col].  The rows lie in slices of
-// 32; entry k of a slice's rows is a run of 32 values from sptr[slice] + 32 k (short rows padded
-// with zeros), so a warp reads its slice coalesced, and neighbouring rows read neighbouring inputs.
+// 32; entry k of a slice's rows is a run of 32 entries from sptr[slice] + 32 k, so a warp reads its
+// slice coalesced, and neighbouring rows read neighbouring inputs.  Short rows are padded with zeros of
+// column `cols`, one past the inputs, where the reader keeps a zero.
+template <typename T>
+struct alignas(2 * sizeof(T)) SellEntry {
+    T val;
+    int col;
+};
 struct Sell {
-    Buf sptr, col, val;
-    int rows = 0;
+    Buf sptr, ent;
+    int rows = 0, cols = 0;
 };
 template <typename T>
 struct SellView {
     const int* sptr = nullptr;
-    const int* col = nullptr;
-    const T* val = nullptr;
-    int rows = 0;
+    const SellEntry<T>* ent = nullptr;
+    int rows = 0, cols = 0;
 };
 
 struct OpTables {

@@ -417,7 +417,7 @@ void free_operators(OpTables& ops) {
 }
 
 void free_sparse(Sell& m) {
-    for (Buf* b : {&m.sptr, &m.col, &m.val}) {
+    for (Buf* b : {&m.sptr, &m.ent}) {
         if (b->ptr) cudaFree(b->ptr);
         b->ptr = nullptr;
         b->cap = 0;
@@ -447,20 +447,18 @@ void build_sparse(Ctx* c, int kind, int p, int rows, Sell& dst) {
         for (int r = 0; r < nr; ++r)
             if (h[(size_t)k * R + r] != 0.0) cols[r].push_back(k);
     const int ns = (nr + 31) / 32;
-    std::vector<int> sptr(ns + 1, 0), col;
-    std::vector<T> val;
+    std::vector<int> sptr(ns + 1, 0);
+    std::vector<SellEntry<T>> ent;
     for (int q = 0; q < ns; ++q) {
         const int n = std::min(32, nr - 32 * q);
         size_t width = 0;
         for (int i = 0; i < n; ++i) width = std::max(width, cols[32 * q + i].size());
         sptr[q + 1] = sptr[q] + 32 * (int)width;
-        col.resize(sptr[q + 1], 0);
-        val.resize(sptr[q + 1], (T)0);
+        ent.resize(sptr[q + 1], SellEntry<T>{(T)0, C});
         for (int i = 0; i < n; ++i) {
             const int r = 32 * q + i;
             for (int k = 0; k < (int)cols[r].size(); ++k) {
-                col[sptr[q] + 32 * k + i] = cols[r][k];
-                val[sptr[q] + 32 * k + i] = (T)h[(size_t)cols[r][k] * R + r];
+                ent[sptr[q] + 32 * k + i] = SellEntry<T>{(T)h[(size_t)cols[r][k] * R + r], cols[r][k]};
             }
         }
     }
@@ -470,9 +468,9 @@ void build_sparse(Ctx* c, int kind, int p, int rows, Sell& dst) {
         if (bytes) cuda_check(cudaMemcpy(b.ptr, src, bytes, cudaMemcpyHostToDevice), "sparse map");
     };
     put(dst.sptr, sptr.data(), sptr.size() * 4);
-    put(dst.col, col.data(), col.size() * 4);
-    put(dst.val, val.data(), val.size() * sizeof(T));
+    put(dst.ent, ent.data(), ent.size() * sizeof(SellEntry<T>));
     dst.rows = nr;
+    dst.cols = C;
 }
 
 void m2l_offsets(std::vector<int>& offs, std::vector<int>& slot_of) {
