@@ -38,12 +38,12 @@
 // multipoles into A and run
 //   A -transposed-> C -Z-> B -Y-> C -coaxial-> B -conversion-> C -Y-> B -Z-> C -transposed-> B -> locals
 // on [row][pair] buffers, the Y and coaxial stages as register-tiled products (4 output rows x 4 pairs
-// per thread).  The next chunk's gather is issued after the first Z stage.  Where a box's row is a
+// per thread, one row x 2 pairs in FP64).  The next chunk's gather is issued after the first Z stage.  Where a box's row is a
 // multiple of 16 bytes (FP64; FP32 of even p) the gather copies 16 bytes at a time to [pair][row] and a
 // pair's result leaves as one bulk addition; the index work of 4-byte copies and of one
 // atomicAdd per coefficient was a third of the kernel's instructions.  Products at p = 12, FP32, ms with 4-byte
 // copies and atomicAdd (odd p still) / so: cloud of 100,003, 0.64 M pairs 1.45 / 1.19; ring of 2^18,
-// 0.50 M pairs 1.14 / 0.94; FP64 ring of 2^15 9.15 / 9.11 (FP64 pipe).  What bounds it: issue slots and the
+// 0.50 M pairs 1.14 / 0.94; FP64 ring of 2^15 9.15 / 9.11 (4 x 4 tiles).  What bounds it: issue slots and the
 // shared-memory pipe, each at about 60 % (two 16-byte reads for 16 multiply-adds), and the seven
 // barriers a chunk with 16 warps an SM; 384 and 512 threads a CTA were slower (1.23, 1.47).
 #include <cuda_runtime.h>
@@ -370,16 +370,28 @@ struct RcrArgs {
     int wide;            // a box's row is a multiple of 16 bytes
 };
 
-template <typename T>
-__device__ __forceinline__ void fma44(T (&acc)[4][4], Quad<T> x, Quad<T> v) {
-    const T xs[4] = {x.x, x.y, x.z, x.w};
+// Rows and pairs of a thread's register tile in the Y and coaxial stages.  FP32 wants reuse: two 16-byte
+// reads feed 16 multiply-adds.  In FP64 a warp's multiply-add holds its quarter of the SM for 64 cycles and
+// the reads are free; what counts is that the few items of a chunk of eight pairs (p = 12) load the
+// quarters evenly and no row is padded.  Products of the ring of 32,768 in FP64, ms: 4 x 4 tiles 9.1,
+// 2 x 4 6.9, 2 x 2 5.8, 1 x 4 5.8, 2 x 1 5.4, 1 x 2 5.2 (its multiply-adds alone: 3.9).
+template <typename T> struct RcrTile {
+    static constexpr int R = 4, C = 4;
+};
+template <> struct RcrTile<double> {
+    static constexpr int R = 1, C = 2;
+};
+// consecutive values, read and written 16 bytes at a time
+template <typename T, int N> struct alignas(N * sizeof(T) < 16 ? N * sizeof(T) : 16) Run {
+    T v[N];
+};
+
+template <typename T, int R, int C>
+__device__ __forceinline__ void fma_tile(T (&acc)[R][C], Run<T, R> x, Run<T, C> v) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        acc[j][0] = fma(xs[j], v.x, acc[j][0]);
-        acc[j][1] = fma(xs[j], v.y, acc[j][1]);
-        acc[j][2] = fma(xs[j], v.z, acc[j][2]);
-        acc[j][3] = fma(xs[j], v.w, acc[j][3]);
-    }
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+        for (int k = 0; k < C; ++k) acc[j][k] = fma(x.v[j], v.v[k], acc[j][k]);
 }
 
 // Work item k of a stage for this thread: items are dealt in rounds of RA_THREADS, in
@@ -389,9 +401,10 @@ __device__ __forceinline__ int stage_item(int k) {
 }
 
 // S -> D by the Y blocks: rows q P + n^2 + member(i) of each class of each degree.
-template <typename T, int NCP, int NCG>
+template <typename T, int NCP, int NC>
 __device__ __forceinline__ void y_stage(const RcrArgs<T>& a, const int* rg_y, const int* yo, const T* Y,
                                         const T* S, T* D) {
+    constexpr int TR = RcrTile<T>::R, TC = RcrTile<T>::C, NCG = NC / TC;
     const int P = a.p * a.p, total = a.nrg_y * NCG;
     for (int k = 0; k * RA_THREADS < total; ++k) {
         const int it = stage_item(k);
@@ -399,36 +412,40 @@ __device__ __forceinline__ void y_stage(const RcrArgs<T>& a, const int* rg_y, co
         const int rg = it / NCG, cg = it - rg * NCG;
         const int code = rg_y[rg], q = code & 1, odd = (code >> 1) & 1, n = (code >> 2) & 31, og = code >> 7;
         const int sz = odd ? n : n + 1, W = pad4(sz);
-        const T* x = Y + yo[n] + (odd ? (n + 1) * pad4(n + 1) : 0) + og * 4;
-        const T* s = S + (q * P + n * n) * NCP + cg * 4;
-        T acc[4][4] = {};
+        const T* x = Y + yo[n] + (odd ? (n + 1) * pad4(n + 1) : 0) + og * TR;
+        const T* s = S + (q * P + n * n) * NCP + cg * TC;
+        T acc[TR][TC] = {};
         if (odd) {
 #pragma unroll 4
             for (int i = 0; i < sz; ++i)
-                fma44(acc, *reinterpret_cast<const Quad<T>*>(x + i * W),
-                      *reinterpret_cast<const Quad<T>*>(s + odd_member(i) * NCP));
+                fma_tile(acc, *reinterpret_cast<const Run<T, TR>*>(x + i * W),
+                         *reinterpret_cast<const Run<T, TC>*>(s + odd_member(i) * NCP));
         } else {
 #pragma unroll 4
             for (int i = 0; i < sz; ++i)
-                fma44(acc, *reinterpret_cast<const Quad<T>*>(x + i * W),
-                      *reinterpret_cast<const Quad<T>*>(s + even_member(i) * NCP));
+                fma_tile(acc, *reinterpret_cast<const Run<T, TR>*>(x + i * W),
+                         *reinterpret_cast<const Run<T, TC>*>(s + even_member(i) * NCP));
         }
-        T* d = D + (q * P + n * n) * NCP + cg * 4;
+        T* d = D + (q * P + n * n) * NCP + cg * TC;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int o = og * 4 + j;
-            if (o < sz)
-                *reinterpret_cast<Quad<T>*>(d + (odd ? odd_member(o) : even_member(o)) * NCP) =
-                    make_quad<T>(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+        for (int j = 0; j < TR; ++j) {
+            const int o = og * TR + j;
+            if (o < sz) {
+                Run<T, TC> v;
+#pragma unroll
+                for (int c = 0; c < TC; ++c) v.v[c] = acc[j][c];
+                *reinterpret_cast<Run<T, TC>*>(d + (odd ? odd_member(o) : even_member(o)) * NCP) = v;
+            }
         }
     }
 }
 
 // S (rotated S-basis multipoles) -> D (rotated R-basis locals): the coaxial translation A_m
 // of each order, the same for phi and chi, Re and Im.
-template <typename T, int NCP, int NCG>
+template <typename T, int NCP, int NC>
 __device__ __forceinline__ void coax_stage(const RcrArgs<T>& a, const int* rg_cx, const int* co, const T* CX,
                                            const T* S, T* D) {
+    constexpr int TR = RcrTile<T>::R, TC = RcrTile<T>::C, NCG = NC / TC;
     const int p = a.p, P = p * p, total = a.nrg_cx * NCG;
     for (int kk = 0; kk * RA_THREADS < total; ++kk) {
         const int it = stage_item(kk);
@@ -436,20 +453,24 @@ __device__ __forceinline__ void coax_stage(const RcrArgs<T>& a, const int* rg_cx
         const int rg = it / NCG, cg = it - rg * NCG;
         const int code = rg_cx[rg], q = code & 1, r = (code >> 1) & 1, m = (code >> 2) & 31, og = code >> 7;
         const int k = p - m, K = pad4(k), mo = m ? 2 * m - 1 : 0;
-        const T* blk = CX + co[m] + og * 4;
-        const T* s = S + (q * P + mo + r) * NCP + cg * 4;
-        T acc[4][4] = {};
+        const T* blk = CX + co[m] + og * TR;
+        const T* s = S + (q * P + mo + r) * NCP + cg * TC;
+        T acc[TR][TC] = {};
 #pragma unroll 4
         for (int i = 0; i < k; ++i) {
             const int n = m + i;
-            fma44(acc, *reinterpret_cast<const Quad<T>*>(blk + i * K), *reinterpret_cast<const Quad<T>*>(s + n * n * NCP));
+            fma_tile(acc, *reinterpret_cast<const Run<T, TR>*>(blk + i * K),
+                     *reinterpret_cast<const Run<T, TC>*>(s + n * n * NCP));
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n2 = m + og * 4 + j;
-            if (n2 < p)
-                *reinterpret_cast<Quad<T>*>(D + (q * P + n2 * n2 + mo + r) * NCP + cg * 4) =
-                    make_quad<T>(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+        for (int j = 0; j < TR; ++j) {
+            const int n2 = m + og * TR + j;
+            if (n2 < p) {
+                Run<T, TC> v;
+#pragma unroll
+                for (int c = 0; c < TC; ++c) v.v[c] = acc[j][c];
+                *reinterpret_cast<Run<T, TC>*>(D + (q * P + n2 * n2 + mo + r) * NCP + cg * TC) = v;
+            }
         }
     }
 }
@@ -581,16 +602,19 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
     const int tid = threadIdx.x;
     if (tid == 0) {
         // row groups longest first
+        constexpr int TR = RcrTile<T>::R;
         int g = 0;
         for (int n = p - 1; n >= 0; --n)
             for (int q = 0; q < 2; ++q)
                 for (int odd = 0; odd < 2; ++odd)
-                    for (int og = 0; og * 4 < (odd ? n : n + 1); ++og) rg_y[g++] = q | (odd << 1) | (n << 2) | (og << 7);
+                    for (int og = 0; og * TR < (odd ? n : n + 1); ++og)
+                        rg_y[g++] = q | (odd << 1) | (n << 2) | (og << 7);
         g = 0;
         for (int m = 0; m < p; ++m)
             for (int q = 0; q < 2; ++q)
                 for (int r = 0; r < (m ? 2 : 1); ++r)
-                    for (int og = 0; og * 4 < p - m; ++og) rg_cx[g++] = q | (r << 1) | (m << 2) | (og << 7);
+                    for (int og = 0; og * TR < p - m; ++og)
+                        rg_cx[g++] = q | (r << 1) | (m << 2) | (og << 7);
         for (int k = 0; k <= p; ++k) {
             yo[k] = y_off(k);
             co[k] = coax_off(p, k);
@@ -633,9 +657,9 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
         if (chunk + 1 < c1) {  // A is free: the next chunk's multipoles arrive during the stages
             gather(a.chunks[chunk + 1]);
         }
-        y_stage<T, NCP, NCG>(a, rg_y, yo, Yf, B, C);
+        y_stage<T, NCP, NC>(a, rg_y, yo, Yf, B, C);
         __syncthreads();
-        coax_stage<T, NCP, NCG>(a, rg_cx, co, CX, C, B);
+        coax_stage<T, NCP, NC>(a, rg_cx, co, CX, C, B);
         __syncthreads();
         // B -> C: the conversion of Eq. rcr1, per (n, m) and 4 pairs:
         // Re phi~ = Re phi - tau Im chi, Im phi~ = Im phi + tau Re chi, chi~_n = chi_n - sigma chi_{n+1}
@@ -683,7 +707,7 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
             }
         }
         __syncthreads();
-        y_stage<T, NCP, NCG>(a, rg_y, yo, Yb, C, B);
+        y_stage<T, NCP, NC>(a, rg_y, yo, Yb, C, B);
         __syncthreads();
         z_stage<T, NCP, NCG>(p, units, Zb, B, C);
         __syncthreads();
@@ -710,22 +734,26 @@ __global__ void __launch_bounds__(RA_THREADS) k_rcr_m2l(RcrArgs<T> a) {
 int slot_floats(int p) { return 2 * y_off(p) + 8 * p; }
 int coax_floats(int p) { return coax_off(p, p) + pad4(2 * p * p); }
 
-int rg_y_count(int p) {
+int tile_rows(int size) { return size == 8 ? RcrTile<double>::R : RcrTile<float>::R; }
+
+int rg_y_count(int p, int size) {
+    const int tr = tile_rows(size);
     int g = 0;
-    for (int n = 0; n < p; ++n) g += pad4(n + 1) / 4 + pad4(n) / 4;
+    for (int n = 0; n < p; ++n) g += (n + tr) / tr + (n + tr - 1) / tr;
     return 2 * g;
 }
 
-int rg_cx_count(int p) {
+int rg_cx_count(int p, int size) {
+    const int tr = tile_rows(size);
     int g = 0;
-    for (int m = 0; m < p; ++m) g += (m ? 2 : 1) * (pad4(p - m) / 4);
+    for (int m = 0; m < p; ++m) g += (m ? 2 : 1) * ((p - m + tr - 1) / tr);
     return 2 * g;
 }
 
 int apply_smem(int p, int nc, int size) {
     const int P = p * p;
     const int floats = slot_floats(p) + coax_floats(p) + 3 * (2 * P) * (nc + 4);
-    const int ints = rg_y_count(p) + rg_cx_count(p) + RCR_PMAX * (RCR_PMAX + 1) / 2 + 2 * (RCR_PMAX + 1) + nc;
+    const int ints = rg_y_count(p, size) + rg_cx_count(p, size) + RCR_PMAX * (RCR_PMAX + 1) / 2 + 2 * (RCR_PMAX + 1) + nc;
     return floats * size + ints * 4;
 }
 
@@ -950,8 +978,8 @@ void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const T* mult, T* loc, 
     a.p = rt.p;
     a.slot_floats = rt.slot_floats;
     a.coax_floats = rt.coax_floats;
-    a.nrg_y = rg_y_count(rt.p);
-    a.nrg_cx = rg_cx_count(rt.p);
+    a.nrg_y = rg_y_count(rt.p, sizeof(T));
+    a.nrg_cx = rg_cx_count(rt.p, sizeof(T));
     a.wide = 2 * rt.p * rt.p * sizeof(T) % 16 == 0 && ld * sizeof(T) % 16 == 0;
     switch (rt.nc) {
         case 32: launch_apply<T, 32>(c, rt, a); break;
