@@ -281,13 +281,13 @@ __global__ void __launch_bounds__(P2P_TILE / TPT) k_p2p(const int* __restrict__ 
     if (threadIdx.x == 0 && my_pairs) atomicAdd(pairs, my_pairs);
 }
 
-// The same sums with S source strands (FP64): a block of P2P_TILE threads takes P2P_TILE / S targets
-// of a tile, thread t target t % (P2P_TILE / S) over the sources of strand t / (P2P_TILE / S) of every
-// stage; the strands' totals are added at the end.  A leaf of ten elements fills 8 % of k_p2p's
-// block and 62 % of this one's at S = 8; past P2P_TILE / 2 elements a leaf S = 1 (k_p2p) wastes less than
-// half.  FP64 ring of 32768 elements (10 a leaf): 12.4 ms a launch with k_p2p, 4.4 ms with
-// S = 8.
-template <typename T, bool SMOOTH, int S, int CH>
+// The same sums with source strands (FP64): the nt targets of a tile take S = P2P_TILE / nt threads each,
+// thread t target t % nt over the sources t / nt, t / nt + S, ... of every stage; the strands'
+// totals are added at the end.  A leaf of ten elements fills 8 % of k_p2p's block and 94 % of this
+// one's; past P2P_TILE / 2 elements a leaf S = 1.  FP64 ring of 32768 elements (10 a leaf): 12.4 ms a
+// launch with k_p2p, 4.35 with eight strands of 16 targets for every leaf, 4.09 now; the FP64 pipe is full (the lanes of
+// a warp take all three branches of the core).
+template <typename T, bool SMOOTH, int CH>
 __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict__ ntiles_dev,
                                                          const int2* __restrict__ tiles, int* __restrict__ work,
                                                          const int* __restrict__ bbeg, const int* __restrict__ bend,
@@ -300,7 +300,6 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
                                                          vec4_t<T>* __restrict__ vout, vec4_t<T>* __restrict__ sout,
                                                          CoreConsts<T> cc, int near,
                                                          unsigned long long* __restrict__ pairs) {
-    constexpr int TW = P2P_TILE / S;     // targets per work item
     constexpr int NA = 9;
     __shared__ vec4_t<T> sx[CH];
     __shared__ vec4_t<T> sw[CH];
@@ -308,8 +307,7 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
     __shared__ T part[NA][P2P_TILE];
     __shared__ int cbeg[27], cpre[28];
     __shared__ int cur;
-    const int nitems = *ntiles_dev * S;
-    const int strand = threadIdx.x / TW, tg = threadIdx.x % TW;
+    const int nitems = *ntiles_dev;
     unsigned long long my_pairs = 0;
     for (;;) {
         __syncthreads();
@@ -317,10 +315,9 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
         __syncthreads();
         const int item = cur;
         if (item >= nitems) break;
-        const int2 tw = tiles[item / S];
-        const int leaf = tw.x, t0 = tw.y + (item % S) * TW;
-        const int tend = min(bend[leaf], tw.y + P2P_TILE);
-        if (t0 >= tend) continue;  // block-uniform
+        const int2 tw = tiles[item];
+        const int leaf = tw.x, t0 = tw.y, nt = min(bend[leaf] - t0, P2P_TILE), S = P2P_TILE / nt;
+        const int strand = threadIdx.x / nt, tg = threadIdx.x - strand * nt;
         if (threadIdx.x < 32) {  // lane q < 27 reads colleague q; a warp scan gives the prefix counts
             int cnt = 0, beg = 0;
             if (threadIdx.x < 27) {
@@ -343,7 +340,7 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
             if (threadIdx.x == 26) cpre[27] = incl;
         }
         const int ti = t0 + tg;
-        const bool act = ti < tend;
+        const bool act = strand < S;
         const vec4_t<T> xi = act ? xs[ti] : vec4_t<T>{};
         const vec4_t<T> wi = act ? ws[ti] : vec4_t<T>{};
         T hi[NA], lo[NA];
@@ -351,8 +348,7 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
         for (int a = 0; a < NA; ++a) hi[a] = lo[a] = 0;
         __syncthreads();
         const int nsrc = near ? cpre[27] : 0;
-        if (threadIdx.x == 0 && near)
-            my_pairs += (unsigned long long)min(TW, tend - t0) * (unsigned long long)(nsrc - 1);
+        if (threadIdx.x == 0 && near) my_pairs += (unsigned long long)nt * (unsigned long long)(nsrc - 1);
         int qrun = 0;  // colleague of this thread's last staged source (its sources only move forward)
         for (int s0 = 0; s0 < nsrc; s0 += CH) {
             for (int v = s0 + threadIdx.x; v < min(nsrc, s0 + CH); v += P2P_TILE) {
@@ -399,12 +395,12 @@ __global__ void __launch_bounds__(P2P_TILE) k_p2p_strands(const int* __restrict_
 #pragma unroll
         for (int a = 0; a < NA; ++a) part[a][threadIdx.x] = hi[a] + lo[a];
         __syncthreads();
-        if (strand == 0 && act) {
+        if (strand == 0) {
             T r[NA];
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
                 r[a] = part[a][tg];
-                for (int q = 1; q < S; ++q) r[a] += part[a][q * TW + tg];
+                for (int q = 1; q < S; ++q) r[a] += part[a][q * nt + tg];
             }
             vec4_t<T> vf{}, sf{};
             if (vfar) {
@@ -1257,27 +1253,22 @@ void run_p2p(Ctx* c, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs, 
     const bool wide = ctx_p2p_sources(c) == 256;
     // FP64 at one target per thread (the default): source strands where the mean leaf fills less
     // than half of a tile
-    int strands = 1;
+    bool strands = false;
     if constexpr (!std::is_same<T, float>::value) {
-        if (ctx_p2p_tpt(c) == 1)
-            while (strands < 8 && n * strands < (int64_t)lv.leaves * (P2P_TILE / 2)) strands *= 2;
-        auto launch_strands = [&](auto st) {
-            constexpr int S = decltype(st)::value;
+        strands = ctx_p2p_tpt(c) == 1 && n < (int64_t)lv.leaves * (P2P_TILE / 2);
+        if (strands) {
             int per_sm = 1, sms = 152, dev = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            auto kern = cc.smooth ? k_p2p_strands<T, true, S, 128> : k_p2p_strands<T, false, S, 128>;
+            auto kern = cc.smooth ? k_p2p_strands<T, true, 128> : k_p2p_strands<T, false, 128>;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P2P_TILE, 0);
-            const int grid = (int)std::min<int64_t>(max_tiles * S, (int64_t)sms * std::max(per_sm, 1));
+            const int grid = (int)std::min<int64_t>(max_tiles, (int64_t)sms * std::max(per_sm, 1));
             kern<<<grid, P2P_TILE, 0, s>>>(tb.tile_count.as<int>(), tb.tiles.as<int2>(), work, tb.bbeg.as<int>() + o,
                                            tb.bend.as<int>() + o, tb.bcol.as<int>() + (int64_t)o * 27, xs, ws, perm,
                                            vfar, sfar, v_out, s_out, cc, near ? 1 : 0, pair_counter);
-        };
-        if (strands == 2) launch_strands(I2{});
-        else if (strands == 4) launch_strands(I4{});
-        else if (strands == 8) launch_strands(std::integral_constant<int, 8>{});
+        }
     }
-    if (strands == 1) switch (ctx_p2p_tpt(c)) {
+    if (!strands) switch (ctx_p2p_tpt(c)) {
         case 2: wide ? launch(I2{}, C256{}) : launch(I2{}, C128{}); break;
         case 4: wide ? launch(I4{}, C256{}) : launch(I4{}, C128{}); break;
         default: wide ? launch(I1{}, C256{}) : launch(I1{}, C128{}); break;
