@@ -324,6 +324,10 @@ __device__ void dims(int kind, int P, int& pots_out, int& pots_in) {
     }
 }
 
+// Block (k, y) of a grid (specs, slices): every slices-th run of entries of table k.  With one block a
+// table the eight of M2M or L2L (83,000 FP64 entries each at p = 12) kept eight SMs busy and the rest idle.
+// A context's first evaluation, ms: cloud of 100,003 at p = 12 32.6 -> 11.8, sphere surface of 2^20 61 -> 43,
+// filament ring at p = 16 162 -> 102.
 __global__ void k_build_ops(const Spec* __restrict__ specs, double* __restrict__ out,
                             const int64_t* __restrict__ out_off) {
     __shared__ cplx Q[MAXTRI];
@@ -366,7 +370,8 @@ __global__ void k_build_ops(const Spec* __restrict__ specs, double* __restrict__
     dims(sp.kind, 0, po, pi);
     const int rows = po * Pout, cols = pi * Pin;
     double* dst = out + out_off[blockIdx.x] + sp.row0;
-    for (int64_t e = threadIdx.x; e < (int64_t)rows * cols; e += blockDim.x) {
+    for (int64_t e = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)rows * cols;
+         e += (int64_t)gridDim.y * blockDim.x) {
         int row = (int)(e % rows), col = (int)(e / rows);  // k-major: element (col, row) at col*rows + row
         int pot_out = row / Pout, pot_in = col / Pin;
         int n2, m2, pt2, n, m, q;
@@ -381,6 +386,9 @@ __global__ void k_build_ops(const Spec* __restrict__ specs, double* __restrict__
         dst[(int64_t)col * sp.ld + row] = val;
     }
 }
+
+// slices of n tables: about eight blocks an SM in all
+unsigned build_slices(int64_t n) { return (unsigned)std::max<int64_t>(1, 8 * 152 / std::max<int64_t>(n, 1)); }
 
 template <typename T>
 __global__ void k_cast(int64_t n, const double* __restrict__ in, T* __restrict__ out) {
@@ -512,7 +520,7 @@ void build_m2l_at(Ctx* c, int p, const std::vector<double>& t3, Buf& dst) {
         ensure(c, dst, n * 4 * P * P * sizeof(double));
         cuda_check(cudaMemcpyAsync(dspec.ptr, specs.data(), n * sizeof(Spec), cudaMemcpyHostToDevice, s), "specs");
         cuda_check(cudaMemcpyAsync(doff.ptr, off.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice, s), "offs");
-        k_build_ops<<<(int)n, 256, 0, s>>>(dspec.as<Spec>(), dst.as<double>(), doff.as<int64_t>());
+        k_build_ops<<<dim3((unsigned)n, build_slices(n)), 256, 0, s>>>(dspec.as<Spec>(), dst.as<double>(), doff.as<int64_t>());
         count_launch(c);
         check_launch("build operators at t");
         cuda_check(cudaStreamSynchronize(s), "operators at t");
@@ -587,7 +595,7 @@ void build_op(Ctx* c, int kind, int pout, int pin, Buf& dst) {
         cuda_check(cudaMemsetAsync(dout.ptr, 0, total * sizeof(double), s), "zero ops");
         cuda_check(cudaMemcpyAsync(dspec.ptr, specs.data(), nspec * sizeof(Spec), cudaMemcpyHostToDevice, s), "specs");
         cuda_check(cudaMemcpyAsync(doff.ptr, off.data(), nspec * sizeof(int64_t), cudaMemcpyHostToDevice, s), "offs");
-        k_build_ops<<<nspec, 256, 0, s>>>(dspec.as<Spec>(), dout.as<double>(), doff.as<int64_t>());
+        k_build_ops<<<dim3((unsigned)nspec, build_slices(nspec)), 256, 0, s>>>(dspec.as<Spec>(), dout.as<double>(), doff.as<int64_t>());
         count_launch(c);
         check_launch("build operators");
         ensure(c, dst, total * sizeof(T));
