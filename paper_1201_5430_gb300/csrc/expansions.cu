@@ -616,7 +616,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.mode = GEMM_ATOMIC;
         a.scale = (T)1;
         a.pairs_hint = lv.real[l + 1];
-        a.may_split_k = 1;
+        a.between = BETWEEN_LEVELS;
         if (!oct_tc(c, pl, TRANS_M2M, pl.m2m_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }
@@ -645,11 +645,10 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
         a.ldin = pl.ld;
         a.out = loc;
         a.ldout = pl.ld;
-        a.swap = 1;
         a.mode = GEMM_ATOMIC;  // one parent per child: the plain sum, issued without waiting for the old value
         a.scale = (T)1;
         a.pairs_hint = lv.real[l + 1];
-        a.may_split_k = 1;
+        a.between = BETWEEN_LEVELS | BETWEEN_SWAPPED;
         if (!oct_tc(c, pl, TRANS_L2L, pl.l2l_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }

@@ -125,7 +125,10 @@ constexpr int GG_THREADS = 256;
 constexpr int KC = 16;  // operator rows (input coefficients) staged per step
 constexpr int GG_DEPTH = 4;  // steps of operator rows in flight
 
-// RT = 16 * TM output rows per work item; NC columns, TN = NC / 16 per thread.
+// RT = 16 * TM output rows per work item; NC columns, TN = NC / 16 per thread.  SPLIT: the translations
+// between levels (split K, chunks in parts, pairs swapped, items in turn); M2L's instances stay free of
+// all that.  GemmArgs grows with care: two more ints in it, and the compiler gave the NC = 32, TM = 8
+// instance 79 registers instead of 106 (M2L of levels of p = 18 to 20 45 ms instead of 35).
 template <typename T, int NC, int TM, bool SPLIT>
 __global__ void __launch_bounds__(GG_THREADS) k_group_gemm(GemmArgs<T> a) {
     constexpr int TN = NC / 16;
@@ -144,31 +147,38 @@ __global__ void __launch_bounds__(GG_THREADS) k_group_gemm(GemmArgs<T> a) {
     // segments' partial products meet in the atomic adds of the epilogue
     const int nks = SPLIT && a.ksplit > 1 ? a.ksplit : 1;
     const int kper = SPLIT ? (a.C + nks * KC - 1) / (nks * KC) * KC : a.C;
-    const int nwork = (c_end - c_beg) * a.sub * nrt * nks;
+    const int sub = SPLIT && (a.between & BETWEEN_WIDE) ? TC_PAIRS / NC : 1;  // parts of a chunk
+    const int nwork = SPLIT ? (c_end - c_beg) * sub * nrt * nks : (c_end - c_beg) * nrt;
     int last_key = -1;
-    for (int turn = blockIdx.x;; turn += gridDim.x) {
+    int turn = SPLIT ? (int)blockIdx.x : 0;
+    for (;;) {
         __syncthreads();
-        if (a.work) {
+        int w;
+        if (SPLIT && !a.work) {
+            w = turn;
+            turn += gridDim.x;
+        } else {
             if (t == 0) s_work = atomicAdd(a.work, 1);
             __syncthreads();
+            w = s_work;
         }
-        const int w = a.work ? s_work : turn;
         if (w >= nwork) break;
         const int ks = SPLIT ? w % nks : 0, wc = SPLIT ? w / nks : w;
         const int part = wc / nrt, rt = wc % nrt;  // part: NC pairs of a chunk
         const int kseg0 = ks * kper, kseg1 = SPLIT ? min(a.C, kseg0 + kper) : a.C;
         if (kseg0 >= kseg1) continue;  // block-uniform: an empty last segment
-        const int4 ch = a.chunks[c_beg + part / a.sub];
-        const int g = ch.x, skip = part % a.sub * NC, p0 = ch.y + skip, np = min(NC, ch.z - skip);
-        if (np <= 0) continue;
+        const int4 ch = a.chunks[c_beg + (SPLIT ? part / sub : part)];
+        const int skip = SPLIT ? part % sub * NC : 0;
+        const int g = ch.x, p0 = ch.y + skip, np = SPLIT ? min(NC, ch.z - skip) : ch.z;
+        if (SPLIT && np <= 0) continue;
         const int r0 = rt * RT;
         const int key = part * nks + ks;
         if (key != last_key) {
             if (t < NC) {
                 if (t < np) {
                     const int2 pr = a.pairs[p0 + t];
-                    s_src[t] = a.swap ? pr.y : pr.x;
-                    s_dst[t] = a.swap ? pr.x : pr.y;
+                    s_src[t] = SPLIT && (a.between & BETWEEN_SWAPPED) ? pr.y : pr.x;
+                    s_dst[t] = SPLIT && (a.between & BETWEEN_SWAPPED) ? pr.x : pr.y;
                 } else {
                     s_src[t] = -1;
                     s_dst[t] = -1;
@@ -272,7 +282,7 @@ void launch_gemm(Ctx* c, GemmArgs<T> a) {
     // block), are handed out by a counter, which costs the clearing (FP64 ring of 32,768, M2M 0.90 ms in
     // turn, 0.75 by the counter)
     const int64_t items = (a.pairs_hint / NC + (a.g1 - a.g0)) * ((a.R + 16 * TM - 1) / (16 * TM)) * std::max(a.ksplit, 1);
-    if (a.pairs_hint > 0 && items <= (int64_t)sms * per_sm) a.work = nullptr;
+    if (SPLIT && a.pairs_hint > 0 && items <= (int64_t)sms * per_sm) a.work = nullptr;
     else cuda_check(cudaMemsetAsync(a.work, 0, 4, stream_of(c)), "gemm work");
     k_group_gemm<T, NC, TM, SPLIT><<<sms * per_sm, GG_THREADS, smem, stream_of(c)>>>(a);
     count_launch(c);
@@ -369,7 +379,7 @@ void run_group_gemm(Ctx* c, const Grouped& gp, GemmArgs<T> a) {
     a.work = gp.work.as<int>();
     // a list of the tensor cores' wide chunks: each as several items of 16 pairs
     const int nc = gp.nc == TC_PAIRS ? 16 : gp.nc;
-    a.sub = gp.nc / nc;
+    if (nc != gp.nc) a.between |= BETWEEN_WIDE;
     // rows per tile 16 TM: the tallest tile that still leaves every SM a few work items
     // (a small level's few chunks would otherwise run as a handful of long serial tiles)
     int tm = 8;
@@ -380,11 +390,11 @@ void run_group_gemm(Ctx* c, const Grouped& gp, GemmArgs<T> a) {
     // split K when the items would leave most resident blocks idle (a short level's few chunks
     // each run one long serial K loop); only where the outputs are added atomically anyway
     a.ksplit = 1;
-    if (a.may_split_k && nc == 16 && a.mode == GEMM_ATOMIC && a.pairs_hint > 0) {
+    if (a.between && nc == 16 && a.mode == GEMM_ATOMIC && a.pairs_hint > 0) {
         const int64_t items = (a.pairs_hint / nc + (a.g1 - a.g0)) * ((a.R + 16 * tm - 1) / (16 * tm));
         while (a.ksplit < 8 && items * a.ksplit < 2 * 152 * 4 && a.C >= 4 * KC * a.ksplit) a.ksplit *= 2;
     }
-    if (a.ksplit > 1 && nc == 16) launch_tm<16, true>(c, a, tm);
+    if (a.between && nc == 16) launch_tm<16, true>(c, a, tm);
     else if (nc == 64) launch_tm<64>(c, a, tm);
     else if (nc == 32) launch_tm<32>(c, a, tm);
     else launch_tm<16>(c, a, tm);

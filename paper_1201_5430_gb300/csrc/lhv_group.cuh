@@ -8,6 +8,10 @@ namespace lhv {
 
 enum GemmMode : int { GEMM_STORE = 0, GEMM_ADD = 1, GEMM_ATOMIC = 2 };
 
+// Bits of GemmArgs::between: levels; the pairs are (destination, source); chunks of TC_PAIRS pairs, taken in
+// parts of 16 (set by run_group_gemm).
+enum Between : int { BETWEEN_LEVELS = 1, BETWEEN_SWAPPED = 2, BETWEEN_WIDE = 4 };
+
 struct Grouped {
     int ngroups = 0;
     int nc = 64;                 // pairs per chunk (columns of one GEMM work item)
@@ -28,8 +32,6 @@ struct GemmArgs {
     const T* ops;         // operator of group g at ops + (g % ops_mod) * C * R, k-major [C][R]
     int ops_mod;
     int R, C;
-    int sub;              // items of a chunk (set by run_group_gemm where the list's chunks are wider than its kernel)
-    int swap;             // 1: the pairs are (destination, source)
     int psplit;           // > 0: rows >= psplit use inputs >= psplit_c only (zero lower-left block)
     int psplit_c;         // column of that split (0: the same as psplit)
     const T* in;          // source vectors: in + src * ldin, C entries
@@ -39,7 +41,7 @@ struct GemmArgs {
     int mode;             // GemmMode
     T scale;
     int64_t pairs_hint;   // about how many pairs this launch covers (0: unknown); picks the tile height
-    int may_split_k;      // 1: run_group_gemm may split K (GEMM_ATOMIC only; the translations between levels)
+    int between;          // translations between levels: BETWEEN_* bits (GEMM_ATOMIC; K may be split); else 0
     int ksplit;           // > 1: K in this many segments, one work item each (set by run_group_gemm)
 };
 
