@@ -22,8 +22,8 @@
  *    (w_x, w_y, w_z); lane 3 is ignored on input and written 0 on output.
  *  - Outputs are in the caller's element order.
  *  - All work is enqueued on the stream given to lhv_create, in stream order.
- *    Calls that build a tree read a few sizes back to the host (two short
- *    synchronisations of that stream per tree build), except the steps replayed
+ *    Calls that build a tree read a few sizes back to the host (one short
+ *    synchronisation of that stream per tree build), except the steps replayed
  *    from a captured graph (lhv_set_graph: one synchronisation per RK4 step).
  *  - Every call returns a status code (LHV_OK = 0, negative on error); no C++
  *    exception crosses the ABI.  After an error the outputs are unspecified and
@@ -306,9 +306,8 @@ int lhv_set_graph(lhv_ctx* ctx, int enable);
  * real potentials phi and chi, p^2 reals each.  M2L by the fused real tables [[T, C12 T],
  * [0, C22 T]] (translation and conversion) or by an equal route that costs less: on the
  * tensor cores (LHV_TF32X3, p a multiple of 4) the translation T of both potentials with
- * the conversion applied to the sums, on the CUDA cores with one 4 <= p <= 20 at every
- * level (FP64: up to the p whose tables fit an SM's shared memory, 16) the RCR
- * translations below, unless lhv_set_launch_shape asks for a CUDA-core chunk of the fused
+ * the conversion applied to the sums, on the CUDA cores with one 4 <= p <= 16 at every
+ * level the RCR translations below, unless lhv_set_launch_shape asks for a CUDA-core chunk of the fused
  * tables.  The routes agree to rounding.  M2M and L2L use the fused tables, or on the
  * tensor cores their translation and conversion apart.
  * LHV_FORM_PSI: one complex harmonic function Psi = phi + i chi (Eq. chf1), stored as
@@ -384,7 +383,7 @@ int lhv_export(lhv_ctx* ctx, int what, int level, void* dst, int64_t capacity_by
  * memory: a real-time loop that shares the GPU with other streams, a host
  * callback, or an application that owns a fixed memory budget.  It allocates nothing (no
  * cudaMalloc/cudaFree, no allocating library routine): every temporary lives in
- * one file-scope device array of fixed size (about 12.3 MiB, present once the
+ * one file-scope device array of fixed size (about 12.5 MiB, present once the
  * library's module is loaded on a device), whose address the first call on each
  * device looks up (cudaGetSymbolAddress).  That first call also loads the
  * library's kernels on the device; make it before any stream capture begins and

@@ -223,7 +223,7 @@ static void ensure_ops(Ctx* c) {
 }
 
 // Operator table (kind, p_out, p_in) in T from the cache, built on first use.
-// kind 5 is the tensor-core tile set of M2L(p, p).
+// kinds 5, 6 and 7 are the tensor-core tile sets of M2L, M2M and L2L(p, p).
 template <typename T>
 static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
     if (c->opcache_type != (int)sizeof(T)) {
@@ -236,11 +236,10 @@ static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
     if (it != c->opcache.end()) return it->second.as<T>();
     Buf& b = c->opcache[key];
     StageScope sc(c, LHV_STAGE_OPS);
-    if (kind == 5) {
-        // tensor-core tiles of M2L(p, p)
+    if (kind >= 5) {
         if constexpr (sizeof(T) == 4) {
-            const float* m2l = cached_op<float>(c, OP_M2L, pout, pout);
-            tc_trans_tiles(c, TRANS_M2L, m2l, pout, false, c->opcache[key]);
+            const float* op = cached_op<float>(c, kind == 5 ? OP_M2L : kind == 6 ? OP_M2M : OP_L2L, pout, pout);
+            tc_trans_tiles(c, kind == 5 ? TRANS_M2L : kind == 6 ? TRANS_M2M : TRANS_L2L, op, pout, false, c->opcache[key]);
         }
     } else {
         build_op<T>(c, kind, pout, pin, b);
@@ -317,11 +316,15 @@ static void ensure_psi_ops(Ctx* c) {
 // (640,584 pairs), RCR against the fused tables, ms: FP32 p = 4 0.24 / 0.32, p = 8 0.62 / 1.13, p = 12
 // 1.48 / 5.76, p = 16 2.94 / 20.9, p = 20 6.34 / 62.6; FP64 (32,768 elements, 640,206 pairs) p = 4
 // 1.29 / 3.72, p = 8 6.80 / 14.3, p = 12 21.5 / 92.9, p = 16 44.3 / 216.  Below p = 4 the tables were
-// not compared.
-constexpr int RCR_MIN_P = 4;
+// not compared.  Above p = 16 RCR stays with lhv_set_form: a schedule of several p (the learned form picks 18 to
+// 20 for eps = 1e-6 in FP32) has the fused tables alone, and there it is measured against a uniform p
+// of the same products (cube of 2^18: 38 ms against 49 at p = 18, 6.8 by RCR).
+constexpr int RCR_MIN_P = 4, RCR_MAX_P = 16;
 template <typename T>
 static bool default_rcr(Ctx* c) {
-    if (c->form != LHV_FORM_PHI_CHI || c->tune_nc != 0 || c->rcr_failed || c->cfg.p < RCR_MIN_P) return false;
+    if (c->form != LHV_FORM_PHI_CHI || c->tune_nc != 0 || c->rcr_failed || c->cfg.p < RCR_MIN_P ||
+        c->cfg.p > RCR_MAX_P)
+        return false;
     if (sizeof(T) == 4 && ctx_m2l_tc(c) && tc_trans_supported(TRANS_M2L, c->cfg.p)) return false;
     return rcr_chunk(c->cfg.p, sizeof(T), nullptr) > 0;
 }
@@ -397,6 +400,12 @@ static Plan<T> make_plan(Ctx* c, int L) {
         if (tc && tc_trans_supported(TRANS_M2L, pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
         if (l < L) pl.m2m[l] = cached_op<T>(c, OP_M2M, pl.p[l], pl.p[l + 1]);
         if (l > 2) pl.l2l[l] = cached_op<T>(c, OP_L2L, pl.p[l], pl.p[l - 1]);
+    }
+    // a schedule of one p (not the context's): the translations between levels on the tensor cores too
+    if (pl.uniform && tc && ctx_m2l_tc(c) && L > 2) {
+        const int p = pl.p[L];
+        if (tc_trans_supported(TRANS_M2M, p)) pl.m2m_tiles = cached_op<float>(c, 6, p, p);
+        if (tc_trans_supported(TRANS_L2L, p)) pl.l2l_tiles = cached_op<float>(c, 7, p, p);
     }
     return pl;
 }

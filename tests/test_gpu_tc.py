@@ -116,3 +116,22 @@ def test_levels_of_many_boxes_take_the_tensor_cores(p, n, leaf):
     """Low p: a level needs p^4 boxes > 1.6e7 for the tensor cores; the levels above stay with the
     grouped GEMM, which splits the same list's chunks of 128.  Bound as above."""
     test_levels_translate_like_the_fused_tables(p, n, leaf, 1)
+
+
+@pytest.mark.parametrize("p", [8, 16, 20])
+def test_a_schedule_of_one_p_equals_the_context_of_that_p(p):
+    """set_level_p with one p at every level (M2L, M2M and L2L tiles of a p that is not the context's) against
+    a context of that p: the same products, bound as for the levels above, 1.2e-5; far field."""
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(20000, 8)
+    got = []
+    for schedule in (True, False):
+        ctx = LHV(p=12 if schedule else p, leaf_max=8, core_a=0.0, precision="tf32x3", terms="far")
+        if schedule:
+            ctx.set_level_p([p] * 12)
+        v4, s4 = ctx.evaluate_velocity_stretching(dev(x, "fp32"), dev(w, "fp32"))
+        assert ctx.stats()["leaf_level"] >= 4
+        got.append((host3(v4), host3(s4)))
+        ctx.close()
+    for a, b in zip(*got):
+        assert rel(a, b) < 1.2e-5, rel(a, b)
