@@ -78,6 +78,67 @@ __device__ inline void for_each_Q(int p, T x, T y, T z, const QTab<T>& q, F&& f,
     }
 }
 
+// The same walk for N points at once: f(n, m, sum of w Re Q, sum of w Im Q).  A table entry is read
+// once for the N points, and their chains interleave.
+template <int N, typename T, typename F>
+__device__ inline void for_each_Q_sum(int p, const T (&x)[N], const T (&y)[N], const T (&z)[N], const T (&w)[N],
+                                      const QTab<T>& q, F&& f, int par) {
+    T r2[N], dre[N], dim[N];  // Q_m^m w
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        r2[i] = x[i] * x[i] + y[i] * y[i] + z[i] * z[i];
+        dre[i] = w[i];
+        dim[i] = 0;
+    }
+    const auto put = [&](int n, int m, const T(&re)[N], const T(&im)[N]) {
+        T a = re[0], b = im[0];
+#pragma unroll
+        for (int i = 1; i < N; ++i) {
+            a += re[i];
+            b += im[i];
+        }
+        f(n, m, a, b);
+    };
+    for (int m = 0; m < p; ++m) {
+        if (m > 0) {
+            const T c = q.cm[m];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const T nre = c * (x[i] * dre[i] - y[i] * dim[i]);
+                dim[i] = c * (x[i] * dim[i] + y[i] * dre[i]);
+                dre[i] = nre;
+            }
+        }
+        if ((m & 1) != par) continue;
+        put(m, m, dre, dim);
+        if (m + 1 >= p) continue;
+        T pre[N], pim[N], qre[N], qim[N];  // Q_{n-2}, Q_{n-1}
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const T c1 = q.c1[m] * z[i];
+            pre[i] = dre[i];
+            pim[i] = dim[i];
+            qre[i] = c1 * dre[i];
+            qim[i] = c1 * dim[i];
+        }
+        put(m + 1, m, qre, qim);
+        for (int n = m + 2; n < p; ++n) {
+            const T A = q.A[m * q.p + n], B = q.B[m * q.p + n];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const T a = A * z[i], b = B * r2[i];
+                const T nre = a * qre[i] - b * pre[i];
+                const T nim = a * qim[i] - b * pim[i];
+                pre[i] = qre[i];
+                pim[i] = qim[i];
+                qre[i] = nre;
+                qim[i] = nim;
+            }
+            put(n, m, qre, qim);
+        }
+    }
+}
+
 // out[r] = sum of the sparse map's row r over `in` (shared memory, in[cols] = 0), f(r, sum): the warps of
 // a block take the slices in turn.
 template <typename T, typename F>
@@ -125,6 +186,11 @@ size_t p2m_smem(int p, int most, int& chunk) {
     while (chunk > 32 && sizeof(T) * (chunk * row + qtab_reals(p)) > 80 * 1024) chunk /= 2;
     return sizeof(T) * (chunk * row + qtab_reals(p));
 }
+
+// Gauss points of a segment that one walk of the harmonics takes.  One at a time, every point added to the
+// element's row in shared memory: P2M of the filament ring of 2^18 (p = 16, eight points) 1.21 ms; four at a
+// time (two in FP64, by registers) 0.59.
+template <typename T> constexpr int SEG_POINTS = sizeof(T) == 4 ? 4 : 2;
 
 // Work items are the tiles of at most P2P_TILE consecutive elements of one leaf
 // (the near-field tiles), so a crowded leaf is spread over several blocks; each
@@ -206,36 +272,44 @@ __global__ void __launch_bounds__(THREADS) k_p2m_w(const int* __restrict__ ntile
                     }
                 }
                 T* g = gh + (size_t)e * gs;
-                const int nq = SEG ? rule.nq : 1;
-                for (int j = 0; j < nq; ++j) {
-                    double px = (double)xv.x, py = (double)xv.y, pz = (double)xv.z;
-                    T wq = 1;
-                    if constexpr (SEG) {  // Gauss point j of the segment (Eq. vf6)
-                        const vec4_t<T> wv = ws[c0 + e];
-                        const double t = 0.5 * (1.0 + rule.xi[j]);
-                        px += t * (double)wv.x;
-                        py += t * (double)wv.y;
-                        pz += t * (double)wv.z;
-                        wq = (T)rule.w[j];
+                // i^m conj(Q) to the element's row, or added to it
+                auto put = [&](int n, int m, T qr, T qi, bool add) {
+                    T re, im;
+                    switch (m & 3) {
+                        case 0: re = qr; im = -qi; break;
+                        case 1: re = qi; im = qr; break;
+                        case 2: re = -qr; im = qi; break;
+                        default: re = -qi; im = -qr; break;
                     }
-                    const T rx = (T)((px - bg.x) * bg.w), ry = (T)((py - bg.y) * bg.w), rz = (T)((pz - bg.z) * bg.w);
-                    for_each_Q<T>(p, rx, ry, rz, qt, [&](int n, int m, T qr, T qi) {
-                        T re, im;  // i^m conj(Q)
-                        switch (m & 3) {
-                            case 0: re = qr; im = -qi; break;
-                            case 1: re = qi; im = qr; break;
-                            case 2: re = -qr; im = qi; break;
-                            default: re = -qi; im = -qr; break;
+                    const int k0 = m == 0 ? n * n : n * n + 2 * m - 1;
+                    g[k0] = add ? g[k0] + re : re;
+                    if (m > 0) g[k0 + 1] = add ? g[k0 + 1] + im : im;
+                };
+                if constexpr (SEG) {
+                    // the Gauss points of the segment (Eq. vf6) SEG_POINTS at a time, in FP64 up to their rounding
+                    const vec4_t<T> wv = ws[c0 + e];
+                    const double ox = ((double)xv.x - bg.x) * bg.w, oy = ((double)xv.y - bg.y) * bg.w,
+                                 oz = ((double)xv.z - bg.z) * bg.w;
+                    const double lx = (double)wv.x * bg.w, ly = (double)wv.y * bg.w, lz = (double)wv.z * bg.w;
+                    constexpr int N = SEG_POINTS<T>;
+                    for (int j0 = 0; j0 < rule.nq; j0 += N) {
+                        T rx[N], ry[N], rz[N], wq[N];
+#pragma unroll
+                        for (int i = 0; i < N; ++i) {  // past the last point: the last again, of weight zero
+                            const int j = min(j0 + i, rule.nq - 1);
+                            const double t = 0.5 * (1.0 + rule.xi[j]);
+                            rx[i] = (T)fma(t, lx, ox);
+                            ry[i] = (T)fma(t, ly, oy);
+                            rz[i] = (T)fma(t, lz, oz);
+                            wq[i] = j0 + i < rule.nq ? (T)rule.w[j] : (T)0;
                         }
-                        const int k0 = m == 0 ? n * n : n * n + 2 * m - 1;
-                        if (j == 0) {
-                            g[k0] = wq * re;
-                            if (m > 0) g[k0 + 1] = wq * im;
-                        } else {
-                            g[k0] += wq * re;
-                            if (m > 0) g[k0 + 1] += wq * im;
-                        }
-                    }, par);
+                        for_each_Q_sum<N>(p, rx, ry, rz, wq, qt,
+                                          [&](int n, int m, T qr, T qi) { put(n, m, qr, qi, j0 > 0); }, par);
+                    }
+                } else {
+                    const T rx = (T)(((double)xv.x - bg.x) * bg.w), ry = (T)(((double)xv.y - bg.y) * bg.w),
+                            rz = (T)(((double)xv.z - bg.z) * bg.w);
+                    for_each_Q<T>(p, rx, ry, rz, qt, [&](int n, int m, T qr, T qi) { put(n, m, qr, qi, false); }, par);
                 }
             }
             __syncthreads();

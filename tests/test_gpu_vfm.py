@@ -87,3 +87,21 @@ def test_rejects_a_smoothed_context():
     with pytest.raises(LHVError) as e:
         c.evaluate_filaments([0, 4], [True], dev(np.zeros((4, 3), np.float32), "fp32"), torch.ones(4, device="cuda"))
     assert e.value.status == -6
+
+
+@pytest.mark.parametrize("p", [3, 6, 9, 10, 14])
+def test_every_number_of_gauss_points(p):
+    """Quadratures that do not fill the walks of four (FP32) and two (FP64) points: 2, 3, 5, 5 and 7 points.  Far
+    field of a ring, FP32 against FP64: 2 p^2 rounded terms a coefficient through five stages,
+    5 sqrt(2 14^2) 2^-24 = 6e-6."""
+    import torch
+    from paper_1201_5430_gb300 import LHV
+    th = 2 * np.pi * np.arange(4000) / 4000
+    x = np.stack([np.cos(th), np.sin(th), 0.1 * np.sin(3 * th)], axis=1).astype(np.float32)
+    out = []
+    for prec in ("fp32", "fp64"):
+        ctx = LHV(p=p, leaf_max=16, core_a=0.0, precision=prec, terms="far")
+        g = torch.ones(4000, device="cuda", dtype=torch.float64 if prec == "fp64" else torch.float32)
+        out.append(ctx.evaluate_filaments([0, 4000], [True], dev(x, prec), g)[:, :3].double().cpu().numpy())
+        ctx.close()
+    assert np.linalg.norm(out[0] - out[1]) < 6e-6 * np.linalg.norm(out[1])
