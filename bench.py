@@ -54,9 +54,9 @@ SINGLE = {"leapfrog": "leapfrog_rings_4194304", "ring_262144": "ring_262144"}
 # s += g (w_i . d)(w_j x d) (6) = 46 flops
 P2P_FLOPS_PER_PAIR = 46
 # extra FP32 flops of a pair inside the core radius r_K (the evaluation of K, Eq. vem1, on top of
-# the singular terms, in the form K / r^3 = 1/r^3 - exp(-x^2/2) G(a/r) / (a r^2)): t 2, degree-7
-# polynomial 14, exp argument 2 (the exp on the SFU), f 3, g 3
-P2P_CORE_FLOPS_PER_PAIR = 24
+# the singular terms, in the form K / r^3 = 1/r^3 - exp(-x^2/2) G(a/r) / (a r^2)): t 2, degree-5
+# polynomial 10, exp argument 1 (the exp on the SFU), f 3, g 3
+P2P_CORE_FLOPS_PER_PAIR = 19
 # the oracle sample of the CPU legs: the headline geometry at 2 x 2048 elements
 CPU_SAMPLE_PER_RING = 2048
 
@@ -446,6 +446,15 @@ def rcr_macs(p, padded=True):
     return 2 * 2 * (y + z) + 2 * cx + conv
 
 
+def m2l_flops_per_pair(p, tc):
+    """Useful flops of one M2L pair: on the tensor cores the translation block T of both potentials (the
+    conversion follows in the epilogue); on the CUDA cores the RCR products where they are the default
+    (4 <= p <= 16), else the fused table's three p^2 x p^2 blocks."""
+    if tc:
+        return 4 * p ** 4
+    return 2 * rcr_macs(p, padded=False) if 4 <= p <= 16 else 6 * p ** 4
+
+
 def m2l_forms(torch, LHV, n=1 << 20, ps=(12, 16, 20), reps=2, fma_peak=None):
     """M2L products by the fused tables on the tensor cores (TF32x3) against RCR translations
     on the CUDA cores (FP32), uniform cube of n elements, far field only: time per evaluation
@@ -479,7 +488,7 @@ def m2l_forms(torch, LHV, n=1 << 20, ps=(12, 16, 20), reps=2, fma_peak=None):
                                              / torch.linalg.norm(vs["fused_tf32x3"]))
         row["rcr_useful_flops_per_pair"] = 2 * rcr_macs(p, padded=False)
         row["rcr_issued_flops_per_pair"] = 2 * rcr_macs(p)
-        row["fused_useful_flops_per_pair"] = 6 * p ** 4
+        row["fused_useful_flops_per_pair"] = m2l_flops_per_pair(p, True)
         tf = row["rcr_issued_flops_per_pair"] * row["pairs"] / (row["rcr_fp32_ms"] / 1e3) / 1e12
         row["rcr_tflops_issued"] = tf
         if fma_peak:
@@ -666,9 +675,9 @@ def run_single(args, torch, LHV, local, world, rank, dist):
     fma_peak = max(probes["ffma"]["rate"] or 0.0, probes["ffma2"]["rate"] or 0.0)
     m2l_ms = st["stage_ms"].get("m2l_products", 0.0) / max(st["stage_launches"].get("m2l_products", 0), 1)
     m2l_p = st["level_p"][-1] if st["level_p"] else spec["p"]
-    m2l_flops = 6.0 * m2l_p ** 4 * st["m2l_pairs"]
-    tf32_peak = probes["tf32_mma"]["rate"]
     tc = head != "plain_fp32"
+    m2l_flops = float(m2l_flops_per_pair(m2l_p, tc)) * st["m2l_pairs"]
+    tf32_peak = probes["tf32_mma"]["rate"]
 
     # end to end through the C ABI with host buffers (H2D, step, D2H inside the timed region),
     # L2 flushed before each step as in the device-timed arm
@@ -726,7 +735,7 @@ def run_single(args, torch, LHV, local, world, rank, dist):
                                               "core_fraction_sample": "2000 targets of the initial tree"},
                      "frac_singular_only": achieved_singular / fma_peak if fma_peak else None,
                      "mean_launch_ms": p2p_ms},
-        "roofline_m2l": {"kernel": "M2L products, " + ("tcgen05 TF32 x3 (k_tc_gemm)" if tc else "CUDA cores"),
+        "roofline_m2l": {"kernel": "M2L products, " + ("tcgen05 TF32 x3 (k_tc_m2l)" if tc else "CUDA cores (k_rcr_m2l)"),
                          "bound": "tensor" if tc else "alu",
                          "achieved": m2l_flops / (m2l_ms / 1e3) / 1e12 if m2l_ms else None,
                          "peak": tf32_peak if tc else fma_peak, "unit": "TFLOP/s",
@@ -734,7 +743,7 @@ def run_single(args, torch, LHV, local, world, rank, dist):
                          if m2l_ms and (tf32_peak if tc else fma_peak) else None,
                          "peak_kind": "measured in this run: tcgen05.mma kind::tf32 probe" if tc
                          else "measured FP32 FMA probe", "box_pairs": st["m2l_pairs"],
-                         "flops_per_pair": 6 * m2l_p ** 4, "useful_only": "split products issue 3x these flops",
+                         "flops_per_pair": m2l_flops_per_pair(m2l_p, tc), "useful_only": "split products issue 3x these flops",
                          "frac_issued": (3.0 if tc else 1.0) * (m2l_flops / (m2l_ms / 1e3) / 1e12)
                          / (tf32_peak if tc else fma_peak) if m2l_ms and (tf32_peak if tc else fma_peak) else None,
                          "mean_launch_ms": m2l_ms},

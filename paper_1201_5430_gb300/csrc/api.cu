@@ -315,8 +315,9 @@ static void ensure_psi_ops(Ctx* c) {
 // smaller (sphere surface, p = 12: v 3.1e-7 against 3.6e-7).  Products of a cube of 100,003 elements
 // (640,584 pairs), RCR against the fused tables, ms: FP32 p = 4 0.24 / 0.32, p = 8 0.62 / 1.13, p = 12
 // 1.48 / 5.76, p = 16 2.94 / 20.9, p = 20 6.34 / 62.6; FP64 (32,768 elements, 640,206 pairs) p = 4
-// 1.29 / 3.72, p = 8 6.80 / 14.3, p = 12 21.5 / 92.9, p = 16 44.3 / 216.  Below p = 4 the tables were
-// not compared.  Above p = 16 RCR stays with lhv_set_form: a schedule of several p (the learned form picks 18 to
+// 1.29 / 3.72, p = 8 6.80 / 14.3, p = 12 21.5 / 92.9, p = 16 44.3 / 216.  (Before the
+// 16-byte gathers and the FP64 tiles of rcr.cu: p = 12 now 1.19 in FP32, and in FP64 4 / 7 of its time.)  Below
+// p = 4 the tables were not compared.  Above p = 16 RCR stays with lhv_set_form: a schedule of several p (the learned form picks 18 to
 // 20 for eps = 1e-6 in FP32) has the fused tables alone, and there it is measured against a uniform p
 // of the same products (cube of 2^18: 38 ms against 49 at p = 18, 6.8 by RCR).
 constexpr int RCR_MIN_P = 4, RCR_MAX_P = 16;

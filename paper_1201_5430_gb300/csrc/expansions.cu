@@ -646,8 +646,8 @@ static int oct_nc(const Plan<T>& pl, const float* tiles) {
 
 // One level of M2M or L2L on the tensor cores (LHV_TF32X3, one p a multiple of 4), true if it ran
 // there.  The grouped GEMM streams 250 KB of operator for every 16 boxes (p = 12), here one block T for
-// 128; M2M + L2L, ms: sphere surface of 2^20 2.74 -> 0.56, offset rings of 2^21 (p = 16) 1.13 -> 0.43,
-// 16 blob systems 0.61 -> 0.27.  A level of few boxes (b boxes with b p^4 up to OCT_TC_MIN) stays with the
+// 128; M2M + L2L, ms: sphere surface of 2^20 2.74 -> 0.44, offset rings of 2^21 (p = 16) 1.13 -> 0.34,
+// 16 blob systems 0.61 -> 0.20 (with the lists of k_oct_list and the bulk additions).  A level of few boxes (b boxes with b p^4 up to OCT_TC_MIN) stays with the
 // grouped GEMM, which splits its sums over the idle SMs: about 12 us at p = 12, 17 at p = 16, where the
 // MMA's one pass over T and its epilogue take 29 and 36.  M2M + L2L of a filament's eleven levels 0.88 -> 0.71, of the
 // ring of 32,768 elements 0.23 -> 0.20, the others as before (twice the limit: offset rings 0.35 -> 0.37).
