@@ -372,6 +372,11 @@ __global__ void __launch_bounds__(P2M_APPLY_THREADS) k_p2m_apply(const int* __re
 // ---------------------------------------------------------------------------
 constexpr int L2P_THREADS = 128;
 
+// Vector j = r / P of row r = j P + i (r < 12 P) of the L2P map without a division a row: the upper half of r per, per =
+// floor((2^32 - 1) / P) + 1, exact for 2 <= P <= 24^2.  At P = 1 that reciprocal is 2^32, past its 32 bits, and j = r.
+__device__ inline unsigned row_reciprocal(int P) { return P > 1 ? 0xffffffffu / (unsigned)P + 1u : 0u; }
+__device__ inline int row_vector(int r, int P, unsigned per) { return P > 1 ? (int)__umulhi((unsigned)r, per) : r; }
+
 // GRAD: the 12 vectors of v and grad v, else the 3 of v (sfar unused)
 template <typename T, int THREADS, bool GRAD>
 __global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ ntiles_dev,
@@ -388,7 +393,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ nt
     T* lh = cf + CS * P;                     // [2P] the leaf's local expansion, then a zero
     const int ntiles = *ntiles_dev;
     if (threadIdx.x == 0) lh[2 * P] = 0;
-    const unsigned per = 0xffffffffu / (unsigned)P + 1u;  // r / P = the upper half of r per, r < 12 P
+    const unsigned per = row_reciprocal(P);
     const QTab<T> qt = load_qtab(lh + 2 * P + 4, qtab, p);  // visible after the tile loop's first barrier
     // a block takes a contiguous range of tiles; the tiles of a leaf are consecutive, so the
     // leaf's coefficient vectors are staged once per leaf, not once per tile
@@ -404,7 +409,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_eval(const int* __restrict__ nt
             for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) lh[i] = loc[(int64_t)b * ld + i];
             __syncthreads();
             sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {  // r = j P + i: vector j, entry i
-                const int j = (int)__umulhi((unsigned)r, per), i = r - j * P;
+                const int j = row_vector(r, P, per), i = r - j * P;
                 cf[i * CS + j] = v;
             });
             __syncthreads();
@@ -481,7 +486,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_scalar(const int* __restrict__ 
     T* lh = cf + 4 * P;                      // [2P] (L_hat, 0), then a zero
     const int ntiles = *ntiles_dev;
     if (threadIdx.x == 0) lh[2 * P] = 0;
-    const unsigned per = 0xffffffffu / (unsigned)P + 1u;
+    const unsigned per = row_reciprocal(P);
     const QTab<T> qt = load_qtab(lh + 2 * P + 4, qtab, p);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int2 tw = tiles[t];
@@ -493,7 +498,7 @@ __global__ void __launch_bounds__(THREADS) k_l2p_scalar(const int* __restrict__ 
         // vector j = 0: phi itself, 1..3: rows of v_x, v_y, v_z
         for (int i = threadIdx.x; i < P; i += blockDim.x) cf[i * 4] = lh[i];
         sparse_rows(e, lh, threadIdx.x >> 5, THREADS / 32, [&](int r, T v) {
-            const int j = (int)__umulhi((unsigned)r, per), i = r - j * P;
+            const int j = row_vector(r, P, per), i = r - j * P;
             cf[i * 4 + 1 + j] = v;
         });
         __syncthreads();

@@ -45,3 +45,53 @@ def test_filaments_need_only_the_velocity(n):
         got.append(host3(c.evaluate_filaments([0, n], [True], dev(x, prec), torch.ones(n, device="cuda", dtype=t))))
         c.close()
     assert rel(got[0], got[1]) < 2e-6, rel(got[0], got[1])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64", "tf32x3"])
+@pytest.mark.parametrize("n,leaf", [(600, 8), (4000, 300)])
+def test_one_term_expansions(prec, n, leaf):
+    """p = 1, the smallest truncation number: a far field of constants per leaf, so v, s and grad phi are zero
+    and phi is the oracle's, for vortex elements, filaments, the scalar case and a leaf level of p = 1 below
+    longer expansions.  Positive charges: phi adds positive terms, at most the elements of a leaf, 8 L children and
+    189 L pairs in a chain, each one rounding, 20 more for the tables' own."""
+    import torch
+    from oracle import scalar
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n, 5)
+    q = np.abs(workloads.charges(n, 6))
+    e = "fp64" if prec == "fp64" else "fp32"
+    t = torch.float64 if prec == "fp64" else torch.float32
+    ref = scalar.fmm_scalar(x, q, 1, leaf_max=leaf, near=False)
+    assert ref.tree.L >= 2
+    c = LHV(p=1, leaf_max=leaf, core_a=0.0, precision=prec, terms="far")
+    v4, s4 = c.evaluate_velocity_stretching(dev(x, e), dev(w, e))
+    assert c.stats()["leaf_level"] == ref.tree.L
+    assert not v4.any() and not s4.any()
+    pg = c.evaluate_potential_gradient(dev(x, e), torch.from_numpy(q.astype(np.float64)).to("cuda", t))
+    assert not pg[:, :3].any()
+    eps = 2.0 ** (-53 if prec == "fp64" else -24)
+    bound = (leaf + 197 * ref.tree.L + 20) * eps
+    assert np.max(np.abs(pg[:, 3].double().cpu().numpy() - ref.phi) / ref.phi) < bound
+    assert not c.evaluate_filaments([0, n], [True], dev(x, e), torch.ones(n, device="cuda", dtype=t)).any()
+    c.close()
+    c = LHV(p=6, leaf_max=leaf, core_a=0.0, precision=prec, terms="far")
+    c.set_level_p([0] * ref.tree.L + [1])
+    v4, s4 = c.evaluate_velocity_stretching(dev(x, e), dev(w, e))
+    assert not v4.any() and not s4.any()
+    c.close()
+
+
+@pytest.mark.parametrize("n,leaf", [(600, 8), (4000, 300)])
+def test_two_term_expansions(n, leaf):
+    """p = 2: v and s of the FP64 context are the oracle's (1e-10, as at every other p), the FP32 one's
+    to 2e-6 as above."""
+    from oracle import fmm
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n, 5)
+    ref = fmm.fmm(x, w, 2, leaf_max=leaf, near=False)
+    assert ref.tree.L >= 2
+    for prec, tol in (("fp64", 1e-10), ("fp32", 2e-6)):
+        c = LHV(p=2, leaf_max=leaf, core_a=0.0, precision=prec, terms="far")
+        v4, s4 = c.evaluate_velocity_stretching(dev(x, prec), dev(w, prec))
+        assert rel(host3(v4), ref.v) < tol and rel(host3(s4), ref.s) < tol, (rel(host3(v4), ref.v), rel(host3(s4), ref.s))
+        c.close()
