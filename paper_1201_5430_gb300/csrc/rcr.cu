@@ -39,7 +39,7 @@
 //   A -transposed-> C -Z-> B -Y-> C -coaxial-> B -conversion-> C -Y-> B -Z-> C -transposed-> B -> locals
 // on [row][pair] buffers, the Y and coaxial stages as register-tiled products (4 output rows x 4 pairs
 // per thread, one row x 2 pairs in FP64).  The next chunk's gather is issued after the first Z stage.  Where a box's row is a
-// multiple of 16 bytes (FP64; FP32 of even p) the gather copies 16 bytes at a time to [pair][row] and a
+// multiple of 16 bytes (FP64; FP32 of even p from 4 on) the gather copies 16 bytes at a time to [pair][row] and a
 // pair's result leaves as one bulk addition; the index work of 4-byte copies and of one
 // atomicAdd per coefficient was a third of the kernel's instructions.  Products at p = 12, FP32, ms with 4-byte
 // copies and atomicAdd (odd p still) / so: cloud of 100,003, 0.64 M pairs 1.45 / 1.19; ring of 2^18,
@@ -367,7 +367,7 @@ struct RcrArgs {
     int p;
     int slot_floats, coax_floats;
     int nrg_y, nrg_cx;   // register-tile row groups of the Y / coaxial stages
-    int wide;            // a box's row is a multiple of 16 bytes
+    int wide;            // rcr_wide, and a box's row in global memory starts on 16 bytes
 };
 
 // Rows and pairs of a thread's register tile in the Y and coaxial stages.  FP32 wants reuse: two 16-byte
@@ -533,7 +533,7 @@ __device__ __forceinline__ void gather_async(const RcrArgs<T>& a, int p0, int np
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
-// The same where a row is a multiple of 16 bytes: A as [pair][row], in 16-byte pieces, a row one piece
+// The same where rcr_wide allows it: A as [pair][row], in 16-byte pieces, a row one piece
 // longer than R so that one piece of consecutive pairs spreads over the banks.
 template <typename T, int NC>
 __device__ __forceinline__ void gather_wide(const RcrArgs<T>& a, int p0, int np, T* A) {
@@ -755,6 +755,14 @@ int apply_smem(int p, int nc, int size) {
     const int floats = slot_floats(p) + coax_floats(p) + 3 * (2 * P) * (nc + 4);
     const int ints = rg_y_count(p, size) + rg_cx_count(p, size) + RCR_PMAX * (RCR_PMAX + 1) / 2 + 2 * (RCR_PMAX + 1) + nc;
     return floats * size + ints * 4;
+}
+
+// Whether a chunk may take the 16-byte route: a row of whole 16-byte pieces, and nc rows each a piece longer,
+// [pair][R + VE], no larger than the buffer [R][nc + 4] they share with the stages (FP32: nc <= R, which 32
+// pairs at p = 2 are not).
+bool rcr_wide(int p, int size, int nc) {
+    const int R = 2 * p * p, VE = 16 / size;
+    return R % VE == 0 && nc * VE <= 4 * R;
 }
 
 template <typename T, int NC>
@@ -980,7 +988,7 @@ void rcr_apply(Ctx* c, const RcrTables& rt, Grouped& gp, const T* mult, T* loc, 
     a.coax_floats = rt.coax_floats;
     a.nrg_y = rg_y_count(rt.p, sizeof(T));
     a.nrg_cx = rg_cx_count(rt.p, sizeof(T));
-    a.wide = 2 * rt.p * rt.p * sizeof(T) % 16 == 0 && ld * sizeof(T) % 16 == 0;
+    a.wide = rcr_wide(rt.p, sizeof(T), rt.nc) && ld * sizeof(T) % 16 == 0;
     switch (rt.nc) {
         case 32: launch_apply<T, 32>(c, rt, a); break;
         case 24: launch_apply<T, 24>(c, rt, a); break;

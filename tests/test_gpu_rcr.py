@@ -179,3 +179,26 @@ def test_pair_list_against_the_definition(n, leaf, nsys):
         got.append(st["m2l_pairs"])
         c.close()
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("n,leaf", [(700, 8), (40000, 8)])
+def test_form_of_few_terms_equals_the_fused_tables(p, n, leaf):
+    """LHV_FORM_RCR at the smallest p, one and many chunks a block: rows of 8 to 128 bytes, of which those of
+    p = 2 are whole 16-byte pieces but too short for the 16-byte route.  The locals of every level and the far
+    field against the fused tables', to the rounding of the sums as above (2e-6)."""
+    from paper_1201_5430_gb300 import LHV
+    x, w = workloads.cube(n, 12)
+    got = []
+    for form in ("rcr", "phi_chi"):
+        c = LHV(p=p, leaf_max=leaf, core_a=0.0, precision="fp32", terms="far")
+        c.set_form(form)
+        if form == "phi_chi":
+            c.set_launch_shape(m2l_pairs_per_chunk=64)
+        v4, s4 = c.evaluate_velocity_stretching(dev(x, "fp32"), dev(w, "fp32"))
+        L = c.stats()["leaf_level"]
+        assert L >= 2
+        got.append([host3(v4), host3(s4)] + [c.export("local", l).double().cpu().numpy() for l in range(2, L + 1)])
+        c.close()
+    for a, b in zip(*got):
+        assert np.linalg.norm(a - b) <= 2e-6 * np.linalg.norm(b), (np.linalg.norm(a - b), np.linalg.norm(b))
