@@ -284,7 +284,8 @@ int lhv_set_level_p(lhv_ctx* ctx, const int* p, int nlevels);
  * Applies to lhv_step, lhv_step_batched and lhv_step_host on FP32 / TF32X3 contexts with
  * one truncation number at every level and the selector off (other steps run as usual).
  * The first step after enabling (and after any change of n, the system offsets, the
- * x4 / w4 pointers, dt, p, precision, form or launch shapes) runs uncaptured, then in the
+ * x4 / w4 pointers, dt, p, precision, form or launch shapes, or a call in between that
+ * moved a buffer of the context to a larger one) runs uncaptured, then in the
  * captured layout, and is captured for the next calls; each later step is one
  * cudaGraphLaunch on the context stream followed by one 4-byte read and a stream
  * synchronisation.  The captured layout: the leaf level of the capture's first tree is

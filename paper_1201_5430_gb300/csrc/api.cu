@@ -76,6 +76,8 @@ struct Ctx {
     bool graph_on = false;
     int graph_L = -1;                   // >= 0 while a step runs in the captured layout (leaf level)
     bool capturing = false;
+    int64_t given_back = 0;             // buffers that have moved to a larger allocation: a captured step
+                                        // holds the addresses of its time
     bool lv_captured = false;           // the last tree was built in the captured layout
     cudaGraphExec_t graph_exec = nullptr;
     std::vector<double> graph_key;      // what the instantiated graph was captured for
@@ -125,7 +127,10 @@ void ensure(Ctx* c, Buf& b, int64_t bytes) {
     if ((size_t)bytes <= b.cap) return;
     // a capture follows an uncaptured step in the same layout, which sized every buffer
     if (c->capturing) throw Error{LHV_ECUDA, "buffer growth inside a graph capture"};
-    if (b.ptr) cudaFree(b.ptr);
+    if (b.ptr) {
+        cudaFree(b.ptr);
+        ++c->given_back;
+    }
     b.ptr = nullptr;
     b.cap = 0;
     size_t want = (size_t)bytes + (size_t)bytes / 4 + 256;
@@ -1033,7 +1038,7 @@ static std::vector<double> graph_key(Ctx* c, int64_t n, int nsys, const int64_t*
                                      const void* w4, double dt) {
     std::vector<double> k = {(double)n, (double)nsys, (double)(uintptr_t)x4, (double)(uintptr_t)w4, dt,
                              (double)c->cfg.p, (double)c->cfg.precision, (double)c->form, (double)c->tune_tpt,
-                             (double)c->tune_ch, (double)c->tune_nc, (double)c->tune_tc};
+                             (double)c->tune_ch, (double)c->tune_nc, (double)c->tune_tc, (double)c->given_back};
     for (int i = 0; i <= nsys; ++i) k.push_back((double)sysoff[i]);
     return k;
 }
@@ -1064,8 +1069,7 @@ static bool layout_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, floa
 
 static int graphed_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, float4* x4, float4* w4, double dt) {
     if (n == 0) return LHV_OK;
-    std::vector<double> key = graph_key(c, n, nsys, sysoff, x4, w4, dt);
-    if (c->graph_exec && key == c->graph_key) {
+    if (c->graph_exec && graph_key(c, n, nsys, sysoff, x4, w4, dt) == c->graph_key) {
         cuda_check(cudaGraphLaunch(c->graph_exec, c->stream), "graph launch");
         c->launches += c->graph_kernels;
         ++c->graph_replays;
@@ -1114,7 +1118,7 @@ static int graphed_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, floa
     }
     c->graph_kernels = c->launches - before;
     c->launches = before;
-    c->graph_key = key;
+    c->graph_key = graph_key(c, n, nsys, sysoff, x4, w4, dt);  // the buffers as this capture found them
     ++c->graph_captures;
     return LHV_OK;
 }

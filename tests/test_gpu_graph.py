@@ -120,3 +120,27 @@ def test_graph_needs_a_stream():
             c.set_graph(True)
         assert ei.value.status == -6
     assert c.lib.lhv_set_graph(c.h, 3) == -1
+
+
+def test_a_call_that_moves_the_buffers_ends_the_captured_step():
+    """A larger evaluation between two steps of one context moves its buffers: the next step is captured
+    again instead of replaying kernels that hold the old addresses, and equals the uncaptured step."""
+    import torch
+    x, w = workloads.ring(6000, 6)
+    xl, wl = workloads.ring(60000, 7)
+    s, g, e = _pair()
+    out = []
+    for ctx in (g, e):
+        with torch.cuda.stream(s):
+            x4, w4 = dev(x, "fp32"), dev(w, "fp32")
+            ctx.step(x4, w4, 1e-3)
+            ctx.evaluate_velocity_stretching(dev(xl, "fp32"), dev(wl, "fp32"))
+            states = []
+            for _ in range(2):
+                ctx.step(x4, w4, 1e-3)
+                states.append((host3(x4), host3(w4)))
+        s.synchronize()
+        out.append(states)
+    st = g.stats()["graph"]
+    assert st["captures"] == 2 and st["replays"] == 1 and st["fallbacks"] == 0, st
+    _close(out[0], out[1], x.astype(np.float64), w.astype(np.float64))
