@@ -1070,6 +1070,13 @@ static bool layout_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, floa
 static int graphed_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, float4* x4, float4* w4, double dt) {
     if (n == 0) return LHV_OK;
     if (c->graph_exec && graph_key(c, n, nsys, sysoff, x4, w4, dt) == c->graph_key) {
+        // the captured kernels read the system offsets that the last uncaptured tree uploaded
+        const std::vector<int64_t> offsets(sysoff, sysoff + nsys + 1);
+        if (c->tb.offsets != offsets) {
+            cuda_check(cudaMemcpyAsync(c->tb.sysoff.ptr, sysoff, offsets.size() * 8, cudaMemcpyHostToDevice, c->stream),
+                       "system offsets");
+            c->tb.offsets = offsets;
+        }
         cuda_check(cudaGraphLaunch(c->graph_exec, c->stream), "graph launch");
         c->launches += c->graph_kernels;
         ++c->graph_replays;

@@ -130,6 +130,7 @@ struct TreeBufs {
     Buf params;                // TreeParams, then a block counter per system (device)
     Buf cubes;                 // SysCube[nsys] (device)
     Buf sysoff;                // int64[nsys + 1] element offsets of the systems (device)
+    std::vector<int64_t> offsets;  // what it holds
     Buf counts;                // int32[64] (device)
     Buf bkey, bbeg, bend, bparent, bcbeg, bcend, bcol;  // per box (global index)
     Buf tiles, tile_count;     // P2P work items: int2 (leaf, first element)

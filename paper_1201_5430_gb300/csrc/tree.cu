@@ -980,12 +980,15 @@ int build_tree(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const vec4_t<
     ensure(c, tb.counts, 64 * 4);
     ensure(c, tb.cubes, (int64_t)nsys * sizeof(SysCube));
     ensure(c, tb.sysoff, (int64_t)(nsys + 1) * 8);
-    // a captured step uploads its system offsets once, before the capture
+    // a captured step uploads its system offsets before the capture, and again before a replay that
+    // follows another tree
     const int L_graph = ctx_graph_level(c);
     const bool graph = L_graph >= 0;
-    if (!graph)
+    if (!graph) {
         cuda_check(cudaMemcpyAsync(tb.sysoff.ptr, sysoff, (nsys + 1) * 8, cudaMemcpyHostToDevice, s),
                    "system offsets");
+        tb.offsets.assign(sysoff, sysoff + nsys + 1);
+    }
 
     TreeParams* tp = tb.params.as<TreeParams>();
     int* counts = tb.counts.as<int>();

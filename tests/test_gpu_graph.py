@@ -144,3 +144,29 @@ def test_a_call_that_moves_the_buffers_ends_the_captured_step():
     st = g.stats()["graph"]
     assert st["captures"] == 2 and st["replays"] == 1 and st["fallbacks"] == 0, st
     _close(out[0], out[1], x.astype(np.float64), w.astype(np.float64))
+
+
+@pytest.mark.parametrize("nsys", [1, 3])
+def test_a_smaller_call_between_replays(nsys):
+    """A smaller evaluation between two steps leaves the captured step's buffers where they are but
+    uploads its own system offsets: the next step is a replay over its own ones."""
+    import torch
+    parts = [workloads.ring(7000 - 1500 * k, 11 + k) for k in range(nsys)]
+    x, w = (np.concatenate([q[k] for q in parts]) for k in (0, 1))
+    off = [0] + list(np.cumsum([q[0].shape[0] for q in parts]))
+    xo, wo = workloads.ring(2000, 30)
+    s, g, e = _pair(max_level=4)   # one leaf level in every stage, as above
+    out = []
+    for ctx in (g, e):
+        with torch.cuda.stream(s):
+            x4, w4 = dev(x, "fp32"), dev(w, "fp32")
+            states = []
+            for k in range(3):
+                ctx.step_batched(off, x4, w4, 1e-3)
+                states.append((host3(x4), host3(w4)))
+                ctx.evaluate_velocity_stretching(dev(xo, "fp32"), dev(wo, "fp32"))
+        s.synchronize()
+        out.append(states)
+    st = g.stats()["graph"]
+    assert st["captures"] == 1 and st["replays"] == 2 and st["fallbacks"] == 0, st
+    _close(out[0], out[1], x.astype(np.float64), w.astype(np.float64))
