@@ -2,6 +2,7 @@
 // step (Sec. 5.3), statistics and array export.  See include/lhv.h.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -82,6 +83,12 @@ struct Ctx {
     cudaGraphExec_t graph_exec = nullptr;
     std::vector<double> graph_key;      // what the instantiated graph was captured for
     int64_t graph_kernels = 0;          // kernels in it
+    struct Last {                       // what the host says of the last tree and its expansions
+        Levels lv;
+        bool captured = false, far = false;
+        int64_t n = 0;
+        int p[MAX_LEVELS + 1] = {}, ld = 0;
+    } graph_last;                       // as the capture left it: a replay builds the same layout
     int64_t graph_replays = 0, graph_captures = 0, graph_fallbacks = 0;
     // complex form Psi = phi + i chi (lhv_set_form)
     int form = LHV_FORM_PHI_CHI;
@@ -581,6 +588,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
     {
         StageScope sc(c, LHV_STAGE_TREE);
         if (build_tree<T>(c, n, 1, off, x4, nullptr, c->tb, c->lv, c->hp, err) != LHV_OK) throw err;
+        c->lv_captured = false;
         c->tree_n = n;
         ensure(c, c->xs, n * (int64_t)sizeof(vec4_t<T>));
         ensure(c, c->qs, n * (int64_t)sizeof(T));
@@ -1043,6 +1051,26 @@ static std::vector<double> graph_key(Ctx* c, int64_t n, int nsys, const int64_t*
     return k;
 }
 
+static Ctx::Last last_tree(Ctx* c) {
+    Ctx::Last r;
+    r.lv = c->lv;
+    r.captured = c->lv_captured;
+    r.far = c->have_far;
+    r.n = c->tree_n;
+    std::copy(c->eval_p, c->eval_p + MAX_LEVELS + 1, r.p);
+    r.ld = c->eval_ld;
+    return r;
+}
+
+static void set_last_tree(Ctx* c, const Ctx::Last& r) {
+    c->lv = r.lv;
+    c->lv_captured = r.captured;
+    c->have_far = r.far;
+    c->tree_n = r.n;
+    std::copy(r.p, r.p + MAX_LEVELS + 1, c->eval_p);
+    c->eval_ld = r.ld;
+}
+
 static void drop_graph(Ctx* c) {
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     c->graph_exec = nullptr;
@@ -1078,6 +1106,7 @@ static int graphed_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, floa
             c->tb.offsets = offsets;
         }
         cuda_check(cudaGraphLaunch(c->graph_exec, c->stream), "graph launch");
+        set_last_tree(c, c->graph_last);
         c->launches += c->graph_kernels;
         ++c->graph_replays;
         int abort_word = 0;
@@ -1126,6 +1155,7 @@ static int graphed_step(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, floa
     c->graph_kernels = c->launches - before;
     c->launches = before;
     c->graph_key = graph_key(c, n, nsys, sysoff, x4, w4, dt);  // the buffers as this capture found them
+    c->graph_last = last_tree(c);
     ++c->graph_captures;
     return LHV_OK;
 }

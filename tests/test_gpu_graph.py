@@ -170,3 +170,34 @@ def test_a_smaller_call_between_replays(nsys):
     st = g.stats()["graph"]
     assert st["captures"] == 1 and st["replays"] == 2 and st["fallbacks"] == 0, st
     _close(out[0], out[1], x.astype(np.float64), w.astype(np.float64))
+
+
+def test_stats_and_export_follow_the_last_tree():
+    """After a replay the statistics are those of the replayed step's tree and lhv_export refuses its
+    boxes, whatever other tree came before it; after a scalar evaluation both are the scalar tree's."""
+    import torch
+    from paper_1201_5430_gb300 import LHVError
+    x, w = workloads.ring(7000, 11)
+    xo, wo = workloads.ring(1500, 30)
+    s, g, _ = _pair(a=0.0)  # the scalar case takes the singular kernel
+    with torch.cuda.stream(s):
+        x4, w4, o4, u4 = (dev(a, "fp32") for a in (x, w, xo, wo))
+        g.step(x4, w4, 0.0)
+        g.step(x4, w4, 0.0)
+        want = g.stats()
+        g.evaluate_velocity_stretching(o4, u4)
+        other = g.stats()
+        g.step(x4, w4, 0.0)
+        st = g.stats()
+        assert st["graph"]["replays"] == 2
+        assert (st["n"], st["leaf_level"], st["nbox"]) == (7000, want["leaf_level"], want["nbox"])
+        assert other["n"] == 1500 and other["nbox"] != want["nbox"]
+        for what in ("box_keys", "multipole"):
+            with pytest.raises(LHVError) as ei:
+                g.export(what, 2)
+            assert ei.value.status == -6
+        g.evaluate_potential_gradient(o4, torch.ones(1500, device="cuda"))
+        st = g.stats()
+        assert (st["n"], st["leaf_level"]) == (1500, other["leaf_level"])
+        assert g.export("box_keys", 2).numel() == st["nbox"][2]
+    s.synchronize()
