@@ -149,6 +149,15 @@ void ensure(Ctx* c, Buf& b, int64_t bytes) {
     b.cap = want;
 }
 
+// A plain cudaMemcpy may return before its transfer is done and is ordered on the default stream alone, which a
+// non-blocking stream of the context does not wait for.
+void upload(Ctx* c, Buf& b, const void* src, int64_t bytes, const char* what) {
+    ensure(c, b, bytes);
+    if (bytes <= 0) return;
+    cuda_check(cudaMemcpyAsync(b.ptr, src, (size_t)bytes, cudaMemcpyHostToDevice, c->stream), what);
+    cuda_check(cudaStreamSynchronize(c->stream), what);
+}
+
 static void release(Buf& b) {
     if (b.ptr) cudaFree(b.ptr);
     b.ptr = nullptr;

@@ -558,8 +558,7 @@ void build_qtab(Ctx* c, int p, Buf& dst) {
         cm[m] = m > 0 ? (T)-std::sqrt((2.0 * m - 1.0) / (2.0 * m)) : (T)0;
         c1[m] = (T)std::sqrt(2.0 * m + 1.0);
     }
-    ensure(c, dst, (int64_t)(h.size() * sizeof(T)));
-    cuda_check(cudaMemcpy(dst.ptr, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice), "recurrence table");
+    upload(c, dst, h.data(), (int64_t)(h.size() * sizeof(T)), "recurrence table");
 }
 
 // Blocks of a persistent kernel: as many as are resident at once, at most `items`.

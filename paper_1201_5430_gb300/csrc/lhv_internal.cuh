@@ -87,6 +87,8 @@ cudaStream_t stream_of(Ctx* c);
 void check_launch(const char* what);                 // throws Error{LHV_ECUDA} on a launch failure
 void cuda_check(cudaError_t e, const char* what);    // throws Error{LHV_ECUDA}
 void ensure(Ctx* c, Buf& b, int64_t bytes);          // grow b to >= bytes (throws Error{LHV_ENOMEM})
+// b = `bytes` bytes of pageable host memory, in order on the context's stream, `src` free on return
+void upload(Ctx* c, Buf& b, const void* src, int64_t bytes, const char* what);
 int ctx_leaf_max(Ctx* c);
 int ctx_max_level(Ctx* c);
 double ctx_rK(Ctx* c);

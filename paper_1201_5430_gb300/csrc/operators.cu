@@ -471,12 +471,8 @@ void build_sparse(Ctx* c, int kind, int p, int rows, Sell& dst) {
         }
     }
     free_sparse(dst);
-    auto put = [&](Buf& b, const void* src, size_t bytes) {
-        ensure(c, b, (int64_t)bytes);
-        if (bytes) cuda_check(cudaMemcpy(b.ptr, src, bytes, cudaMemcpyHostToDevice), "sparse map");
-    };
-    put(dst.sptr, sptr.data(), sptr.size() * 4);
-    put(dst.ent, ent.data(), ent.size() * sizeof(SellEntry<T>));
+    upload(c, dst.sptr, sptr.data(), (int64_t)sptr.size() * 4, "sparse map");
+    upload(c, dst.ent, ent.data(), (int64_t)(ent.size() * sizeof(SellEntry<T>)), "sparse map");
     dst.rows = nr;
     dst.cols = C;
 }
