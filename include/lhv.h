@@ -267,6 +267,10 @@ int lhv_autotune_batched(lhv_ctx* ctx, int nsys, const int64_t* offsets, const f
  * them).  LHV_EINVAL otherwise. */
 int lhv_set_launch_shape(lhv_ctx* ctx, int p2p_targets_per_thread, int p2p_sources_per_stage,
                          int m2l_pairs_per_chunk, int m2l_tensor_cores);
+/* Polls after which a device-side wait of the tensor-core translations (LHV_TF32X3) gives up, 1 ..
+ * 2^24; 0: the default, 2^24 (seconds).  Every block then ends with its copies and products waited for, the
+ * outputs are invalid, and the next lhv_get_stats returns LHV_ETIMEOUT once.  LHV_EINVAL otherwise. */
+int lhv_set_wait_limit(lhv_ctx* ctx, int64_t polls);
 
 /* Truncation number per octree level (variable truncation, which the paper
  * mentions but does not use, Sec. 5).  p[l] for the levels l < nlevels (host

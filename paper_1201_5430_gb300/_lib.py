@@ -56,6 +56,7 @@ SIGNATURES = {
     "lhv_autotune": (_int, [_vp, _i64, _vp, _vp, _vp, _vp]),
     "lhv_autotune_batched": (_int, [_vp, _int, ctypes.POINTER(_i64), _vp, _vp, _vp, _vp]),
     "lhv_set_launch_shape": (_int, [_vp, _int, _int, _int, _int]),
+    "lhv_set_wait_limit": (_int, [_vp, ctypes.c_int64]),
     "lhv_set_selector": (_int, [_vp, _vp, _vp, _dbl, _int, _int]),
     "lhv_selector_features": (_int, [_vp, _i64, _vp, _vp, _dbl, _vp, _int, ctypes.POINTER(_int)]),
     "lhv_mlp_forward": (_int, [_int, _vp, _vp, _vp, _vp, _vp]),

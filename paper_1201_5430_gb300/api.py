@@ -181,6 +181,10 @@ class LHV:
                                                   int(m2l_pairs_per_chunk), int(m2l_tensor_cores)),
                     "set_launch_shape")
 
+    def set_wait_limit(self, polls=0):
+        """Polls after which a device wait of the tensor-core translations gives up (0: the default)."""
+        self._check(self.lib.lhv_set_wait_limit(self.h, int(polls)), "set_wait_limit")
+
     def set_selector(self, W=None, b=None, eps=1e-6, check_every=1, check_samples=1000):
         """Switch the learned form on with network weights W (bfloat16 [LHV_MLP_NW]) and
         biases b (float32 [LHV_MLP_NB]), host or device tensors; W = None switches it off."""

@@ -62,6 +62,7 @@ struct Ctx {
     int tune_tpt = 1;                   // P2P targets per thread
     int tune_ch = 128;                  // P2P sources per shared-memory stage
     int tune_nc = 0;                    // M2L pairs per SIMT GEMM chunk (0: the largest that fits)
+    int64_t wait_limit = WAIT_LIMIT_DEFAULT;  // lhv_set_wait_limit
     int tune_tc = 1;                    // TF32x3: M2L products on the tensor cores (1) or CUDA cores (0)
     double tune_ms[12] = {0};           // measured stage times of the candidates
     // learned form (lhv_set_selector)
@@ -115,6 +116,7 @@ double ctx_rK(Ctx* c) { return c->rK; }
 int& ctx_sort_levels(Ctx* c) { return c->sort_levels; }
 Buf& ctx_tmp(Ctx* c, int i) { return c->tmp[i]; }
 bool ctx_use_tc(Ctx* c) { return c->cfg.precision == LHV_TF32X3; }
+int64_t ctx_wait_limit(Ctx* c) { return c->wait_limit; }
 int* ctx_err_flag(Ctx* c) { return reinterpret_cast<int*>(c->counters.as<unsigned long long>() + 2); }
 int ctx_p2p_tpt(Ctx* c) { return c->tune_tpt; }
 int ctx_p2p_sources(Ctx* c) { return c->tune_ch; }
@@ -1055,7 +1057,7 @@ static std::vector<double> graph_key(Ctx* c, int64_t n, int nsys, const int64_t*
                                      const void* w4, double dt) {
     std::vector<double> k = {(double)n, (double)nsys, (double)(uintptr_t)x4, (double)(uintptr_t)w4, dt,
                              (double)c->cfg.p, (double)c->cfg.precision, (double)c->form, (double)c->tune_tpt,
-                             (double)c->tune_ch, (double)c->tune_nc, (double)c->tune_tc, (double)c->given_back};
+                             (double)c->tune_ch, (double)c->tune_nc, (double)c->tune_tc, (double)c->given_back, (double)c->wait_limit};
     for (int i = 0; i <= nsys; ++i) k.push_back((double)sysoff[i]);
     return k;
 }
@@ -1694,6 +1696,12 @@ int lhv_set_launch_shape(lhv_ctx* ctx, int p2p_targets_per_thread, int p2p_sourc
     ctx->c.tune_ch = p2p_sources_per_stage;
     ctx->c.tune_nc = nc;
     ctx->c.tune_tc = m2l_tensor_cores;
+    return LHV_OK;
+}
+
+int lhv_set_wait_limit(lhv_ctx* ctx, int64_t polls) {
+    if (!ctx || polls < 0 || polls > lhv::WAIT_LIMIT_DEFAULT) return LHV_EINVAL;
+    ctx->c.wait_limit = polls ? polls : lhv::WAIT_LIMIT_DEFAULT;
     return LHV_OK;
 }
 

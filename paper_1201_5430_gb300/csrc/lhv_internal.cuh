@@ -16,6 +16,7 @@ constexpr int MAX_LEVELS = LHV_MAX_LEVELS;
 constexpr int NUM_OFFSETS = 316;       // M2L offsets: [-3,3]^3 minus [-1,1]^3
 constexpr int P2P_TILE = 128;          // targets per P2P work item
 constexpr int TC_PAIRS = 128;          // box pairs per tensor-core M2L chunk (the MMA's M)
+constexpr int64_t WAIT_LIMIT_DEFAULT = 1ll << 24;  // polls of a device wait of the tensor-core translations
 
 // 32-byte aligned four-double element (the _f64 element layout).
 struct alignas(32) dbl4 {
@@ -96,6 +97,7 @@ int& ctx_sort_levels(Ctx* c);                        // Morton levels the next t
 Buf& ctx_tmp(Ctx* c, int i);                         // scratch buffers 0..13 owned by the context
 bool ctx_use_tc(Ctx* c);                             // LHV_TF32X3: dense maps on the tensor cores
 int* ctx_err_flag(Ctx* c);                           // device word set by a timed-out device wait
+int64_t ctx_wait_limit(Ctx* c);                      // polls of a device wait of the tensor-core translations
 int ctx_p2p_tpt(Ctx* c);                             // P2P targets per thread (autotuned; 1, 2 or 4)
 int ctx_p2p_sources(Ctx* c);                         // P2P sources per shared-memory stage (128 or 256)
 int ctx_m2l_nc(Ctx* c, int dflt);                    // M2L pairs per SIMT GEMM chunk (autotuned, <= dflt)

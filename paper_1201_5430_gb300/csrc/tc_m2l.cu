@@ -72,7 +72,6 @@ constexpr int M2_X_TILE = TC_PAIRS * TC_KC * 4;  // bytes of one operand tile of
 constexpr int M2_BAND = 64;                // columns (a potential) staged at once
 constexpr int M2_STG_LD = M2_BAND + 4;     // staging [pair][column]: a quad of a pair to a bank group of its own
 constexpr int M2_TMEM = 512;               // TMEM columns: one or two accumulator buffers
-constexpr long long M2_WAIT_LIMIT = 1ll << 24;
 constexpr int M2_SMEM_MAX = 226 * 1024;    // dynamic shared memory (the static part is below 1 KB)
 
 struct M2lArgs {
@@ -98,6 +97,7 @@ struct M2lArgs {
     float chi_scale;         // chi^ = chi_scale T chi (1; L2L 1/2, M2M 2)
     int ngroups;             // operators (a group's is g % ngroups)
     int* err;
+    int64_t wait_limit;      // polls after which a wait gives up
 };
 
 // floats of the conversion table, padded for the reads of the eight orders of a last unit
@@ -108,13 +108,12 @@ struct M2lShared {
     uint64_t acc_full[2], acc_empty[2], done;
     uint32_t tmem;
     int abort;       // set by a role whose wait gave up
-    int epi_abort;   // the epilogue's own verdict, read by all its warps after a barrier
 };
 
 // bounded wait that also ends when another role has given up
-__device__ __forceinline__ bool m2_wait(uint64_t* bar, uint32_t parity, M2lShared& sh, int* err) {
+__device__ __forceinline__ bool m2_wait(uint64_t* bar, uint32_t parity, M2lShared& sh, const M2lArgs& args) {
     const uint32_t a = smem_u32(bar);
-    for (long long it = 0; it < M2_WAIT_LIMIT; ++it) {
+    for (int64_t it = 0; it < args.wait_limit; ++it) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -126,7 +125,7 @@ __device__ __forceinline__ bool m2_wait(uint64_t* bar, uint32_t parity, M2lShare
         if ((it & 63) == 63 && *(volatile int*)&sh.abort) return false;
     }
     *(volatile int*)&sh.abort = 1;
-    atomicExch(err, 1);
+    atomicExch(args.err, 1);
     return false;
 }
 
@@ -146,7 +145,19 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t b
 // epilogue reads the column before a degree
 __device__ __forceinline__ uint32_t acc_base(int range) { return range ? 16u : 0u; }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// Barrier of the 256 epilogue threads; whether any of them passed `leave`, the same answer for all.  (A word in
+// shared memory that each reads after the barrier is not: a fast warp can set it for its next item before a slow one has
+// read it for this one, and the two would part at different barriers.)
+__device__ __forceinline__ bool epi_any(bool leave) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(any)
+        : "r"((uint32_t)leave)
+        : "memory");
+    return any != 0;
+}
 // the two epilogue warps of a lane quarter
 __device__ __forceinline__ void quarter_sync(int quarter) {
     asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
@@ -314,7 +325,6 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
         }
         mbar_init(&sh.done, 1);
         sh.abort = 0;
-        sh.epi_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (NPOT == 2) {
@@ -385,7 +395,7 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                 load(cur, k2, w);
             }
             const int st = g % S;
-            if (!__all_sync(0xffffffffu, m2_wait(&sh.empty[st], ((uint32_t)(g / S) & 1u) ^ 1u, sh, a.err))) break;
+            if (!__all_sync(0xffffffffu, m2_wait(&sh.empty[st], ((uint32_t)(g / S) & 1u) ^ 1u, sh, a))) break;
             unsigned char* base = smem + (size_t)st * a.stage_bytes;
 #pragma unroll
             for (int q = 0; q < NPOT; ++q)
@@ -426,7 +436,7 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                 const uint32_t bytes = (uint32_t)a.nlen[r] * TC_KC * 4 * 2;
                 const float* src = a.tiles + (int64_t)slot * a.group_stride + a.roff[r];
                 for (int k = 0; k < nk; ++k) {
-                    ok = m2_wait(&sh.empty[st], ph, sh, a.err);
+                    ok = m2_wait(&sh.empty[st], ph, sh, a);
                     if (!ok) break;
                     mbar_expect_tx(&sh.full_b[st], bytes);
                     bulk_copy(smem + (size_t)st * a.stage_bytes + 2 * NPOT * M2_X_TILE, src + (int64_t)(nk - 1 - k) * (bytes / 4),
@@ -455,10 +465,10 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                 const int nlen = a.nlen[item % a.nranges], b = n % a.nbuf;
                 const uint32_t idesc = make_idesc(TC_PAIRS, nlen);
                 const uint32_t d0 = tmem + (uint32_t)(b * (M2_TMEM / a.nbuf)) + acc_base(item % a.nranges);
-                ok = m2_wait(&sh.acc_empty[b], ((uint32_t)(n / a.nbuf) & 1u) ^ 1u, sh, a.err);
+                ok = m2_wait(&sh.acc_empty[b], ((uint32_t)(n / a.nbuf) & 1u) ^ 1u, sh, a);
                 if (!ok) break;
                 for (int k = 0; k < nk; ++k) {
-                    ok = m2_wait(&sh.full_a[st], ph, sh, a.err) && m2_wait(&sh.full_b[st], ph, sh, a.err);
+                    ok = m2_wait(&sh.full_a[st], ph, sh, a) && m2_wait(&sh.full_b[st], ph, sh, a);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t base = smem_u32(smem + (size_t)st * a.stage_bytes);
@@ -507,10 +517,8 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
             const int2 pr = row < ch.z ? a.pairs[ch.y + row] : make_int2(-1, -1);
             const int dst = a.swap ? pr.x : pr.y;
             float* out = a.out + (int64_t)dst * a.ld;  // not used where dst < 0
-            // a wait that gave up is seen by every epilogue warp after this barrier: all leave together
-            if (!m2_wait(&sh.acc_full[b], (uint32_t)(n / a.nbuf) & 1u, sh, a.err)) *(volatile int*)&sh.epi_abort = 1;
-            epi_sync();
-            if (*(volatile int*)&sh.epi_abort) break;
+            // where a wait gave up, all epilogue warps leave together, at this item
+            if (epi_any(!m2_wait(&sh.acc_full[b], (uint32_t)(n / a.nbuf) & 1u, sh, a))) break;
             tc_fence_after();
             const int n0 = a.n0[r], n1 = a.n1[r], c0 = a.c0[r], nlen = a.nlen[r];
             const uint32_t tp =
@@ -760,6 +768,7 @@ void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int
     a.tvec = a.conv + conv_floats(p);
     a.chi_scale = kind == TRANS_M2L ? 1.0f : kind == TRANS_L2L ? 0.5f : 2.0f;
     a.err = err;
+    a.wait_limit = ctx_wait_limit(c);
     // above half an SM's shared memory: one CTA (and its 512 TMEM columns) per SM
     const size_t smem =
         std::max<size_t>((size_t)a.nstages * a.stage_bytes + m2l_fixed_smem(p, scalar ? 1 : 2), 120 * 1024);

@@ -135,3 +135,38 @@ def test_a_schedule_of_one_p_equals_the_context_of_that_p(p):
         ctx.close()
     for a, b in zip(*got):
         assert rel(a, b) < 1.2e-5, rel(a, b)
+
+
+@pytest.mark.parametrize("scalar", [False, True])
+def test_waits_that_give_up_end_the_translations(scalar):
+    """Short limits let the waits of a launch's roles run out at any of its items: every call ends, the
+    status says so once, and with the default limit the same context gives its first results again."""
+    import torch
+    from paper_1201_5430_gb300 import LHV, LHVError
+    from paper_1201_5430_gb300 import _lib
+    x, w = workloads.cube(20000, 8)
+    x4, w4 = dev(x, "fp32"), dev(w, "fp32")
+    q = torch.from_numpy(workloads.charges(20000, 3)).cuda()
+    ctx = LHV(p=12, leaf_max=16, core_a=0.0, precision="tf32x3", terms="far")
+    call = (lambda: ctx.evaluate_potential_gradient(x4, q)) if scalar else \
+        (lambda: ctx.evaluate_velocity_stretching(x4, w4)[0])
+    want = call().double().cpu().numpy()
+    ctx.stats()
+    gave_up = 0
+    for limit in [1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64, 128, 256, 1024] * 3:
+        ctx.set_wait_limit(limit)
+        call()
+        torch.cuda.synchronize()
+        try:
+            ctx.stats()
+        except LHVError as e:
+            assert e.status == _lib.LHV_ETIMEOUT
+            gave_up += 1
+    assert gave_up > 0
+    ctx.set_wait_limit()
+    got = call().double().cpu().numpy()
+    ctx.stats()
+    assert rel(got, want) < 2e-6
+    for bad in (-1, (1 << 24) + 1):
+        assert ctx.lib.lhv_set_wait_limit(ctx.h, bad) == _lib.LHV_EINVAL
+    ctx.close()
