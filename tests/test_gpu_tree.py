@@ -141,3 +141,35 @@ def test_keys_and_order_at_the_edges_of_the_sort(n, kind):
 def test_colleagues_of_many_leaves():
     """Enough leaves (above 8192) that their colleagues come from the parents'."""
     _check(workloads.cube(30000, 3)[0], 4)
+
+
+@pytest.mark.parametrize("n", [4194304, 4194305])
+def test_boxes_at_the_change_of_items_a_thread(n):
+    """The two passes over the sorted keys take more elements a thread above 4,194,304: the boxes of every level
+    against the runs of equal key prefixes, ranges, and the colleagues' number."""
+    import torch
+    from paper_1201_5430_gb300 import LHV
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    x4 = torch.zeros((n, 4), device="cuda")
+    x4[:, :3] = torch.rand((n, 3), generator=g, device="cuda")
+    ctx = LHV(p=4, leaf_max=64, max_level=5)
+    ctx.build_tree(x4)
+    st = ctx.stats()
+    assert st["leaf_level"] == 5
+    keys = ctx.export("keys")
+    assert bool((keys[1:] >= keys[:-1]).all())
+    assert torch.equal(ctx.export("perm").long().sort().values, torch.arange(n, device="cuda"))
+    for l in range(6):
+        want, cnt = torch.unique_consecutive(keys >> (3 * (21 - l)), return_counts=True)
+        end = cnt.cumsum(0)
+        assert st["nbox"][l] == want.numel()
+        assert torch.equal(ctx.export("box_keys", l), want)
+        rng = ctx.export("box_range", l).reshape(-1, 2).long()
+        assert torch.equal(rng[:, 0], end - cnt) and torch.equal(rng[:, 1], end)
+        col = ctx.export("colleagues", l).reshape(-1, 27).long()
+        assert torch.equal(col[:, 13], torch.arange(want.numel(), device="cuda"))
+        if l == 5:  # a full level: 3 m - 2 neighbours along each axis of m boxes, summed
+            assert want.numel() == 32 ** 3
+            assert int((col >= 0).sum()) == (3 * 32 - 2) ** 3
+    ctx.close()
