@@ -54,9 +54,9 @@ extern "C" {
 #define LHV_FP32 0  /* all kernels in FP32 (CUDA cores); operator tables built in FP64, stored FP32 */
 #define LHV_FP64 1  /* all kernels in FP64 (use the _f64 entry points) */
 #define LHV_TF32X3 2 /* mixed precision: as LHV_FP32, but the products of M2L, and with one p at every
-                        level of M2M (p <= 16) and L2L, run on the tensor cores in TF32 with split
-                        operands (hi.hi + hi.lo + lo.hi, FP32 accumulation) where p is a multiple
-                        of 4; other p and the other maps run as in LHV_FP32 */
+                        level of L2L, run on the tensor cores in TF32 with split operands (hi.hi +
+                        hi.lo + lo.hi, FP32 accumulation) where p is a multiple of 4; other p and
+                        the other maps run as in LHV_FP32 */
 
 /* ---- which parts of Eq. fmm1 to evaluate (lhv_config.terms) ------------ */
 #define LHV_TERMS_NEAR 1  /* sparse part only: direct sum over colleague leaves */
@@ -313,8 +313,8 @@ int lhv_set_graph(lhv_ctx* ctx, int enable);
  * tensor cores (LHV_TF32X3, p a multiple of 4) the translation T of both potentials with
  * the conversion applied to the sums, on the CUDA cores with one 4 <= p <= 16 at every
  * level the RCR translations below, unless lhv_set_launch_shape asks for a CUDA-core chunk of the fused
- * tables.  The routes agree to rounding.  M2M and L2L use the fused tables, or on the
- * tensor cores their translation and conversion apart.
+ * tables.  The routes agree to rounding.  M2M and L2L use the fused tables, L2L on the
+ * tensor cores translation and conversion apart.
  * LHV_FORM_PSI: one complex harmonic function Psi = phi + i chi (Eq. chf1), stored as
  * 2 p^2 reals (Re / Im of Psi_n^m for m >= 0, then of Psi_n^{-m}; Im Psi_n^0 in place of
  * the m = 0 entry of the second half), translated by one dense real table per offset or

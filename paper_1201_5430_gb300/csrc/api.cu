@@ -43,7 +43,7 @@ struct Ctx {
     bool have_m2l = false;              // ops.m2l is built
     Buf tmp[14];
     Buf xs, ws, mult, loc, table, vfar, sfar, counters, W;
-    Grouped gp_m2m, gp_m2l, gp_l2l;
+    Grouped gp_m2m, gp_m2l;  // gp_m2m: of L2L too
     Buf rk[6];         // kv, ks, ax, aw, sx, sw
     Buf hx, hw;        // device copies for lhv_step_host
     bool have_far = false;
@@ -100,7 +100,7 @@ struct Ctx {
     bool rcr_failed = false;            // its tables failed their check: the default form keeps the fused ones
     // scalar reference case (lhv_evaluate_potential_gradient)
     Buf s_m2l, s_m2m, s_l2l;            // translation blocks of the fused tables
-    Buf s_tiles, s_m2m_tiles, s_l2l_tiles;  // and their TF32 tiles
+    Buf s_tiles, s_l2l_tiles;           // TF32 tiles of M2L and L2L
     int s_p = 0, s_type = 0;
     Buf qs, pgfar;
     // filament segments (lhv_evaluate_filaments)
@@ -235,18 +235,16 @@ static void ensure_ops(Ctx* c) {
     if constexpr (sizeof(T) == 4) {
         if (ctx_use_tc(c)) {
             const int p = c->cfg.p;
-            if (tc_trans_supported(TRANS_M2L, p))
+            if (tc_trans_supported(p)) {
                 tc_trans_tiles(c, TRANS_M2L, fused_m2l<float>(c), p, false, c->ops.m2l_tiles);
-            if (tc_trans_supported(TRANS_M2M, p))
-                tc_trans_tiles(c, TRANS_M2M, c->ops.m2m.as<float>(), p, false, c->ops.m2m_tiles);
-            if (tc_trans_supported(TRANS_L2L, p))
                 tc_trans_tiles(c, TRANS_L2L, c->ops.l2l.as<float>(), p, false, c->ops.l2l_tiles);
+            }
         }
     }
 }
 
 // Operator table (kind, p_out, p_in) in T from the cache, built on first use.
-// kinds 5, 6 and 7 are the tensor-core tile sets of M2L, M2M and L2L(p, p).
+// kinds 5 and 6 are the tensor-core tile sets of M2L and L2L(p, p).
 template <typename T>
 static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
     if (c->opcache_type != (int)sizeof(T)) {
@@ -261,8 +259,8 @@ static const T* cached_op(Ctx* c, int kind, int pout, int pin) {
     StageScope sc(c, LHV_STAGE_OPS);
     if (kind >= 5) {
         if constexpr (sizeof(T) == 4) {
-            const float* op = cached_op<float>(c, kind == 5 ? OP_M2L : kind == 6 ? OP_M2M : OP_L2L, pout, pout);
-            tc_trans_tiles(c, kind == 5 ? TRANS_M2L : kind == 6 ? TRANS_M2M : TRANS_L2L, op, pout, false, c->opcache[key]);
+            const float* op = cached_op<float>(c, kind == 5 ? OP_M2L : OP_L2L, pout, pout);
+            tc_trans_tiles(c, kind == 5 ? TRANS_M2L : TRANS_L2L, op, pout, false, c->opcache[key]);
         }
     } else {
         build_op<T>(c, kind, pout, pin, b);
@@ -349,7 +347,7 @@ static bool default_rcr(Ctx* c) {
     if (c->form != LHV_FORM_PHI_CHI || c->tune_nc != 0 || c->rcr_failed || c->cfg.p < RCR_MIN_P ||
         c->cfg.p > RCR_MAX_P)
         return false;
-    if (sizeof(T) == 4 && ctx_m2l_tc(c) && tc_trans_supported(TRANS_M2L, c->cfg.p)) return false;
+    if (sizeof(T) == 4 && ctx_m2l_tc(c) && tc_trans_supported(c->cfg.p)) return false;
     return rcr_chunk(c->cfg.p, sizeof(T), nullptr) > 0;
 }
 
@@ -408,10 +406,7 @@ static Plan<T> make_plan(Ctx* c, int L) {
         pl.qtab = c->ops.qtab.as<T>();
         pl.p2m_sp = view<T>(c->ops.p2m_sp);
         pl.l2p_sp = view<T>(c->ops.l2p_sp);
-        if (tiles) {
-            pl.m2m_tiles = c->ops.m2m_tiles.as<float>();
-            pl.l2l_tiles = c->ops.l2l_tiles.as<float>();
-        }
+        if (tiles) pl.l2l_tiles = c->ops.l2l_tiles.as<float>();
         return pl;
     }
     pl.p2m_sp = cached_sparse<T>(c, OP_P2M, pl.p[L]);
@@ -421,16 +416,13 @@ static Plan<T> make_plan(Ctx* c, int L) {
     pl.l2p_sp = cached_sparse<T>(c, OP_L2P, pl.p[L]);
     for (int l = 2; l <= L; ++l) {
         pl.m2l[l] = cached_op<T>(c, OP_M2L, pl.p[l], pl.p[l]);
-        if (tc && tc_trans_supported(TRANS_M2L, pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
+        if (tc && tc_trans_supported(pl.p[l])) pl.m2l_tiles[l] = cached_op<float>(c, 5, pl.p[l], pl.p[l]);
         if (l < L) pl.m2m[l] = cached_op<T>(c, OP_M2M, pl.p[l], pl.p[l + 1]);
         if (l > 2) pl.l2l[l] = cached_op<T>(c, OP_L2L, pl.p[l], pl.p[l - 1]);
     }
-    // a schedule of one p (not the context's): the translations between levels on the tensor cores too
-    if (pl.uniform && tc && ctx_m2l_tc(c) && L > 2) {
-        const int p = pl.p[L];
-        if (tc_trans_supported(TRANS_M2M, p)) pl.m2m_tiles = cached_op<float>(c, 6, p, p);
-        if (tc_trans_supported(TRANS_L2L, p)) pl.l2l_tiles = cached_op<float>(c, 7, p, p);
-    }
+    // a schedule of one p (not the context's): L2L on the tensor cores too
+    if (pl.uniform && tc && ctx_m2l_tc(c) && L > 2 && tc_trans_supported(pl.p[L]))
+        pl.l2l_tiles = cached_op<float>(c, 6, pl.p[L], pl.p[L]);
     return pl;
 }
 
@@ -517,7 +509,7 @@ static int evaluate(Ctx* c, int64_t n, int nsys, const int64_t* sysoff, const ve
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, lv, c->gp_m2m, loc);
         }
         vfar = c->vfar.as<vec4_t<T>>();
         sfar = c->sfar.as<vec4_t<T>>();
@@ -572,11 +564,10 @@ static void ensure_scalar_ops(Ctx* c) {
     if constexpr (sizeof(T) == 4) {
         const int p = c->cfg.p;
         auto tiles = [&](TransKind kind, const float* fused, Buf& dst) {
-            if (ctx_use_tc(c) && tc_trans_supported(kind, p)) tc_trans_tiles(c, kind, fused, p, true, dst);
+            if (ctx_use_tc(c) && tc_trans_supported(p)) tc_trans_tiles(c, kind, fused, p, true, dst);
             else release(dst);
         };
         tiles(TRANS_M2L, c->ops.m2l.as<float>(), c->s_tiles);
-        tiles(TRANS_M2M, c->ops.m2m.as<float>(), c->s_m2m_tiles);
         tiles(TRANS_L2L, c->ops.l2l.as<float>(), c->s_l2l_tiles);
     }
     cuda_check(cudaStreamSynchronize(c->stream), "scalar tables");
@@ -632,10 +623,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
             pl.m2l_tiles[l] = c->s_tiles.ptr ? c->s_tiles.as<float>() : nullptr;
         }
         pl.qtab = c->ops.qtab.as<T>();
-        if (sizeof(T) == 4 && ctx_m2l_tc(c)) {
-            pl.m2m_tiles = c->s_m2m_tiles.as<float>();
-            pl.l2l_tiles = c->s_l2l_tiles.as<float>();
-        }
+        if (sizeof(T) == 4 && ctx_m2l_tc(c)) pl.l2l_tiles = c->s_l2l_tiles.as<float>();
         pl.l2p_sp = velocity_rows<T>(c, p);
         const int64_t nbt = lv.off[L + 1];
         ensure(c, c->mult, nbt * pl.ld * (int64_t)sizeof(T));
@@ -662,7 +650,7 @@ static int evaluate_scalar(Ctx* c, int64_t n, const vec4_t<T>* x4, const T* q, v
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, lv, c->gp_m2m, loc);
         }
         pgfar = c->pgfar.as<vec4_t<T>>();
         {
@@ -807,7 +795,7 @@ static int evaluate_filaments(Ctx* c, int nfil, const int64_t* offsets, const in
         }
         {
             StageScope sc(c, LHV_STAGE_L2L);
-            run_l2l<T>(c, pl, c->tb, lv, c->gp_m2m, c->gp_l2l, loc);
+            run_l2l<T>(c, pl, lv, c->gp_m2m, loc);
         }
         vfar = c->vfar.as<vec4_t<T>>();
         {
@@ -1345,7 +1333,7 @@ void lhv_destroy(lhv_ctx* ctx) {
     c.qtabs.clear();
     c.spcache.clear();
     for (auto* b : {&c.sel_W, &c.sel_b, &c.sel_X, &c.sel_Z, &c.sel_choice, &c.sel_idx, &c.sel_dv, &c.sel_ds, &c.sel_err,
-                    &c.s_m2l, &c.s_m2m, &c.s_l2l, &c.s_tiles, &c.s_m2m_tiles, &c.s_l2l_tiles, &c.qs, &c.pgfar, &c.psi_m2l, &c.psi_m2m,
+                    &c.s_m2l, &c.s_m2m, &c.s_l2l, &c.s_tiles, &c.s_l2l_tiles, &c.qs, &c.pgfar, &c.psi_m2l, &c.psi_m2m,
                     &c.psi_l2l, &c.psi_tiles, &c.f_off, &c.f_closed, &c.f_seg, &c.f_next, &c.f_segs, &c.f_nexts})
         lhv::release(*b);
     lhv::TreeBufs& t = c.tb;
@@ -1357,7 +1345,7 @@ void lhv_destroy(lhv_ctx* ctx) {
     lhv::Buf* rest[] = {&c.xs, &c.ws, &c.mult, &c.loc, &c.table, &c.vfar, &c.sfar, &c.counters, &c.hx, &c.hw,
                         &c.W};
     for (auto* b : rest) lhv::release(*b);
-    for (lhv::Grouped* g : {&c.gp_m2m, &c.gp_m2l, &c.gp_l2l}) {
+    for (lhv::Grouped* g : {&c.gp_m2m, &c.gp_m2l}) {
         lhv::Buf* gb[] = {&g->gcount, &g->goff, &g->gcursor, &g->choff, &g->chunks, &g->pairs, &g->tmp,
                           &g->scan_tmp, &g->work};
         for (auto* b : gb) lhv::release(*b);

@@ -638,31 +638,35 @@ void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
     launch_p2m_apply<T>(c, pl, tb, lv, W, mult);
 }
 
-// chunk width for the translations between levels: the MMA's on the tensor cores, else set by the
+// chunk width of the list of M2M and L2L: the MMA's where L2L may run on the tensor cores, else set by the
 // widest input
 template <typename T>
-static int oct_nc(const Plan<T>& pl, const float* tiles) {
-    if (tiles) return TC_PAIRS;
+static int oct_nc(const Plan<T>& pl) {
+    if (pl.l2l_tiles) return TC_PAIRS;
     int pmax = 1;
     for (int l = 2; l <= pl.L; ++l) pmax = std::max(pmax, pl.p[l]);
     return std::min(16, gemm_nc<T>(2 * pmax * pmax));  // levels hold few boxes: many short items
 }
 
-// One level of M2M or L2L on the tensor cores (LHV_TF32X3, one p a multiple of 4), true if it ran
-// there.  The grouped GEMM streams 250 KB of operator for every 16 boxes (p = 12), here one block T for
-// 128; M2M + L2L, ms: sphere surface of 2^20 2.74 -> 0.44, offset rings of 2^21 (p = 16) 1.13 -> 0.34,
-// 16 blob systems 0.61 -> 0.20 (with the lists of k_oct_list and the bulk additions).  A level of few boxes (b boxes with b p^4 up to OCT_TC_MIN) stays with the
-// grouped GEMM, which splits its sums over the idle SMs: about 12 us at p = 12, 17 at p = 16, where the
-// MMA's one pass over T and its epilogue take 29 and 36.  M2M + L2L of a filament's eleven levels 0.88 -> 0.71, of the
-// ring of 32,768 elements 0.23 -> 0.20, the others as before (twice the limit: offset rings 0.35 -> 0.37).
+// One level of L2L on the tensor cores (LHV_TF32X3, one p a multiple of 4), true if it ran there.  The
+// grouped GEMM streams 250 KB of operator for every 16 boxes (p = 12), here one block T for 128; L2L, ms: sphere
+// surface of 2^20 1.38 -> 0.19, offset rings of 2^21 (p = 16) 0.55 -> 0.15, 16 blob systems 0.26 -> 0.079, a
+// filament's eleven levels 0.75 -> 0.32, ring of 32,768 0.12 -> 0.084.  A level of few boxes (b boxes with b p^4
+// up to OCT_TC_MIN) stays with the grouped GEMM, which splits its sums over the idle SMs: about 12 us at p = 12, 17
+// at p = 16, where the MMA's one pass over T and its epilogue take 29 and 36.
+//
+// M2M stays with the grouped GEMM at every level.  Against the exact map of the same inputs the split products put
+// 1.06e-7 on a level's multipoles of a sphere surface (p = 8 to 16) where FP32 puts 5.1e-8 (scalar case 6.5e-8 and
+// 4.8e-8), whether or not the cross products of all K come first; L2L's locals come out nearer than FP32's,
+// 6.0e-8 against 0.6 to 1.2e-7.  On the tensor cores M2M of the sphere surface of 2^20 took 0.24 ms, here 1.50.
 constexpr int64_t OCT_TC_MIN = 16000000;
 template <typename T>
-static bool oct_tc(Ctx* c, const Plan<T>& pl, TransKind kind, const float* tiles, const Grouped& gp,
-                   const GemmArgs<T>& a) {
+static bool l2l_tc(Ctx* c, const Plan<T>& pl, const Grouped& gp, const GemmArgs<T>& a) {
     if constexpr (sizeof(T) == 4) {
         const int64_t P = pl.p[pl.L] * pl.p[pl.L];
-        if (tiles && a.pairs_hint * P * P > OCT_TC_MIN) {
-            run_tc_trans(c, kind, gp, a.g0, a.g1, pl.p[pl.L], pl.scalar, tiles, a.in, a.out, a.ldin, ctx_err_flag(c));
+        if (pl.l2l_tiles && a.pairs_hint * P * P > OCT_TC_MIN) {
+            run_tc_trans(c, TRANS_L2L, gp, a.g0, a.g1, pl.p[pl.L], pl.scalar, pl.l2l_tiles, a.in, a.out, a.ldin,
+                         ctx_err_flag(c));
             return true;
         }
     }
@@ -675,7 +679,7 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
     if (L < 3) return;
     // parents of the levels 2 .. L-1 accumulate atomically
     fill_level_rows<T>(c, lv, tb.counts.as<int>(), 2, L - 1, pl.ld, 0, mult, (T)0);
-    oct_list(c, tb, lv, gp, oct_nc(pl, pl.m2m_tiles));
+    oct_list(c, tb, lv, gp, oct_nc(pl));
     for (int l = L - 1; l >= 2; --l) {
         const int Pout = pl.p[l] * pl.p[l], Pin = pl.p[l + 1] * pl.p[l + 1];
         GemmArgs<T> a{};
@@ -695,19 +699,14 @@ void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Gr
         a.scale = (T)1;
         a.pairs_hint = lv.real[l + 1];
         a.between = BETWEEN_LEVELS;
-        if (!oct_tc(c, pl, TRANS_M2M, pl.m2m_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
+        run_group_gemm<T>(c, gp, a);
     }
 }
 
 template <typename T>
-void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const Grouped& up, Grouped& own, T* loc) {
+void run_l2l(Ctx* c, const Plan<T>& pl, const Levels& lv, const Grouped& gp, T* loc) {
     const int L = lv.L;
     if (L < 3) return;
-    // M2M's list serves with the pairs swapped, unless its chunks have another width (p > 16 on the
-    // tensor cores, which take L2L but not M2M there)
-    const int nc = oct_nc(pl, pl.l2l_tiles);
-    if (up.nc != nc) oct_list(c, tb, lv, own, nc);
-    const Grouped& gp = up.nc != nc ? own : up;
     for (int l = 2; l < L; ++l) {
         const int Pout = pl.p[l + 1] * pl.p[l + 1], Pin = pl.p[l] * pl.p[l];
         GemmArgs<T> a{};
@@ -727,7 +726,7 @@ void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
         a.scale = (T)1;
         a.pairs_hint = lv.real[l + 1];
         a.between = BETWEEN_LEVELS | BETWEEN_SWAPPED;
-        if (!oct_tc(c, pl, TRANS_L2L, pl.l2l_tiles, gp, a)) run_group_gemm<T>(c, gp, a);
+        if (!l2l_tc(c, pl, gp, a)) run_group_gemm<T>(c, gp, a);
     }
 }
 
@@ -793,7 +792,7 @@ void run_l2p_scalar(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels&
     template void run_p2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,            \
                              const vec4_t<T>*, T*, T*);                                                         \
     template void run_m2m<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, Grouped&, T*);              \
-    template void run_l2l<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const Grouped&, Grouped&, T*); \
+    template void run_l2l<T>(Ctx*, const Plan<T>&, const Levels&, const Grouped&, T*);                          \
     template void run_l2p<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,            \
                              const vec4_t<T>*, const T*, vec4_t<T>*, vec4_t<T>*);                      \
     template void run_p2m_scalar<T>(Ctx*, const Plan<T>&, const TreeBufs&, const Levels&, const vec4_t<T>*,     \

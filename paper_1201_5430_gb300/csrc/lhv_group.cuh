@@ -106,11 +106,11 @@ void run_tc_gemm(Ctx* c, Grouped& gp, GemmArgs<float> a, const float* tiles, con
                  const float* in_lo, int* err);
 
 // Tensor-core translations of the two-potential and scalar forms (tc_m2l.cu), one p a multiple of
-// 4.  tc_trans_tiles lays out the translation blocks of the fused tables (316 of M2L, 8 of M2M or
-// L2L) and the conversion's tables; run_tc_trans adds the translated (and, unless scalar,
+// 4.  tc_trans_tiles lays out the translation blocks of the fused tables (316 of M2L, 8 of L2L)
+// and the conversion's tables; run_tc_trans adds the translated (and, unless scalar,
 // converted) rows of the groups [g0, g1) to out (L2L: of the pairs (child, parent) of M2M).
-enum TransKind : int { TRANS_M2L = 0, TRANS_M2M = 1, TRANS_L2L = 2 };
-bool tc_trans_supported(TransKind kind, int p);
+enum TransKind : int { TRANS_M2L = 0, TRANS_L2L = 1 };
+bool tc_trans_supported(int p);
 void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scalar, Buf& tiles);
 void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int p, bool scalar, const float* tiles,
                   const float* in, float* out, int64_t ld, int* err);

@@ -193,8 +193,8 @@ struct OpTables {
     Buf m2l;                   // [316][2P][2P] fused (S|R) + Eq. drt10 per offset slot (built when a route needs it)
     Buf m2m;                   // [8][2P][2P]   fused (S|S) + Eq. drt11 per child octant
     Buf l2l;                   // [8][2P][2P]   fused (R|R) + Eq. drt10 per child octant
-    // TF32 hi/lo tiles of the translation blocks of the three tables (LHV_TF32X3, tc_m2l.cu)
-    Buf m2l_tiles, m2m_tiles, l2l_tiles;
+    // TF32 hi/lo tiles of the translation blocks of M2L and L2L (LHV_TF32X3, tc_m2l.cu)
+    Buf m2l_tiles, l2l_tiles;
     // sparse maps (structural zeros dropped): P2M 3P -> 2P (Eq. eve4 for w = i_x, i_y, i_z), L2P
     // 2P -> 12P (v_k of Eq. evf3, u_lk of Eq. dt3), and the 3P rows v_k of it alone (built on first use)
     Sell p2m_sp, l2p_sp, l2pv_sp;
@@ -245,8 +245,7 @@ struct Plan {
     const T* l2l[MAX_LEVELS + 1] = {};     // [l]: level l-1 -> l, 8 x [2P(l-1)][2P(l)]
     const T* m2l[MAX_LEVELS + 1] = {};     // [l]: 316 x [2P(l)][2P(l)]
     const float* m2l_tiles[MAX_LEVELS + 1] = {};  // tensor-core tiles of m2l[l] (LHV_TF32X3), or null
-    const float* m2m_tiles = nullptr;      // tensor-core tiles of m2m / l2l (LHV_TF32X3, one p), or null
-    const float* l2l_tiles = nullptr;
+    const float* l2l_tiles = nullptr;      // tensor-core tiles of l2l (LHV_TF32X3, one p), or null
     const T* qtab = nullptr;               // recurrence coefficients of the harmonics for p[L]
     SellView<T> p2m_sp, l2p_sp;            // P2M(p[L]), L2P(p[L]) (v_k alone: filaments, scalar case)
     bool uniform = true;                   // p[l] equal over l = 2..L
@@ -271,9 +270,9 @@ void run_p2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, co
 // M2M for all levels L-1 .. 2 (mult of the levels < L is overwritten).
 template <typename T>
 void run_m2m(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, Grouped& gp, T* mult);
-// L2L for all levels 2 -> 3 .. L-1 -> L (adds into loc).
+// L2L for all levels 2 -> 3 .. L-1 -> L (adds into loc); gp: the list of run_m2m.
 template <typename T>
-void run_l2l(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const Grouped& up, Grouped& own, T* loc);
+void run_l2l(Ctx* c, const Plan<T>& pl, const Levels& lv, const Grouped& gp, T* loc);
 // L2P at the leaves (sfar null: v alone, with the v_k rows of the map in pl.l2p_sp).
 template <typename T>
 void run_l2p(Ctx* c, const Plan<T>& pl, const TreeBufs& tb, const Levels& lv, const vec4_t<T>* xs,

@@ -414,7 +414,7 @@ int m2l_slot_host(int dx, int dy, int dz) {
 
 void free_operators(OpTables& ops) {
     Buf* all[] = {&ops.m2l, &ops.m2m, &ops.l2l, &ops.qtab, &ops.offsets, &ops.slot_of, &ops.m2l_tiles,
-                  &ops.m2m_tiles, &ops.l2l_tiles};
+                  &ops.l2l_tiles};
     for (Buf* b : all) {
         if (b->ptr) cudaFree(b->ptr);
         b->ptr = nullptr;

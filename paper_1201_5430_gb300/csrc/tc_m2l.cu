@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05, TF32) translations: M2L, and M2M and L2L with the same kernel.
+// Tensor-core (tcgen05, TF32) translations: M2L, and L2L with the same kernel.
 //
 // The fused operator of a translation t is [[T, C12 T], [0, C22 T]] (Eqs. mr3, drt10, drt11): the
 // same translation T for both potentials, then the conversion, which couples each (n, m) to
@@ -14,11 +14,8 @@
 //   f = -sqrt((n+1-m)(n+1+m)) / (n+1)   (d = e = f = 0 at n = p - 1: the chi_p term is dropped);
 //   at m = 0 the m - 1 terms are the conjugates of the m + 1 terms: a and e doubled, b = d = 0.
 // L2L converts in the same (R) basis; its T block carries the change of scale from the parent's
-// box to the child's of phi, and chi takes half of it (one length more, Eq. 4).  M2M converts in
-// the S basis (Eq. drt11), chi~ from the degree below:
-//   a = -sqrt((n-m)(n+m+1)) / 2(n+1),  b = sqrt((n+m)(n-m+1)) / 2(n+1),  z = -m / (n+1),
-//   d = -sqrt((n+m)(n+m-1)) / 2n,  e = sqrt((n-m)(n-m-1)) / 2n,  f = sqrt((n-m)(n+m)) / n  (0 at n = 0),
-// and chi takes twice the T block's scale of phi.
+// box to the child's of phi, and chi takes half of it (one length more, Eq. 4).  M2M is not taken here: its
+// error would be larger than in FP32 (run_l2l's rule in expansions.cu).
 // The scalar reference case is the same kernel with one potential and no conversion.
 //
 // D (128 pairs x N) = X (128 x P) T^T (P x N) per potential, D in TMEM in FP32 (phi^ and chi^
@@ -94,7 +91,7 @@ struct M2lArgs {
     int nbuf;                // accumulator buffers (each M2_TMEM / nbuf columns)
     const float* conv;       // [p (p + 1) / 2 + 8][8]: a, b, z, d | e, f, 0, 0 of (n, m) at n (n + 1) / 2 + m
     const float* tvec;       // [ngroups][4]: t of each operator, in box sides of the conversion's basis
-    float chi_scale;         // chi^ = chi_scale T chi (1; L2L 1/2, M2M 2)
+    float chi_scale;         // chi^ = chi_scale T chi (1; L2L 1/2)
     int ngroups;             // operators (a group's is g % ngroups)
     int* err;
     int64_t wait_limit;      // polls after which a wait gives up
@@ -206,9 +203,6 @@ __device__ __forceinline__ void order_zero(uint32_t (&x)[N]) {
     x[3] = 0u;
 }
 
-// What the epilogue does with the translated potentials.
-enum TransMode : int { TM_SCALAR = 0, TM_R = 1, TM_S = 2 };  // one potential; Eq. drt10; Eq. drt11
-
 // (Re, Im) of the orders M .. M + 3 (M a multiple of 4) of degree n to d[0 .. 8), d = the column of Re of
 // order M.  Orders past n are not stored, and order 0 is the one real v[1].  An odd degree's
 // orders start on a quad (n^2 - 1 = 0 mod 4), whose first column belongs to the degree below where M = 0;
@@ -239,17 +233,15 @@ __device__ __forceinline__ void store_orders(float* d, const float (&v)[8], int 
 }
 
 // Converts the orders [mb, mb + 8) of degree n of this thread's pair and writes them to the
-// staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n (R basis; S basis:
-// n - 1) as read by tmem_orders with order_zero applied; on return that of the next degree, so
+// staging columns op (phi) and oc (chi), column n^2 at op[0].  x: chi of degree n as
+// read by tmem_orders with order_zero applied; on return that of the next degree, so
 // that a run of degrees reads each once.
-template <int MODE>
 __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uint32_t tc, int c0, int p, int n,
                                                int mb, float tx, float ty, float tz, float cs, uint32_t (&x)[20],
                                                float* op, float* oc) {
     uint32_t y[20], f[16];
-    const int nx = MODE == TM_R ? n + 1 : n;  // the degree read here
-    const bool up = nx < p;
-    if (up) tmem_orders(tc + (uint32_t)(nx * nx - c0 + 2 * mb - 3), nx, mb, y);
+    const bool up = n + 1 < p;
+    if (up) tmem_orders(tc + (uint32_t)((n + 1) * (n + 1) - c0 + 2 * mb - 3), n + 1, mb, y);
     if (n > 0) tmem_ld16_async(tp + (uint32_t)(n * n - c0 + 2 * mb - 1), f);
     else tmem_ld1(tp - (uint32_t)c0, f[1]);
     tmem_wait(f);
@@ -276,12 +268,10 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
             const float ax = g.x * tx, ay = g.x * ty, bx = g.y * tx, by = g.y * ty, z = g.z * tz;
             const float dx = g.w * tx, dy = g.w * ty, ex = e.x * tx, ey = e.x * ty, fz = e.y * tz;
             auto F = [](uint32_t u) { return __uint_as_float(u); };
-            const uint32_t* u = MODE == TM_R ? x : y;  // degree n
-            const uint32_t* w = MODE == TM_R ? y : x;  // degree n + 1 (R), n - 1 (S)
-            const float mr = F(u[2 * i]), mi = F(u[2 * i + 1]), cr = F(u[2 * i + 2]), ci = F(u[2 * i + 3]);
-            const float pr = m < n ? F(u[2 * i + 4]) : 0.f, pi = m < n ? F(u[2 * i + 5]) : 0.f;
-            const float umr = F(w[2 * i]), umi = F(w[2 * i + 1]), ucr = F(w[2 * i + 2]), uci = F(w[2 * i + 3]),
-                        upr = F(w[2 * i + 4]), upi = F(w[2 * i + 5]);
+            const float mr = F(x[2 * i]), mi = F(x[2 * i + 1]), cr = F(x[2 * i + 2]), ci = F(x[2 * i + 3]);
+            const float pr = m < n ? F(x[2 * i + 4]) : 0.f, pi = m < n ? F(x[2 * i + 5]) : 0.f;
+            const float umr = F(y[2 * i]), umi = F(y[2 * i + 1]), ucr = F(y[2 * i + 2]), uci = F(y[2 * i + 3]),
+                        upr = F(y[2 * i + 4]), upi = F(y[2 * i + 5]);  // degree n + 1
             const float o0 = fmaf(ax, pr, fmaf(-ay, pi, fmaf(bx, mr, fmaf(by, mi, fmaf(-z, ci, F(f[2 * i]))))));
             const float q0 = fmaf(ey, upr, fmaf(ex, upi, fmaf(dy, umr, fmaf(-dx, umi, fmaf(fz, ucr, cs * cr)))));
             const float o1 = fmaf(ax, pi, fmaf(ay, pr, fmaf(bx, mi, fmaf(-by, mr, fmaf(z, cr, F(f[2 * i + 1]))))));
@@ -299,9 +289,9 @@ __device__ __forceinline__ void convert_orders(const float* cv, uint32_t tp, uin
     for (int k = 0; k < 20; ++k) x[k] = y[k];
 }
 
-template <int MODE>
+// NPOT: two potentials, converted in the epilogue, or the one of the scalar case
+template <int NPOT>
 __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant__ M2lArgs a) {
-    constexpr int NPOT = MODE == TM_SCALAR ? 1 : 2;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ M2lShared sh;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -577,18 +567,12 @@ __global__ void __launch_bounds__(M2_THREADS, 1) k_tc_m2l(const __grid_constant_
                         }
                         if (d0 >= d1) continue;
                         uint32_t x[20];
-                        const int dx = MODE == TM_R ? d0 : d0 - 1;
-                        if (dx >= 0) {
-                            tmem_orders(tc + (uint32_t)(dx * dx - c0 + 2 * mb - 3), dx, mb, x);
-                            tmem_wait(x);
-                            if (mb == 0) order_zero(x);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 20; ++k) x[k] = 0u;
-                        }
+                        tmem_orders(tc + (uint32_t)(d0 * d0 - c0 + 2 * mb - 3), d0, mb, x);
+                        tmem_wait(x);
+                        if (mb == 0) order_zero(x);
                         for (int dn = d0; dn < d1; ++dn) {
                             const int at = dn * dn - s0;
-                            convert_orders<MODE>(conv, tp, tc, c0, a.p, dn, mb, tv.x, tv.y, tv.z, a.chi_scale, x,
+                            convert_orders(conv, tp, tc, c0, a.p, dn, mb, tv.x, tv.y, tv.z, a.chi_scale, x,
                                                  st_p + at, st_c + at);
                         }
                     }
@@ -698,11 +682,7 @@ M2lArgs m2l_layout(int p, int npot, int ngroups) {
 
 }  // namespace
 
-bool tc_trans_supported(TransKind kind, int p) {
-    // above p = 16 the accumulators are split into ranges of degrees whose halo is the degree above;
-    // M2M's conversion reads the degree below
-    return p % 4 == 0 && p >= 4 && p <= (kind == TRANS_M2M ? 16 : 24);
-}
+bool tc_trans_supported(int p) { return p % 4 == 0 && p >= 4 && p <= 24; }
 
 void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scalar, Buf& tiles) {
     const int ng = kind == TRANS_M2L ? NUM_OFFSETS : 8;
@@ -715,19 +695,12 @@ void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scal
         for (int m = 0; m <= n; ++m) {
             float* v = &tab[(size_t)(n * (n + 1) / 2 + m) * 8];
             const double two = m ? 1.0 : 2.0, one = m ? 1.0 : 0.0;
-            const double den = kind == TRANS_M2M ? n + 1.0 : (double)n;
-            if (den > 0.0) {
-                v[0] = (float)(-two * in_chi * std::sqrt((double)(n - m) * (n + m + 1)) / (2.0 * den));
-                v[1] = (float)(one * in_chi * std::sqrt((double)(n + m) * (n - m + 1)) / (2.0 * den));
-                v[2] = (float)((kind == TRANS_M2M ? -1.0 : 1.0) * in_chi * m / den);
+            if (n > 0) {
+                v[0] = (float)(-two * in_chi * std::sqrt((double)(n - m) * (n + m + 1)) / (2.0 * n));
+                v[1] = (float)(one * in_chi * std::sqrt((double)(n + m) * (n - m + 1)) / (2.0 * n));
+                v[2] = (float)(in_chi * m / n);
             }
-            if (kind == TRANS_M2M) {
-                if (n > 0) {
-                    v[3] = (float)(-one * std::sqrt((double)(n + m) * (n + m - 1)) / (2.0 * n));
-                    v[4] = (float)(two * std::sqrt((double)(n - m) * std::max(n - m - 1, 0)) / (2.0 * n));
-                    v[5] = (float)(std::sqrt((double)(n - m) * (n + m)) / n);
-                }
-            } else if (n + 1 < p) {
+            if (n + 1 < p) {
                 v[3] = (float)(one * in_chi * std::sqrt((double)(n - m + 1) * (n - m + 2)) / (2.0 * (n + 1)));
                 v[4] = (float)(-two * in_chi * std::sqrt((double)(n + m + 1) * (n + m + 2)) / (2.0 * (n + 1)));
                 v[5] = (float)(-in_chi * std::sqrt((double)(n + 1 - m) * (n + 1 + m)) / (n + 1));
@@ -737,9 +710,9 @@ void tc_trans_tiles(Ctx* c, TransKind kind, const float* fused, int p, bool scal
     m2l_offsets(offs, slot_of);
     for (int g = 0; g < ng; ++g)
         for (int k = 0; k < 4; ++k) {
-            // M2L: t = target - source = -offset; child octant o: t = 0.5 - o (M2M), o - 0.5 (L2L), in child sides
+            // M2L: t = target - source = -offset; L2L of child octant o: o - 0.5, in child sides
             const float o = (float)((g >> k) & 1);
-            tab.push_back(k == 3 ? 0.f : kind == TRANS_M2L ? (float)-offs[3 * g + k] : kind == TRANS_M2M ? 0.5f - o : o - 0.5f);
+            tab.push_back(k == 3 ? 0.f : kind == TRANS_M2L ? (float)-offs[3 * g + k] : o - 0.5f);
         }
     ensure(c, tiles, (nt + (int64_t)tab.size()) * (int64_t)sizeof(float));
     k_m2l_tiles<<<ng, 256, 0, stream_of(c)>>>(fused, 4 * (int64_t)a.P * a.P, 2 * a.P, a, tiles.as<float>());
@@ -766,13 +739,13 @@ void run_tc_trans(Ctx* c, TransKind kind, const Grouped& gp, int g0, int g1, int
     a.tiles = tiles;
     a.conv = tiles + a.group_stride * a.ngroups;
     a.tvec = a.conv + conv_floats(p);
-    a.chi_scale = kind == TRANS_M2L ? 1.0f : kind == TRANS_L2L ? 0.5f : 2.0f;
+    a.chi_scale = kind == TRANS_M2L ? 1.0f : 0.5f;
     a.err = err;
     a.wait_limit = ctx_wait_limit(c);
     // above half an SM's shared memory: one CTA (and its 512 TMEM columns) per SM
     const size_t smem =
         std::max<size_t>((size_t)a.nstages * a.stage_bytes + m2l_fixed_smem(p, scalar ? 1 : 2), 120 * 1024);
-    auto kernel = scalar ? k_tc_m2l<TM_SCALAR> : kind == TRANS_M2M ? k_tc_m2l<TM_S> : k_tc_m2l<TM_R>;
+    auto kernel = scalar ? k_tc_m2l<1> : k_tc_m2l<2>;
     cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "translation smem");
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);

@@ -170,3 +170,27 @@ def test_waits_that_give_up_end_the_translations(scalar):
     for bad in (-1, (1 << 24) + 1):
         assert ctx.lib.lhv_set_wait_limit(ctx.h, bad) == _lib.LHV_EINVAL
     ctx.close()
+
+
+@pytest.mark.parametrize("p", [8, 12, 16])
+def test_multipoles_are_as_exact_as_in_fp32(p):
+    """M2M of a TF32x3 context runs in FP32: the multipoles of every level with a thousand boxes below it are no
+    further from the FP64 context's than the FP32 context's.  Both add the same products in another order; the
+    norm of 1000 x 2 p^2 rounding errors scatters by about a percent, and ten are allowed."""
+    from paper_1201_5430_gb300 import LHV
+    x = np.random.default_rng(6).standard_normal((100003, 3))
+    x = (x / np.linalg.norm(x, axis=1)[:, None]).astype(np.float32)
+    w = np.random.default_rng(7).standard_normal((100003, 3)).astype(np.float32)
+    got = {}
+    for prec in ("tf32x3", "fp32", "fp64"):
+        ctx = LHV(p=p, leaf_max=32, core_a=0.0, precision=prec, terms="far")
+        e = "fp64" if prec == "fp64" else "fp32"
+        ctx.evaluate_velocity_stretching(dev(x, e), dev(w, e))
+        st = ctx.stats()
+        L = st["leaf_level"]
+        levels = [l for l in range(2, L) if st["nbox"][l + 1] >= 1000]
+        got[prec] = [ctx.export("multipole", l).double().cpu().numpy() for l in levels]
+        ctx.close()
+    assert len(levels) >= 2
+    for a, b, c in zip(got["tf32x3"], got["fp32"], got["fp64"]):
+        assert np.linalg.norm(a - c) <= 1.1 * np.linalg.norm(b - c), (rel(a, c), rel(b, c))
