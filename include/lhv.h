@@ -403,8 +403,8 @@ int lhv_export(lhv_ctx* ctx, int what, int level, void* dst, int64_t capacity_by
  * one without core radius and level cap (21 bits per axis, stable order of
  * equal keys).  Work is enqueued on cuda_stream (a cudaStream_t,
  * NULL = legacy default stream); the call returns after that stream has
- * finished it (one device-to-host read of the non-finite flag).  The only
- * scratch state that must start at zero (the non-finite flag) is cleared by the
+ * finished it (one device-to-host read of the non-finite flag).  The scratch
+ * state that must start at zero (the non-finite flag, a block counter) is cleared by the
  * call's first kernel.  Returns LHV_ETOOBIG for n > LHV_NOALLOC_MAX_N,
  * LHV_EINVAL for n < 0, null or misaligned pointers, LHV_ENONFINITE for NaN/Inf,
  * LHV_ECUDA if a CUDA call failed, LHV_OK for n = 0 (nothing done).  A CUDA

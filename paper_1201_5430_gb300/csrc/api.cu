@@ -333,14 +333,13 @@ static void ensure_psi_ops(Ctx* c) {
 // rotation, O(p^3) a pair, instead of the fused tables, O(p^4), on the CUDA cores: always where its
 // tables fit, unless a chunk of the fused-table GEMM was asked for (lhv_set_launch_shape) or the
 // tensor cores run the products.  The far field's error against FP64 is that of the fused tables or
-// smaller (sphere surface, p = 12: v 3.1e-7 against 3.6e-7).  Products of a cube of 100,003 elements
-// (640,584 pairs), RCR against the fused tables, ms: FP32 p = 4 0.24 / 0.32, p = 8 0.62 / 1.13, p = 12
-// 1.48 / 5.76, p = 16 2.94 / 20.9, p = 20 6.34 / 62.6; FP64 (32,768 elements, 640,206 pairs) p = 4
-// 1.29 / 3.72, p = 8 6.80 / 14.3, p = 12 21.5 / 92.9, p = 16 44.3 / 216.  (Before the
-// 16-byte gathers and the FP64 tiles of rcr.cu: p = 12 now 1.19 in FP32, and in FP64 4 / 7 of its time.)  Below
-// p = 4 the tables were not compared.  Above p = 16 RCR stays with lhv_set_form: a schedule of several p (the learned form picks 18 to
-// 20 for eps = 1e-6 in FP32) has the fused tables alone, and there it is measured against a uniform p
-// of the same products (cube of 2^18: 38 ms against 49 at p = 18, 6.8 by RCR).
+// smaller (sphere surface, p = 12: v 3.1e-7 against 3.6e-7); in FP64 the two differ by 0.7e-15 (p = 4) to 1.6e-15
+// (p = 16) of v.  Products of a cube, RCR against the fused tables, ms: FP32, 100,003 elements (640,584 pairs),
+// p = 4 0.26 / 0.32, p = 8 0.57 / 1.13, p = 12 1.19 / 5.76, p = 16 2.58 / 20.9, p = 20 5.35 / 62.5; FP64, 32,768
+// elements (2,755,324 pairs), p = 4 3.27 / 15.6, p = 8 17.0 / 60.0, p = 12 52.6 / 393, p = 16 134 / 941.  Below
+// p = 4 the two were not timed.  Above p = 16 RCR would be the faster too, but stays with lhv_set_form: a schedule of
+// several p (the learned form picks 18 to 20 for eps = 1e-6 in FP32) has the fused tables alone, and is
+// compared with a uniform p of the same products (cube of 2^18: 38 ms against 49 at p = 18, 6.8 by RCR).
 constexpr int RCR_MIN_P = 4, RCR_MAX_P = 16;
 template <typename T>
 static bool default_rcr(Ctx* c) {

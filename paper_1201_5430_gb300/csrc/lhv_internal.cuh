@@ -315,7 +315,6 @@ void m2l_apply(Ctx* c, const Plan<T>& pl, const Levels& lv, const int* count, Gr
 constexpr int RCR_PMAX = 20;
 struct RcrTables {
     int p = 0;
-    int type = 0;         // sizeof(T) of the tables
     int nc = 0;           // box pairs per chunk of the grouped pair list
     int slot_floats = 0;  // reals of one offset slot's rotation tables [Y fwd | Y back | Z fwd | Z back]
     int coax_floats = 0;  // reals of one distance's coaxial blocks and conversion coefficients

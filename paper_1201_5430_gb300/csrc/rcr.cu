@@ -958,7 +958,6 @@ void rcr_build(Ctx* c, int p, RcrTables& rt) {
         throw Error{LHV_EUNSUPPORTED, "RCR tables failed their structural check"};
     }
     rt.p = p;
-    rt.type = (int)sizeof(T);
     rt.slot_floats = sf;
     rt.coax_floats = cf;
     rt.resid = resid;
