@@ -38,9 +38,10 @@
 // Measured (products, ms an evaluation, fused-table kernel before / this one with the additions by
 // atomicAdd / by bulk reductions): sphere surface of 2^20 at p = 12, 4.13 M pairs 7.26 / 4.56 / 4.24; scalar
 // cube of 2^20 at p = 12, 6.04 M pairs 4.01 / 2.28 / 1.96; offset rings of 2^21 at p = 16, 1.33 M
-// pairs 4.33 / 2.54 / 2.32.  Without the epilogue the first takes 1.97: what bounds it is the
-// conversion (tcgen05.ld and its latency), which runs in turn with the products where one accumulator
-// set fills TMEM.  Operand traffic a pair at p = 12: 1.15 KB of source (split here instead of two
+// pairs 4.33 / 2.54 / 2.32.  Without the epilogue the first takes 1.97: the conversion runs in turn with
+// the products where one accumulator set fills TMEM.  No unit is near its rate (sphere surface of 2^19, 3.81 M
+// pairs, ncu): tensor pipe 20 %, issue slots 42 %, L1 and shared memory 45 %, ALU 31 %, FMA 18 %; of the stalls the
+// long scoreboard (the gathers and the reads of TMEM) leads with 5.8 warps an issue.  Operand traffic a pair at p = 12: 1.15 KB of source (split here instead of two
 // arrays) and 1.3 KB of operator, against 3.5 and 3.9 of the fused tables.
 //
 // Every mbarrier wait gives up after a fixed number of polls, sets the error word for the host
